@@ -273,7 +273,6 @@ void enqueue_step(lbe_ctx *c)
         launch_integrate(L, c->P, c->d.particle_mode, s);
         if (c->d.particle_mode != LBE_PARTICLES_STATIC) {
             uint32_t *oo = c->owner[c->ocur], *on = c->owner[1 - c->ocur];
-            launch_geom(L, c->P, s);
             launch_claim(L, c->P, 0, on, s);
             launch_transition(st, L, c->P, fout, c->type, oo, on, 0, s);
             launch_reset(L, c->P, 1, oo, s);
@@ -774,8 +773,10 @@ int32_t lbe_kernels_per_step(const lbe_ctx *c)
     else
         k = 1 + (c->np > 0 ? 2 : 0) + (c->d.walls_z ? 1 : 0);
     if (c->np > 0) {
-        k += 6;  // links, pair cells (count, prefix, fill), pairs, integrate
-        if (c->d.particle_mode != LBE_PARTICLES_STATIC) k += 4;  // geometry, claim, transition, reset
+        // links, pairs, the update (with the geometry of the new coverage);
+        // from pairs_by_cells on the cell list (count, prefix, fill)
+        k += 3 + (pairs_by_cells(c->np) ? 3 : 0);
+        if (c->d.particle_mode != LBE_PARTICLES_STATIC) k += 3;  // claim, transition, reset
     }
     return k;
 }

@@ -465,8 +465,13 @@ void launch_links(int storage, const Lat &L, const Parts &P, void *fnew, const f
 void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
                  const Parts &P, void *fout, cudaStream_t s);
 void launch_pairs(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, cudaStream_t s);
+// Whether the pair forces of np particles take the cell list (three more
+// kernels) or a loop over all partners.
+bool pairs_by_cells(int np);
+// The update of the particles and, unless they are static, the geometry of
+// their new coverage.
 void launch_integrate(const Lat &L, const Parts &P, int mode, cudaStream_t s);
-// Coverage geometry of the particles (old and current), once per update;
+// Coverage geometry of particles just placed (old = current);
 // geom_bytes_per_particle() is the size of one particle's record.
 void launch_geom(const Lat &L, const Parts &P, cudaStream_t s);
 size_t geom_bytes_per_particle();

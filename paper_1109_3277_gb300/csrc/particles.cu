@@ -46,7 +46,9 @@ __device__ __forceinline__ double node_disp(const Lat &L, int k, int xi, double 
 {
     if (periodic_dim(L, k)) {
         int n = ext_of(L, k);
-        double s = rint(__ddiv_rn(s_((double)xi, X), (double)n));
+        const double d = s_((double)xi, X);
+        if (fabs(d) < 0.49 * n) return d;  // no shift: the same value without the division
+        double s = rint(__ddiv_rn(d, (double)n));
         return s_((double)((long long)xi - (long long)s * n), X);
     }
     return s_((double)xi, X);
@@ -57,6 +59,7 @@ __device__ __forceinline__ double pair_disp(const Lat &L, int k, double a, doubl
     double r = s_(b, a);
     if (periodic_dim(L, k)) {
         double n = (double)ext_of(L, k);
+        if (fabs(r) < 0.49 * n) return r;  // no shift: the same value without the division
         r = s_(r, m_(n, rint(__ddiv_rn(r, n))));
     }
     return r;
@@ -329,6 +332,7 @@ __device__ __forceinline__ void for_candidates(const Box &b, const Geo &g, const
 struct PGeom {
     Geo g;
     double X[3];
+    double lo[3], hi[3];  // the box as box_of gives it, before finish_box
     int Xi[3];
     float Xf[3];
     Box box;
@@ -343,49 +347,179 @@ struct PGeom2 {
     Box uni;
 };
 
-__device__ void pgeom_of(const Lat &L, const double *X, const double *q, double rp, double ro, PGeom &o)
+// ---- four lanes per particle ------------------------------------------------
+// The Newton-Euler update and the geometry are chains of FP64 operations,
+// and this part issues a warp's FP64 instruction over many cycles whether
+// one lane or 32 are active: what counts is the number of warp
+// instructions.  Four neighbouring lanes therefore share a particle: lane k
+// = 0..2 carries axis k of every vector and lane l = 0..3 component l of
+// the quaternion, so the three (four) like operations of a vector
+// (quaternion) are one instruction.  Every operation and its order are those
+// of the scalar formulas.  With one thread per particle the update and the
+// geometry took 19 + 23 us for a single particle and 39 + 45 us for 25,033;
+// as one kernel of quads 15 and 58 us.
+__device__ __forceinline__ double quad(double v, int l) { return __shfl_sync(0xffffffffu, v, l, 4); }
+
+// A vector given around axis k (its components k, k+1, k+2 cyclically) in
+// the order 0, 1, 2.
+__device__ __forceinline__ void order3(int k, double d, double n, double p, double o[3])
 {
-    geo_of(q, rp, ro, o.g);
-    double lo[3], hi[3];
-    box_of(L, X, o.g.R, rp, ro, lo, hi);
-    finish_box(L, lo, hi, o.box);
-    for (int k = 0; k < 3; k++) {
-        o.X[k] = X[k];
-        // X = Xi + Xf, Xi integral: the FP32 displacement (u - Xi) - Xf
-        // carries no large cancellation (box_of bounds |X| < 1e9)
-        const double fl = floor(X[k]);
-        o.Xi[k] = o.box.count ? (int)fl : 0;
-        o.Xf[k] = (float)(X[k] - fl);
+    o[0] = k == 0 ? d : (k == 1 ? p : n);
+    o[1] = k == 0 ? n : (k == 1 ? d : p);
+    o[2] = k == 0 ? p : (k == 1 ? n : d);
+}
+
+// Row and column k of the rotation matrix of q (rotmat's operations).
+__device__ __forceinline__ void quad_rot(int k, const double q[4], double row[3], double col[3])
+{
+    const double w = q[0];
+    const double a = k == 0 ? q[1] : (k == 1 ? q[2] : q[3]);
+    const double b = k == 0 ? q[2] : (k == 1 ? q[3] : q[1]);
+    const double c = k == 0 ? q[3] : (k == 1 ? q[1] : q[2]);
+    const double d = s_(1.0, m_(2.0, a_(m_(b, b), m_(c, c))));
+    const double ab = m_(a, b), ac = m_(a, c), wc = m_(w, c), wb = m_(w, b);
+    order3(k, d, m_(2.0, s_(ab, wc)), m_(2.0, a_(ac, wb)), row);
+    order3(k, d, m_(2.0, a_(ab, wc)), m_(2.0, s_(ac, wb)), col);
+}
+
+// Axis k of box_of for centre X and half-extent h.
+__device__ __forceinline__ void box_axis(double X, double h, double &lo, double &hi)
+{
+    lo = floor(X - h) - 1.0;
+    hi = ceil(X + h) + 1.0;
+    if (!(lo <= hi) || !(fabs(X) < 1e9) || !(h < 1e9)) {
+        lo = 1.0;
+        hi = 0.0;
     }
 }
 
-__device__ __forceinline__ void geom_body(const Lat &L, const Parts &P, int p)
+// Whether the box whose axis k this lane holds is empty on any axis.
+__device__ __forceinline__ bool quad_empty(double lo, double hi)
 {
-    PGeom2 &G = reinterpret_cast<PGeom2 *>(P.geo)[p];
-    pgeom_of(L, P.Xold + 3 * p, P.qold + 4 * p, P.rp[p], P.ro[p], G.old_);
-    pgeom_of(L, P.X + 3 * p, P.q + 4 * p, P.rp[p], P.ro[p], G.now);
-    double lo[3], hi[3], lo2[3], hi2[3];
-    for (int k = 0; k < 3; k++) G.Xu[k] = P.Xold[3 * p + k] + pair_disp(L, k, P.Xold[3 * p + k], P.X[3 * p + k]);
-    box_of(L, P.Xold + 3 * p, G.old_.g.R, P.rp[p], P.ro[p], lo, hi);
-    box_of(L, G.Xu, G.now.g.R, P.rp[p], P.ro[p], lo2, hi2);
-    if (box_empty(lo, hi)) {
-        for (int k = 0; k < 3; k++) {
-            lo[k] = lo2[k];
-            hi[k] = hi2[k];
-        }
-    } else if (!box_empty(lo2, hi2)) {
-        for (int k = 0; k < 3; k++) {
-            lo[k] = fmin(lo[k], lo2[k]);
-            hi[k] = fmax(hi[k], hi2[k]);
-        }
+    const unsigned bad = __ballot_sync(0xffffffffu, !(lo <= hi));
+    return ((bad >> (threadIdx.x & 28)) & 7u) != 0;
+}
+
+// finish_box for axis k (lanes 0..2 of a quad write their axis, lane 0 the
+// count).
+__device__ __forceinline__ int quad_box(const Lat &L, int k, bool wr, bool empty, double lo, double hi, Box &b)
+{
+    const double n = (double)ext_of(L, k);
+    int fullp = 0;
+    if (empty) {
+        lo = 0.0;
+        hi = -1.0;
+    } else if (!periodic_dim(L, k)) {
+        lo = fmax(lo, 0.0);
+        hi = fmin(hi, n - 1.0);
+    } else if (hi - lo + 1.0 > n) {
+        lo = 0.0;
+        hi = n - 1.0;
+        fullp = 1;
     }
-    finish_box(L, lo, hi, G.uni);
+    const int ext = hi >= lo ? (int)(hi - lo + 1.0) : 0;
+    const int count = __shfl_sync(0xffffffffu, ext, 0, 4) * __shfl_sync(0xffffffffu, ext, 1, 4) *
+                      __shfl_sync(0xffffffffu, ext, 2, 4);
+    if (wr) {
+        b.lo[k] = hi >= lo ? (int)lo : 0;
+        b.ext[k] = ext;
+        b.full[k] = fullp;
+        if (k == 0) b.count = count;
+    }
+    return count;
+}
+
+// Geometry of particle p after an update: the last geometry becomes the old
+// one and the new one is formed from this lane's X (axis k) and q.  first:
+// placement, the old geometry is the new one.  Called by whole warps; act:
+// the quad has a particle.
+__device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, bool act, bool first, double X,
+                                          double Xold, const double q[4])
+{
+    const int lane = threadIdx.x & 3, k = lane == 3 ? 0 : lane;
+    const bool wr = act && lane < 3;
+    PGeom2 &G = reinterpret_cast<PGeom2 *>(P.geo)[p];
+    constexpr int GW = (int)(sizeof(PGeom) / 8);
+    static_assert(sizeof(PGeom) % 8 == 0, "PGeom is copied in 8-byte words");
+    auto copy_now = [&] {  // old_ = now
+        const double *src = reinterpret_cast<const double *>(&G.now);
+        double *dst = reinterpret_cast<double *>(&G.old_);
+        if (act)
+            for (int w = lane; w < GW; w += 4) dst[w] = src[w];
+        __syncwarp();
+    };
+    if (!first) copy_now();
+    const double rp = P.rp[p], ro = P.ro[p];
+    double row[3], col[3];
+    quad_rot(k, q, row, col);
+    const double h = sqrt(rp * rp * row[0] * row[0] + ro * ro * (row[1] * row[1] + row[2] * row[2]));
+    double lo, hi;
+    box_axis(X, h, lo, hi);
+    const bool empty = quad_empty(lo, hi);
+    const int count = quad_box(L, k, wr, empty, lo, hi, G.now.box);
+    const double fl = floor(X);
+    if (wr) {
+        for (int j = 0; j < 3; j++) {
+            G.now.g.R[k][j] = row[j];
+            G.now.g.R32[k][j] = (float)row[j];
+        }
+        G.now.X[k] = X;
+        G.now.lo[k] = lo;
+        G.now.hi[k] = hi;
+        // X = Xi + Xf, Xi integral: the FP32 displacement (u - Xi) - Xf
+        // carries no large cancellation (box_axis bounds |X| < 1e9)
+        G.now.Xi[k] = count ? (int)fl : 0;
+        G.now.Xf[k] = (float)(X - fl);
+    }
+    if (first && act && lane < 2) {  // the radii never change
+        const double inv = __ddiv_rn(1.0, lane == 0 ? m_(rp, rp) : m_(ro, ro));
+        (lane == 0 ? G.now.g.ip2 : G.now.g.io2) = inv;
+        (lane == 0 ? G.now.g.ip2f : G.now.g.io2f) = (float)inv;
+    }
+    // the new centre next to the old one, and the union of the two boxes
+    const double Xu = Xold + pair_disp(L, k, Xold, X);
+    double lu, hu;
+    box_axis(Xu, h, lu, hu);
+    const bool eu = quad_empty(lu, hu);
+    double lo0 = first ? lo : G.old_.lo[k], hi0 = first ? hi : G.old_.hi[k];
+    const bool e0 = quad_empty(lo0, hi0);
+    if (e0) {
+        lo0 = lu;
+        hi0 = hu;
+    } else if (!eu) {
+        lo0 = fmin(lo0, lu);
+        hi0 = fmax(hi0, hu);
+    }
+    quad_box(L, k, wr, e0 && eu, lo0, hi0, G.uni);
+    if (wr) G.Xu[k] = Xu;
+    __syncwarp();
+    if (first) copy_now();
+}
+
+// Geometry from the particle's state in memory.
+__device__ __forceinline__ void geom_body(const Lat &L, const Parts &P, int p, bool act, bool first)
+{
+    const int lane = threadIdx.x & 3, k = lane == 3 ? 0 : lane;
+    double q[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) q[j] = P.q[4 * p + j];
+    geom_quad(L, P, p, act, first, P.X[3 * p + k], P.Xold[3 * p + k], q);
+}
+
+// The particle of this quad in a launch of four lanes per particle: quads
+// past the end work on the last particle and write nothing.
+__device__ __forceinline__ int quad_particle(int n, bool &act)
+{
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    act = g < n;
+    return act ? g : n - 1;
 }
 
 __global__ void k_geom(Lat L, Parts P)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < P.n) geom_body(L, P, p);
+    bool act;
+    const int p = quad_particle(P.n, act);
+    geom_body(L, P, p, act, true);
 }
 
 // Fixed-order block reduction of K doubles (PT threads).
@@ -764,46 +898,6 @@ __device__ double hertz_bp(double K, double rp, double ro, const double r[3], co
     return sigma;
 }
 
-// The Hertz and lubrication (Eq. 9 with 2R -> σ, R^2 -> (σ/2)^2, only for
-// gaps 0 < r - σ < Δc, opposing the normal approach) contribution of
-// partner j to particle i.  The lubrication coefficient K (1/h - 1/Δc) is
-// capped at the pair's reduced mass M_i M_j / (M_i + M_j): at the cap one
-// update (Δt = 1) removes the normal approach speed; above it the explicit
-// update would reverse the approach with growing speed as h -> 0.  A pair
-// is evaluated in FP64 only when the FP32 distance of the centres is within
-// reach_i + reach_j + Δc (+0.05 for the FP32 error).
-
-__device__ void pair_term(const Lat &L, const Parts &P, const Pair &pp, int i, int j, const double oi[3],
-                          double F[3], double T[3])
-{
-    int a = i < j ? i : j, b = i < j ? j : i;  // the pair is taken as (a, b), a < b
-    double r[3];
-    for (int k = 0; k < 3; k++) r[k] = pair_disp(L, k, P.X[3 * a + k], P.X[3 * b + k]);
-    double Rj[3][3];
-    rotmat(P.q + 4 * j, Rj);
-    double oj[3] = {Rj[0][0], Rj[1][0], Rj[2][0]};
-    const double *oa = i < j ? oi : oj, *ob = i < j ? oj : oi;
-    double rp = 0.5 * (P.rp[a] + P.rp[b]), ro = 0.5 * (P.ro[a] + P.ro[b]);
-    double fb[3], ta[3], tb[3];
-    double sigma = hertz_bp(pp.k_hertz, rp, ro, r, oa, ob, fb, ta, tb);
-    for (int k = 0; k < 3; k++) {
-        F[k] += i == b ? fb[k] : -fb[k];
-        T[k] += i == a ? ta[k] : tb[k];
-    }
-    double rl = sqrt(dot3(r, r));
-    double h = rl - sigma;
-    if (pp.lub_cut > 0 && h > 0 && h < pp.lub_cut) {
-        double rh[3] = {r[0] / rl, r[1] / rl, r[2] / rl};
-        double du[3] = {P.V[3 * a] - P.V[3 * b], P.V[3 * a + 1] - P.V[3 * b + 1], P.V[3 * a + 2] - P.V[3 * b + 2]};
-        double K = 3.0 * M_PI * pp.mu * sigma * sigma / 8.0;
-        double gam = K * (1.0 / h - 1.0 / pp.lub_cut);
-        const double mred = P.M[a] * P.M[b] / (P.M[a] + P.M[b]);
-        if (gam > mred) gam = mred;
-        double s = gam * dot3(rh, du);
-        for (int k = 0; k < 3; k++) F[k] += i == a ? -s * rh[k] : s * rh[k];
-    }
-}
-
 // FP32 prefilter of a pair (centres and reaches in xyzw): nearest-image
 // distance within reach_i + reach_j + extra.  Pairs it drops contribute
 // exactly zero, so it decides nothing but the work done.
@@ -818,6 +912,131 @@ __device__ __forceinline__ bool near_pair(float4 me, float4 o, const float nl[3]
     return __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, dz * dz)) <= reach * reach;
 }
 
+// ---- eight lanes per particle ------------------------------------------------
+// A particle's pair terms are long FP64 chains (divisions, square roots)
+// and few (about 4 partners pass the prefilter in a dense emulsion), and a
+// warp instruction costs the same for one active lane as for 32: eight lanes
+// share a particle, test eight partners at a time and evaluate up to eight
+// terms at once.  The terms are then added one after the other in the order
+// of the partners' indices, one component per lane, which gives the sums of
+// a plain loop bit for bit.  525
+// particles (150 x 141 x 133, 10 %): 81 us with one lane per particle, 34
+// now; 25,033: 127 and 175 us, where the other lanes' work had filled the
+// warps (1.7 % of that step).
+//
+// Up to PAIRS_SCAN_MAX particles the loop over all partners replaces the
+// cell list: its three kernels and the clearing cost about 10 us however few
+// the particles (1 particle: 18 -> 4 us; 40: 38 -> 17 us), and 256 prefilter
+// rounds of eight stay below that.
+constexpr int PAIRS_SCAN_MAX = 256;
+constexpr int PG = 8;                  // lanes per particle
+constexpr int PAIR_GROUPS = 128 / PG;  // particles per CTA
+constexpr int CAND_MAX = 96;           // candidates held per particle; beyond that a full scan
+
+struct PairGroup {
+    int cand[CAND_MAX];    // partners waiting for evaluation
+    int sorted[CAND_MAX];
+    double term[PG][9];    // Hertz force and torque, lubrication force
+};
+
+// The Hertz and lubrication (Eq. 9 with 2R -> σ, R^2 -> (σ/2)^2, only for
+// gaps 0 < r - σ < Δc, opposing the normal approach) contribution of
+// partner j to particle i.  The lubrication coefficient K (1/h - 1/Δc) is
+// capped at the pair's reduced mass M_i M_j / (M_i + M_j): at the cap one
+// update (Δt = 1) removes the normal approach speed; above it the explicit
+// update would reverse the approach with growing speed as h -> 0.  A pair
+// is evaluated in FP64 only when the FP32 distance of the centres is within
+// reach_i + reach_j + Δc (+0.05 for the FP32 error).
+// t gets the Hertz force and torque and, with lub set, the lubrication force.
+__device__ void pair_parts(const Lat &L, const Parts &P, const Pair &pp, int i, int j, const double oi[3],
+                           double *t, bool &lub)
+{
+    int a = i < j ? i : j, b = i < j ? j : i;  // the pair is taken as (a, b), a < b
+    double r[3];
+    for (int k = 0; k < 3; k++) r[k] = pair_disp(L, k, P.X[3 * a + k], P.X[3 * b + k]);
+    double Rj[3][3];
+    rotmat(P.q + 4 * j, Rj);
+    double oj[3] = {Rj[0][0], Rj[1][0], Rj[2][0]};
+    const double *oa = i < j ? oi : oj, *ob = i < j ? oj : oi;
+    double rp = 0.5 * (P.rp[a] + P.rp[b]), ro = 0.5 * (P.ro[a] + P.ro[b]);
+    double fb[3], ta[3], tb[3];
+    double sigma = hertz_bp(pp.k_hertz, rp, ro, r, oa, ob, fb, ta, tb);
+    for (int k = 0; k < 3; k++) {
+        t[k] = i == b ? fb[k] : -fb[k];
+        t[3 + k] = i == a ? ta[k] : tb[k];
+    }
+    double rl = sqrt(dot3(r, r));
+    double h = rl - sigma;
+    lub = pp.lub_cut > 0 && h > 0 && h < pp.lub_cut;
+    if (lub) {
+        double rh[3] = {r[0] / rl, r[1] / rl, r[2] / rl};
+        double du[3] = {P.V[3 * a] - P.V[3 * b], P.V[3 * a + 1] - P.V[3 * b + 1], P.V[3 * a + 2] - P.V[3 * b + 2]};
+        double K = 3.0 * M_PI * pp.mu * sigma * sigma / 8.0;
+        double gam = K * (1.0 / h - 1.0 / pp.lub_cut);
+        const double mred = P.M[a] * P.M[b] / (P.M[a] + P.M[b]);
+        if (gam > mred) gam = mred;
+        double s = gam * dot3(rh, du);
+        for (int k = 0; k < 3; k++) t[6 + k] = i == a ? -s * rh[k] : s * rh[k];
+    }
+}
+
+// Evaluate the n <= 8 partners list[0..n) and add their terms in list order
+// to acc, which is component l of (force, torque) on lane l < 6.  Called by
+// the eight lanes of a group (mask m).
+__device__ __forceinline__ void pair_flush(const Lat &L, const Parts &P, const Pair &pp, int i, const int *list, int n,
+                                           const double oi[3], PairGroup &g, unsigned m, double &acc)
+{
+    const int l = threadIdx.x & (PG - 1);
+    bool lub = false;
+    if (l < n) pair_parts(L, P, pp, i, list[l], oi, g.term[l], lub);
+    const unsigned bl = __ballot_sync(m, lub) >> (threadIdx.x & 24);
+    __syncwarp(m);
+    if (l < 6)
+        for (int k = 0; k < n; k++) {
+            acc += g.term[k][l];
+            if (l < 3 && ((bl >> k) & 1u)) acc += g.term[k][6 + l];
+        }
+    __syncwarp(m);
+}
+
+// Pair sums of particle i over all partners in index order: eight at a
+// time through the prefilter, those that pass queued and evaluated eight at
+// a time.  Returns component l of (force, torque) on lane l < 6.
+__device__ __forceinline__ double pairs_scan(const Lat &L, const Parts &P, const Pair &pp, int i, float4 me,
+                                             const double oi[3], PairGroup &g, unsigned m)
+{
+    const int l = threadIdx.x & (PG - 1);
+    const float nl[3] = {(float)L.nx, (float)L.ny, (float)L.nz};
+    const float inv[3] = {1.f / nl[0], 1.f / nl[1], 1.f / nl[2]};
+    const float extra = (float)pp.lub_cut + 0.05f;
+    double acc = 0.0;
+    int n = 0;
+    for (int j0 = 0; j0 < P.n; j0 += PG) {
+        const int j = j0 + l;
+        const bool near = j < P.n && j != i && near_pair(me, P.X32[j], nl, inv, !L.walls, extra);
+        const unsigned b = (__ballot_sync(m, near) >> (threadIdx.x & 24)) & 0xFFu;
+        if (near) g.cand[n + __popc(b & ((1u << l) - 1u))] = j;
+        n += __popc(b);
+        __syncwarp(m);
+        if (n >= PG) {
+            pair_flush(L, P, pp, i, g.cand, PG, oi, g, m, acc);
+            const int v = l < n - PG ? g.cand[PG + l] : 0;
+            __syncwarp(m);
+            if (l < n - PG) g.cand[l] = v;
+            n -= PG;
+            __syncwarp(m);
+        }
+    }
+    if (n > 0) pair_flush(L, P, pp, i, g.cand, n, oi, g, m, acc);
+    return acc;
+}
+
+__device__ __forceinline__ void pairs_store(const Parts &P, int i, double acc)
+{
+    const int l = threadIdx.x & (PG - 1);
+    if (l < 6) P.ppart[(size_t)l * P.n + i] = acc;
+}
+
 // ---------------------------------------------------------------- cells
 // Per step: count the particles of each cell, exclusive prefix over the
 // cells (one CTA), place each particle's index, then each particle gathers
@@ -825,7 +1044,8 @@ __device__ __forceinline__ bool near_pair(float4 me, float4 o, const float nl[3]
 // axis has fewer than 3 cells), keeps those the FP32 prefilter passes, and
 // sums the pair terms in increasing partner index: the same terms in the
 // same order as a loop over all partners, so the sums do not depend on the
-// order the cells were filled in.
+// order the cells were filled in.  Lattices of at most PAIRS_SCAN_MAX
+// particles take the loop over all partners instead.
 
 __device__ __forceinline__ int cell_axis(float x, float n, float inv, int nc, bool periodic)
 {
@@ -882,20 +1102,15 @@ __global__ void k_cell_fill(Parts P, Cells C)
     C.idx[C.start[c] + atomicAdd(&C.fill[c], 1)] = i;
 }
 
-constexpr int CAND_MAX = 96;  // candidates held per particle; beyond that a full scan
-
-__global__ void __launch_bounds__(128) k_pairs(Lat L, Parts P, Pair pp, Cells C)
+__device__ __forceinline__ double pairs_cells(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, int i,
+                                              float4 me, const double oi[3], PairGroup &g, unsigned m)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const float4 me = P.X32[i];
+    const int l = threadIdx.x & (PG - 1);
     const float nl[3] = {(float)L.nx, (float)L.ny, (float)L.nz};
     const float inv[3] = {1.f / nl[0], 1.f / nl[1], 1.f / nl[2]};
     const bool per_z = !L.walls;
     const float extra = (float)pp.lub_cut + 0.05f;
-    int cand[CAND_MAX];
     int nc = 0;
-    bool overflow = false;
     const int c0 = C.cid[i];
     const int ci[3] = {c0 % C.n[0], (c0 / C.n[0]) % C.n[1], c0 / (C.n[0] * C.n[1])};
     int lo[3], hi[3];
@@ -921,40 +1136,52 @@ __global__ void __launch_bounds__(128) k_pairs(Lat L, Parts P, Pair pp, Cells C)
             for (int dx = lo[0]; dx <= hi[0]; dx++) {
                 const int x = C.n[0] >= 3 ? (dx + C.n[0]) % C.n[0] : dx;
                 const int c = x + C.n[0] * (y + C.n[1] * z);
-                for (int k = C.start[c]; k < C.start[c + 1]; k++) {
-                    const int j = C.idx[k];
-                    if (j == i || !near_pair(me, P.X32[j], nl, inv, per_z, extra)) continue;
-                    if (nc < CAND_MAX)
-                        cand[nc++] = j;
-                    else
-                        overflow = true;
+                const int k1 = C.start[c + 1];
+                for (int k0 = C.start[c]; k0 < k1; k0 += PG) {
+                    const int j = k0 + l < k1 ? C.idx[k0 + l] : i;
+                    const bool near = j != i && near_pair(me, P.X32[j], nl, inv, per_z, extra);
+                    const unsigned b = (__ballot_sync(m, near) >> (threadIdx.x & 24)) & 0xFFu;
+                    const int at = nc + __popc(b & ((1u << l) - 1u));
+                    if (near && at < CAND_MAX) g.cand[at] = j;
+                    nc += __popc(b);
                 }
             }
         }
     }
+    if (nc > CAND_MAX) return pairs_scan(L, P, pp, i, me, oi, g, m);  // very dense
+    __syncwarp(m);
+    for (int a = l; a < nc; a += PG) {  // by increasing partner index (all distinct)
+        int r = 0;
+        for (int b = 0; b < nc; b++) r += g.cand[b] < g.cand[a];
+        g.sorted[r] = g.cand[a];
+    }
+    __syncwarp(m);
+    double acc = 0.0;
+    for (int a = 0; a < nc; a += PG) pair_flush(L, P, pp, i, g.sorted + a, min(PG, nc - a), oi, g, m, acc);
+    return acc;
+}
+
+// Pair sums of particle i by its group of eight lanes; cells null: over all
+// partners.
+__device__ __forceinline__ void pairs_body(const Lat &L, const Parts &P, const Pair &pp, const Cells *C, int i,
+                                           PairGroup &g)
+{
+    const unsigned m = 0xFFu << (threadIdx.x & 24);
+    const float4 me = P.X32[i];
     double Ri[3][3];
     rotmat(P.q + 4 * i, Ri);
     const double oi[3] = {Ri[0][0], Ri[1][0], Ri[2][0]};
-    double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-    if (!overflow) {
-        for (int a = 1; a < nc; a++) {  // insertion sort: increasing partner index
-            const int v = cand[a];
-            int b = a - 1;
-            while (b >= 0 && cand[b] > v) {
-                cand[b + 1] = cand[b];
-                b--;
-            }
-            cand[b + 1] = v;
-        }
-        for (int a = 0; a < nc; a++) pair_term(L, P, pp, i, cand[a], oi, F, T);
-    } else {  // very dense: every partner in index order
-        for (int j = 0; j < P.n; j++)
-            if (j != i && near_pair(me, P.X32[j], nl, inv, per_z, extra)) pair_term(L, P, pp, i, j, oi, F, T);
-    }
-    for (int k = 0; k < 3; k++) {
-        P.ppart[(size_t)k * P.n + i] = F[k];
-        P.ppart[(size_t)(3 + k) * P.n + i] = T[k];
-    }
+    const double acc = C ? pairs_cells(L, P, pp, *C, i, me, oi, g, m) : pairs_scan(L, P, pp, i, me, oi, g, m);
+    pairs_store(P, i, acc);
+}
+
+template <bool CELLS>
+__global__ void __launch_bounds__(128) k_pairs(Lat L, Parts P, Pair pp, Cells C)
+{
+    __shared__ PairGroup g[PAIR_GROUPS];
+    const int i = (blockIdx.x * 128 + threadIdx.x) / PG;
+    if (i >= P.n) return;  // whole groups
+    pairs_body(L, P, pp, CELLS ? &C : nullptr, i, g[threadIdx.x / PG]);
 }
 
 // ------------------------------------------------------------ integrate
@@ -963,117 +1190,121 @@ __global__ void __launch_bounds__(128) k_pairs(Lat L, Parts P, Pair pp, Cells C)
 // momentum exchange + pair forces + the fill/empty momentum of the last
 // coverage update.
 
-__device__ void qmul(const double a[4], const double b[4], double o[4])
+// One update of particle p by its quad; X and q get the new centre (axis k)
+// and orientation, Xold the old centre.  The quads of a warp may differ in
+// mode (boxes of a batch), so all take part in every exchange between lanes.
+__device__ __forceinline__ void integrate_quad(const Lat &L, const Parts &P, int mode, int p, bool act, double &X,
+                                               double &Xold, double q[4])
 {
-    o[0] = a[0] * b[0] - a[1] * b[1] - a[2] * b[2] - a[3] * b[3];
-    o[1] = a[0] * b[1] + a[1] * b[0] + a[2] * b[3] - a[3] * b[2];
-    o[2] = a[0] * b[2] - a[1] * b[3] + a[2] * b[0] + a[3] * b[1];
-    o[3] = a[0] * b[3] + a[1] * b[2] - a[2] * b[1] + a[3] * b[0];
-}
-
-__device__ void rotate_by_body_omega(double q[4], const double wb[3])
-{
-    double h[3] = {0.5 * wb[0], 0.5 * wb[1], 0.5 * wb[2]};
-    double hn = sqrt(dot3(h, h));
-    double dq[4] = {1.0, 0.0, 0.0, 0.0};
-    if (hn > 0) {
-        double s = sin(hn) / hn;
-        dq[0] = cos(hn);
-        dq[1] = s * h[0];
-        dq[2] = s * h[1];
-        dq[3] = s * h[2];
+    const int lane = threadIdx.x & 3, k = lane == 3 ? 0 : lane;
+    const bool wr = act && lane < 3;
+    const int e = 3 * p + k;
+    // link sums: FP64 from the two-pass link kernel, or 2^-40 fixed point
+    // from the fused kernel (the other one is zero)
+    const double fl = P.Flink[e] + (double)(long long)P.fix[6 * p + k] * FIXED_UNIT;
+    const double tl = P.Tlink[e] + (double)(long long)P.fix[6 * p + 3 + k] * FIXED_UNIT;
+    double fp = 0.0, tp = 0.0;
+    for (int sp = 0; sp < P.nsplit; sp++) {
+        fp += P.ppart[((size_t)sp * 6 + k) * P.n + p];
+        tp += P.ppart[((size_t)sp * 6 + 3 + k) * P.n + p];
     }
-    double qn[4];
-    qmul(q, dq, qn);
-    double nn = sqrt(qn[0] * qn[0] + qn[1] * qn[1] + qn[2] * qn[2] + qn[3] * qn[3]);
-    for (int k = 0; k < 4; k++) q[k] = qn[k] / nn;
-}
-
-__device__ __forceinline__ void integrate_body(const Lat &L, const Parts &P, int mode, int p)
-{
-    double F[3], T[3];
-    for (int k = 0; k < 3; k++) {
-        // link sums: FP64 from the two-pass link kernel, or 2^-40 fixed point
-        // from the fused kernel (the other one is zero)
-        const double fl = P.Flink[3 * p + k] + (double)(long long)P.fix[6 * p + k] * FIXED_UNIT;
-        const double tl = P.Tlink[3 * p + k] + (double)(long long)P.fix[6 * p + 3 + k] * FIXED_UNIT;
+    const double F = fl + fp + P.Fpend[e], T = tl + tp + P.Tpend[e];
+    Xold = X = P.X[e];
+    double V = P.V[e], W = P.W[e];
+    const double qc = P.q[4 * p + lane];
+    __syncwarp();  // every lane has read before any writes
+    if (wr) {
         P.fix[6 * p + k] = 0ull;
         P.fix[6 * p + 3 + k] = 0ull;
-        double fp = 0.0, tp = 0.0;
-        for (int sp = 0; sp < P.nsplit; sp++) {
-            fp += P.ppart[((size_t)sp * 6 + k) * P.n + p];
-            tp += P.ppart[((size_t)sp * 6 + 3 + k) * P.n + p];
+        P.Fpair[e] = fp;
+        P.Tpair[e] = tp;
+        P.F[e] = F;
+        P.T[e] = T;
+        P.Fpend[e] = 0.0;
+        P.Tpend[e] = 0.0;
+        P.Flink[e] = 0.0;
+        P.Tlink[e] = 0.0;
+        P.Xold[e] = X;
+    }
+    if (act) P.qold[4 * p + lane] = qc;
+#pragma unroll
+    for (int j = 0; j < 4; j++) q[j] = quad(qc, j);
+    if (__all_sync(0xffffffffu, mode == LBE_PARTICLES_STATIC)) return;
+    const bool moves = act && mode != LBE_PARTICLES_STATIC, free_ = mode == LBE_PARTICLES_FREE;
+    double row[3], col[3];
+    quad_rot(k, q, row, col);
+    double wb = col[0] * quad(W, 0) + col[1] * quad(W, 1) + col[2] * quad(W, 2);
+    {
+        const double tb = col[0] * quad(T, 0) + col[1] * quad(T, 1) + col[2] * quad(T, 2);
+        const double I = k == 0 ? P.Ipar[p] : P.Iperp[p];
+        const double Lb = I * wb;
+        const int k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+        const double wl = quad(wb, k1) * quad(Lb, k2) - quad(wb, k2) * quad(Lb, k1);
+        if (free_) {
+            V += F / P.M[p];
+            wb += (tb - wl) / I;
         }
-        P.Fpair[3 * p + k] = fp;
-        P.Tpair[3 * p + k] = tp;
-        F[k] = fl + fp + P.Fpend[3 * p + k];
-        T[k] = tl + tp + P.Tpend[3 * p + k];
-        P.F[3 * p + k] = F[k];
-        P.T[3 * p + k] = T[k];
-        P.Fpend[3 * p + k] = 0.0;
-        P.Tpend[3 * p + k] = 0.0;
-        P.Flink[3 * p + k] = 0.0;
-        P.Tlink[3 * p + k] = 0.0;
-        P.Xold[3 * p + k] = P.X[3 * p + k];
+        X += V;
     }
-    double q[4];
-    for (int k = 0; k < 4; k++) q[k] = P.qold[4 * p + k] = P.q[4 * p + k];
-    if (mode == LBE_PARTICLES_STATIC) return;
-    double X[3], V[3], W[3];
-    for (int k = 0; k < 3; k++) {
-        X[k] = P.X[3 * p + k];
-        V[k] = P.V[3 * p + k];
-        W[k] = P.W[3 * p + k];
-    }
-    double R[3][3];
-    rotmat(q, R);
-    double wb[3];
-    for (int k = 0; k < 3; k++) wb[k] = R[0][k] * W[0] + R[1][k] * W[1] + R[2][k] * W[2];
-    if (mode == LBE_PARTICLES_PRESCRIBED) {
-        for (int k = 0; k < 3; k++) X[k] += V[k];
-        rotate_by_body_omega(q, wb);
-    } else {
-        double M = P.M[p];
-        for (int k = 0; k < 3; k++) {
-            V[k] += F[k] / M;
-            X[k] += V[k];
+    // q <- normalise(q (x) exp(ω_body / 2)): component l of the product is
+    // a0 b_l ± a1 b_{l^1} ± a2 b_{l^2} ± a3 b_{l^3}
+    {
+        const double h = 0.5 * wb;
+        const double h0 = quad(h, 0), h1 = quad(h, 1), h2 = quad(h, 2);
+        const double x = h0 * h0 + h1 * h1 + h2 * h2;
+        double c, s;  // cos |h|, sin |h| / |h|
+        if (x < 1.0 / 256.0) {
+            // Taylor series in x = |h|^2: the first terms left out are below
+            // x^6 / 12! < 1e-23, so only rounding remains, and the square
+            // root, the division and the general sine and cosine go
+            c = 1.0 + x * (-1.0 / 2 + x * (1.0 / 24 + x * (-1.0 / 720 + x * (1.0 / 40320 + x * (-1.0 / 3628800)))));
+            s = 1.0 + x * (-1.0 / 6 + x * (1.0 / 120 + x * (-1.0 / 5040 + x * (1.0 / 362880 + x * (-1.0 / 39916800)))));
+        } else {
+            const double hn = sqrt(x);
+            s = hn > 0 ? sin(hn) / hn : 0.0;
+            c = hn > 0 ? cos(hn) : 1.0;
         }
-        double tb[3];
-        for (int k = 0; k < 3; k++) tb[k] = R[0][k] * T[0] + R[1][k] * T[1] + R[2][k] * T[2];
-        double I[3] = {P.Ipar[p], P.Iperp[p], P.Iperp[p]};
-        double Lb[3] = {I[0] * wb[0], I[1] * wb[1], I[2] * wb[2]};
-        double wl[3];
-        cross3(wb, Lb, wl);
-        for (int k = 0; k < 3; k++) wb[k] += (tb[k] - wl[k]) / I[k];
-        rotate_by_body_omega(q, wb);
-        rotmat(q, R);
-        for (int k = 0; k < 3; k++) W[k] = R[k][0] * wb[0] + R[k][1] * wb[1] + R[k][2] * wb[2];
+        const double b = lane == 0 ? c : (x > 0 ? s * (lane == 1 ? h0 : (lane == 2 ? h1 : h2)) : 0.0);
+        const double b1 = quad(b, lane ^ 1), b2 = quad(b, lane ^ 2), b3 = quad(b, lane ^ 3);
+        const double t1 = q[1] * b1, t2 = q[2] * b2, t3 = q[3] * b3;
+        double o = q[0] * b;
+        o += (lane & 1) ? t1 : -t1;
+        o += lane == 1 || lane == 2 ? t2 : -t2;
+        o += lane >= 2 ? t3 : -t3;
+        const double o0 = quad(o, 0), o1 = quad(o, 1), o2 = quad(o, 2), o3 = quad(o, 3);
+        const double nn = sqrt(o0 * o0 + o1 * o1 + o2 * o2 + o3 * o3);
+        const double qn = o / nn;
+        if (moves) P.q[4 * p + lane] = qn;
+#pragma unroll
+        for (int j = 0; j < 4; j++) q[j] = quad(qn, j);
     }
-    for (int k = 0; k < 3; k++) {
-        if (periodic_dim(L, k)) {
-            double n = (double)ext_of(L, k);
-            if (X[k] < 0) X[k] += n;
-            if (X[k] >= n) X[k] -= n;
-        }
-        P.X[3 * p + k] = X[k];
-        P.V[3 * p + k] = V[k];
-        P.W[3 * p + k] = W[k];
+    quad_rot(k, q, row, col);
+    const double Wn = row[0] * quad(wb, 0) + row[1] * quad(wb, 1) + row[2] * quad(wb, 2);
+    if (free_) W = Wn;
+    if (periodic_dim(L, k)) {
+        const double n = (double)ext_of(L, k);
+        if (X < 0) X += n;
+        if (X >= n) X -= n;
     }
-    for (int k = 0; k < 4; k++) P.q[4 * p + k] = q[k];
-    float4 x32 = P.X32[p];
-    x32.x = (float)X[0];
-    x32.y = (float)X[1];
-    x32.z = (float)X[2];
-    P.X32[p] = x32;
-    P.K32[2 * p] = make_float4((float)V[0], (float)V[1], (float)V[2], 0.f);
-    P.K32[2 * p + 1] = make_float4((float)W[0], (float)W[1], (float)W[2], 0.f);
+    if (wr && moves) {
+        P.X[e] = X;
+        P.V[e] = V;
+        P.W[e] = W;
+        reinterpret_cast<float *>(P.X32 + p)[k] = (float)X;
+        reinterpret_cast<float *>(P.K32 + 2 * p)[k] = (float)V;
+        reinterpret_cast<float *>(P.K32 + 2 * p + 1)[k] = (float)W;
+    }
 }
 
-__global__ void k_integrate(Lat L, Parts P, int mode)
+// The update and, for particles that move, the geometry of their new
+// coverage, in one launch.
+__global__ void __launch_bounds__(128) k_integrate(Lat L, Parts P, int mode)
 {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P.n) return;
-    integrate_body(L, P, mode, p);
+    bool act;
+    const int p = quad_particle(P.n, act);
+    double X, Xold, q[4];
+    integrate_quad(L, P, mode, p, act, X, Xold, q);
+    if (mode != LBE_PARTICLES_STATIC) geom_quad(L, P, p, act, false, X, Xold, q);
 }
 
 // ---------------------------------------------------------------- claim
@@ -1389,52 +1620,36 @@ __global__ void __launch_bounds__(PT) k_reset_batch(BatchIndex B, int total)
     reset_body(bx.L, bx.P, g - B.part0[b], 1, bx.owner[B.par[2 * b + 1]]);
 }
 
-__global__ void k_geom_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(128) k_geom_batch(BatchIndex B, int total)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= total) return;
+    bool act;
+    const int g = quad_particle(total, act);
     const int b = find_box(B.part0, B.nbox, g);
     const BoxDev &bx = B.box[b];
-    if (bx.mode == LBE_PARTICLES_STATIC) return;
-    geom_body(bx.L, bx.P, g - B.part0[b]);
+    // the quads of a warp may belong to boxes of either kind: all take part
+    geom_body(bx.L, bx.P, g - B.part0[b], act && bx.mode != LBE_PARTICLES_STATIC, false);
 }
 
-__global__ void k_integrate_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(128) k_integrate_batch(BatchIndex B, int total)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= total) return;
+    bool act;
+    const int g = quad_particle(total, act);
     const int b = find_box(B.part0, B.nbox, g);
     const BoxDev &bx = B.box[b];
-    integrate_body(bx.L, bx.P, bx.mode, g - B.part0[b]);
+    double X, Xold, q[4];
+    integrate_quad(bx.L, bx.P, bx.mode, g - B.part0[b], act, X, Xold, q);
 }
 
-// Pair forces within each box: one thread per particle over its box's
-// particles in index order (the same terms in the same order as the cell
-// list of a lattice stepped alone).
-__global__ void k_pairs_batch(BatchIndex B, int total)
+// Pair forces within each box, over its box's particles in index order (the
+// same terms in the same order as the cell list of a lattice stepped alone).
+__global__ void __launch_bounds__(128) k_pairs_batch(BatchIndex B, int total)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ PairGroup gr[PAIR_GROUPS];
+    const int g = (blockIdx.x * 128 + threadIdx.x) / PG;
     if (g >= total) return;
     const int b = find_box(B.part0, B.nbox, g);
     const BoxDev &bx = B.box[b];
-    const Lat &L = bx.L;
-    const Parts &P = bx.P;
-    const int i = g - B.part0[b];
-    double Ri[3][3];
-    rotmat(P.q + 4 * i, Ri);
-    const double oi[3] = {Ri[0][0], Ri[1][0], Ri[2][0]};
-    const float4 me = P.X32[i];
-    const float nl[3] = {(float)L.nx, (float)L.ny, (float)L.nz};
-    const float inv[3] = {1.f / nl[0], 1.f / nl[1], 1.f / nl[2]};
-    const bool per_z = !L.walls;
-    const float extra = (float)bx.pair.lub_cut + 0.05f;
-    double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-    for (int j = 0; j < P.n; j++)
-        if (j != i && near_pair(me, P.X32[j], nl, inv, per_z, extra)) pair_term(L, P, bx.pair, i, j, oi, F, T);
-    for (int k = 0; k < 3; k++) {
-        P.ppart[(size_t)k * P.n + i] = F[k];
-        P.ppart[(size_t)(3 + k) * P.n + i] = T[k];
-    }
+    pairs_body(bx.L, bx.P, bx.pair, nullptr, g - B.part0[b], gr[threadIdx.x / PG]);
 }
 
 // End of a batched step: flip each box's parities.
@@ -1474,17 +1689,17 @@ __global__ void k_verify(Lat L, const uint8_t *type, const uint32_t *owner)
 
 void launch_pairs_batch(const BatchIndex &B, int total, cudaStream_t s)
 {
-    if (total > 0) k_pairs_batch<<<(total + 127) / 128, 128, 0, s>>>(B, total);
+    if (total > 0) k_pairs_batch<<<(total + PAIR_GROUPS - 1) / PAIR_GROUPS, 128, 0, s>>>(B, total);
 }
 
 void launch_integrate_batch(const BatchIndex &B, int total, cudaStream_t s)
 {
-    if (total > 0) k_integrate_batch<<<(total + 127) / 128, 128, 0, s>>>(B, total);
+    if (total > 0) k_integrate_batch<<<(4 * total + 127) / 128, 128, 0, s>>>(B, total);
 }
 
 void launch_geom_batch(const BatchIndex &B, int total, cudaStream_t s)
 {
-    if (total > 0) k_geom_batch<<<(total + 127) / 128, 128, 0, s>>>(B, total);
+    if (total > 0) k_geom_batch<<<(4 * total + 127) / 128, 128, 0, s>>>(B, total);
 }
 
 void launch_claim_batch(const BatchIndex &B, int total, cudaStream_t s)
@@ -1530,21 +1745,27 @@ void launch_links(int storage, const Lat &L, const Parts &P, void *fnew, const f
     LBE_DISPATCH(storage, (k_links<S><<<P.n, PT, 0, s>>>(L, P, (typename S::P *)fnew, rho, type, owner)));
 }
 
+bool pairs_by_cells(int np) { return np > PAIRS_SCAN_MAX; }
+
 void launch_pairs(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, cudaStream_t s)
 {
     if (P.n == 0) return;
-    const int b = (P.n + 127) / 128;
+    const int b = (P.n + 127) / 128, bp = (P.n + PAIR_GROUPS - 1) / PAIR_GROUPS;
+    if (!pairs_by_cells(P.n)) {
+        k_pairs<false><<<bp, 128, 0, s>>>(L, P, pp, C);
+        return;
+    }
     cudaMemsetAsync(C.count, 0, (size_t)C.ncell * sizeof(int), s);
     k_cell_count<<<b, 128, 0, s>>>(L, P, C);
     k_cell_scan<<<1, 1024, 0, s>>>(C);
     k_cell_fill<<<b, 128, 0, s>>>(P, C);
-    k_pairs<<<b, 128, 0, s>>>(L, P, pp, C);
+    k_pairs<true><<<bp, 128, 0, s>>>(L, P, pp, C);
 }
 
 void launch_geom(const Lat &L, const Parts &P, cudaStream_t s)
 {
     if (P.n == 0) return;
-    k_geom<<<(P.n + 127) / 128, 128, 0, s>>>(L, P);
+    k_geom<<<(4 * P.n + 127) / 128, 128, 0, s>>>(L, P);
 }
 
 size_t geom_bytes_per_particle() { return sizeof(PGeom2); }
@@ -1552,7 +1773,7 @@ size_t geom_bytes_per_particle() { return sizeof(PGeom2); }
 void launch_integrate(const Lat &L, const Parts &P, int mode, cudaStream_t s)
 {
     if (P.n == 0) return;
-    k_integrate<<<(P.n + 127) / 128, 128, 0, s>>>(L, P, mode);
+    k_integrate<<<(4 * P.n + 127) / 128, 128, 0, s>>>(L, P, mode);
 }
 
 void launch_claim(const Lat &L, const Parts &P, int, uint32_t *owner_new, cudaStream_t s)
