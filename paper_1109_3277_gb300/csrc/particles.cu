@@ -236,6 +236,106 @@ __device__ __forceinline__ void row_span(const Geo &g, const double X[3], const 
 
 __device__ __forceinline__ bool box_full(const Box &b) { return b.full[0] || b.full[1] || b.full[2]; }
 
+// The nodes of a row that the inside test accepts form one interval (the
+// quadric is convex along x; three neighbouring nodes on its level 1 would
+// need radii beyond 1e6).  Two bounds of it from FP32 quadrics, whose error
+// (below 1e-5) is far inside the margins: outer [oa, ob] holds every
+// accepted node, inner [ia, ib] only accepted ones.  They differ in the few
+// nodes within 1e-3 of the surface, which alone need the FP64 test.  Empty
+// intervals have a > b.
+struct RowSpan {
+    int oa, ob, ia, ib;
+};
+
+struct RowEval {  // the FP32 quadric along a row
+    float bx[3], R0[3], w1, w2;
+    int Xi;
+    float Xf;
+    __device__ __forceinline__ float operator()(int ux) const
+    {
+        const float d = (float)(ux - Xi) - Xf;
+        float e[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) e[k] = __fmaf_rn(R0[k], d, bx[k]);
+        return __fmaf_rn(e[0] * e[0], w1, __fmaf_rn(e[1], e[1], e[2] * e[2]) * w2);
+    }
+};
+
+__device__ __forceinline__ RowSpan span_of(const Geo &g, const double X[3], const int Xi[3], const float Xf[3],
+                                           const Box &b, int u1, int u2)
+{
+    RowSpan r;
+    row_span(g, X, b, u1, u2, r.oa, r.ob);
+    RowEval q;
+    const float dy = (float)(u1 - Xi[1]) - Xf[1], dz = (float)(u2 - Xi[2]) - Xf[2];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        q.R0[k] = g.R32[0][k];
+        q.bx[k] = __fmaf_rn(g.R32[1][k], dy, g.R32[2][k] * dz);
+    }
+    q.w1 = g.ip2f;
+    q.w2 = g.io2f;
+    q.Xi = Xi[0];
+    q.Xf = Xf[0];
+    while (r.oa <= r.ob && q(r.oa) > 1.001f) r.oa++;
+    while (r.oa <= r.ob && q(r.ob) > 1.001f) r.ob--;
+    r.ia = r.oa;
+    r.ib = r.ob;
+    while (r.ia <= r.ib && !(q(r.ia) < 0.999f)) r.ia++;
+    while (r.ia <= r.ib && !(q(r.ib) < 0.999f)) r.ib--;
+    return r;
+}
+
+// Rows of a box that is no whole period along any axis, 32 at a time per
+// warp (one a lane): f(valid, u1, u2) is called by whole warps.
+template <class F>
+__device__ __forceinline__ void for_rows(const Box &b, F f)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int rows = b.ext[1] * b.ext[2];
+    for (int r0 = warp * 32; r0 < rows; r0 += nw * 32) {
+        const int r = r0 + lane;
+        const bool valid = r < rows;
+        f(valid, b.lo[1] + (valid ? r % b.ext[1] : 0), b.lo[2] + (valid ? r / b.ext[1] : 0));
+    }
+}
+
+// Every node of the intervals [a, b] of the warp's 32 rows (u1, u2): f(node)
+// by groups of eight lanes along x, so that a row's accesses stay together.
+template <class F>
+__device__ __forceinline__ void fill_rows(const Lat &L, int a, int b, int u1, int u2, F f)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int xw = wrapi(a, L.nx), row = L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
+    const int len = max(0, b - a + 1);
+    if (!__any_sync(full, len > 0)) return;
+#pragma unroll
+    for (int it = 0; it < 8; it++) {
+        const int src = it * 4 + (lane >> 3);
+        const int x0 = __shfl_sync(full, xw, src), n0 = __shfl_sync(full, row, src), ln = __shfl_sync(full, len, src);
+        for (int k = lane & 7; k < ln; k += 8) {
+            int x = x0 + k;
+            if (x >= L.nx) x -= L.nx;  // len <= nx
+            f(n0 + x);
+        }
+    }
+}
+
+// Every node of a box that spans a whole period along some axis, once each.
+template <class F>
+__device__ __forceinline__ void for_box(const Box &b, F f)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int k0 = warp * 32; k0 < b.count; k0 += nw * 32) {
+        const int k = k0 + lane;
+        const bool valid = k < b.count;
+        const int kk = valid ? k : 0;
+        const int t = kk / b.ext[0];
+        f(valid, b.lo[0] + kk % b.ext[0], b.lo[1] + t % b.ext[1], b.lo[2] + t / b.ext[1]);
+    }
+}
+
 // Every candidate node of a particle's box, each visited once.  Each warp
 // takes chunks of 32 rows: lane l computes the NSEG disjoint segments
 // [xs[j], xe[j]] of row l of the chunk (spans(u1, u2, xs, xe), empty when
@@ -1315,25 +1415,47 @@ __device__ __forceinline__ void claim_body(const Lat &L, const Parts &P, int p, 
 {
     const PGeom &G = reinterpret_cast<const PGeom2 *>(P.geo)[p].now;
     const Box &box = G.box;
-    for_candidates(box, G.g, G.X, [&](int ux, int u1, int u2, bool valid) {
-        if (!valid) return;
-        const int u[3] = {ux, u1, u2};
-        const int x = wrapi(ux, L.nx), y = wrapi(u1, L.ny), z = wrapi(u2, L.nz);
-        if (is_wall_z(L, z)) return;
-        float d32[3];
+    if (box_full(box)) {
+        for_box(box, [&](bool valid, int ux, int u1, int u2) {
+            if (!valid) return;
+            const int u[3] = {ux, u1, u2};
+            const int x = wrapi(ux, L.nx), y = wrapi(u1, L.ny), z = wrapi(u2, L.nz);
+            if (is_wall_z(L, z)) return;
+            float d32[3];
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-            d32[a] = box.full[a] ? (float)node_disp(L, a, a == 0 ? x : (a == 1 ? y : z), G.X[a])
-                                 : (float)(u[a] - G.Xi[a]) - G.Xf[a];
-        float q32;
-        bool in = inside_q32(G.g, d32, q32);
-        if (!in && q32 <= 1.001f) {
-            double dx[3] = {box_disp(L, box, 0, u[0], x, G.X[0]), box_disp(L, box, 1, u[1], y, G.X[1]),
-                            box_disp(L, box, 2, u[2], z, G.X[2])};
-            in = inside_exact(G.g, dx);
+            for (int a = 0; a < 3; a++)
+                d32[a] = box.full[a] ? (float)node_disp(L, a, a == 0 ? x : (a == 1 ? y : z), G.X[a])
+                                     : (float)(u[a] - G.Xi[a]) - G.Xf[a];
+            float q32;
+            bool in = inside_q32(G.g, d32, q32);
+            if (!in && q32 <= 1.001f) {
+                double dx[3] = {box_disp(L, box, 0, u[0], x, G.X[0]), box_disp(L, box, 1, u[1], y, G.X[1]),
+                                box_disp(L, box, 2, u[2], z, G.X[2])};
+                in = inside_exact(G.g, dx);
+            }
+            int n = x + L.nx * (y + L.ny * z);
+            if (in && idx_ok(L, n, L.N, 4)) atomicMin(owner_new + n, (uint32_t)p);
+        });
+        return;
+    }
+    for_rows(box, [&](bool valid, int u1, int u2) {
+        int a = 1, b = 0;
+        if (valid && !is_wall_z(L, wrapi(u2, L.nz))) {
+            const RowSpan r = span_of(G.g, G.X, G.Xi, G.Xf, box, u1, u2);
+            // the FP64 test for the nodes between the two bounds
+            auto in = [&](int ux) {
+                const double dx[3] = {s_((double)ux, G.X[0]), s_((double)u1, G.X[1]), s_((double)u2, G.X[2])};
+                return inside_exact(G.g, dx);
+            };
+            const bool core = r.ia <= r.ib;
+            a = r.oa;
+            b = r.ob;
+            while (a <= b && !(core && a >= r.ia) && !in(a)) a++;
+            while (a <= b && !(core && b <= r.ib) && !in(b)) b--;
         }
-        int n = x + L.nx * (y + L.ny * z);
-        if (in && idx_ok(L, n, L.N, 4)) atomicMin(owner_new + n, (uint32_t)p);
+        fill_rows(L, a, b, u1, u2, [&](int n) {
+            if (idx_ok(L, n, L.N, 4)) atomicMin(owner_new + n, (uint32_t)p);
+        });
     });
 }
 
@@ -1351,139 +1473,190 @@ __global__ void __launch_bounds__(PT) k_claim(Lat L, Parts P, uint32_t *__restri
 //    that momentum;  both through the pending force/torque.
 // With placement != 0 (particles just added) nodes only change type.
 
+//
+// A node whose owner changes with p the lower of the two owners is inside
+// the particle's old ellipsoid or its new one but not both, so it lies in
+// the outer bound of one and outside the inner bound of the other: only
+// those few nodes of each row are looked at, and their two owners decide.
+// The fill or empty of a changed node is the work of a whole warp (one
+// direction, or one neighbour's populations, per lane).  512^3 Pickering:
+// 731 us when every candidate's two owners were read and one lane did each
+// change, 501 now; 40 dragged particles, of which some change every step:
+// 67 and 22 us.
+
+// What a particle takes over with (o == NONE, covered) or gives to (w ==
+// NONE, uncovered) node (x, y, z): momentum mom.  Called by a whole warp.
 template <class S>
-__device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, int p, typename S::P *__restrict__ f,
-                                                uint8_t *__restrict__ type, const uint32_t *__restrict__ own_old,
-                                                const uint32_t *__restrict__ own_new, int placement)
+__device__ __forceinline__ void change_node(const Lat &L, const Parts &P, int p, typename S::P *f, int x, int y, int z,
+                                            bool covered, const uint32_t *own_old, const uint32_t *own_new,
+                                            double acc[6])
 {
-    __shared__ double red[6][PT / 32];
-    const PGeom2 &G2 = reinterpret_cast<const PGeom2 *>(P.geo)[p];
-    const Box &box = G2.uni;
-    const Geo &gold = G2.old_.g, &gnew = G2.now.g;
-    const double *sXo = G2.old_.X, *sXu = G2.Xu;
-    const double sX[3] = {P.X[3 * p], P.X[3 * p + 1], P.X[3 * p + 2]};
-    const double sV[3] = {P.V[3 * p], P.V[3 * p + 1], P.V[3 * p + 2]};
-    const double sW[3] = {P.W[3 * p], P.W[3 * p + 1], P.W[3 * p + 2]};
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    // a node whose owner changed lies in the old or the new ellipsoid of the
-    // lower of its owners: the candidates of the old, then those of the new
-    // not already visited
-    auto visit = [&](int x, int y, int z) {
-        int n = x + L.nx * (y + L.ny * z);
-        if (!idx_ok(L, n, L.N, 5)) return;
-        uint32_t o = own_old[n], w = own_new[n];
-        if (o == w) return;
-        if (min(o, w) != (uint32_t)p) return;
-        if (o == NONE) {
-            type[n] = PART;
-            if (placement) return;
-            double mom[3] = {0, 0, 0};
-#pragma unroll
-            for (int c = 0; c < 2; c++)
-#pragma unroll
-                for (int i = 0; i < Q; i++) {
-                    const float2 v2 = ld2f<S>(f, L, i, n);
-                    float v = c ? v2.y : v2.x;
-                    if (cx(i)) mom[0] += cx(i) * (double)v;
-                    if (cy(i)) mom[1] += cy(i) * (double)v;
-                    if (cz(i)) mom[2] += cz(i) * (double)v;
-                }
-            double r[3] = {node_disp(L, 0, x, sX[0]), node_disp(L, 1, y, sX[1]), node_disp(L, 2, z, sX[2])};
-            double t[3];
-            cross3(r, mom, t);
-            for (int k2 = 0; k2 < 3; k2++) {
-                acc[k2] += mom[k2];
-                acc[3 + k2] += t[k2];
-            }
-        } else if (w == NONE) {
-            type[n] = FLUID;
-            if (placement) return;
-            float sr0 = 0.f, sr1 = 0.f;
-            int cnt = 0;
-            for (int i = 1; i < Q; i++) {
-                int m = nbr_node(L, x, y, z, i);
-                if (m < 0 || !idx_ok(L, m, L.N, 6)) continue;
-                int mz = m / (L.nx * L.ny);
-                if (is_wall_z(L, mz) || own_old[m] != NONE || own_new[m] != NONE) continue;
-                float a0 = 0.f, a1 = 0.f;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int n = x + L.nx * (y + L.ny * z);
+    const double r[3] = {node_disp(L, 0, x, P.X[3 * p]), node_disp(L, 1, y, P.X[3 * p + 1]),
+                         node_disp(L, 2, z, P.X[3 * p + 2])};
+    const int i = lane < Q ? lane : 0;
+    const int c[3] = {cdir(CXP, i), cdir(CYP, i), cdir(CZP, i)};
+    float2 v = make_float2(0.f, 0.f);  // this lane's direction, both components
+    if (covered) {
+        v = ld2f<S>(f, L, i, n);
+    } else {
+        // lane i: ρ of neighbour i, if it is fluid before and after
+        float a0 = 0.f, a1 = 0.f;
+        bool ok = false;
+        if (lane >= 1 && lane < Q) {
+            int xx = x + c[0], yy = y + c[1], zz = z + c[2];
+            xx = xx < 0 ? xx + L.nx : (xx >= L.nx ? xx - L.nx : xx);
+            yy = yy < 0 ? yy + L.ny : (yy >= L.ny ? yy - L.ny : yy);
+            ok = !L.walls || (zz > 0 && zz < L.nz - 1);
+            if (!L.walls) zz = zz < 0 ? zz + L.nz : (zz >= L.nz ? zz - L.nz : zz);
+            const int m = xx + L.nx * (yy + L.ny * zz);
+            ok = ok && idx_ok(L, m, L.N, 6) && own_old[m] == NONE && own_new[m] == NONE;
+            if (ok) {
 #pragma unroll
                 for (int j = 0; j < Q; j++) {
                     const float2 v2 = ld2f<S>(f, L, j, m);
                     a0 += v2.x;
                     a1 += v2.y;
                 }
-                sr0 += a0;
-                sr1 += a1;
-                cnt++;
-            }
-            float rb0 = cnt ? sr0 / cnt : (float)L.rho_ref[0];
-            float rb1 = cnt ? sr1 / cnt : (float)L.rho_ref[1];
-            double r[3] = {node_disp(L, 0, x, sX[0]), node_disp(L, 1, y, sX[1]), node_disp(L, 2, z, sX[2])};
-            float us[3] = {(float)(sV[0] + sW[1] * r[2] - sW[2] * r[1]),
-                           (float)(sV[1] + sW[2] * r[0] - sW[0] * r[2]),
-                           (float)(sV[2] + sW[0] * r[1] - sW[1] * r[0])};
-            float uu = us[0] * us[0] + us[1] * us[1] + us[2] * us[2];
-            double mom[3] = {0, 0, 0};
-            float fe2[2][Q];
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-                float rc = c ? rb1 : rb0;
-#pragma unroll
-                for (int i = 0; i < Q; i++) {
-                    float cu = cx(i) * us[0] + cy(i) * us[1] + cz(i) * us[2];
-                    float fe = wgt(i) * rc * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * uu);
-                    fe2[c][i] = fe;
-                    if (cx(i)) mom[0] += cx(i) * (double)fe;
-                    if (cy(i)) mom[1] += cy(i) * (double)fe;
-                    if (cz(i)) mom[2] += cz(i) * (double)fe;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < Q; i++) st2f<S>(f, L, i, n, make_float2(fe2[0][i], fe2[1][i]));
-            double t[3];
-            cross3(r, mom, t);
-            for (int k2 = 0; k2 < 3; k2++) {
-                acc[k2] -= mom[k2];
-                acc[3 + k2] -= t[k2];
             }
         }
-    };
-    // per row: the old span, then the new span's parts left and right of it
-    for_segments<3>(
-        box,
-        [&](int u1, int u2, int *xs, int *xe) {
-            int a0, b0, a1, b1;
-            row_span(gold, sXo, box, u1, u2, a0, b0);
-            row_span(gnew, sXu, box, u1, u2, a1, b1);
-            xs[0] = a0;
-            xe[0] = b0;
-            xs[1] = a1;
-            xe[1] = a0 <= b0 ? min(b1, a0 - 1) : b1;
-            xs[2] = a0 <= b0 ? max(a1, b0 + 1) : 1;
-            xe[2] = a0 <= b0 ? b1 : 0;
-        },
-        [&](int ux, int u1, int u2, bool valid) {
-            if (valid) visit(wrapi(ux, L.nx), wrapi(u1, L.ny), wrapi(u2, L.nz));
-        });
-    if (placement) return;
-    block_sum<6>(acc, red);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 3; k++) {
-            P.Fpend[3 * p + k] = acc[k];
-            P.Tpend[3 * p + k] = acc[3 + k];
+        const unsigned have = __ballot_sync(full, ok);
+        float sr0 = 0.f, sr1 = 0.f;
+        for (unsigned m = have; m; m &= m - 1) {  // in the order of the directions
+            sr0 += __shfl_sync(full, a0, __ffs(m) - 1);
+            sr1 += __shfl_sync(full, a1, __ffs(m) - 1);
         }
+        const int cnt = __popc(have);
+        const float rb0 = cnt ? sr0 / cnt : (float)L.rho_ref[0], rb1 = cnt ? sr1 / cnt : (float)L.rho_ref[1];
+        const double V[3] = {P.V[3 * p], P.V[3 * p + 1], P.V[3 * p + 2]};
+        const double W[3] = {P.W[3 * p], P.W[3 * p + 1], P.W[3 * p + 2]};
+        const float us[3] = {(float)(V[0] + W[1] * r[2] - W[2] * r[1]), (float)(V[1] + W[2] * r[0] - W[0] * r[2]),
+                             (float)(V[2] + W[0] * r[1] - W[1] * r[0])};
+        const float uu = us[0] * us[0] + us[1] * us[1] + us[2] * us[2];
+        const float wi = i == 0 ? wgt(0) : (i < 7 ? wgt(1) : wgt(7));
+        const float cu = c[0] * us[0] + c[1] * us[1] + c[2] * us[2];
+        v.x = wi * rb0 * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * uu);
+        v.y = wi * rb1 * (1.f + 3.f * cu + 4.5f * cu * cu - 1.5f * uu);
+        __syncwarp();
+        if (lane < Q)
+            f[pidx(L, i, n)] = S::enc2(make_float2(v.x - L.base[0][i], v.y - L.base[1][i]));
+    }
+    // Σ f c: every term is an FP32 value, whose sums over a node are exact
+    // in FP64 (or differ in the last place) whatever the order
+    const double both = lane < Q ? (double)v.x + (double)v.y : 0.0;
+    double mom[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        double a = c[k] * both;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(full, a, o);
+        mom[k] = a;
+    }
+    double t[3];
+    cross3(r, mom, t);
+    for (int k = 0; k < 3; k++) {
+        acc[k] += covered ? mom[k] : -mom[k];
+        acc[3 + k] += covered ? t[k] : -t[k];
     }
 }
 
-// Compiled for eight CTAs per SM (64 registers): most candidates only
-// compare two owner words, and the occupancy hides their latency; the
-// rare fill and empty spill a few registers.
 template <class S>
-__global__ void __launch_bounds__(PT, 8) k_transition(Lat L, Parts P, typename S::P *__restrict__ f,
-                                                   uint8_t *__restrict__ type,
+__device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, int p, typename S::P *f, uint8_t *type,
+                                                const uint32_t *__restrict__ own_old,
+                                                const uint32_t *__restrict__ own_new, int placement)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double part[PT / 32][6];
+    const PGeom2 &G2 = reinterpret_cast<const PGeom2 *>(P.geo)[p];
+    const Box &box = G2.uni;
+    double acc[6] = {0, 0, 0, 0, 0, 0};  // the same on every lane
+    bool any = false;
+    // one node a lane (cand: it has one): the changed ones go through
+    // change_node one after the other
+    auto visit = [&](bool cand, int ux, int u1, int u2) {
+        int x = 0, y = 0, z = 0;
+        uint32_t o = NONE, w = NONE;
+        if (cand) {
+            x = wrapi(ux, L.nx);
+            y = wrapi(u1, L.ny);
+            z = wrapi(u2, L.nz);
+            const int n = x + L.nx * (y + L.ny * z);
+            if (idx_ok(L, n, L.N, 5)) {
+                o = own_old[n];
+                w = own_new[n];
+                if (o != w && min(o, w) == (uint32_t)p && (o == NONE || w == NONE))
+                    type[n] = o == NONE ? PART : FLUID;
+                else
+                    o = w;
+            }
+        }
+        unsigned m = __ballot_sync(full, o != w);
+        if (placement) return;
+        for (; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            change_node<S>(L, P, p, f, __shfl_sync(full, x, src), __shfl_sync(full, y, src), __shfl_sync(full, z, src),
+                           __shfl_sync(full, (int)(o == NONE), src) != 0, own_old, own_new, acc);
+            any = true;
+        }
+    };
+    if (box_full(box)) {
+        for_box(box, visit);
+    } else {
+        for_rows(box, [&](bool valid, int u1, int u2) {
+            int a = 1, b = 0, ca = 1, cb = 0;  // nodes [a, b] but for [ca, cb]
+            if (valid) {
+                const float uf[3] = {(float)(G2.Xu[0] - floor(G2.Xu[0])), (float)(G2.Xu[1] - floor(G2.Xu[1])),
+                                     (float)(G2.Xu[2] - floor(G2.Xu[2]))};
+                const int ui[3] = {(int)floor(G2.Xu[0]), (int)floor(G2.Xu[1]), (int)floor(G2.Xu[2])};
+                const RowSpan s0 = span_of(G2.old_.g, G2.old_.X, G2.old_.Xi, G2.old_.Xf, box, u1, u2);
+                const RowSpan s1 = span_of(G2.now.g, G2.Xu, ui, uf, box, u1, u2);
+                if (s0.oa > s0.ob) {
+                    a = s1.oa;
+                    b = s1.ob;
+                } else if (s1.oa > s1.ob) {
+                    a = s0.oa;
+                    b = s0.ob;
+                } else {
+                    a = min(s0.oa, s1.oa);
+                    b = max(s0.ob, s1.ob);
+                    if (!placement && s0.ia <= s0.ib && s1.ia <= s1.ib) {
+                        ca = max(s0.ia, s1.ia);
+                        cb = min(s0.ib, s1.ib);
+                    }
+                }
+            }
+            if (a == ca && ca <= cb) a = cb + 1;
+            while (__any_sync(full, a <= b)) {
+                visit(a <= b, a, u1, u2);
+                if (++a == ca && ca <= cb) a = cb + 1;
+            }
+        });
+    }
+    if (placement) return;
+    if (!__syncthreads_or(any)) {
+        if (threadIdx.x < 3) {
+            P.Fpend[3 * p + threadIdx.x] = 0.0;
+            P.Tpend[3 * p + threadIdx.x] = 0.0;
+        }
+        return;
+    }
+    if (lane == 0)
+        for (int k = 0; k < 6; k++) part[warp][k] = acc[k];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        double a = 0.0;
+        for (int w = 0; w < PT / 32; w++) a += part[w][threadIdx.x];
+        (threadIdx.x < 3 ? P.Fpend + 3 * p + threadIdx.x : P.Tpend + 3 * p + threadIdx.x - 3)[0] = a;
+    }
+}
+
+template <class S>
+__global__ void __launch_bounds__(PT) k_transition(Lat L, Parts P, typename S::P *f, uint8_t *type,
                                                    const uint32_t *__restrict__ own_old,
-                                                   const uint32_t *__restrict__ own_new,
-                                                   int placement)
+                                                   const uint32_t *__restrict__ own_new, int placement)
 {
     transition_body<S>(L, P, blockIdx.x, f, type, own_old, own_new, placement);
 }
@@ -1497,13 +1670,23 @@ __device__ __forceinline__ void reset_body(const Lat &L, const Parts &P, int p, 
 {
     // The map holds, over this particle's box, only nodes inside its
     // ellipsoid (its own) or inside other particles' (cleared by them), so
-    // clearing its own candidates empties the map.
+    // clearing the outer bound of its own rows empties the map.
     const PGeom2 &G2 = reinterpret_cast<const PGeom2 *>(P.geo)[p];
     const PGeom &G = use_old ? G2.old_ : G2.now;
-    for_candidates(G.box, G.g, G.X, [&](int ux, int u1, int u2, bool valid) {
-        if (!valid) return;
-        int n = wrapi(ux, L.nx) + L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
-        if (idx_ok(L, n, L.N, 7)) owner[n] = NONE;
+    if (box_full(G.box)) {
+        for_box(G.box, [&](bool valid, int ux, int u1, int u2) {
+            if (!valid) return;
+            const int n = wrapi(ux, L.nx) + L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
+            if (idx_ok(L, n, L.N, 7)) owner[n] = NONE;
+        });
+        return;
+    }
+    for_rows(G.box, [&](bool valid, int u1, int u2) {
+        int a = 1, b = 0;
+        if (valid) row_span(G.g, G.X, G.box, u1, u2, a, b);
+        fill_rows(L, a, b, u1, u2, [&](int n) {
+            if (idx_ok(L, n, L.N, 7)) owner[n] = NONE;
+        });
     });
 }
 
