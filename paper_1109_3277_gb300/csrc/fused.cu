@@ -71,24 +71,30 @@ struct Cfg {
     // (any τ: 512), which the node arithmetic needs without spilling.
     static constexpr int by_regs = (GEN ? 512 : 768) / NT;
     static constexpr size_t twords = SELF ? 0 : (size_t)NT * 4 * sizeof(uint32_t);  // type words in flight
+    static constexpr int MSLOTS = SELF ? 8 : 4;  // ring slots of the solid bits
     static constexpr size_t other =
-        4 * HN * sizeof(float2) + 4 * HY * sizeof(unsigned long long) + twords + 128 + 1024;
+        4 * HN * sizeof(float2) + MSLOTS * HY * sizeof(unsigned long long) + twords + 128 + 1024;
     static constexpr int ctas_for(int nst)
     {
         const int m = (int)((228 * 1024) / (nst * pstride + nst * 8 + other));
         return m < by_regs ? (m > 0 ? m : 1) : by_regs;
     }
     // stage buffers: any τ with SELF re-reads plane z's box one iteration
-    // after its densities (three); otherwise a box is done with in the
-    // iteration it arrives, and a third buffer lets the copies run two
-    // planes ahead where it costs no CTA per SM
-    static constexpr int NST = (GEN && SELF) ? 3 : (SELF ? 2 : (ctas_for(3) >= ctas_for(2) ? 3 : 2));
+    // after its densities (three; at 16 bit: in FP32 three boxes would leave
+    // one CTA per SM, and the pairs come from L2 again); otherwise a box is
+    // done with in the iteration it arrives: two at 16 bit, and one in FP32,
+    // where it is refilled during the collision and the other two of the
+    // three CTAs it leaves room for cover the copy (two boxes: one CTA of
+    // eight warps per SM).  Without SELF a third buffer lets the copies run
+    // two planes ahead where it costs no CTA per SM
+    static constexpr bool RELAX_STAGE = GEN && SELF && E == 4;
+    static constexpr int NST = RELAX_STAGE ? 3 : (SELF ? (E == 8 ? 1 : 2) : (ctas_for(3) >= ctas_for(2) ? 3 : 2));
     static constexpr int CTAS = ctas_for(NST);
     // dynamic shared memory (bytes from a 128-byte aligned base)
     static constexpr size_t stage = 0;                              // P [NST][Q][BY][BX]
     static constexpr size_t sps = stage + NST * pstride;            // float2 [4][HN] (ψ_b, ψ_r)
-    static constexpr size_t smask = sps + 4 * HN * sizeof(float2);  // uint64 [4][HY] solid bits per row
-    static constexpr size_t stw = smask + 4 * HY * sizeof(unsigned long long);  // uint32 [NT][4] type words
+    static constexpr size_t smask = sps + 4 * HN * sizeof(float2);  // uint64 [MSLOTS][HY] solid bits per row
+    static constexpr size_t stw = smask + MSLOTS * HY * sizeof(unsigned long long);  // uint32 [NT][4] type words
     static constexpr size_t bar = stw + twords;                     // uint64 [NST] mbarriers
     static constexpr size_t bytes = bar + NST * sizeof(unsigned long long) + 128;  // + alignment slack
 };
@@ -113,6 +119,14 @@ struct Counts {
             if (b == j) v[j]++;
     }
 };
+
+// Asynchronous copy of 4 or 8 bytes to shared memory.
+template <int B>
+__device__ __forceinline__ void cp_async(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "n"(B)
+                 : "memory");
+}
 
 // The first 128-byte aligned byte at or after p.  The result is a generic
 // address (rounded through an integer), so the compiler issues generic
@@ -398,6 +412,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
     using P = typename S::P;
     constexpr int HX = C::HX, HN = C::HN, BX = C::BX, BY = C::BY, NST = C::NST;
     constexpr size_t PSTR = C::pstride / sizeof(P);  // pairs from one stage to the next
+    constexpr int BXY = SELF && !TMA ? HN : BX * BY;  // pairs from one direction of a stage to the next
     const P *stage = reinterpret_cast<const P *>(smem + C::stage);
     float2 *sps = reinterpret_cast<float2 *>(smem + C::sps);                                // [slot][e]
     unsigned long long *smask = reinterpret_cast<unsigned long long *>(smem + C::smask);   // [slot][ey]
@@ -421,7 +436,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         e.ring = ey * HX + ex;
         const int lx = x0 - 1 + ex, ly = y0 - 1 + ey;
         if (SELF) {
-            e.st = ey * BX + ex - 1 + C::PADX;
+            e.st = TMA ? ey * BX + ex - 1 + C::PADX : e.ring;
             e.inlat = TMA && lx >= 0 && lx < L.nx && ly >= 0 && ly < L.ny;
         } else {  // only the own entries of active nodes are in the box
             e.st = (ey - 1) * BX + ex - 1;
@@ -458,27 +473,21 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         issued.inc(b);
     };
 
-    // node types one plane ahead, and ψ: SELF loads it for solid nodes
-    // only (once their type is known), otherwise for every node along
-    // with the type
+    // node type of entry e of iteration k's plane
     auto load_type = [&](int k, const Ent &e) -> uint8_t {
         const int p = zb - 1 + k;
         if (!pvalid(p)) return WALL;
         return type[e.xy + (size_t)nxy * gz_of(p)];
     };
-    auto load_psi = [&](int k, const Ent &e, uint8_t t) -> float2 {
-        const int p = zb - 1 + k;
-        if ((SELF && t == FLUID) || !pvalid(p)) return dup2(0.f);
-        const size_t n = e.xy + (size_t)nxy * gz_of(p);
-        return make_float2(psi[n], psi[(size_t)L.N + n]);
-    };
 
-    // Collision of plane z with ring slots s0, s1, s2 (planes z - 1, z,
+    // Collision of plane z with ring planes j, j + 1, j + 2 (z - 1, z,
     // z + 1): the own node's moments from mom_of(), with GEN its stored
     // pairs from stage buffer bst (or global memory) for the relaxation.
-    auto collide_at = [&](int z, int s0, int s1, int s2, int bst, auto mom_of) {
-        const float2 *pl[3] = {sps + s0 * HN, sps + s1 * HN, sps + s2 * HN};
-        const unsigned long long *ml[3] = {smask + s0 * C::HY, smask + s1 * C::HY, smask + s2 * C::HY};
+    auto collide_at = [&](int z, int j, int bst, auto mom_of) {
+        constexpr int M = C::MSLOTS - 1;
+        const float2 *pl[3] = {sps + (j & 3) * HN, sps + ((j + 1) & 3) * HN, sps + ((j + 2) & 3) * HN};
+        const unsigned long long *ml[3] = {smask + (j & M) * C::HY, smask + ((j + 1) & M) * C::HY,
+                                           smask + ((j + 2) & M) * C::HY};
         const bool solid_own = (ml[1][ty + 1] >> (tx + 1)) & 1ull;
         const int n = gx + L.nx * gy + nxy * z;
         if (active && !solid_own) {
@@ -584,7 +593,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                 // the box of plane z (or global memory)
                 const P *fb = stage + (size_t)bst * PSTR + own.st;
                 auto ldf = [&](int i) {
-                    if (TMA) return S::raw2(fb[i * BY * BX]);
+                    if (SELF ? C::RELAX_STAGE : TMA) return S::raw2(fb[i * BXY]);
                     return S::raw2(fin[pidx(L, i, (long long)n)]);
                 };
                 float2 ue[3], um15;
@@ -748,9 +757,9 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             // a copy that never arrived leaves stale shared data: the
             // collision then stores garbage (at valid addresses), and the
             // step is reported as timed out
-            collide_at(z, j & 3, (j + 1) & 3, (j + 2) & 3, b, [&] {
+            collide_at(z, j, b, [&] {
                 const P *sb = stage + (size_t)b * PSTR;
-                if (TMA) return moments([&](int i) { return S::raw2(sb[i * BY * BX + own.st]); });
+                if (TMA) return moments([&](int i) { return S::raw2(sb[i * BXY + own.st]); });
                 const size_t n = own.xy + (size_t)nxy * z;
                 return moments([&](int i) { return S::raw2(fin[pidx(L, i, (long long)n)]); });
             });
@@ -762,99 +771,127 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             }
         }
     } else {
-        if (tid < C::HY) smask[tid] = 0ull;  // slot 0
+        // Iteration k takes in plane zb - 1 + k (densities of its own and at
+        // most one halo entry per thread, from the box) and collides the
+        // plane below.  One CTA barrier per plane suffices: iteration k
+        // writes ring slot k & 3 while slower threads may still collide with
+        // slots k - 1, k - 2, k - 3; a box's buffer is refilled after the
+        // barrier that follows its last reader; the row masks have eight
+        // slots, cleared two iterations before they are filled.
+        constexpr int MS = C::MSLOTS - 1;
+        if (tid < C::HY) smask[tid] = smask[C::HY + tid] = 0ull;  // slots 0 and 1
         __syncthreads();
-        issue(0, 0);
+        // plane copies: issued after the barrier of iteration k is box k +
+        // NST - LAG (with LAG the collision re-reads the box one iteration
+        // after its densities); a thread without TMA copies its own entries
+        // (never read by another) for k + 1 once it has taken in plane k
+        constexpr int LAG = C::RELAX_STAGE ? 2 : 0;
+        auto self_copy = [&](int k, int b) {
+            const int p = zb - 1 + k;
+            if (!pvalid(p)) return;
+            const size_t g = (size_t)nxy * gz_of(p);
+            P *d = const_cast<P *>(stage) + (size_t)b * PSTR;
+#pragma unroll
+            for (int i = 0; i < Q; i++) cp_async<sizeof(P)>(d + i * BXY + own.st, fin + pidx(L, i, (long long)(own.xy + g)));
+            if (has_halo)
+#pragma unroll
+                for (int i = 0; i < Q; i++)
+                    cp_async<sizeof(P)>(d + i * BXY + hal.st, fin + pidx(L, i, (long long)(hal.xy + g)));
+        };
+        // ψ of the solid entries of plane k straight into the ring, in flight
+        // until the plane is taken in
+        auto solid_psi = [&](int k, const Ent &e, uint8_t t) {
+            const int p = zb - 1 + k;
+            if (t == FLUID || !pvalid(p)) return;
+            const size_t n = e.xy + (size_t)nxy * gz_of(p);
+            float2 *d = sps + (k & 3) * HN + e.ring;  // (ψ_b, ψ_r): the partner first
+            cp_async<4>(&d->x, psi + (size_t)L.N + n);
+            cp_async<4>(&d->y, psi + n);
+        };
+        if (TMA) {
+#pragma unroll
+            for (int q = 0; q < NST; q++)
+                if (q < kmax) issue(q, q);
+        } else {
+            self_copy(0, 0);
+        }
         uint8_t t_own = load_type(0, own), t_hal = has_halo ? load_type(0, hal) : WALL;
-        float2 p_own = load_psi(0, own, t_own), p_hal = has_halo ? load_psi(0, hal, t_hal) : dup2(0.f);
+        solid_psi(0, own, t_own);
+        if (has_halo) solid_psi(0, hal, t_hal);
+        uint8_t tn_own = load_type(1, own), tn_hal = has_halo ? load_type(1, hal) : WALL;  // kmax >= 3
         Mom mcur{}, mnext{};
-            int b_cur = 0;  // stage buffer of iteration k
+        int b_cur = 0;  // stage buffer of iteration k
         for (int k = 0; k < kmax; k++) {
             const int b_next = b_cur + 1 == NST ? 0 : b_cur + 1;
             const int b_prev = b_cur == 0 ? NST - 1 : b_cur - 1;
-            if (k + 1 < kmax) issue(k + 1, b_next);
             const int p = zb - 1 + k;
             const bool pv = pvalid(p);
-            // types (and without SELF ψ) of the next plane: in flight during this iteration
-            uint8_t tn_own = WALL, tn_hal = WALL;
-            float2 pn_own = dup2(0.f), pn_hal = dup2(0.f);
-            if (k + 1 < kmax) {
-                tn_own = load_type(k + 1, own);
-                if (has_halo) tn_hal = load_type(k + 1, hal);
-                if (!SELF) {
-                    pn_own = load_psi(k + 1, own, tn_own);
-                    if (has_halo) pn_hal = load_psi(k + 1, hal, tn_hal);
-                }
-            }
             bool late = false;
             if (TMA && pv) {
                 late = !mbar_wait(&bar[b_cur], (unsigned)(waited.get(b_cur) & 1) ^ unreachable, limit);
                 if (!late) waited.inc(b_cur);
             }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            // this plane's entries into ring slot k & 3: ψ of fluid nodes,
+            // solid bits; the own node's moments
+            {
+                const P *sb = stage + (size_t)b_cur * PSTR;
+                const size_t gbase = pv ? (size_t)nxy * gz_of(p) : 0;
+                auto put_psi = [&](const Ent &e, float2 dr) {
+                    const float2 r = add2(make_float2(L.rref[0], L.rref[1]), dr);
+                    sps[(k & 3) * HN + e.ring] = make_float2(1.f - expf(-r.y), 1.f - expf(-r.x));  // (ψ_b, ψ_r)
+                };
+                unsigned long long *mrows = smask + (k & MS) * C::HY;
+                if (t_own == FLUID && pv) {
+                    if (!TMA || own.inlat) {
+                        mnext = moments([&](int i) { return S::raw2(sb[i * BXY + own.st]); });
+                    } else {
+                        const size_t n = own.xy + gbase;
+                        mnext = moments([&](int i) { return S::raw2(fin[pidx(L, i, (long long)n)]); });
+                    }
+                    put_psi(own, mnext.dr);
+                }
+                const unsigned so = __ballot_sync(0xffffffffu, t_own != FLUID);
+                if (tx == 0 && so) atomicOr(&mrows[own.ey], (unsigned long long)so << 1);
+                if (has_halo) {
+                    if (t_hal != FLUID) {
+                        atomicOr(&mrows[hal.ey], 1ull << hal.ex);
+                    } else if (pv) {
+                        float2 dr;
+                        if (!TMA || hal.inlat) {
+                            dr = density_sum([&](int i) { return S::raw2(sb[i * BXY + hal.st]); });
+                        } else {
+                            const size_t n = hal.xy + gbase;
+                            dr = density_sum([&](int i) { return S::raw2(fin[pidx(L, i, (long long)n)]); });
+                        }
+                        put_psi(hal, dr);
+                    }
+                }
+            }
+            if (!TMA && k + 1 < kmax) self_copy(k + 1, b_next);
             if (__syncthreads_or(late)) {
                 ok = false;
                 break;
             }
-            // this plane's entries into ring slot k & 3: ψ (formed here for
-            // fluid nodes with SELF), type, solid bits; the own node's moments
-            {
-                const int slot = k & 3;
-                const P *sb = stage + (size_t)b_cur * PSTR;
-                const size_t gbase = pv ? (size_t)nxy * gz_of(p) : 0;
-                auto entry = [&](const Ent &e, uint8_t t, float2 ps, bool is_own) {
-                    float2 pq = ps;  // (ψ_r, ψ_b)
-                    if (t == FLUID && pv && (SELF || is_own)) {
-                        float2 dr;
-                        if (e.inlat) {
-                            auto ld = [&](int i) { return S::raw2(sb[i * BY * BX + e.st]); };
-                            if (is_own) {
-                                mnext = moments(ld);
-                                dr = mnext.dr;
-                            } else {
-                                dr = density_sum(ld);
-                            }
-                        } else {
-                            const size_t n = e.xy + gbase;
-                            auto ld = [&](int i) { return S::raw2(fin[pidx(L, i, (long long)n)]); };
-                            if (is_own) {
-                                mnext = moments(ld);
-                                dr = mnext.dr;
-                            } else {
-                                dr = density_sum(ld);
-                            }
-                        }
-                        if (SELF) {
-                            const float2 r = add2(make_float2(L.rref[0], L.rref[1]), dr);
-                            pq = make_float2(1.f - expf(-r.x), 1.f - expf(-r.y));
-                        }
-                    }
-                    sps[slot * HN + e.ring] = make_float2(pq.y, pq.x);  // (ψ_b, ψ_r): the partner first
-                    if (t != FLUID) atomicOr(&smask[slot * C::HY + e.ey], 1ull << e.ex);
-                };
-                // without SELF an own entry of an inactive node holds no moments
-                entry(own, t_own, p_own, SELF || active);
-                if (has_halo) entry(hal, t_hal, p_hal, false);
+            // refill, the next plane's solid ψ, the types of the one after it
+            if (TMA && k >= LAG && k + NST - LAG < kmax) issue(k + NST - LAG, LAG == 0 ? b_cur : (b_cur + NST - LAG) % NST);
+            if (tid < C::HY) smask[((k + 2) & MS) * C::HY + tid] = 0ull;
+            if (k + 1 < kmax) {
+                t_own = tn_own;
+                t_hal = tn_hal;
+                solid_psi(k + 1, own, t_own);
+                if (has_halo) solid_psi(k + 1, hal, t_hal);
+                if (k + 2 < kmax) {
+                    tn_own = load_type(k + 2, own);
+                    if (has_halo) tn_hal = load_type(k + 2, hal);
+                }
             }
-            __syncthreads();
             // collision of plane z = p - 1 with ring planes z - 1, z, z + 1
-            if (k >= 2) collide_at(p - 1, (k - 2) & 3, (k - 1) & 3, k & 3, b_prev, [&] { return mcur; });
+            if (k >= 2) collide_at(p - 1, k - 2, b_prev, [&] { return mcur; });
             mcur = mnext;
-            // ring slot (k+1) & 3 was last read by the collision of iteration
-            // k - 1: clear its solid rows for the next iteration
-            if (tid < C::HY) smask[((k + 1) & 3) * C::HY + tid] = 0ull;
-            // SELF: ψ of the next plane's solid entries, now that their types are in
-            t_own = tn_own;
-            t_hal = tn_hal;
-            if (SELF && k + 1 < kmax) {
-                p_own = load_psi(k + 1, own, t_own);
-                if (has_halo) p_hal = load_psi(k + 1, hal, t_hal);
-            } else {
-                p_own = pn_own;
-                p_hal = pn_hal;
-            }
             b_cur = b_next;
-            __syncthreads();
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     if (TMA) {
         if (tid == 0) {
