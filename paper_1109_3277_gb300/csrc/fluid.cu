@@ -142,113 +142,25 @@ __device__ __forceinline__ int site_nb(const Lat &L, const Site &s, int i)
     return nidx(L, b, i);
 }
 
-// Batched form: lanes may belong to different boxes (key: the box, or -1
-// for a lane without a node); lanes of the same box share one atomic on the
-// box's counter.  Called by all 32 lanes.
-__device__ __forceinline__ void append_links_keyed(const LinkList &ll, int key, int n, uint32_t m)
-{
-    if (!__any_sync(0xffffffffu, m != 0)) return;
-    const unsigned grp = __match_any_sync(0xffffffffu, key);
-    const unsigned want = __ballot_sync(0xffffffffu, m != 0) & grp;
-    const int lane = threadIdx.x & 31;
-    const int leader = want ? __ffs(want) - 1 : lane;
-    int base = 0;
-    if (want && lane == leader) base = atomicAdd(ll.count, __popc(want));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (m) {
-        const int k = base + __popc(want & ((1u << lane) - 1u));
-        if (k < ll.cap) ll.ent[k] = make_uint2((unsigned)n, m);
-    }
-}
-
-// Node g of a batch (all boxes' nodes in box order) as a site of its box.
-__device__ __forceinline__ const BoxDev &batch_site(const BatchIndex &B, int g, Site &s)
-{
-    const int b = find_box(B.node0, B.nbox, g);
-    const BoxDev &bx = B.box[b];
-    const int n = g - B.node0[b];
-    s.n = n;
-    s.x = n % bx.L.nx;
-    const int t = n / bx.L.nx;
-    s.y = t % bx.L.ny;
-    s.z = t / bx.L.ny;
-    s.inner = s.x >= 1 && s.x <= bx.L.nx - 2 && s.y >= 1 && s.y <= bx.L.ny - 2 && s.z >= 1 && s.z <= bx.L.nz - 2;
-    return bx;
-}
-
-// Densities of the fluid nodes of all boxes, one node per thread (batched
-// boxes are small).
-template <class S>
-__global__ void __launch_bounds__(256) k_rho_batch(BatchIndex B, int total)
-{
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        Site s;
-        const BoxDev &bx = batch_site(B, g, s);
-        if (bx.type[s.n] != FLUID) continue;
-        const int b = find_box(B.node0, B.nbox, g);
-        const typename S::P *f = (const typename S::P *)bx.f[B.par[2 * b]];
-        const float2 r = node_rho2<S>(f, bx.L, s.n);
-        st_pair(bx.rho, s.n, r);
-        bx.psi[s.n] = 1.f - expf(-r.x);
-        bx.psi[(size_t)bx.L.N + s.n] = 1.f - expf(-r.y);
-    }
-}
-
 // ---------------------------------------------------------- shell fill
 // Solid nodes with at least one fluid neighbour take the mean ρ^c of those
 // neighbours (Eq. 10); the colour Δρ of the owning particle is added to red
-// if positive, else |Δρ| to blue.  Walls take Δρ = 0.  A particle node
-// among them returns the mask of its fluid neighbours (its links), 0
-// otherwise.
-
-__device__ __forceinline__ uint32_t shell_node(const Lat &L, const float *__restrict__ rho, float *__restrict__ psi,
-                                               const uint8_t *__restrict__ type, const uint32_t *__restrict__ owner,
-                                               const double *__restrict__ drho, const Site &s)
-{
-    const uint8_t t = type[s.n];
-    if (t == FLUID) return 0;
-    float dr = 0.f;
-    if (t == PART) {
-        uint32_t o = owner[s.n];
-        if (idx_ok(L, o, L.np, 1)) dr = (float)drho[o];
-    }
-    const uint32_t fm = shell_fill(L, rho, psi, type, s.n, dr, [&](int i) { return site_nb(L, s, i); });
-    return t == PART ? fm : 0u;
-}
+// if positive, else |Δρ| to blue.  Walls take Δρ = 0.
 
 __global__ void __launch_bounds__(128) k_shell(Lat L, const float *__restrict__ rho, float *__restrict__ psi,
                                                const uint8_t *__restrict__ type, const uint32_t *__restrict__ owner,
-                                               const double *__restrict__ drho, LinkList ll)
+                                               const double *__restrict__ drho)
 {
     Site s{};
-    const bool valid = site_of(L, s);
-    const uint32_t fm = valid ? shell_node(L, rho, psi, type, owner, drho, s) : 0u;
-    if (ll.ent) append_links(ll, s.n, fm);
-}
-
-__global__ void __launch_bounds__(256) k_shell_batch(BatchIndex B, int total)
-{
-    // warp-uniform trip count: every lane takes part in the appends
-    const int stride = gridDim.x * blockDim.x;
-    for (int w0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < total; w0 += stride) {
-        const int g = w0 + (threadIdx.x & 31);
-        int key = -1, n = 0;
-        uint32_t fm = 0;
-        LinkList ll{nullptr, nullptr, 0};
-        if (g < total) {
-            Site s;
-            const BoxDev &bx = batch_site(B, g, s);
-            const int b = find_box(B.node0, B.nbox, g);
-            fm = shell_node(bx.L, bx.rho, bx.psi, bx.type, bx.owner[B.par[2 * b + 1]], bx.P.drho, s);
-            ll = bx.links;
-            if (ll.ent)
-                key = b;
-            else
-                fm = 0;
-            n = s.n;
-        }
-        append_links_keyed(ll, key, n, fm);
+    if (!site_of(L, s)) return;
+    const uint8_t t = type[s.n];
+    if (t == FLUID) return;
+    float dr = 0.f;
+    if (t == PART) {
+        const uint32_t o = owner[s.n];
+        if (idx_ok(L, o, L.np, 1)) dr = (float)drho[o];
     }
+    shell_fill(L, rho, psi, type, s.n, dr, [&](int i) { return site_nb(L, s, i); });
 }
 
 // ------------------------------------------------------ collide + stream
@@ -560,27 +472,11 @@ void launch_rho(int storage, const Lat &L, const void *f, const uint8_t *type, f
                  (k_rho<S><<<blocks_for(L.N, 256), 256, 0, s>>>(L, (const typename S::P *)f, type, rho, psi)));
 }
 
-static unsigned batch_grid(int total)
-{
-    unsigned g = (unsigned)((total + 255) / 256);
-    return g > 8 * 152 ? 8 * 152 : (g ? g : 1);
-}
-
-void launch_rho_batch(int storage, const BatchIndex &B, int total_nodes, cudaStream_t s)
-{
-    LBE_DISPATCH(storage, (k_rho_batch<S><<<batch_grid(total_nodes), 256, 0, s>>>(B, total_nodes)));
-}
-
-void launch_shell_batch(const BatchIndex &B, int total_nodes, cudaStream_t s)
-{
-    k_shell_batch<<<batch_grid(total_nodes), 256, 0, s>>>(B, total_nodes);
-}
-
 void launch_shell(const Lat &L, const float *rho, float *psi, const uint8_t *type, const uint32_t *owner,
-                  const double *drho, const LinkList &ll, cudaStream_t s)
+                  const double *drho, cudaStream_t s)
 {
     dim3 grid((L.nx + 127) / 128, L.ny, L.nz);
-    k_shell<<<grid, 128, 0, s>>>(L, rho, psi, type, owner, drho, ll);
+    k_shell<<<grid, 128, 0, s>>>(L, rho, psi, type, owner, drho);
 }
 
 void launch_collide_stream(int storage, const Lat &L, const void *fin, void *fout, const float *psi,

@@ -10,13 +10,13 @@
 // per-row bitmask of solid nodes of the tile and a one-node halo go into a
 // four-slot ring of planes; the collision of plane z reads planes z-1, z
 // and z+1 of it.  Two configurations fill the ring:
-//  - ψ formed on chip (lattices without particles): the box also holds a
+//  - ψ formed on chip (lattices with no or few particles, batches): the box also holds a
 //    one-node halo (x widened to 16-byte boundaries), and each thread sums
 //    the densities of its node and of at most one halo node, so ψ of the
 //    tile and its halo comes from the stage; halo nodes beyond the lattice
 //    edge wrap around and are read from global memory.  Solid nodes (walls)
 //    take their ψ from the shell fill.
-//  - ψ from memory (lattices with particles): the density pass and the
+//  - ψ from memory (lattices with many particles): the density pass and the
 //    shell fill have written ψ of every node a fluid node sees.  The ring
 //    entries of plane z + 2 arrive by asynchronous copies issued before the
 //    collision of plane z and waited for after it.
@@ -35,6 +35,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "lbe_internal.cuh"
@@ -230,7 +231,6 @@ __device__ __forceinline__ void tma_box(void *dst, const CUtensorMap *map, int x
 // like its scalar form; the subtraction, which has no intrinsic, in PTX):
 // every component's result has the bits of the scalar sequence.
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b)
 {
@@ -923,49 +923,47 @@ __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF>::CTAS))
 }
 
 // Persistent multi-lattice variant: CTAs take tiles of all boxes of a batch
-// from one queue (largest boxes first in the queue order set by the host).
-// It runs the any-τ configuration with ψ from memory (the batch runs the
-// density kernel), which stores exactly what the other configurations
-// store: τ = 1 takes f^eq in the relaxation, and ψ from memory has the
-// bits of ψ formed in the kernel.
+// from one queue (largest boxes first in the queue order set by the host);
+// the first tile of a CTA is its own index.  ψ is formed on chip: a batch's
+// boxes hold few particles each.  GEN: some box needs any τ or
+// 64-bit offsets (it stores exactly what the τ = 1 configuration stores: τ =
+// 1 takes f^eq in the relaxation); otherwise all are τ = 1 with 32-bit offsets.
 constexpr int BATCH_TY = FUSED_TY_BATCH;
 
-template <class S>
-__global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, true, false>::CTAS)) k_fused_batch(BatchIndex B, int total)
+template <class S, bool GEN>
+__global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true>::CTAS)) k_fused_batch(BatchIndex B, int total)
 {
     constexpr int NT = TX * BATCH_TY;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = align128(smem_raw);
-    __shared__ int s_tile, s_box;
+    __shared__ int s_tile;
     __shared__ BoxDev sb;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_tile = atomicAdd(B.counter, 1);
-            s_box = s_tile < total ? find_box(B.tile0, B.nbox, s_tile) : 0;
-        }
-        __syncthreads();
-        const int t = s_tile;
-        if (t >= total) break;
+    int t = blockIdx.x;
+    while (t < total) {
         // the box descriptor into shared memory (word copy)
-        const int *src = reinterpret_cast<const int *>(B.box + s_box);
+        const int box = find_box(B.tile0, B.nbox, t);
+        const int *src = reinterpret_cast<const int *>(B.box + box);
         int *dstw = reinterpret_cast<int *>(&sb);
         for (int k = threadIdx.x; k < (int)(sizeof(BoxDev) / 4); k += NT) dstw[k] = src[k];
         __syncthreads();
-        const int lt = t - B.tile0[s_box];
+        const int lt = t - B.tile0[box];
         const int bx = lt % sb.ntx, by = (lt / sb.ntx) % sb.nty, bz = lt / (sb.ntx * sb.nty);
-        const int cur = B.par[2 * s_box];
+        const int cur = B.par[2 * box];
         // the tensor map stays in global memory (a TMA operand cannot be in shared memory)
-        const CUtensorMap *tm = &B.box[s_box].tmap[cur];
+        const CUtensorMap *tm = &B.box[box].tmap[cur];
         using P = typename S::P;
         bool ok;
         if (sb.tma)
-            ok = fused_tile<S, BATCH_TY, true, false, true, false>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
-                                                            sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
+            ok = fused_tile<S, BATCH_TY, GEN, true, true, !GEN>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
+                                                          sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         else
-            ok = fused_tile<S, BATCH_TY, true, false, false, false>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
-                                                             sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
+            ok = fused_tile<S, BATCH_TY, GEN, true, false, !GEN>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
+                                                           sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         if (!ok) break;
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = gridDim.x + atomicAdd(B.counter, 1);
+        __syncthreads();
+        t = s_tile;
     }
 }
 
@@ -980,15 +978,31 @@ __global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, true, false>::
         }                                                             \
     } while (0)
 
-int fused_zchunk(const Lat &L, int ty)
+int fused_zchunk(const Lat &L, int ty, int es, bool self, double share)
 {
-    // About 16 waves of CTAs (three per SM on 152 SMs), so the last wave's
-    // idle SMs cost little, each chunk long enough (>= 16 planes where the
-    // lattice allows) that its two extra halo planes cost little.
-    long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
-    int zc = L.nz;
-    while (zc > 16 && cols * ((L.nz + zc - 1) / zc) < 48 * 152) zc = (zc + 1) / 2;
-    return zc;
+    // A CTA's time is about (zc + 3) planes (two of halo, the start and the
+    // end), and a plane takes longer the more CTAs share the SM: measured 2.6
+    // us alone, 3.5 with two, 4.4 with three (64^3 f32).  The chunk that
+    // minimises this over the SMs (share: the part of the machine this
+    // lattice gets) keeps small lattices from leaving SMs idle, e.g. 64^3: 4
+    // planes 25 us, 16 planes 53.  With ψ formed on chip, chunks of more than
+    // 8 planes (FP32: 4) let the halo rows of the next chunk and the next
+    // rows of tiles leave L2 before they are read again: 256^3 f16 598 us at
+    // 8 planes, 652 at 16, 805 at 48; f32 964 at 4, 1095 at 16.  With ψ from
+    // memory (256^3 bijel, f16) 564 at 16, 601 at 64.
+    const long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
+    const int cap = self ? (es == 4 ? 4 : 8) : 16, slots = 3 * 8 / ty;
+    int best = 1;
+    double bt = 1e30;
+    for (int zc = 1; zc <= L.nz && zc <= cap; zc++) {
+        const double ctas = std::ceil(cols * std::ceil((double)L.nz / zc) / (152 * share));
+        const double t = (zc + 3) * (ctas <= slots ? 1.7 + 0.9 * ctas * ty / 8 : 4.4 * ctas / slots);
+        if (t < bt * 0.999) {
+            bt = t;
+            best = zc;
+        }
+    }
+    return best;
 }
 
 bool fused_tau1(const Lat &L) { return L.itau[0] == 1.f && L.itau[1] == 1.f; }
@@ -1100,7 +1114,7 @@ void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const 
                   const CUtensorMap *tmap, cudaStream_t s, int zc, int ty, int wait_limit, bool self)
 {
     const int rows = fused_rows(L, ty, tmap != nullptr);
-    if (zc <= 0) zc = fused_zchunk(L, rows);
+    if (zc <= 0) zc = fused_zchunk(L, rows, storage == LBE_STORE_F32 ? 4 : 2, self, 1.0);
     if (zc > L.nz) zc = L.nz;
     if (self)
         LBE_DISPATCH(storage, (launch_fused_t<S, true>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
@@ -1108,29 +1122,54 @@ void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const 
         LBE_DISPATCH(storage, (launch_fused_t<S, false>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
 }
 
-template <class S>
-static void launch_fused_batch_t(const BatchIndex &B, int total, int ctas, cudaStream_t s)
+template <class S, bool GEN>
+static void batch_configure()
 {
-    using C = Cfg<S, BATCH_TY, true, false>;
-    static bool configured = false;
+    static bool configured = false;  // the attribute is per function and process
     if (!configured) {
-        cudaFuncSetAttribute(k_fused_batch<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes);
+        cudaFuncSetAttribute(k_fused_batch<S, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)Cfg<S, BATCH_TY, GEN, true>::bytes);
         configured = true;
     }
-    k_fused_batch<S><<<ctas, C::NT, C::bytes, s>>>(B, total);
 }
 
-void launch_fused_batch(int storage, const BatchIndex &B, int total_tiles, int ctas, cudaStream_t s)
+template <class S, bool GEN>
+static void launch_fused_batch_t(const BatchIndex &B, int total, int ctas, cudaStream_t s)
 {
-    LBE_DISPATCH(storage, (launch_fused_batch_t<S>(B, total_tiles, ctas, s)));
+    using C = Cfg<S, BATCH_TY, GEN, true>;
+    batch_configure<S, GEN>();
+    k_fused_batch<S, GEN><<<ctas < total ? ctas : total, C::NT, C::bytes, s>>>(B, total);
 }
 
-int fused_batch_ctas_per_sm(int storage)
+// CTAs of the batched kernel an SM holds.  The shared-memory attribute comes
+// first: without it the query answers 0 for more than 48 KB, and batches ran
+// one CTA per SM (7 boxes of 48 x 48 x 40 f32: 131 us).
+template <class S, bool GEN>
+static int batch_occupancy()
 {
     int n = 0;
-    LBE_DISPATCH(storage, (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S>, TX * BATCH_TY,
-                                                                         Cfg<S, BATCH_TY, true, false>::bytes)));
+    batch_configure<S, GEN>();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S, GEN>, TX * BATCH_TY,
+                                                  Cfg<S, BATCH_TY, GEN, true>::bytes);
     return n > 0 ? n : 1;
+}
+
+void launch_fused_batch(int storage, const BatchIndex &B, int total_tiles, int ctas, bool general, cudaStream_t s)
+{
+    if (general)
+        LBE_DISPATCH(storage, (launch_fused_batch_t<S, true>(B, total_tiles, ctas, s)));
+    else
+        LBE_DISPATCH(storage, (launch_fused_batch_t<S, false>(B, total_tiles, ctas, s)));
+}
+
+int fused_batch_ctas_per_sm(int storage, bool general)
+{
+    int n = 1;
+    if (general)
+        LBE_DISPATCH(storage, (n = batch_occupancy<S, true>()));
+    else
+        LBE_DISPATCH(storage, (n = batch_occupancy<S, false>()));
+    return n;
 }
 
 }  // namespace lbe

@@ -34,6 +34,8 @@ struct lbe_ctx {
     double *mass_partials = nullptr, *mass_out = nullptr;
     // particles
     int np = 0, cap = 0;
+    double rmax = 0.0;     // largest radius of any particle
+    double area = 0.0;     // surface area of all particles (an upper estimate)
     double *pbuf = nullptr;
     float4 *x32 = nullptr;
     double *ppart = nullptr;
@@ -99,6 +101,7 @@ void bind_parts(lbe_ctx *c)
     auto at = [&](int off) { return b + (size_t)off * cp; };
     Parts &P = c->P;
     P.n = c->np;
+    P.rmax = std::nextafter((float)c->rmax, INFINITY);
     P.X = at(OX);
     P.q = at(OQ);
     P.V = at(OV);
@@ -203,11 +206,16 @@ __global__ void k_set_types(Lat L, uint8_t *type)
     type[n] = (L.walls && (z == 0 || z == L.nz - 1)) ? WALL : FLUID;
 }
 
-// The fused kernel forms ψ of the fluid nodes itself when no particle needs
-// the densities from memory (a lattice without particles runs no density
-// kernel); with particles, the density kernel feeds the shell fill and the
-// fused kernel reads ψ.
-bool fused_self(const lbe_ctx *c) { return c->np == 0; }
+// Whether the step runs the density pass and reads ψ from memory, or forms ψ
+// in the fused kernel (and sums the few densities the shell fill needs there).
+// The pass costs 76 B (FP32: 152 B) a node at the HBM rate, 12 ps in f16,
+// and forming ψ on chip about 10 ps a node more than reading it; the gathers
+// of the shell fill cost about 0.35 ns per fluid node next to a particle (479
+// us for 1.4 M of them), so the pass wins as soon as those are more than a
+// few percent of the lattice: 15 % oblate particles in 256^3 (f16) 786 + 100
+// us with the pass, 728 + 479 without.  Below, it saves the pass and a launch
+// (a single particle in 64^3 f32: 9 us of 55).
+bool fused_self(const lbe_ctx *c) { return 50.0 * c->area < (double)c->L.N; }
 
 // Tensor map of buffer `buf` for the fused kernel's mode and tile height
 // (null without TMA).
@@ -225,21 +233,16 @@ void enqueue_step(lbe_ctx *c)
     int st = c->d.storage;
     void *fin = c->f[c->cur], *fout = c->f[1 - c->cur];
     const bool two_pass = (c->d.flags & LBE_FLAG_TWO_PASS) != 0;
-    const bool links = c->np > 0 && !two_pass;
     if (two_pass) {
         launch_moments(st, L, fin, c->type, c->rho, c->psi, s);
-        launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, LinkList{nullptr, nullptr, 0}, s);
+        launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, s);
     } else {
-        if (links) cudaMemsetAsync(c->ll.count, 0, sizeof(int), s);
         // the solid nodes a fluid node can see: the particles' own nodes and
-        // the wall planes (none for a periodic lattice without particles);
-        // without particles the fused kernel forms the densities itself
-        if (c->np > 0) {
-            c->P.n = c->np;
-            launch_rho(st, L, fin, c->type, c->rho, c->psi, s);
-            launch_shell_particles(L, c->P, c->rho, c->psi, c->type, c->owner[c->ocur], c->ll, s);
-        }
-        launch_shell_walls(st, L, fin, c->psi, c->type, s);
+        // the wall planes (none for a periodic lattice without particles)
+        c->P.n = c->np;
+        const bool dense = !fused_self(c);
+        if (dense) launch_rho(st, L, fin, c->type, c->rho, c->psi, s);
+        launch_shell_fill(st, L, c->P, dense, fin, c->rho, c->psi, c->type, c->owner[c->ocur], c->ll, s);
     }
     if (c->profiling) {
         if (c->ev_used + 2 > c->ev.size()) {
@@ -604,6 +607,13 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
     CK(c, cudaMemcpy(c->x32, x32.data(), x32.size() * sizeof(float4), cudaMemcpyHostToDevice));
     c->np = np;
     c->L.np = np;
+    c->rmax = c->area = 0.0;
+    for (int p = 0; p < np; p++) {
+        const double rp = blk[ORP * cp + p], ro = blk[ORO * cp + p];
+        c->rmax = std::fmax(c->rmax, std::fmax(rp, ro));
+        // mean of the squared radii of the three axes (at least the area)
+        c->area += 4.0 * M_PI * std::sqrt((rp * rp * ro * ro * 2.0 + ro * ro * ro * ro) / 3.0);
+    }
     bind_parts(c);
     drop_graphs(c);
     cudaStream_t s = c->stream;
@@ -656,7 +666,7 @@ lbe_status lbe_read_fields(lbe_ctx *c, double *rho, double *vel, uint8_t *node_t
     const Lat &L = c->L;
     size_t N = (size_t)L.N;
     launch_moments(c->d.storage, L, c->f[c->cur], c->type, c->rho, c->psi, s);
-    launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, LinkList{nullptr, nullptr, 0}, s);
+    launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, s);
     double *dr = nullptr, *dv = nullptr;
     if (rho) CK(c, lib_malloc_async((void **)&dr, 2 * N * sizeof(double), s));
     if (vel) {
@@ -765,13 +775,13 @@ int32_t lbe_kernels_per_step(const lbe_ctx *c)
     if (!c) return 0;
     const bool two_pass = (c->d.flags & LBE_FLAG_TWO_PASS) != 0;
     // two-pass: densities, shell sweep, collide + stream; fused: the fused
-    // kernel, with particles the densities and the shell fill per
-    // particle, with walls the shell fill of the wall planes
+    // kernel, with particles or walls the shell fill, with many particles
+    // the densities
     int k = 0;
     if (two_pass)
         k = 3;
     else
-        k = 1 + (c->np > 0 ? 2 : 0) + (c->d.walls_z ? 1 : 0);
+        k = 1 + (c->np > 0 || c->d.walls_z ? 1 : 0) + (fused_self(c) ? 0 : 1);
     if (c->np > 0) {
         // links, pairs, the update (with the geometry of the new coverage);
         // from pairs_by_cells on the cell list (count, prefix, fill)
@@ -830,7 +840,10 @@ lbe_status lbe_autotune(lbe_ctx *c, int32_t *chosen_zc)
     // the next step overwrites anyway, so the state is not changed.
     const Lat &L = c->L;
     std::vector<int> zcs;
-    for (int zc = 4; zc < L.nz; zc *= 2) zcs.push_back(zc);
+    for (int zc = 2; zc < L.nz; zc *= 2) {
+        zcs.push_back(zc);
+        if (zc + zc / 2 < L.nz) zcs.push_back(zc + zc / 2);
+    }
     zcs.push_back(L.nz);
     std::vector<int> tys = {8};
     if (fused_rows(L, 4, c->tma) == 4) tys.push_back(4);
@@ -839,20 +852,22 @@ lbe_status lbe_autotune(lbe_ctx *c, int32_t *chosen_zc)
     CK(c, cudaEventCreate(&e1));
     void *fin = c->f[c->cur], *fout = c->f[1 - c->cur];
     // ψ of the solid nodes, as the step's shell fill gives them
-    launch_rho(c->d.storage, L, fin, c->type, c->rho, c->psi, c->stream);
-    launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, LinkList{nullptr, nullptr, 0}, c->stream);
+    c->P.n = c->np;
+    const bool self = fused_self(c);
+    if (!self) launch_rho(c->d.storage, L, fin, c->type, c->rho, c->psi, c->stream);
+    launch_shell_fill(c->d.storage, L, c->P, !self, fin, c->rho, c->psi, c->type, c->owner[c->ocur],
+                      LinkList{nullptr, nullptr, 0}, c->stream);
     float best = 1e30f;
     int best_zc = 0, best_ty = 8;
     for (int ty : tys)
         for (int zc : zcs) {
             const CUtensorMap *tm = fused_map(c, c->cur, ty);
-            const bool self = fused_self(c);
             launch_fused(c->d.storage, L, fin, fout, c->psi, c->type, tm, c->stream, zc, ty, FUSED_WAIT_LIMIT,
                          self);  // warm-up
             cudaEventRecord(e0, c->stream);
             for (int r = 0; r < 3; r++)
                 launch_fused(c->d.storage, L, fin, fout, c->psi, c->type, tm, c->stream, zc, ty, FUSED_WAIT_LIMIT,
-                             self);
+                         self);
             cudaEventRecord(e1, c->stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) break;
             float ms = 0.f;
@@ -904,7 +919,7 @@ lbe_status lbe_get_tile(const lbe_ctx *c, int32_t *rows, int32_t *zc)
         return LBE_OK;
     }
     *rows = fused_rows(c->L, c->ty_tuned, c->tma);
-    *zc = c->zc_tuned > 0 ? c->zc_tuned : fused_zchunk(c->L, *rows);
+    *zc = c->zc_tuned > 0 ? c->zc_tuned : fused_zchunk(c->L, *rows, (int)c->esize, fused_self(c), 1.0);
     return LBE_OK;
 }
 
@@ -937,7 +952,9 @@ struct lbe_batch {
     BoxDev *d_box = nullptr;
     int *d_idx = nullptr;             // tile0 | node0 | part0 | par | counter
     BatchIndex idx{};
-    int total_tiles = 0, total_nodes = 0, total_parts = 0;
+    int total_tiles = 0, total_parts = 0, total_walls = 0;
+    int ext[3] = {1, 1, 1};           // bound of the particle boxes
+    bool general = false;             // some member is not τ = 1 with 32-bit offsets
     int ctas_per_sm = 0;
     cudaGraphExec_t graph = nullptr;
     std::string err;
@@ -948,10 +965,9 @@ namespace {
 void batch_enqueue_step(lbe_batch *b)
 {
     cudaStream_t s = b->stream;
-    launch_rho_batch(b->storage, b->idx, b->total_nodes, s);
-    launch_shell_batch(b->idx, b->total_nodes, s);
-    cudaMemsetAsync(b->idx.counter, 0, sizeof(int), s);
-    launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * b->ctas_per_sm, s);
+    launch_begin_batch(b->idx, s);
+    launch_shell_batch(b->storage, b->idx, b->ext, b->total_parts, b->total_walls, s);
+    launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * b->ctas_per_sm, b->general, s);
     if (b->total_parts > 0) {
         launch_link_batch(b->storage, b->idx, s);
         launch_pairs_batch(b->idx, b->total_parts, s);
@@ -1030,8 +1046,10 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         b->order.push_back(idx0[k]);
     }
     std::vector<BoxDev> box(n);
+    double nodes = 0.0;
+    for (lbe_ctx *c : b->members) nodes += (double)c->L.N;
     std::vector<int> idx(3 * (n + 1) + 2 * n + 1, 0);
-    int *tile0 = idx.data(), *node0 = tile0 + (n + 1), *part0 = node0 + (n + 1), *par = part0 + (n + 1);
+    int *tile0 = idx.data(), *part0 = tile0 + (n + 1), *wall0 = part0 + (n + 1), *par = wall0 + (n + 1);
     for (int k = 0; k < n; k++) {
         lbe_ctx *c = b->members[k];
         BoxDev &d = box[k];
@@ -1039,8 +1057,8 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         d.ofs = fused_offsets(c->L);
         d.tma = c->tma ? 1 : 0;
         if (c->tma) {  // the batched kernel's tiles have FUSED_TY_BATCH = 8 rows
-            d.tmap[0] = c->tmap[0][0][0];  // ψ from memory: the batch runs the density kernel
-            d.tmap[1] = c->tmap[0][0][1];
+            d.tmap[0] = c->tmap[1][0][0];  // ψ formed in the kernel
+            d.tmap[1] = c->tmap[1][0][1];
         }
         d.f[0] = c->f[0];
         d.f[1] = c->f[1];
@@ -1054,19 +1072,22 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         d.pair = c->pair;
         d.mode = c->d.particle_mode;
         d.links = c->np > 0 ? c->ll : LinkList{nullptr, nullptr, 0};
-        d.zc = c->zc_tuned > 0 ? c->zc_tuned : fused_zchunk(c->L, FUSED_TY_BATCH);
+        d.zc = c->zc_tuned > 0 ? c->zc_tuned
+                               : fused_zchunk(c->L, FUSED_TY_BATCH, (int)c->esize, true, (double)c->L.N / nodes);
         d.ntx = (c->L.nx + FUSED_TX - 1) / FUSED_TX;
         d.nty = (c->L.ny + FUSED_TY_BATCH - 1) / FUSED_TY_BATCH;
         d.nzc = (c->L.nz + d.zc - 1) / d.zc;
         tile0[k + 1] = tile0[k] + d.ntx * d.nty * d.nzc;
-        node0[k + 1] = node0[k] + c->L.N;
         part0[k + 1] = part0[k] + c->np;
+        wall0[k + 1] = wall0[k] + batch_wall_tiles(c->L);
+        batch_shell_extent(c->L, d.P, b->ext);
+        if (!fused_tau1(c->L) || !fused_rel32(c->L)) b->general = true;
         par[2 * k] = c->cur;
         par[2 * k + 1] = c->ocur;
     }
     b->total_tiles = tile0[n];
-    b->total_nodes = node0[n];
     b->total_parts = part0[n];
+    b->total_walls = wall0[n];
     cudaError_t e = cudaMalloc((void **)&b->d_box, sizeof(BoxDev) * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_idx, idx.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void **)&b->d_quat, sizeof(double) * 4 * n);
@@ -1081,11 +1102,11 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
     b->idx.box = b->d_box;
     b->idx.nbox = n;
     b->idx.tile0 = b->d_idx;
-    b->idx.node0 = b->d_idx + (n + 1);
-    b->idx.part0 = b->d_idx + 2 * (n + 1);
+    b->idx.part0 = b->d_idx + (n + 1);
+    b->idx.wall0 = b->d_idx + 2 * (n + 1);
     b->idx.par = b->d_idx + 3 * (n + 1);
     b->idx.counter = b->idx.par + 2 * n;
-    b->ctas_per_sm = fused_batch_ctas_per_sm(b->storage);
+    b->ctas_per_sm = fused_batch_ctas_per_sm(b->storage, b->general);
     // link lists start empty; the last kernel of each batched step empties them
     for (lbe_ctx *c : b->members)
         if (c->np > 0 && c->ll.count) cudaMemsetAsync(c->ll.count, 0, sizeof(int), c->stream);
@@ -1140,7 +1161,7 @@ lbe_status lbe_batch_autotune(lbe_batch *b, int32_t *chosen_ctas_per_sm)
     // Persistent CTAs per SM for the batched fused kernel, timed on the
     // fused kernel alone (it writes only the spare buffers; the link sums it
     // accumulates are cleared afterwards).
-    const int maxc = fused_batch_ctas_per_sm(b->storage);
+    const int maxc = fused_batch_ctas_per_sm(b->storage, b->general);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -1150,7 +1171,7 @@ lbe_status lbe_batch_autotune(lbe_batch *b, int32_t *chosen_ctas_per_sm)
         for (int r = 0; r < 4; r++) {
             if (r == 1) cudaEventRecord(e0, b->stream);
             cudaMemsetAsync(b->idx.counter, 0, sizeof(int), b->stream);
-            launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * cps, b->stream);
+            launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * cps, b->general, b->stream);
         }
         cudaEventRecord(e1, b->stream);
         if (cudaEventSynchronize(e1) != cudaSuccess) break;

@@ -236,6 +236,7 @@ struct Parts {
     double *Fpend, *Tpend;          // fill/empty momentum for the next update
     double *F, *T;                  // total of the last update
     unsigned long long *fix;        // [6n] link force and torque in 2^-40 fixed point
+    float rmax;                     // largest radius
     int nsplit;                     // pair-force splits of the j range
     double *ppart;                  // [nsplit][6][n] pair-force partial sums
     float4 *X32;                    // FP32 (x, y, z, max radius) for the pair prefilter
@@ -259,27 +260,13 @@ constexpr double FIXED_UNIT = 1.0 / 1099511627776.0;  // 2^-40
 // its fluid neighbours, the colour Δρ added to red if positive, else |Δρ| to
 // blue, then ψ^c = 1 - exp(-ρ^c).  Nothing for a node without a fluid
 // neighbour (never read by a fluid node).  nb(i) is the neighbour index
-// along c_i, -1 beyond a wall; rho_of(m) gives (ρ^red, ρ^blue) of fluid node
-// m.  Returns the mask of fluid neighbours.
-template <class NB, class RHO>
-__device__ __forceinline__ uint32_t shell_fill_with(const Lat &L, float *__restrict__ psi,
-                                                    const uint8_t *__restrict__ type, int n, float dr, NB nb,
-                                                    RHO rho_of)
+// along c_i, -1 beyond a wall.
+// shell_psi takes the sums over its fluid neighbours, added in the order of the
+// directions.
+__device__ __forceinline__ void shell_psi(const Lat &L, float *__restrict__ psi, int n, float dr, float s0, float s1,
+                                          int cnt)
 {
-    float s0 = 0.f, s1 = 0.f;
-    int cnt = 0;
-    uint32_t fm = 0;
-#pragma unroll
-    for (int i = 1; i < Q; i++) {
-        const int m = nb(i);
-        if (m < 0 || type[m] != FLUID) continue;
-        const float2 r = rho_of(m);
-        s0 += r.x;
-        s1 += r.y;
-        cnt++;
-        fm |= 1u << i;
-    }
-    if (cnt == 0) return 0;
+    if (cnt == 0) return;
     float r0 = s0 / (float)cnt, r1 = s1 / (float)cnt;
     if (dr > 0.f)
         r0 += dr;
@@ -287,16 +274,25 @@ __device__ __forceinline__ uint32_t shell_fill_with(const Lat &L, float *__restr
         r1 += fabsf(dr);
     psi[n] = 1.f - expf(-r0);
     psi[(size_t)L.N + n] = 1.f - expf(-r1);
-    return fm;
 }
 
-// The same with the neighbours' densities from the array rho[2][N].
+// The fill of one node with the neighbours' densities from the array rho.
 template <class NB>
-__device__ __forceinline__ uint32_t shell_fill(const Lat &L, const float *__restrict__ rho, float *__restrict__ psi,
-                                               const uint8_t *__restrict__ type, int n, float dr, NB nb)
+__device__ __forceinline__ void shell_fill(const Lat &L, const float *__restrict__ rho, float *__restrict__ psi,
+                                           const uint8_t *__restrict__ type, int n, float dr, NB nb)
 {
-    return shell_fill_with(L, psi, type, n, dr, nb,
-                           [&](int m) { return ld_pair(rho, m); });
+    float s0 = 0.f, s1 = 0.f;
+    int cnt = 0;
+#pragma unroll
+    for (int i = 1; i < Q; i++) {
+        const int m = nb(i);
+        if (m < 0 || type[m] != FLUID) continue;
+        const float2 r = ld_pair(rho, m);
+        s0 += r.x;
+        s1 += r.y;
+        cnt++;
+    }
+    shell_psi(L, psi, n, dr, s0, s1, cnt);
 }
 
 // Append (n, m) for the lanes with m != 0 to a link list: one atomic per
@@ -368,11 +364,12 @@ struct BoxDev {
     int zc, ntx, nty, nzc;   // fused-kernel tiling of this box
 };
 
-// Prefix offsets of the boxes' work items (tiles, nodes, particles).
+// Prefix offsets of the boxes' work items (fused-kernel tiles, particles, wall
+// tiles of the shell fill).
 struct BatchIndex {
     const BoxDev *box;
     int nbox;
-    const int *tile0, *node0, *part0;   // [nbox + 1]
+    const int *tile0, *part0, *wall0;   // [nbox + 1]
     int *par;                           // [2 nbox]: cur, ocur
     int *counter;                       // persistent tile queue of the fused kernel
 };
@@ -384,18 +381,10 @@ void launch_moments(int storage, const Lat &L, const void *f, const uint8_t *typ
                     float *psi, cudaStream_t s);
 void launch_rho(int storage, const Lat &L, const void *f, const uint8_t *type, float *rho, float *psi,
                 cudaStream_t s);
-void launch_shell(const Lat &L, const float *rho, float *psi, const uint8_t *type,
-                  const uint32_t *owner, const double *drho, const LinkList &ll, cudaStream_t s);
-// Shell fill of the particles' own nodes (one CTA per particle over its
-// candidate rows) and of the wall planes: the solid nodes a fluid node can
-// see, without a sweep of the lattice.
-// Shell fill of the particles' own nodes (one CTA per particle over its
-// candidate rows), with the neighbours' densities from rho, and of the wall
-// planes, with the densities of the planes next to the walls computed from
-// the populations f (a lattice without particles runs no density kernel).
-void launch_shell_particles(const Lat &L, const Parts &P, const float *rho, float *psi, const uint8_t *type,
-                            const uint32_t *owner, const LinkList &ll, cudaStream_t s);
-void launch_shell_walls(int storage, const Lat &L, const void *f, float *psi, const uint8_t *type, cudaStream_t s);
+// Shell sweep of a whole lattice with the densities of rho (reads, and the
+// two-pass step).
+void launch_shell(const Lat &L, const float *rho, float *psi, const uint8_t *type, const uint32_t *owner,
+                  const double *drho, cudaStream_t s);
 void launch_collide_stream(int storage, const Lat &L, const void *fin, void *fout, const float *psi,
                            const uint8_t *type, cudaStream_t s);
 void launch_fields(int storage, const Lat &L, const void *f, const float *psi, const uint8_t *type,
@@ -407,10 +396,15 @@ void launch_set_f(int storage, const Lat &L, const double *in, void *f, cudaStre
 int mass_blocks();
 
 // ---- batched launchers (one launch steps every box of a batch) -------------
-void launch_rho_batch(int storage, const BatchIndex &B, int total_nodes, cudaStream_t s);
-void launch_shell_batch(const BatchIndex &B, int total_nodes, cudaStream_t s);
-void launch_fused_batch(int storage, const BatchIndex &B, int total_tiles, int ctas, cudaStream_t s);
-int fused_batch_ctas_per_sm(int storage);
+void launch_begin_batch(const BatchIndex &B, cudaStream_t s);
+// ext: bound of the particle boxes of all members (batch_shell_extent).
+void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, int total_walls,
+                        cudaStream_t s);
+int batch_wall_tiles(const Lat &L);
+void batch_shell_extent(const Lat &L, const Parts &P, int ext[3]);
+// general: some member needs any-τ or 64-bit offsets.
+void launch_fused_batch(int storage, const BatchIndex &B, int total_tiles, int ctas, bool general, cudaStream_t s);
+int fused_batch_ctas_per_sm(int storage, bool general);
 void launch_pairs_batch(const BatchIndex &B, int total_parts, cudaStream_t s);
 void launch_integrate_batch(const BatchIndex &B, int total_parts, cudaStream_t s);
 void launch_geom_batch(const BatchIndex &B, int total_parts, cudaStream_t s);
@@ -433,7 +427,9 @@ constexpr int FUSED_WAIT_LIMIT = 1 << 22;
 // holds ψ of every node (density kernel and shell fill).
 void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
                   const CUtensorMap *tmap, cudaStream_t s, int zc, int ty, int wait_limit, bool self);
-int fused_zchunk(const Lat &L, int ty);
+// The default z chunk for tiles of ty rows, populations of es bytes, and a
+// lattice that gets the given share of the GPU (1, or less in a batch).
+int fused_zchunk(const Lat &L, int ty, int es, bool self, double share);
 // The tile height launch_fused takes for a request (4 only where built).
 int fused_rows(const Lat &L, int ty_request, bool tma);
 bool fused_tau1(const Lat &L);
@@ -460,6 +456,13 @@ __device__ __forceinline__ int find_box(const int *off, int nbox, int i)
 }
 
 // ---- launchers (particles.cu) ---------------------------------------------
+// Shell fill of the particles' own nodes and of the wall planes (the solid
+// nodes a fluid node can see); the particles' nodes with fluid neighbours go
+// into the link list.  dense: rho holds the densities (launch_rho); otherwise
+// those next to the particles are summed from the populations f, and go into
+// rho for the link kernel.  No launch without particles and walls.
+void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
+                       const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s);
 void launch_links(int storage, const Lat &L, const Parts &P, void *fnew, const float *rho,
                   const uint8_t *type, const uint32_t *owner, cudaStream_t s);
 void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,

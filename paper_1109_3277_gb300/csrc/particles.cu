@@ -6,6 +6,9 @@
 // Per-particle work runs one CTA per particle over the particle's bounding
 // box; per-particle sums are FP64 and reduced in a fixed order, so results
 // are bit-reproducible run to run.
+#include <algorithm>
+#include <cmath>
+
 #include "lbe_internal.cuh"
 
 namespace lbe {
@@ -13,6 +16,12 @@ namespace lbe {
 namespace {
 
 constexpr int PT = 128;  // threads per per-particle CTA
+
+// Tiles of a particle's box in the shell fill: nx x ny x nz of them, of 30 x
+// tyi x tzi nodes.
+struct ShellGrid {
+    int nx, ny, nz, tyi, tzi;
+};
 
 // ---------------------------------------------------------- geometry (FP64)
 // The inside test is written with explicit round-to-nearest intrinsics so
@@ -71,17 +80,6 @@ struct Geo {
     double ip2, io2;
     float ip2f, io2f;
 };
-
-__device__ void geo_of(const double *q, double rp, double ro, Geo &g)
-{
-    rotmat(q, g.R);
-    for (int a = 0; a < 3; a++)
-        for (int b = 0; b < 3; b++) g.R32[a][b] = (float)g.R[a][b];
-    g.ip2 = __ddiv_rn(1.0, m_(rp, rp));
-    g.io2 = __ddiv_rn(1.0, m_(ro, ro));
-    g.ip2f = (float)g.ip2;
-    g.io2f = (float)g.io2;
-}
 
 // Inside test: an FP32 evaluation decides unless it lies within 1e-3 of the
 // surface, where the exact FP64 evaluation (oracle operation order) decides.
@@ -204,16 +202,19 @@ __device__ __forceinline__ bool is_wall_z(const Lat &L, int z) { return L.walls 
 // at most 1.  The interval of the quadric at most QSPAN, widened by a node
 // on each side, holds all of them whatever the FP32 rounding of its
 // computation (relative errors ~1e-6 against a margin of ~1% of the radii),
-// so only those candidates are tested.  Boxes that span a whole period use
+// so only those candidates are looked at.  Boxes that span a whole period use
 // the plain box loop.
 constexpr float QSPAN = 1.02f;
 
 // x interval [xa, xb] (unwrapped, clamped to the box) of row (u1, u2) for
-// the ellipsoid g at X; xa > xb when the row misses it.
-__device__ __forceinline__ void row_span(const Geo &g, const double X[3], const Box &b, int u1, int u2, int &xa,
-                                         int &xb)
+// the ellipsoid g at Xi + Xf (integer and fraction, so that FP32 displacements
+// carry no cancellation); xa > xb when the row misses it.  All in FP32: with
+// the conversions in FP64, whose rate is 1/64 of FP32's, they bounded the
+// coverage kernels.
+__device__ __forceinline__ void row_span(const Geo &g, const int Xi[3], const float Xf[3], const Box &b, int u1, int u2,
+                                         int &xa, int &xb)
 {
-    const float dy = (float)((double)u1 - X[1]), dz = (float)((double)u2 - X[2]);
+    const float dy = (float)(u1 - Xi[1]) - Xf[1], dz = (float)(u2 - Xi[2]) - Xf[2];
     const float w[3] = {g.ip2f, g.io2f, g.io2f};
     float A = 0.f, B = 0.f, C = -QSPAN;
 #pragma unroll
@@ -228,10 +229,14 @@ __device__ __forceinline__ void row_span(const Geo &g, const double X[3], const 
     xb = 0;
     if (!(D >= 0.f) || !(A > 0.f)) return;
     const float sq = sqrtf(D), ia = 0.5f / A;
-    const double lo = X[0] + (double)((-B - sq) * ia), hi = X[0] + (double)((-B + sq) * ia);
-    if (!(lo >= -2e9 && hi <= 2e9)) return;
-    xa = max((int)floor(lo) - 1, b.lo[0]);
-    xb = min((int)ceil(hi) + 1, b.lo[0] + b.ext[0] - 1);
+    const float lo = Xf[0] + (-B - sq) * ia, hi = Xf[0] + (-B + sq) * ia;
+    if (!(lo >= -1e6f && hi <= 1e6f)) {  // beyond any lattice: the whole box row
+        xa = b.lo[0];
+        xb = b.lo[0] + b.ext[0] - 1;
+        return;
+    }
+    xa = max(Xi[0] + (int)floorf(lo) - 1, b.lo[0]);
+    xb = min(Xi[0] + (int)ceilf(hi) + 1, b.lo[0] + b.ext[0] - 1);
 }
 
 __device__ __forceinline__ bool box_full(const Box &b) { return b.full[0] || b.full[1] || b.full[2]; }
@@ -261,11 +266,11 @@ struct RowEval {  // the FP32 quadric along a row
     }
 };
 
-__device__ __forceinline__ RowSpan span_of(const Geo &g, const double X[3], const int Xi[3], const float Xf[3],
-                                           const Box &b, int u1, int u2)
+__device__ __forceinline__ RowSpan span_of(const Geo &g, const int Xi[3], const float Xf[3], const Box &b, int u1,
+                                           int u2)
 {
     RowSpan r;
-    row_span(g, X, b, u1, u2, r.oa, r.ob);
+    row_span(g, Xi, Xf, b, u1, u2, r.oa, r.ob);
     RowEval q;
     const float dy = (float)(u1 - Xi[1]) - Xf[1], dz = (float)(u2 - Xi[2]) - Xf[2];
 #pragma unroll
@@ -336,94 +341,6 @@ __device__ __forceinline__ void for_box(const Box &b, F f)
     }
 }
 
-// Every candidate node of a particle's box, each visited once.  Each warp
-// takes chunks of 32 rows: lane l computes the NSEG disjoint segments
-// [xs[j], xe[j]] of row l of the chunk (spans(u1, u2, xs, xe), empty when
-// xs > xe, clamped to the box); a warp prefix over the rows' candidate
-// counts flattens them, and the lanes take consecutive candidates.  No
-// barrier: the warps of a CTA work on their own rows.  node(ux, u1, u2,
-// valid) is called by all 32 lanes of a warp in whole passes (valid =
-// false past the end), so it may use warp votes.  A box that spans a whole
-// period visits all its nodes.
-template <int NSEG, class SP, class F>
-__device__ __forceinline__ void for_segments(const Box &b, SP spans, F node)
-{
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (box_full(b)) {
-        for (int k0 = warp * 32; k0 < b.count; k0 += nw * 32) {
-            const int k = k0 + lane;
-            const bool valid = k < b.count;
-            const int kk = valid ? k : 0;
-            const int t = kk / b.ext[0];
-            node(b.lo[0] + kk % b.ext[0], b.lo[1] + t % b.ext[1], b.lo[2] + t / b.ext[1], valid);
-        }
-        return;
-    }
-    const int rows = b.ext[1] * b.ext[2];
-    for (int r0 = warp * 32; r0 < rows; r0 += nw * 32) {
-        const int r = r0 + lane;
-        int xs[NSEG], len[NSEG];
-        int tot = 0;
-        if (r < rows) {
-            int xe[NSEG];
-            spans(b.lo[1] + r % b.ext[1], b.lo[2] + r / b.ext[1], xs, xe);
-#pragma unroll
-            for (int j = 0; j < NSEG; j++) {
-                len[j] = max(0, xe[j] - xs[j] + 1);
-                tot += len[j];
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < NSEG; j++) {
-                xs[j] = 0;
-                len[j] = 0;
-            }
-        }
-        int incl = tot;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(full, incl, off);
-            if (lane >= off) incl += v;
-        }
-        const int excl = incl - tot;
-        const int total = __shfl_sync(full, incl, 31);
-        for (int k0 = 0; k0 < total; k0 += 32) {
-            const int k = k0 + lane;
-            const bool valid = k < total;
-            // the row (lane) holding candidate k: last lane with excl <= k
-            int src = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int e = __shfl_sync(full, excl, src + step);
-                if (e <= k) src += step;
-            }
-            int rem = k - __shfl_sync(full, excl, src);
-            int ux = 0;
-            bool found = false;
-#pragma unroll
-            for (int j = 0; j < NSEG; j++) {
-                const int xj = __shfl_sync(full, xs[j], src), lj = __shfl_sync(full, len[j], src);
-                if (!found && rem < lj) {
-                    ux = xj + rem;
-                    found = true;
-                } else if (!found) {
-                    rem -= lj;
-                }
-            }
-            const int rr = r0 + src;
-            node(ux, b.lo[1] + rr % b.ext[1], b.lo[2] + rr / b.ext[1], valid);
-        }
-    }
-}
-
-// The candidates of one ellipsoid (g at X) in box b.
-template <class F>
-__device__ __forceinline__ void for_candidates(const Box &b, const Geo &g, const double X[3], F node)
-{
-    for_segments<1>(b, [&](int u1, int u2, int *xs, int *xe) { row_span(g, X, b, u1, u2, xs[0], xe[0]); }, node);
-}
-
 // ---- coverage geometry ----------------------------------------------------
 // The geometry the coverage kernels need of a particle, computed once per
 // step by one thread per particle (k_geom) instead of by every CTA: the
@@ -443,7 +360,8 @@ struct PGeom {
 // the two boxes.
 struct PGeom2 {
     PGeom old_, now;
-    double Xu[3];
+    int Xui[3];    // the new centre next to the old one: integer and fraction
+    float Xuf[3];
     Box uni;
 };
 
@@ -502,7 +420,7 @@ __device__ __forceinline__ bool quad_empty(double lo, double hi)
 
 // finish_box for axis k (lanes 0..2 of a quad write their axis, lane 0 the
 // count).
-__device__ __forceinline__ int quad_box(const Lat &L, int k, bool wr, bool empty, double lo, double hi, Box &b)
+__device__ __forceinline__ void quad_box(const Lat &L, int k, bool wr, bool empty, double lo, double hi, Box &b)
 {
     const double n = (double)ext_of(L, k);
     int fullp = 0;
@@ -526,7 +444,6 @@ __device__ __forceinline__ int quad_box(const Lat &L, int k, bool wr, bool empty
         b.full[k] = fullp;
         if (k == 0) b.count = count;
     }
-    return count;
 }
 
 // Geometry of particle p after an update: the last geometry becomes the old
@@ -556,7 +473,7 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
     double lo, hi;
     box_axis(X, h, lo, hi);
     const bool empty = quad_empty(lo, hi);
-    const int count = quad_box(L, k, wr, empty, lo, hi, G.now.box);
+    quad_box(L, k, wr, empty, lo, hi, G.now.box);
     const double fl = floor(X);
     if (wr) {
         for (int j = 0; j < 3; j++) {
@@ -567,9 +484,10 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
         G.now.lo[k] = lo;
         G.now.hi[k] = hi;
         // X = Xi + Xf, Xi integral: the FP32 displacement (u - Xi) - Xf
-        // carries no large cancellation (box_axis bounds |X| < 1e9)
-        G.now.Xi[k] = count ? (int)fl : 0;
-        G.now.Xf[k] = (float)(X - fl);
+        // carries no large cancellation (box_axis bounds |X| < 1e9); NaN,
+        // which no row meets, for geometry without a box
+        G.now.Xi[k] = empty ? 0 : (int)fl;
+        G.now.Xf[k] = empty ? NAN : (float)(X - fl);
     }
     if (first && act && lane < 2) {  // the radii never change
         const double inv = __ddiv_rn(1.0, lane == 0 ? m_(rp, rp) : m_(ro, ro));
@@ -591,7 +509,11 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
         hi0 = fmax(hi0, hu);
     }
     quad_box(L, k, wr, e0 && eu, lo0, hi0, G.uni);
-    if (wr) G.Xu[k] = Xu;
+    const double flu = floor(Xu);
+    if (wr) {
+        G.Xui[k] = eu ? 0 : (int)flu;
+        G.Xuf[k] = eu ? NAN : (float)(Xu - flu);
+    }
     __syncwarp();
     if (first) copy_now();
 }
@@ -1441,7 +1363,7 @@ __device__ __forceinline__ void claim_body(const Lat &L, const Parts &P, int p, 
     for_rows(box, [&](bool valid, int u1, int u2) {
         int a = 1, b = 0;
         if (valid && !is_wall_z(L, wrapi(u2, L.nz))) {
-            const RowSpan r = span_of(G.g, G.X, G.Xi, G.Xf, box, u1, u2);
+            const RowSpan r = span_of(G.g, G.Xi, G.Xf, box, u1, u2);
             // the FP64 test for the nodes between the two bounds
             auto in = [&](int ux) {
                 const double dx[3] = {s_((double)ux, G.X[0]), s_((double)u1, G.X[1]), s_((double)u2, G.X[2])};
@@ -1608,11 +1530,8 @@ __device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, in
         for_rows(box, [&](bool valid, int u1, int u2) {
             int a = 1, b = 0, ca = 1, cb = 0;  // nodes [a, b] but for [ca, cb]
             if (valid) {
-                const float uf[3] = {(float)(G2.Xu[0] - floor(G2.Xu[0])), (float)(G2.Xu[1] - floor(G2.Xu[1])),
-                                     (float)(G2.Xu[2] - floor(G2.Xu[2]))};
-                const int ui[3] = {(int)floor(G2.Xu[0]), (int)floor(G2.Xu[1]), (int)floor(G2.Xu[2])};
-                const RowSpan s0 = span_of(G2.old_.g, G2.old_.X, G2.old_.Xi, G2.old_.Xf, box, u1, u2);
-                const RowSpan s1 = span_of(G2.now.g, G2.Xu, ui, uf, box, u1, u2);
+                const RowSpan s0 = span_of(G2.old_.g, G2.old_.Xi, G2.old_.Xf, box, u1, u2);
+                const RowSpan s1 = span_of(G2.now.g, G2.Xui, G2.Xuf, box, u1, u2);
                 if (s0.oa > s0.ob) {
                     a = s1.oa;
                     b = s1.ob;
@@ -1683,7 +1602,7 @@ __device__ __forceinline__ void reset_body(const Lat &L, const Parts &P, int p, 
     }
     for_rows(G.box, [&](bool valid, int u1, int u2) {
         int a = 1, b = 0;
-        if (valid) row_span(G.g, G.X, G.box, u1, u2, a, b);
+        if (valid) row_span(G.g, G.Xi, G.Xf, G.box, u1, u2, a, b);
         fill_rows(L, a, b, u1, u2, [&](int n) {
             if (idx_ok(L, n, L.N, 7)) owner[n] = NONE;
         });
@@ -1696,82 +1615,343 @@ __global__ void __launch_bounds__(PT) k_reset(Lat L, Parts P, int use_old, uint3
 }
 
 // ---------------------------------------------------------------- shell
-// Shell fill (Eq. 10 and the colour rule) of the nodes particle p owns,
-// over its candidate rows; its nodes with fluid neighbours enter the link
-// list.  With the wall planes these are all the solid nodes a fluid node
-// can see.
-// The densities of the fluid neighbours come from the density kernel.
-// A particle's link entries go into the list as one contiguous segment
+// Shell fill (Eq. 10 and the colour rule) of the nodes particle p owns and of
+// the wall planes: all the solid nodes a fluid node can see.  The particle
+// nodes with fluid neighbours enter the link list.
+//
+// A CTA takes one tile of a particle's box (30 x TYI x TZI nodes).  The node
+// types of the tile and a one-node halo become one 32-bit mask per row of x
+// (fluid nodes), so that finding the shell nodes (a candidate next to a
+// fluid node) and the fluid nodes next to them is a few shifts per row
+// instead of 18 byte loads per node.  The density of each such fluid node
+// goes into shared memory once, and every shell node takes the mean over its
+// neighbours from there.  The densities are read from rho (DENSE: a density
+// pass over the whole lattice ran before), or summed here from the
+// populations and stored to rho for the link kernel.  The latter needs no
+// pass but gathers 19 scattered 32-byte sectors per node (about 450 nodes per
+// (8, 4, 4) ellipsoid): at 15 % oblate ellipsoids in 256^3 (f16) that was 1.5
+// GB of DRAM traffic, more than the 1.3 GB of the pass, and 479 us against
+// the pass's 225; it pays where particles are few (dense_rho).
+//
+// Tiles: with many particles 22 x 22 rows (an ellipsoid of reach 8 is one
+// tile); with few, 10 x 5 rows, so that one particle spreads over several
+// SMs (the halo rows are then 68 % more rows, which costs less than idle
+// SMs).  Results do not depend on the tiling.
+//
+// A tile's link entries go into the list as one contiguous segment
 // (collected in shared memory, then one reservation and a coalesced copy),
-// so that the link kernel, which walks the list in order, handles the
-// links of one particle together: their slots share cache lines.  Entries
-// beyond the buffer (very large particles) are appended directly.
-constexpr int SHELL_BUF = 1024;
+// so that the link kernel, which walks the list in order, handles
+// neighbouring links together: their slots share cache lines.  Entries
+// beyond the buffer are appended directly.
+constexpr int SHELL_BUF = 1024;   // link entries collected per tile
+constexpr int SHELL_RHO = 1024;   // densities held per tile (the rest are read back from rho)
+constexpr int SHELL_X = 30;       // nodes of a tile along x: a mask word less the halo
+constexpr int SHELL_ROWS = 24 * 24;
 
-__global__ void __launch_bounds__(PT) k_shell_particles(Lat L, Parts P, const float *__restrict__ rho,
-                                                        float *__restrict__ psi, const uint8_t *__restrict__ type,
-                                                        const uint32_t *__restrict__ owner, LinkList ll)
+struct ShellTile {
+    uint32_t S[SHELL_ROWS];      // candidate nodes (bit b: x = x0 - 1 + b), then shell nodes
+    uint32_t F[SHELL_ROWS];      // fluid nodes
+    uint32_t M[SHELL_ROWS];      // particle nodes, then fluid nodes next to a shell node
+    int base[SHELL_ROWS];        // node index of the row's x = 0, -1 beyond a wall
+    uint32_t start[SHELL_ROWS];  // fluid nodes (low half) and shell nodes (high half) of the rows before
+    float2 rho[SHELL_RHO];
+    uint2 buf[SHELL_BUF];
+    uint32_t wsum[PT / 32];
+    int nbuf, lbase;
+};
+
+// The j-th (from 0) set bit of m.
+__device__ __forceinline__ int nth_bit(uint32_t m, int j)
 {
-    __shared__ uint2 buf[SHELL_BUF];
-    __shared__ int nbuf, base;
-    const int p = blockIdx.x;
-    const PGeom &G = reinterpret_cast<const PGeom2 *>(P.geo)[p].now;
-    const Box &box = G.box;
-    const Geo &geo = G.g;
-    const double *sX = G.X;
-    const float dr = (float)P.drho[p];
-    if (threadIdx.x == 0) nbuf = 0;
-    __syncthreads();
-    for_candidates(box, geo, sX, [&](int ux, int u1, int u2, bool valid) {
-        int n = 0;
-        uint32_t fm = 0;
-        if (valid) {
-            const int x = wrapi(ux, L.nx), y = wrapi(u1, L.ny), z = wrapi(u2, L.nz);
-            n = x + L.nx * (y + L.ny * z);
-            if (owner[n] == (uint32_t)p)
-                fm = shell_fill(L, rho, psi, type, n, dr, [&](int i) { return nbr_node(L, x, y, z, i); });
+    int pos = 0;
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+        const int c = __popc(m & ((1u << w) - 1u));
+        if (j >= c) {
+            j -= c;
+            m >>= w;
+            pos += w;
         }
-        if (!ll.ent) return;
-        const unsigned want = __ballot_sync(0xffffffffu, fm != 0);
-        if (!want) return;
-        const int lane = threadIdx.x & 31, leader = __ffs(want) - 1;
-        int k0 = 0;
-        if (lane == leader) k0 = atomicAdd(&nbuf, __popc(want));
-        k0 = __shfl_sync(0xffffffffu, k0, leader);
-        const int k = k0 + __popc(want & ((1u << lane) - 1u));
-        const bool spill = fm != 0 && k >= SHELL_BUF;
-        if (fm && !spill) buf[k] = make_uint2((unsigned)n, fm);
-        append_links(ll, n, spill ? fm : 0u);
-    });
-    if (!ll.ent) return;
-    __syncthreads();
-    const int cnt = min(nbuf, SHELL_BUF);
-    if (threadIdx.x == 0) base = cnt ? atomicAdd(ll.count, cnt) : 0;
-    __syncthreads();
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x)
-        if (base + k < ll.cap) ll.ent[base + k] = buf[k];
+    }
+    return pos;
 }
 
-// Shell fill of the wall planes z = 0 and nz - 1 (Δρ = 0), with the
-// densities of the neighbouring planes' fluid nodes from the populations.
-template <class S>
-__global__ void k_shell_walls(Lat L, const typename S::P *__restrict__ f, float *__restrict__ psi,
-                              const uint8_t *__restrict__ type)
+// Bits of a row that have a neighbour (one of the 18) in the rows m[9] around
+// it (index (dy + 1) + 3 (dz + 1), the row itself at 4).
+__device__ __forceinline__ uint32_t dilate18(const uint32_t m[9])
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nxy = L.nx * L.ny;
-    if (k >= 2 * nxy) return;
-    const int z = k < nxy ? 0 : L.nz - 1, r = k < nxy ? k : k - nxy;
-    const int x = r % L.nx, y = r / L.nx;
-    const int n = x + L.nx * (y + L.ny * z);
-    if (type[n] != WALL) return;
-    shell_fill_with(L, psi, type, n, 0.f, [&](int i) { return nbr_node(L, x, y, z, i); },
-                    [&](int m) { return node_rho2<S>(f, L, m); });
+    uint32_t r = m[0] | m[2] | m[6] | m[8] | (m[4] << 1) | (m[4] >> 1);
+    const uint32_t e = m[1] | m[3] | m[5] | m[7];
+    return r | e | (e << 1) | (e >> 1);
+}
+
+template <class S, bool DENSE>
+__device__ void shell_tile(const Lat &L, const Parts &P, int p, int tile, ShellGrid sg, const typename S::P *__restrict__ f,
+                           float *rho, float *__restrict__ psi, const uint8_t *__restrict__ type,
+                           const uint32_t *__restrict__ owner, const LinkList &ll, ShellTile &sm)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const PGeom &G = reinterpret_cast<const PGeom2 *>(P.geo)[p].now;
+    const Box &box = G.box;
+    const int tx = tile % sg.nx, ty = (tile / sg.nx) % sg.ny, tz = tile / (sg.nx * sg.ny);
+    const int ox = tx * SHELL_X, oy = ty * sg.tyi, oz = tz * sg.tzi;
+    if (ox >= box.ext[0] || oy >= box.ext[1] || oz >= box.ext[2]) return;
+    const int ex = min(SHELL_X, box.ext[0] - ox), ey = min(sg.tyi, box.ext[1] - oy), ez = min(sg.tzi, box.ext[2] - oz);
+    const int x0 = box.lo[0] + ox, y0 = box.lo[1] + oy, z0 = box.lo[2] + oz;
+    const int ny = ey + 2, rows = ny * (ez + 2);
+    const uint32_t inner = (ex >= 31 ? 0xFFFFFFFFu : (1u << ex) - 1u) << 1;  // the tile's own nodes
+    const bool whole = box_full(box);
+    auto inside = [&](int ry, int rz) { return ry >= 1 && ry <= ey && rz >= 1 && rz <= ez; };
+    // candidates of each row
+    for (int r = tid; r < rows; r += PT) {
+        const int ry = r % ny, rz = r / ny, u1 = y0 - 1 + ry, u2 = z0 - 1 + rz;
+        const bool out = L.walls && (u2 < 0 || u2 >= L.nz);
+        uint32_t c = 0;
+        if (inside(ry, rz)) {
+            if (whole) {
+                c = inner;
+            } else {
+                int a, b;
+                row_span(G.g, G.Xi, G.Xf, box, u1, u2, a, b);
+                a = max(a - x0, 0) + 1;
+                b = min(b - x0, ex - 1) + 1;
+                if (a <= b) c = (0xFFFFFFFFu << a) & (0xFFFFFFFFu >> (31 - b));
+            }
+        }
+        sm.S[r] = c;
+        sm.base[r] = out ? -1 : L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
+    }
+    if (tid == 0) sm.nbuf = 0;
+    __syncthreads();
+    // fluid and particle nodes of the rows that a candidate can see
+    const int xw = wrapi(x0 - 1 + lane, L.nx);
+    constexpr int U = 8;  // rows in flight per warp
+    for (int r0 = warp * U; r0 < rows; r0 += (PT / 32) * U) {
+        uint8_t t[U];
+        bool need[U];
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            const int r = r0 + q;
+            uint32_t v = 0;
+            if (r < rows && lane < 9) {
+                const int ry = r % ny + lane % 3 - 1, rz = r / ny + lane / 3 - 1;
+                if (inside(ry, rz)) v = sm.S[ry + ny * rz];
+            }
+            need[q] = __any_sync(0xffffffffu, v != 0) && sm.base[min(r, rows - 1)] >= 0;
+            t[q] = need[q] ? type[sm.base[r] + xw] : WALL;
+        }
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            const uint32_t fl = __ballot_sync(0xffffffffu, t[q] == FLUID), pt = __ballot_sync(0xffffffffu, t[q] == PART);
+            if (lane == 0 && r0 + q < rows) {
+                sm.F[r0 + q] = fl;
+                sm.M[r0 + q] = pt;
+            }
+        }
+    }
+    __syncthreads();
+    // rows around row r of a mask array, 0 outside the tile and its halo
+    auto around = [&](const uint32_t *a, int r, uint32_t m[9]) {
+        const int ry = r % ny, rz = r / ny;
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const int y = ry + k % 3 - 1, z = rz + k / 3 - 1;
+            m[k] = y >= 0 && y < ny && z >= 0 && z < ez + 2 ? a[y + ny * z] : 0u;
+        }
+    };
+    for (int r = tid; r < rows; r += PT) {  // shell nodes
+        uint32_t c = sm.S[r] & sm.M[r];
+        if (c) {
+            uint32_t m[9];
+            around(sm.F, r, m);
+            c &= dilate18(m);
+        }
+        sm.S[r] = c;
+    }
+    __syncthreads();
+    // fluid nodes next to them, and the prefix of both counts over the rows
+    const int per = (rows + PT - 1) / PT, ra = min(tid * per, rows), rb = min(ra + per, rows);
+    uint32_t sum = 0;
+    for (int r = ra; r < rb; r++) {
+        uint32_t m[9];
+        around(sm.S, r, m);
+        const uint32_t n = sm.F[r] & dilate18(m);
+        sm.M[r] = n;
+        sum += (uint32_t)__popc(n) | ((uint32_t)__popc(sm.S[r]) << 16);
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) sm.wsum[warp] = incl;
+    __syncthreads();
+    uint32_t total = 0, run = incl - sum;
+#pragma unroll
+    for (int w = 0; w < PT / 32; w++) {
+        if (w < warp) run += sm.wsum[w];
+        total += sm.wsum[w];
+    }
+    for (int r = ra; r < rb; r++) {
+        sm.start[r] = run;
+        run += (uint32_t)__popc(sm.M[r]) | ((uint32_t)__popc(sm.S[r]) << 16);
+    }
+    __syncthreads();
+    const int nf = (int)(total & 0xFFFFu), ns = (int)(total >> 16);
+    // the row of item k: the last whose prefix (of the half at shift sh) is <= k
+    auto row_of = [&](int k, int sh) {
+        int lo = 0, hi = rows - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((int)((sm.start[mid] >> sh) & 0xFFFFu) <= k)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        return lo;
+    };
+    auto node = [&](int r, int bit) { return sm.base[r] + wrapi(x0 - 1 + bit, L.nx); };
+    for (int k = tid; k < nf; k += PT) {
+        const int r = row_of(k, 0);
+        const int n = node(r, nth_bit(sm.M[r], k - (int)(sm.start[r] & 0xFFFFu)));
+        if (!idx_ok(L, n, L.N, 8)) continue;
+        const float2 v = DENSE ? ld_pair(rho, n) : node_rho2<S>(f, L, n);
+        if (k < SHELL_RHO) sm.rho[k] = v;
+        if (!DENSE) st_pair(rho, n, v);
+    }
+    __syncthreads();
+    const float dr = (float)P.drho[p];
+    for (int k0 = 0; k0 < ns; k0 += PT) {  // whole warps: the appends vote
+        const int k = k0 + tid;
+        int n = 0;
+        uint32_t fm = 0;
+        if (k < ns) {
+            const int r = row_of(k, 16);
+            const int bit = nth_bit(sm.S[r], k - (int)(sm.start[r] >> 16));
+            n = node(r, bit);
+            if (idx_ok(L, n, L.N, 9) && owner[n] == (uint32_t)p) {
+                float s0 = 0.f, s1 = 0.f;
+                int cnt = 0;
+#pragma unroll
+                for (int i = 1; i < Q; i++) {
+                    const int rr = r + cy(i) + ny * cz(i), b = bit + cx(i);
+                    if (!((sm.F[rr] >> b) & 1u)) continue;
+                    const int idx = (int)(sm.start[rr] & 0xFFFFu) + __popc(sm.M[rr] & ((1u << b) - 1u));
+                    const float2 v = idx < SHELL_RHO ? sm.rho[idx] : ld_pair(rho, node(rr, b));
+                    s0 += v.x;
+                    s1 += v.y;
+                    cnt++;
+                    fm |= 1u << i;
+                }
+                shell_psi(L, psi, n, dr, s0, s1, cnt);
+            }
+        }
+        if (!ll.ent) continue;
+        const unsigned want = __ballot_sync(0xffffffffu, fm != 0);
+        if (!want) continue;
+        const int leader = __ffs(want) - 1;
+        int at = 0;
+        if (lane == leader) at = atomicAdd(&sm.nbuf, __popc(want));
+        at = __shfl_sync(0xffffffffu, at, leader) + __popc(want & ((1u << lane) - 1u));
+        const bool spill = fm != 0 && at >= SHELL_BUF;
+        if (fm && !spill) sm.buf[at] = make_uint2((unsigned)n, fm);
+        append_links(ll, n, spill ? fm : 0u);
+    }
+    if (!ll.ent) return;
+    __syncthreads();
+    const int cnt = min(sm.nbuf, SHELL_BUF);
+    if (tid == 0) sm.lbase = cnt ? atomicAdd(ll.count, cnt) : 0;
+    __syncthreads();
+    for (int k = tid; k < cnt; k += PT)
+        if (sm.lbase + k < ll.cap) ll.ent[sm.lbase + k] = sm.buf[k];
+}
+
+// Shell fill of a 32 x 8 tile of a wall plane (z = 0 or nz - 1, Δρ = 0): the
+// densities of the adjacent plane's tile and a one-node halo are summed once
+// into shared memory; each wall node has five neighbours there.
+constexpr int WALL_X = 32, WALL_Y = 8;
+__host__ __device__ inline int wall_tiles(const Lat &L)
+{
+    return L.walls ? 2 * ((L.nx + WALL_X - 1) / WALL_X) * ((L.ny + WALL_Y - 1) / WALL_Y) : 0;
+}
+
+template <class S>
+__device__ void wall_tile(const Lat &L, int tile, const typename S::P *__restrict__ f, float *__restrict__ psi,
+                          const uint8_t *__restrict__ type, ShellTile &sm)
+{
+    constexpr int HX = WALL_X + 2, HN = HX * (WALL_Y + 2);
+    static_assert(HN <= SHELL_RHO && HN <= SHELL_ROWS, "wall tile fits the particle tile's arrays");
+    const int ntx = (L.nx + WALL_X - 1) / WALL_X, nty = (L.ny + WALL_Y - 1) / WALL_Y;
+    const int side = tile / (ntx * nty), t = tile % (ntx * nty);
+    const int x0 = (t % ntx) * WALL_X, y0 = (t / ntx) * WALL_Y;
+    const int zw = side ? L.nz - 1 : 0, zf = side ? L.nz - 2 : 1;
+    for (int e = threadIdx.x; e < HN; e += PT) {
+        const int n = wrapi(x0 - 1 + e % HX, L.nx) + L.nx * (wrapi(y0 - 1 + e / HX, L.ny) + L.ny * zf);
+        const bool fl = type[n] == FLUID;
+        sm.F[e] = fl;
+        if (fl) sm.rho[e] = node_rho2<S>(f, L, n);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < WALL_X * WALL_Y; k += PT) {
+        const int x = x0 + k % WALL_X, y = y0 + k / WALL_X;
+        if (x >= L.nx || y >= L.ny) continue;
+        const int n = x + L.nx * (y + L.ny * zw);
+        if (type[n] != WALL) continue;
+        float s0 = 0.f, s1 = 0.f;
+        int cnt = 0;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if (cz(i) != (side ? -1 : 1)) continue;
+            const int e = (k % WALL_X + 1 + cx(i)) + HX * (k / WALL_X + 1 + cy(i));
+            if (!sm.F[e]) continue;
+            const float2 v = sm.rho[e];
+            s0 += v.x;
+            s1 += v.y;
+            cnt++;
+        }
+        shell_psi(L, psi, n, 0.f, s0, s1, cnt);
+    }
+}
+
+// The tiles of all particles, then those of the walls.
+template <class S, bool DENSE>
+__global__ void __launch_bounds__(PT) k_shell_fill(Lat L, Parts P, ShellGrid sg, const typename S::P *__restrict__ f,
+                                                   float *rho, float *__restrict__ psi, const uint8_t *__restrict__ type,
+                                                   const uint32_t *__restrict__ owner, LinkList ll)
+{
+    __shared__ ShellTile sm;
+    const int nt = sg.nx * sg.ny * sg.nz, npt = P.n * nt, c = blockIdx.x;
+    if (c < npt)
+        shell_tile<S, DENSE>(L, P, c / nt, c % nt, sg, f, rho, psi, type, owner, ll, sm);
+    else
+        wall_tile<S>(L, c - npt, f, psi, type, sm);
 }
 
 // ------------------------------------------------------------- batched
 // One launch for all boxes of a batch: a CTA (or thread) per particle of the
 // batch, in box order; parities come from the batch's device state.
+
+// Start of a batched step: the fused kernel's tile queue is empty again.
+__global__ void k_begin_batch(BatchIndex B) { *B.counter = 0; }
+
+template <class S>
+__global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, int parts)
+{
+    __shared__ ShellTile sm;
+    const int nt = sg.nx * sg.ny * sg.nz, c = blockIdx.x;
+    const bool part = c < parts * nt;
+    const int g = part ? c / nt : c - parts * nt;
+    const int *off = part ? B.part0 : B.wall0;
+    const int b = find_box(off, B.nbox, g);
+    const BoxDev &bx = B.box[b];
+    const int cur = B.par[2 * b], ocur = B.par[2 * b + 1];
+    const typename S::P *f = (const typename S::P *)bx.f[cur];
+    if (part)
+        shell_tile<S, false>(bx.L, bx.P, g - off[b], c % nt, sg, f, bx.rho, bx.psi, bx.type, bx.owner[ocur], bx.links, sm);
+    else
+        wall_tile<S>(bx.L, g - off[b], f, bx.psi, bx.type, sm);
+}
 
 __global__ void __launch_bounds__(PT) k_claim_batch(BatchIndex B, int total)
 {
@@ -1995,18 +2175,64 @@ void launch_link_batch(int storage, const BatchIndex &B, cudaStream_t s)
     LBE_DISPATCH(storage, (k_link_batch<S><<<grid, 256, 0, s>>>(B)));
 }
 
-void launch_shell_particles(const Lat &L, const Parts &P, const float *rho, float *psi, const uint8_t *type,
-                            const uint32_t *owner, const LinkList &ll, cudaStream_t s)
+// Tiles for np particles in boxes of at most ext nodes a side.
+static ShellGrid shell_grid(const int ext[3], int np)
 {
-    if (P.n == 0) return;
-    k_shell_particles<<<P.n, PT, 0, s>>>(L, P, rho, psi, type, owner, ll);
+    auto up = [](int a, int b) { return (a + b - 1) / b; };
+    ShellGrid g{up(ext[0], SHELL_X), up(ext[1], 22), up(ext[2], 22), 22, 22};
+    if ((long long)np * g.nx * g.ny * g.nz < 2 * 152) g = ShellGrid{g.nx, up(ext[1], 10), up(ext[2], 5), 10, 5};
+    return g;
 }
 
-void launch_shell_walls(int storage, const Lat &L, const void *f, float *psi, const uint8_t *type, cudaStream_t s)
+// An upper bound of a particle box's extent (box_axis: 2 h + 5 nodes at
+// most, h <= rmax).
+static void shell_extent(const Lat &L, double rmax, int ext[3])
 {
-    if (!L.walls) return;
-    const int n = 2 * L.nx * L.ny;
-    LBE_DISPATCH(storage, (k_shell_walls<S><<<(n + 255) / 256, 256, 0, s>>>(L, (const typename S::P *)f, psi, type)));
+    const double e = std::floor(2.0 * rmax) + 5.0;
+    const int n[3] = {L.nx, L.ny, L.nz};
+    for (int k = 0; k < 3; k++) ext[k] = std::max(ext[k], e < n[k] ? (int)e : n[k]);
+}
+
+template <class S, bool DENSE>
+static void shell_fill_launch(unsigned ctas, const Lat &L, const Parts &P, const ShellGrid &g, const void *f, float *rho,
+                              float *psi, const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
+{
+    k_shell_fill<S, DENSE><<<ctas, PT, 0, s>>>(L, P, g, (const typename S::P *)f, rho, psi, type, owner, ll);
+}
+
+void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
+                       const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
+{
+    ShellGrid g{0, 0, 0, 1, 1};
+    if (P.n > 0) {
+        int ext[3] = {1, 1, 1};
+        shell_extent(L, P.rmax, ext);
+        g = shell_grid(ext, P.n);
+    }
+    const long long ctas = (long long)P.n * g.nx * g.ny * g.nz + wall_tiles(L);
+    if (ctas == 0) return;
+    if (dense)
+        LBE_DISPATCH(storage, (shell_fill_launch<S, true>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
+    else
+        LBE_DISPATCH(storage, (shell_fill_launch<S, false>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
+}
+
+int batch_wall_tiles(const Lat &L) { return wall_tiles(L); }
+
+void launch_begin_batch(const BatchIndex &B, cudaStream_t s) { k_begin_batch<<<1, 1, 0, s>>>(B); }
+
+void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, int total_walls,
+                        cudaStream_t s)
+{
+    const ShellGrid g = total_parts > 0 ? shell_grid(ext, total_parts) : ShellGrid{0, 0, 0, 1, 1};
+    const long long ctas = (long long)total_parts * g.nx * g.ny * g.nz + total_walls;
+    if (ctas == 0) return;
+    LBE_DISPATCH(storage, (k_shell_batch<S><<<(unsigned)ctas, PT, 0, s>>>(B, g, total_parts)));
+}
+
+void batch_shell_extent(const Lat &L, const Parts &P, int ext[3])
+{
+    if (P.n > 0) shell_extent(L, P.rmax, ext);
 }
 
 void launch_reset(const Lat &L, const Parts &P, int use_old, uint32_t *owner, cudaStream_t s)
