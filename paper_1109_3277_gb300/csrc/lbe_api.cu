@@ -269,11 +269,9 @@ void enqueue_step(lbe_ctx *c)
             launch_links(st, L, c->P, fout, c->rho, c->type, c->owner[c->ocur], s);
         else {
             launch_link(st, L, c->ll, c->rho, c->owner[c->ocur], c->P, fout, s);
-            // the list is empty between steps (batched steps rely on it)
-            cudaMemsetAsync(c->ll.count, 0, sizeof(int), s);
         }
         launch_pairs(L, c->P, c->pair, c->cells, s);
-        launch_integrate(L, c->P, c->d.particle_mode, s);
+        launch_integrate(L, c->P, c->d.particle_mode, c->ll.count, s);  // the list is empty between steps
         if (c->d.particle_mode != LBE_PARTICLES_STATIC) {
             uint32_t *oo = c->owner[c->ocur], *on = c->owner[1 - c->ocur];
             launch_claim(L, c->P, 0, on, s);
@@ -553,10 +551,12 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
                                             (float)blk[OW * cp + 3 * p + 2], 0.f);
     }
     if (!c->ll.ent) {
-        // a fluid node enters the link list at most once per step: N entries
+        // a particle node enters the link list at most once per step, and
+        // LINK_PAD bounds the empty entries
+        const size_t cap_ll = (size_t)c->L.N + LINK_PAD;
         uint2 *ent = nullptr;
         int *cnt = nullptr;
-        CK(c, lib_malloc((void **)&ent, (size_t)c->L.N * sizeof(uint2)));
+        CK(c, lib_malloc((void **)&ent, cap_ll * sizeof(uint2)));
         cudaError_t e = lib_malloc((void **)&cnt, sizeof(int));
         if (e != cudaSuccess) {
             cudaFree(ent);
@@ -565,8 +565,8 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
         CK(c, cudaMemset(cnt, 0, sizeof(int)));
         c->ll.ent = ent;
         c->ll.count = cnt;
-        c->ll.cap = c->L.N;
-        c->bytes += (size_t)c->L.N * sizeof(uint2) + sizeof(int);
+        c->ll.cap = (int)std::min<size_t>(cap_ll, INT32_MAX);
+        c->bytes += cap_ll * sizeof(uint2) + sizeof(int);
     }
     {
         lbe_status cst = build_cells(c, blk, ncap, np);
@@ -809,7 +809,7 @@ size_t lbe_footprint(const lbe_lattice_desc *d, int32_t nparticles)
         b += cap * (PSTRIDE * sizeof(double) + 3 * sizeof(float4) + 6 * sizeof(double) + 2 * sizeof(int) +
                     geom_bytes_per_particle());
         b += (3 * (N / 8) + 1) * sizeof(int);  // cells (at least 2 nodes a side)
-        b += N * sizeof(uint2) + sizeof(int);  // link list
+        b += (N + LINK_PAD) * sizeof(uint2) + sizeof(int);  // link list
     }
     return b;
 }
@@ -969,7 +969,7 @@ void batch_enqueue_step(lbe_batch *b)
     launch_shell_batch(b->storage, b->idx, b->ext, b->total_parts, b->total_walls, s);
     launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * b->ctas_per_sm, b->general, s);
     if (b->total_parts > 0) {
-        launch_link_batch(b->storage, b->idx, s);
+        launch_link_batch(b->storage, b->idx, b->ext, b->total_parts, s);
         launch_pairs_batch(b->idx, b->total_parts, s);
         launch_integrate_batch(b->idx, b->total_parts, s);
         launch_geom_batch(b->idx, b->total_parts, s);

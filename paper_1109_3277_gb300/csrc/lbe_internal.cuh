@@ -246,8 +246,10 @@ struct Parts {
 
 // Particle nodes next to fluid nodes, collected each step by the shell-fill
 // kernel: entry (particle node s, mask of the directions j whose neighbour
-// s + c_j is a fluid node).  A node enters at most once per step, so cap = N
-// cannot overflow.
+// s + c_j is a fluid node).  A node enters at most once per step, and the
+// shell fill adds fewer than LINK_PAD empty entries (mask 0), so cap = N +
+// LINK_PAD cannot overflow.
+constexpr int LINK_PAD = 65536;
 struct LinkList {
     uint2 *ent;   // [cap]
     int *count;   // entries this step (reset before the density kernel)
@@ -293,23 +295,6 @@ __device__ __forceinline__ void shell_fill(const Lat &L, const float *__restrict
         cnt++;
     }
     shell_psi(L, psi, n, dr, s0, s1, cnt);
-}
-
-// Append (n, m) for the lanes with m != 0 to a link list: one atomic per
-// warp.  Called by all 32 lanes.
-__device__ __forceinline__ void append_links(const LinkList &ll, int n, uint32_t m)
-{
-    const unsigned want = __ballot_sync(0xffffffffu, m != 0);
-    if (!want) return;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(want) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(ll.count, __popc(want));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (m) {
-        const int k = base + __popc(want & ((1u << lane) - 1u));
-        if (k < ll.cap) ll.ent[k] = make_uint2((unsigned)n, m);
-    }
 }
 
 // Cell list of the particles for the pair forces: cubic-ish cells of edge
@@ -412,7 +397,7 @@ void launch_claim_batch(const BatchIndex &B, int total_parts, cudaStream_t s);
 void launch_transition_batch(int storage, const BatchIndex &B, int total_parts, cudaStream_t s);
 void launch_reset_batch(const BatchIndex &B, int total_parts, cudaStream_t s);
 void launch_batch_quat(const BatchIndex &B, double *out, cudaStream_t s);
-void launch_link_batch(int storage, const BatchIndex &B, cudaStream_t s);
+void launch_link_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, cudaStream_t s);
 void launch_flip_batch(const BatchIndex &B, cudaStream_t s);
 
 // ---- launchers (fused.cu) -------------------------------------------------
@@ -472,8 +457,8 @@ void launch_pairs(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, 
 // kernels) or a loop over all partners.
 bool pairs_by_cells(int np);
 // The update of the particles and, unless they are static, the geometry of
-// their new coverage.
-void launch_integrate(const Lat &L, const Parts &P, int mode, cudaStream_t s);
+// their new coverage; links (may be null): the link list's counter, set to 0.
+void launch_integrate(const Lat &L, const Parts &P, int mode, int *links, cudaStream_t s);
 // Coverage geometry of particles just placed (old = current);
 // geom_bytes_per_particle() is the size of one particle's record.
 void launch_geom(const Lat &L, const Parts &P, cudaStream_t s);

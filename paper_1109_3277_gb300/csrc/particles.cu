@@ -18,9 +18,9 @@ namespace {
 constexpr int PT = 128;  // threads per per-particle CTA
 
 // Tiles of a particle's box in the shell fill: nx x ny x nz of them, of 30 x
-// tyi x tzi nodes.
+// tyi x tzi nodes; a tile's link entries are filled up to a multiple of pad.
 struct ShellGrid {
-    int nx, ny, nz, tyi, tzi;
+    int nx, ny, nz, tyi, tzi, pad;
 };
 
 // ---------------------------------------------------------- geometry (FP64)
@@ -681,23 +681,27 @@ __device__ __forceinline__ unsigned long long to_fixed(float v)
     return (unsigned long long)__float2ll_rn(v * 1099511627776.f);
 }
 
+// Sum over the lanes of grp of 64-bit two's complement words (exact, by
+// 16/16/32-bit limbs).  Called by the lanes of grp.
+__device__ __forceinline__ unsigned long long reduce_fix(unsigned grp, unsigned long long v)
+{
+    const unsigned lo = (unsigned)v, hi = (unsigned)(v >> 32);
+    const unsigned s0 = __reduce_add_sync(grp, lo & 0xffffu);
+    const unsigned s1 = __reduce_add_sync(grp, lo >> 16);
+    const unsigned s2 = __reduce_add_sync(grp, hi);
+    return ((unsigned long long)s2 << 32) + ((unsigned long long)s1 << 16) + (unsigned long long)s0;
+}
+
 // Add this lane's sums v[6] for particle p (nothing for p < 0) to the
 // particle's totals: lanes of the warp with the same particle are combined
-// first (exact integer reductions over 16/16/32-bit limbs) and one lane per
-// particle does the atomics.  Called by all 32 lanes.
+// first and one lane per particle does the atomics.  Called by all 32 lanes.
 __device__ __forceinline__ void warp_add_fix(int p, const unsigned long long v[6], unsigned long long *fix)
 {
     const unsigned grp = __match_any_sync(0xffffffffu, p);
     const bool leader = (int)(threadIdx.x & 31) == __ffs(grp) - 1;
     unsigned long long tot[6];
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const unsigned lo = (unsigned)v[k], hi = (unsigned)(v[k] >> 32);
-        const unsigned s0 = __reduce_add_sync(grp, lo & 0xffffu);
-        const unsigned s1 = __reduce_add_sync(grp, lo >> 16);
-        const unsigned s2 = __reduce_add_sync(grp, hi);
-        tot[k] = ((unsigned long long)s2 << 32) + ((unsigned long long)s1 << 16) + (unsigned long long)s0;
-    }
+    for (int k = 0; k < 6; k++) tot[k] = reduce_fix(grp, v[k]);
     if (p < 0 || !leader) return;
 #pragma unroll
     for (int k = 0; k < 6; k++) atomicAdd(&fix[6 * p + k], tot[k]);
@@ -715,7 +719,7 @@ constexpr unsigned long long pack_dir(int axis)
 constexpr unsigned long long CXP = pack_dir(0), CYP = pack_dir(1), CZP = pack_dir(2);
 __device__ __forceinline__ int cdir(unsigned long long pack, int j) { return (int)((pack >> (2 * j)) & 3ull) - 1; }
 
-// Per warp of the link kernels: the links of its 32 list entries in
+// Per warp of the link kernels: the links of its list entries in
 // direction-major order, (entry lane, direction) per link.
 struct LinkWarp {
     uint16_t desc[32 * (Q - 1)];
@@ -723,22 +727,25 @@ struct LinkWarp {
     int pre[Q];
 };
 
-// The links of 32 list entries (e = (node, mask of fluid neighbours) per
-// lane; valid = false for a lane without an entry).  The entries' links
-// are laid out direction by direction, so that lanes taking neighbouring
-// links touch the same slot array at neighbouring nodes, and handed out 32
-// at a time: every lane carries one link per round, and the loads of a
-// round are all in flight together.  Called by all 32 lanes.
+// The links of up to 32 list entries (e = (node, mask of fluid neighbours)
+// per lane; mask 0 for a lane without an entry).  The entries' links are
+// laid out direction by direction, so that lanes taking neighbouring links
+// touch the same slot array at neighbouring nodes, and handed out 32 at a
+// time: every lane carries one link per round, and the loads of a round are
+// all in flight together.  What belongs to the entry (its place, the arm from
+// the particle) is formed once by the entry's lane.  Where all entries are of
+// one particle (most warps), each lane adds up its own terms over the rounds
+// and the warp combines them once.  Called by all 32 lanes.
 template <class S>
-__device__ __forceinline__ void link_entries(const Lat &L, uint2 e, bool valid, const float *__restrict__ rho,
+__device__ __forceinline__ void link_entries(const Lat &L, uint2 e, const float *__restrict__ rho,
                                              const uint32_t *__restrict__ owner, const float4 *__restrict__ X32,
                                              const float4 *__restrict__ K32, unsigned long long *fix,
                                              typename S::P *fout, LinkWarp &w)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    uint32_t fm = valid ? e.y : 0u;
-    const int s = valid ? (int)e.x : 0;
+    uint32_t fm = e.y;
+    const int s = (int)e.x;
     int p = -1;
     if (fm) {
         p = (int)owner[s];
@@ -748,6 +755,8 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, bool valid, 
             fm = 0;
         }
     }
+    const unsigned have = __ballot_sync(full, fm != 0);
+    if (!have) return;
     // direction j's links: the lanes of ballot j, after those of 1 .. j-1
     int total = 0;
 #pragma unroll
@@ -765,6 +774,30 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, bool valid, 
         const int k = w.pre[j] + __popc(w.bal[j] & ((1u << lane) - 1u));
         w.desc[k] = (uint16_t)(lane | (j << 5));
     }
+    const int p0 = __shfl_sync(full, p, __ffs(have) - 1);
+    const bool uniform = __all_sync(full, !fm || p == p0);
+    // the entry's node: s - X, nearest image, and the lattice faces it lies on
+    float dx = 0.f, dy = 0.f, dz = 0.f;
+    unsigned face = 0;
+    if (fm) {
+        const float4 X = X32[p];
+        const int x = s % L.nx, t = s / L.nx, y = t % L.ny, z = t / L.ny;
+        dx = (float)x - X.x;
+        dy = (float)y - X.y;
+        dz = (float)z - X.z;
+        if (dx > 0.5f * L.nx) dx -= L.nx;
+        if (dx < -0.5f * L.nx) dx += L.nx;
+        if (dy > 0.5f * L.ny) dy -= L.ny;
+        if (dy < -0.5f * L.ny) dy += L.ny;
+        if (!L.walls) {
+            if (dz > 0.5f * L.nz) dz -= L.nz;
+            if (dz < -0.5f * L.nz) dz += L.nz;
+        }
+        face = (x == L.nx - 1 ? 1u : 0u) | (x == 0 ? 2u : 0u) | (y == L.ny - 1 ? 4u : 0u) | (y == 0 ? 8u : 0u) |
+               (z == L.nz - 1 ? 16u : 0u) | (z == 0 ? 32u : 0u);
+    }
+    float4 V = K32[2 * p0], W = K32[2 * p0 + 1];
+    unsigned long long sum[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
     __syncwarp();
     for (int k0 = 0; k0 < total; k0 += 32) {
         const int k = k0 + lane;
@@ -772,28 +805,25 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, bool valid, 
         const int d = act ? w.desc[k] : 0;
         const int src = d & 31, j = act ? d >> 5 : 1;
         const int sn = __shfl_sync(full, s, src), pn = __shfl_sync(full, p, src);
+        const float ex = __shfl_sync(full, dx, src), ey = __shfl_sync(full, dy, src), ez = __shfl_sync(full, dz, src);
+        const unsigned fc = __shfl_sync(full, face, src);
         unsigned long long acc[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
         if (act) {
-            const float4 X = X32[pn], V = K32[2 * pn], W = K32[2 * pn + 1];
-            const int x = sn % L.nx, t = sn / L.nx, y = t % L.ny, z = t / L.ny;
-            // sn - X, nearest image
-            float dx = (float)x - X.x, dy = (float)y - X.y, dz = (float)z - X.z;
-            if (dx > 0.5f * L.nx) dx -= L.nx;
-            if (dx < -0.5f * L.nx) dx += L.nx;
-            if (dy > 0.5f * L.ny) dy -= L.ny;
-            if (dy < -0.5f * L.ny) dy += L.ny;
-            if (!L.walls) {
-                if (dz > 0.5f * L.nz) dz -= L.nz;
-                if (dz < -0.5f * L.nz) dz += L.nz;
+            if (!uniform) {
+                V = K32[2 * pn];
+                W = K32[2 * pn + 1];
             }
             const int cxj = cdir(CXP, j), cyj = cdir(CYP, j), czj = cdir(CZP, j);
-            int xn = x + cxj, yn = y + cyj, zn = z + czj;  // the fluid node
-            xn = xn < 0 ? xn + L.nx : (xn >= L.nx ? xn - L.nx : xn);
-            yn = yn < 0 ? yn + L.ny : (yn >= L.ny ? yn - L.ny : yn);
-            zn = zn < 0 ? zn + L.nz : (zn >= L.nz ? zn - L.nz : zn);
-            const int yf = xn + L.nx * (yn + L.ny * zn);
+            // the fluid node s + c_j, around the periodic faces
+            int yf = sn + cxj + L.nx * (cyj + L.ny * czj);
+            if (cxj > 0 && (fc & 1u)) yf -= L.nx;
+            if (cxj < 0 && (fc & 2u)) yf += L.nx;
+            if (cyj > 0 && (fc & 4u)) yf -= L.nx * L.ny;
+            if (cyj < 0 && (fc & 8u)) yf += L.nx * L.ny;
+            if (czj > 0 && (fc & 16u)) yf -= L.N;
+            if (czj < 0 && (fc & 32u)) yf += L.N;
             const float fcx = (float)cxj, fcy = (float)cyj, fcz = (float)czj;
-            const float rx = dx + 0.5f * fcx, ry = dy + 0.5f * fcy, rz = dz + 0.5f * fcz;
+            const float rx = ex + 0.5f * fcx, ry = ey + 0.5f * fcy, rz = ez + 0.5f * fcz;
             // surface velocity V + ω × r_b at the link midpoint
             const float usx = __fsub_rn(__fmaf_rn(W.y, rz, V.x), __fmul_rn(W.z, ry));
             const float usy = __fsub_rn(__fmaf_rn(W.z, rx, V.y), __fmul_rn(W.x, rz));
@@ -820,38 +850,55 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, bool valid, 
             acc[4] = to_fixed(__fsub_rn(__fmul_rn(rz, Fx), __fmul_rn(rx, Fz)));
             acc[5] = to_fixed(__fsub_rn(__fmul_rn(rx, Fy), __fmul_rn(ry, Fx)));
         }
-        warp_add_fix(act ? pn : -1, acc, fix);
+        if (uniform) {
+#pragma unroll
+            for (int c = 0; c < 6; c++) sum[c] += acc[c];
+        } else {
+            warp_add_fix(act ? pn : -1, acc, fix);
+        }
+    }
+    if (uniform) {
+        unsigned long long t = 0ull;
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const unsigned long long v = reduce_fix(full, sum[c]);
+            if (lane == c) t = v;
+        }
+        if (lane < 6) atomicAdd(&fix[6 * p0 + lane], t);
     }
     __syncwarp();
 }
 
-// Warp-uniform trip count over the entries (every lane takes part in the
-// reductions).
+// A warp takes group entries of the list at a time: 32, or 8 where the list
+// is short (lists of small tiles, whose groups of 8 are of one particle), so
+// that the links of one particle spread over many warps.  One ellipsoid (6,
+// 3): 18.6 us with 32 and a reduction per round, 8.1 with 8; 40 dragged
+// ellipsoids: 86 and 8.5 us.
 template <class S>
 __device__ __forceinline__ void link_list(const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
-                                          const Parts &P, typename S::P *fout, int first, int stride, LinkWarp &w)
+                                          const Parts &P, typename S::P *fout, int group, LinkWarp &w)
 {
-    const int count = min(*ll.count, ll.cap);
-    for (int w0 = first + (int)(threadIdx.x & ~31u); w0 < count; w0 += stride) {
-        const int e = w0 + (threadIdx.x & 31);
-        const bool valid = e < count;
-        link_entries<S>(L, valid ? ll.ent[e] : make_uint2(0u, 0u), valid, rho, owner, P.X32, P.K32, P.fix, fout, w);
+    const int count = min(*ll.count, ll.cap), lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (blockDim.x >> 5), w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    for (int e0 = w0 * group; e0 < count; e0 += nw * group) {
+        const bool valid = lane < group && e0 + lane < count;
+        link_entries<S>(L, valid ? ll.ent[e0 + lane] : make_uint2(0u, 0u), rho, owner, P.X32, P.K32, P.fix, fout, w);
     }
 }
 
 template <class S>
 __global__ void __launch_bounds__(256) k_link(Lat L, LinkList ll, const float *rho, const uint32_t *owner, Parts P,
-                                              typename S::P *fout)
+                                              typename S::P *fout, int group)
 {
     __shared__ LinkWarp w[256 / 32];
-    link_list<S>(L, ll, rho, owner, P, fout, blockIdx.x * blockDim.x, gridDim.x * blockDim.x, w[threadIdx.x >> 5]);
+    link_list<S>(L, ll, rho, owner, P, fout, group, w[threadIdx.x >> 5]);
 }
 
 // Batched: blockIdx.y is the box; LINK_BATCH_CTAS CTAs per box.
-constexpr int LINK_BATCH_CTAS = 4;
+constexpr int LINK_BATCH_CTAS = 8;
 
 template <class S>
-__global__ void __launch_bounds__(256) k_link_batch(BatchIndex B)
+__global__ void __launch_bounds__(256) k_link_batch(BatchIndex B, int group)
 {
     const int b = blockIdx.y;
     const BoxDev &bx = B.box[b];
@@ -859,7 +906,7 @@ __global__ void __launch_bounds__(256) k_link_batch(BatchIndex B)
     const int cur = B.par[2 * b], ocur = B.par[2 * b + 1];
     __shared__ LinkWarp w[256 / 32];
     link_list<S>(bx.L, bx.links, bx.rho, bx.owner[ocur], bx.P, (typename S::P *)bx.f[1 - cur],
-                 blockIdx.x * blockDim.x, gridDim.x * blockDim.x, w[threadIdx.x >> 5]);
+                 group, w[threadIdx.x >> 5]);
 }
 
 // --------------------------------------------------------- pair forces
@@ -1319,9 +1366,10 @@ __device__ __forceinline__ void integrate_quad(const Lat &L, const Parts &P, int
 }
 
 // The update and, for particles that move, the geometry of their new
-// coverage, in one launch.
-__global__ void __launch_bounds__(128) k_integrate(Lat L, Parts P, int mode)
+// coverage, in one launch; it also empties the step's link list.
+__global__ void __launch_bounds__(128) k_integrate(Lat L, Parts P, int mode, int *links)
 {
+    if (links && blockIdx.x == 0 && threadIdx.x == 0) *links = 0;  // ready for the next step's list
     bool act;
     const int p = quad_particle(P.n, act);
     double X, Xold, q[4];
@@ -1638,51 +1686,40 @@ __global__ void __launch_bounds__(PT) k_reset(Lat L, Parts P, int use_old, uint3
 // SMs (the halo rows are then 68 % more rows, which costs less than idle
 // SMs).  Results do not depend on the tiling.
 //
-// A tile's link entries go into the list as one contiguous segment
-// (collected in shared memory, then one reservation and a coalesced copy),
-// so that the link kernel, which walks the list in order, handles
-// neighbouring links together: their slots share cache lines.  Entries
-// beyond the buffer are appended directly.
-constexpr int SHELL_BUF = 1024;   // link entries collected per tile
-constexpr int SHELL_RHO = 1024;   // densities held per tile (the rest are read back from rho)
-constexpr int SHELL_X = 30;       // nodes of a tile along x: a mask word less the halo
-constexpr int SHELL_ROWS = 24 * 24;
+// A tile's link entries go into the list as one contiguous segment in row
+// order (one reservation, while the densities come in), so that the link
+// kernel, which walks the list in order, handles neighbouring links together:
+// their slots share cache lines.  With the small tiles a segment is filled up
+// to a multiple of 8 with empty entries, so that the link kernel's groups of
+// 8 belong to one particle.
+//
+// The kernel is bound by instruction issue: rows are handled by (plane: warp,
+// row: lane) without a division, and node lists are written out once instead
+// of a search per node.  512^3 Pickering, DENSE: 965 us with a search per node
+// and divisions, 658 now; before the masks 1,420.
+constexpr int SHELL_ITEMS = 1024;  // nodes of a list held at once, and densities held per tile
+constexpr int SHELL_X = 30;        // nodes of a tile along x: a mask word less the halo
+constexpr int SHELL_MAX = 22;      // rows of a tile along y and z
+constexpr int RS = SHELL_MAX + 4;  // rows with the halo, and an empty row on each side
+constexpr int SHELL_PLANES = (SHELL_MAX + 2 + PT / 32 - 1) / (PT / 32);  // planes of rows per warp
 
 struct ShellTile {
-    uint32_t S[SHELL_ROWS];      // candidate nodes (bit b: x = x0 - 1 + b), then shell nodes
-    uint32_t F[SHELL_ROWS];      // fluid nodes
-    uint32_t M[SHELL_ROWS];      // particle nodes, then fluid nodes next to a shell node
-    int base[SHELL_ROWS];        // node index of the row's x = 0, -1 beyond a wall
-    uint32_t start[SHELL_ROWS];  // fluid nodes (low half) and shell nodes (high half) of the rows before
-    float2 rho[SHELL_RHO];
-    uint2 buf[SHELL_BUF];
-    uint32_t wsum[PT / 32];
-    int nbuf, lbase;
+    uint32_t S[RS * RS];     // candidate nodes (bit b: x = x0 - 1 + b), then shell nodes
+    uint32_t F[RS * RS];     // fluid nodes
+    uint32_t M[RS * RS];     // particle nodes, then fluid nodes next to a shell node
+    int base[RS * RS];       // node index of the row's x = 0, -1 beyond a wall
+    uint16_t start[RS * RS];  // fluid nodes of M in the rows before
+    uint16_t fl[SHELL_ITEMS], sl[SHELL_ITEMS];  // lists of fluid and shell nodes: row << 5 | bit
+    float2 rho[SHELL_ITEMS];
+    uint32_t plane[SHELL_MAX + 2];  // fluid nodes | shell nodes << 16 of a plane of rows
+    int owned, next, lbase;
 };
 
-// The j-th (from 0) set bit of m.
-__device__ __forceinline__ int nth_bit(uint32_t m, int j)
+// Bits of row r that have a neighbour (one of the 18) in the mask rows a.
+__device__ __forceinline__ uint32_t dilate18(const uint32_t *a, int r)
 {
-    int pos = 0;
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const int c = __popc(m & ((1u << w) - 1u));
-        if (j >= c) {
-            j -= c;
-            m >>= w;
-            pos += w;
-        }
-    }
-    return pos;
-}
-
-// Bits of a row that have a neighbour (one of the 18) in the rows m[9] around
-// it (index (dy + 1) + 3 (dz + 1), the row itself at 4).
-__device__ __forceinline__ uint32_t dilate18(const uint32_t m[9])
-{
-    uint32_t r = m[0] | m[2] | m[6] | m[8] | (m[4] << 1) | (m[4] >> 1);
-    const uint32_t e = m[1] | m[3] | m[5] | m[7];
-    return r | e | (e << 1) | (e >> 1);
+    const uint32_t e = a[r - 1] | a[r + 1] | a[r - RS] | a[r + RS], c = a[r];
+    return a[r - RS - 1] | a[r - RS + 1] | a[r + RS - 1] | a[r + RS + 1] | e | ((c | e) << 1) | ((c | e) >> 1);
 }
 
 template <class S, bool DENSE>
@@ -1690,6 +1727,7 @@ __device__ void shell_tile(const Lat &L, const Parts &P, int p, int tile, ShellG
                            float *rho, float *__restrict__ psi, const uint8_t *__restrict__ type,
                            const uint32_t *__restrict__ owner, const LinkList &ll, ShellTile &sm)
 {
+    const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const PGeom &G = reinterpret_cast<const PGeom2 *>(P.geo)[p].now;
     const Box &box = G.box;
@@ -1698,173 +1736,221 @@ __device__ void shell_tile(const Lat &L, const Parts &P, int p, int tile, ShellG
     if (ox >= box.ext[0] || oy >= box.ext[1] || oz >= box.ext[2]) return;
     const int ex = min(SHELL_X, box.ext[0] - ox), ey = min(sg.tyi, box.ext[1] - oy), ez = min(sg.tzi, box.ext[2] - oz);
     const int x0 = box.lo[0] + ox, y0 = box.lo[1] + oy, z0 = box.lo[2] + oz;
-    const int ny = ey + 2, rows = ny * (ez + 2);
-    const uint32_t inner = (ex >= 31 ? 0xFFFFFFFFu : (1u << ex) - 1u) << 1;  // the tile's own nodes
-    const bool whole = box_full(box);
-    auto inside = [&](int ry, int rz) { return ry >= 1 && ry <= ey && rz >= 1 && rz <= ez; };
-    // candidates of each row
-    for (int r = tid; r < rows; r += PT) {
-        const int ry = r % ny, rz = r / ny, u1 = y0 - 1 + ry, u2 = z0 - 1 + rz;
-        const bool out = L.walls && (u2 < 0 || u2 >= L.nz);
-        uint32_t c = 0;
-        if (inside(ry, rz)) {
-            if (whole) {
-                c = inner;
-            } else {
-                int a, b;
-                row_span(G.g, G.Xi, G.Xf, box, u1, u2, a, b);
-                a = max(a - x0, 0) + 1;
-                b = min(b - x0, ex - 1) + 1;
-                if (a <= b) c = (0xFFFFFFFFu << a) & (0xFFFFFFFFu >> (31 - b));
-            }
-        }
-        sm.S[r] = c;
-        sm.base[r] = out ? -1 : L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
-    }
-    if (tid == 0) sm.nbuf = 0;
-    __syncthreads();
-    // fluid and particle nodes of the rows that a candidate can see
-    const int xw = wrapi(x0 - 1 + lane, L.nx);
-    constexpr int U = 8;  // rows in flight per warp
-    for (int r0 = warp * U; r0 < rows; r0 += (PT / 32) * U) {
-        uint8_t t[U];
-        bool need[U];
-#pragma unroll
-        for (int q = 0; q < U; q++) {
-            const int r = r0 + q;
-            uint32_t v = 0;
-            if (r < rows && lane < 9) {
-                const int ry = r % ny + lane % 3 - 1, rz = r / ny + lane / 3 - 1;
-                if (inside(ry, rz)) v = sm.S[ry + ny * rz];
-            }
-            need[q] = __any_sync(0xffffffffu, v != 0) && sm.base[min(r, rows - 1)] >= 0;
-            t[q] = need[q] ? type[sm.base[r] + xw] : WALL;
-        }
-#pragma unroll
-        for (int q = 0; q < U; q++) {
-            const uint32_t fl = __ballot_sync(0xffffffffu, t[q] == FLUID), pt = __ballot_sync(0xffffffffu, t[q] == PART);
-            if (lane == 0 && r0 + q < rows) {
-                sm.F[r0 + q] = fl;
-                sm.M[r0 + q] = pt;
-            }
-        }
-    }
-    __syncthreads();
-    // rows around row r of a mask array, 0 outside the tile and its halo
-    auto around = [&](const uint32_t *a, int r, uint32_t m[9]) {
-        const int ry = r % ny, rz = r / ny;
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            const int y = ry + k % 3 - 1, z = rz + k / 3 - 1;
-            m[k] = y >= 0 && y < ny && z >= 0 && z < ez + 2 ? a[y + ny * z] : 0u;
-        }
+    const int xs = wrapi(x0 - 1, L.nx);
+    auto xnode = [&](int bit) {
+        const int x = xs + bit;
+        return x < L.nx ? x : (L.nx >= 32 ? x - L.nx : x % L.nx);
     };
-    for (int r = tid; r < rows; r += PT) {  // shell nodes
-        uint32_t c = sm.S[r] & sm.M[r];
-        if (c) {
-            uint32_t m[9];
-            around(sm.F, r, m);
-            c &= dilate18(m);
+    // Rows: lane ry = 0 .. ey + 1 of plane rz = 0 .. ez + 1 (the halo first and
+    // last), plane rz by warp rz mod 4; row index r.
+    auto row = [&](int ry, int rz) { return ry + 1 + RS * (rz + 1); };
+    for (int r = tid; r < RS * RS; r += PT) sm.S[r] = sm.F[r] = 0u;
+    if (tid == 0) sm.owned = sm.next = 0;
+    __syncthreads();
+    // candidates of each row
+    for (int rz = warp; rz < ez + 2; rz += PT / 32) {
+        if (lane >= ey + 2) continue;
+        const int u1 = y0 - 1 + lane, u2 = z0 - 1 + rz;
+        uint32_t c = 0;
+        if (lane >= 1 && lane <= ey && rz >= 1 && rz <= ez) {
+            int a = x0, b = x0 + ex - 1;
+            if (!box_full(box)) {
+                row_span(G.g, G.Xi, G.Xf, box, u1, u2, a, b);
+                a = max(a, x0);
+                b = min(b, x0 + ex - 1);
+            }
+            if (a <= b) c = (0xFFFFFFFFu << (a - x0 + 1)) & (0xFFFFFFFFu >> (30 - (b - x0)));
         }
-        sm.S[r] = c;
+        const bool out = L.walls && (u2 < 0 || u2 >= L.nz);
+        sm.S[row(lane, rz)] = c;
+        sm.base[row(lane, rz)] = out ? -1 : L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
     }
     __syncthreads();
-    // fluid nodes next to them, and the prefix of both counts over the rows
-    const int per = (rows + PT - 1) / PT, ra = min(tid * per, rows), rb = min(ra + per, rows);
-    uint32_t sum = 0;
-    for (int r = ra; r < rb; r++) {
-        uint32_t m[9];
-        around(sm.S, r, m);
-        const uint32_t n = sm.F[r] & dilate18(m);
-        sm.M[r] = n;
-        sum += (uint32_t)__popc(n) | ((uint32_t)__popc(sm.S[r]) << 16);
+    // fluid and particle nodes of the rows that a candidate can see: a row's
+    // 32 types by one load of the warp, eight rows in flight
+    const int xl = xnode(lane);
+    for (int rz = warp; rz < ez + 2; rz += PT / 32) {
+        const int r = row(min(lane, ey + 1), rz);
+        const int mybase = sm.base[r];
+        uint32_t near = 0;
+#pragma unroll
+        for (int k = 0; k < 9; k++) near |= sm.S[r + k % 3 - 1 + RS * (k / 3 - 1)];
+        unsigned todo = __ballot_sync(full, lane < ey + 2 && near != 0 && mybase >= 0);
+        uint32_t fl = 0, pt = 0;
+        while (todo) {
+            uint8_t t[8];
+            int rr[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                rr[q] = todo ? __ffs(todo) - 1 : -1;
+                todo &= todo - 1;
+                const int b = __shfl_sync(full, mybase, max(rr[q], 0));
+                t[q] = rr[q] >= 0 ? type[b + xl] : WALL;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const uint32_t bf = __ballot_sync(full, t[q] == FLUID), bp = __ballot_sync(full, t[q] == PART);
+                if (lane == rr[q]) {
+                    fl = bf;
+                    pt = bp;
+                }
+            }
+        }
+        if (lane < ey + 2) {
+            sm.F[r] = fl;
+            sm.M[r] = pt;
+        }
     }
-    uint32_t incl = sum;
+    __syncthreads();
+    for (int rz = warp; rz < ez + 2; rz += PT / 32) {  // shell nodes
+        if (lane >= ey + 2) continue;
+        const int r = row(lane, rz);
+        const uint32_t c = sm.S[r] & sm.M[r];
+        sm.S[r] = c ? c & dilate18(sm.F, r) : 0u;
+    }
+    __syncthreads();
+    // fluid nodes next to them, and the counts of both per plane
+    uint32_t excl[SHELL_PLANES];
+#pragma unroll
+    for (int q = 0; q < SHELL_PLANES; q++) {
+        const int rz = warp + q * (PT / 32);
+        excl[q] = 0;
+        if (rz >= ez + 2) continue;  // the same for the whole warp
+        uint32_t v = 0;
+        if (lane < ey + 2) {
+            const int r = row(lane, rz);
+            const uint32_t n = sm.F[r] & dilate18(sm.S, r);
+            sm.M[r] = n;
+            v = (uint32_t)__popc(n) | ((uint32_t)__popc(sm.S[r]) << 16);
+        }
+        uint32_t incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += u;
+        }
+        excl[q] = incl - v;
+        if (lane == 31) sm.plane[rz] = incl;
+    }
+    __syncthreads();
+    uint32_t pl = lane < ez + 2 ? sm.plane[lane] : 0u;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+        const uint32_t u = __shfl_up_sync(full, pl, o);
+        if (lane >= o) pl += u;
     }
-    if (lane == 31) sm.wsum[warp] = incl;
-    __syncthreads();
-    uint32_t total = 0, run = incl - sum;
-#pragma unroll
-    for (int w = 0; w < PT / 32; w++) {
-        if (w < warp) run += sm.wsum[w];
-        total += sm.wsum[w];
-    }
-    for (int r = ra; r < rb; r++) {
-        sm.start[r] = run;
-        run += (uint32_t)__popc(sm.M[r]) | ((uint32_t)__popc(sm.S[r]) << 16);
-    }
-    __syncthreads();
+    const uint32_t total = __shfl_sync(full, pl, 31);
     const int nf = (int)(total & 0xFFFFu), ns = (int)(total >> 16);
-    // the row of item k: the last whose prefix (of the half at shift sh) is <= k
-    auto row_of = [&](int k, int sh) {
-        int lo = 0, hi = rows - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if ((int)((sm.start[mid] >> sh) & 0xFFFFu) <= k)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        return lo;
-    };
-    auto node = [&](int r, int bit) { return sm.base[r] + wrapi(x0 - 1 + bit, L.nx); };
-    for (int k = tid; k < nf; k += PT) {
-        const int r = row_of(k, 0);
-        const int n = node(r, nth_bit(sm.M[r], k - (int)(sm.start[r] & 0xFFFFu)));
-        if (!idx_ok(L, n, L.N, 8)) continue;
-        const float2 v = DENSE ? ld_pair(rho, n) : node_rho2<S>(f, L, n);
-        if (k < SHELL_RHO) sm.rho[k] = v;
-        if (!DENSE) st_pair(rho, n, v);
+#pragma unroll
+    for (int q = 0; q < SHELL_PLANES; q++) {  // prefix over all rows
+        const int rz = warp + q * (PT / 32);
+        const uint32_t before = __shfl_sync(full, pl, max(rz - 1, 0) & 31);
+        if (rz > 0) excl[q] += before;
+        if (rz < ez + 2 && lane < ey + 2) sm.start[row(lane, rz)] = (uint16_t)(excl[q] & 0xFFFFu);
     }
-    __syncthreads();
+    // items [w, w + SHELL_ITEMS) of the fluid (sh = 0) or shell (16) nodes
+    auto expand = [&](const uint32_t *mask, int sh, int w, uint16_t *list) {
+#pragma unroll
+        for (int q = 0; q < SHELL_PLANES; q++) {
+            const int rz = warp + q * (PT / 32);
+            if (rz >= ez + 2 || lane >= ey + 2) continue;
+            const int r = row(lane, rz);
+            int k = (int)((excl[q] >> sh) & 0xFFFFu) - w;
+            for (uint32_t m = mask[r]; m; m &= m - 1, k++)
+                if (k >= 0 && k < SHELL_ITEMS) list[k] = (uint16_t)(r << 5 | (__ffs(m) - 1));
+        }
+    };
+    auto node = [&](int it) { return sm.base[it >> 5] + xnode(it & 31); };
     const float dr = (float)P.drho[p];
-    for (int k0 = 0; k0 < ns; k0 += PT) {  // whole warps: the appends vote
-        const int k = k0 + tid;
-        int n = 0;
-        uint32_t fm = 0;
-        if (k < ns) {
-            const int r = row_of(k, 16);
-            const int bit = nth_bit(sm.S[r], k - (int)(sm.start[r] >> 16));
-            n = node(r, bit);
-            if (idx_ok(L, n, L.N, 9) && owner[n] == (uint32_t)p) {
+    expand(sm.M, 0, 0, sm.fl);
+    for (int ws = 0; ws < ns; ws += SHELL_ITEMS) {
+        const int cs = min(ns - ws, SHELL_ITEMS);
+        if (ws) {
+            __syncthreads();
+            if (tid == 0) sm.owned = sm.next = 0;
+        }
+        expand(sm.S, 16, ws, sm.sl);
+        __syncthreads();
+        // nodes of another particle (overlaps) drop out; the link list's
+        // segment is reserved while the densities come in
+        int mine = 0;
+        for (int k = tid; k < cs; k += PT) {
+            const int n = node(sm.sl[k]);
+            if (idx_ok(L, n, L.N, 9) && owner[n] == (uint32_t)p)
+                mine++;
+            else
+                sm.sl[k] = 0xFFFFu;
+        }
+        mine = __reduce_add_sync(full, mine);
+        if (lane == 0 && mine) atomicAdd(&sm.owned, mine);
+        __syncthreads();
+        const int owned = sm.owned, padded = (owned + sg.pad - 1) / sg.pad * sg.pad;
+        int reserved = 0;
+        if (tid == 0 && ll.ent && owned) reserved = atomicAdd(ll.count, padded);
+        if (ws == 0)
+            for (int wf = 0; wf < nf; wf += SHELL_ITEMS) {
+                if (wf) {
+                    __syncthreads();
+                    expand(sm.M, 0, wf, sm.fl);
+                    __syncthreads();
+                }
+                for (int k = tid; k < min(nf - wf, SHELL_ITEMS); k += PT) {
+                    const int n = node(sm.fl[k]);
+                    if (!idx_ok(L, n, L.N, 8)) continue;
+                    const float2 v = DENSE ? ld_pair(rho, n) : node_rho2<S>(f, L, n);
+                    if (wf == 0) sm.rho[k] = v;
+                    if (!DENSE) st_pair(rho, n, v);
+                }
+            }
+        if (tid == 0) sm.lbase = reserved;
+        __syncthreads();
+        for (int k0 = 0; k0 < cs; k0 += PT) {  // whole warps: positions by vote
+            const int k = k0 + tid;
+            const int it = k < cs ? sm.sl[k] : 0xFFFFu;
+            const bool have = it != 0xFFFFu;
+            int n = 0;
+            uint32_t fm = 0;
+            if (have) {
+                n = node(it);
+                const int r = it >> 5, bit = it & 31;
                 float s0 = 0.f, s1 = 0.f;
-                int cnt = 0;
+                // the neighbour rows' masks and starts, then the 18 in order;
+                // a neighbour that is no fluid node adds zero
+                uint32_t m[9];
+                int st[9];
+#pragma unroll
+                for (int q = 0; q < 9; q++) {
+                    m[q] = sm.M[r + q % 3 - 1 + RS * (q / 3 - 1)];
+                    st[q] = sm.start[r + q % 3 - 1 + RS * (q / 3 - 1)];
+                }
 #pragma unroll
                 for (int i = 1; i < Q; i++) {
-                    const int rr = r + cy(i) + ny * cz(i), b = bit + cx(i);
-                    if (!((sm.F[rr] >> b) & 1u)) continue;
-                    const int idx = (int)(sm.start[rr] & 0xFFFFu) + __popc(sm.M[rr] & ((1u << b) - 1u));
-                    const float2 v = idx < SHELL_RHO ? sm.rho[idx] : ld_pair(rho, node(rr, b));
+                    const int q = cy(i) + 1 + 3 * (cz(i) + 1), b = bit + cx(i);
+                    const bool on = (m[q] >> b) & 1u;
+                    const int idx = st[q] + __popc(m[q] & ((1u << b) - 1u));
+                    float2 v = make_float2(0.f, 0.f);
+                    if (on) v = idx < SHELL_ITEMS ? sm.rho[idx] : ld_pair(rho, sm.base[r + cy(i) + RS * cz(i)] + xnode(b));
                     s0 += v.x;
                     s1 += v.y;
-                    cnt++;
-                    fm |= 1u << i;
+                    fm |= on ? 1u << i : 0u;
                 }
-                shell_psi(L, psi, n, dr, s0, s1, cnt);
+                shell_psi(L, psi, n, dr, s0, s1, __popc(fm));
             }
+            if (!ll.ent) continue;
+            int at = k;
+            if (owned != cs) {  // a segment without gaps
+                const unsigned want = __ballot_sync(full, have);
+                int first = 0;
+                if (want && lane == __ffs(want) - 1) first = atomicAdd(&sm.next, __popc(want));
+                if (want) first = __shfl_sync(full, first, __ffs(want) - 1);
+                at = first + __popc(want & ((1u << lane) - 1u));
+            }
+            if (have && sm.lbase + at < ll.cap) ll.ent[sm.lbase + at] = make_uint2((unsigned)n, fm);
         }
-        if (!ll.ent) continue;
-        const unsigned want = __ballot_sync(0xffffffffu, fm != 0);
-        if (!want) continue;
-        const int leader = __ffs(want) - 1;
-        int at = 0;
-        if (lane == leader) at = atomicAdd(&sm.nbuf, __popc(want));
-        at = __shfl_sync(0xffffffffu, at, leader) + __popc(want & ((1u << lane) - 1u));
-        const bool spill = fm != 0 && at >= SHELL_BUF;
-        if (fm && !spill) sm.buf[at] = make_uint2((unsigned)n, fm);
-        append_links(ll, n, spill ? fm : 0u);
+        if (ll.ent)
+            for (int k = owned + tid; k < padded; k += PT)
+                if (sm.lbase + k < ll.cap) ll.ent[sm.lbase + k] = make_uint2(0u, 0u);
     }
-    if (!ll.ent) return;
-    __syncthreads();
-    const int cnt = min(sm.nbuf, SHELL_BUF);
-    if (tid == 0) sm.lbase = cnt ? atomicAdd(ll.count, cnt) : 0;
-    __syncthreads();
-    for (int k = tid; k < cnt; k += PT)
-        if (sm.lbase + k < ll.cap) ll.ent[sm.lbase + k] = sm.buf[k];
 }
 
 // Shell fill of a 32 x 8 tile of a wall plane (z = 0 or nz - 1, Δρ = 0): the
@@ -1881,7 +1967,7 @@ __device__ void wall_tile(const Lat &L, int tile, const typename S::P *__restric
                           const uint8_t *__restrict__ type, ShellTile &sm)
 {
     constexpr int HX = WALL_X + 2, HN = HX * (WALL_Y + 2);
-    static_assert(HN <= SHELL_RHO && HN <= SHELL_ROWS, "wall tile fits the particle tile's arrays");
+    static_assert(HN <= SHELL_ITEMS && HN <= RS * RS, "wall tile fits the particle tile's arrays");
     const int ntx = (L.nx + WALL_X - 1) / WALL_X, nty = (L.ny + WALL_Y - 1) / WALL_Y;
     const int side = tile / (ntx * nty), t = tile % (ntx * nty);
     const int x0 = (t % ntx) * WALL_X, y0 = (t / ntx) * WALL_Y;
@@ -2133,10 +2219,10 @@ void launch_geom(const Lat &L, const Parts &P, cudaStream_t s)
 
 size_t geom_bytes_per_particle() { return sizeof(PGeom2); }
 
-void launch_integrate(const Lat &L, const Parts &P, int mode, cudaStream_t s)
+void launch_integrate(const Lat &L, const Parts &P, int mode, int *links, cudaStream_t s)
 {
     if (P.n == 0) return;
-    k_integrate<<<(4 * P.n + 127) / 128, 128, 0, s>>>(L, P, mode);
+    k_integrate<<<(4 * P.n + 127) / 128, 128, 0, s>>>(L, P, mode, links);
 }
 
 void launch_claim(const Lat &L, const Parts &P, int, uint32_t *owner_new, cudaStream_t s)
@@ -2160,27 +2246,16 @@ void launch_transition_batch(int storage, const BatchIndex &B, int total, cudaSt
     LBE_DISPATCH(storage, (k_transition_batch<S><<<total, PT, 0, s>>>(B, total)));
 }
 
-void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
-                 const Parts &P, void *fout, cudaStream_t s)
-{
-    if (P.n == 0 || !ll.ent) return;
-    int blocks = (L.N + 255) / 256;
-    if (blocks > 8 * 152) blocks = 8 * 152;
-    LBE_DISPATCH(storage, (k_link<S><<<blocks, 256, 0, s>>>(L, ll, rho, owner, P, (typename S::P *)fout)));
-}
-
-void launch_link_batch(int storage, const BatchIndex &B, cudaStream_t s)
-{
-    dim3 grid(LINK_BATCH_CTAS, B.nbox);
-    LBE_DISPATCH(storage, (k_link_batch<S><<<grid, 256, 0, s>>>(B)));
-}
-
-// Tiles for np particles in boxes of at most ext nodes a side.
+// Tiles for np particles in boxes of at most ext nodes a side.  The small
+// tiles are at most 15 times as many as the large ones, fewer than 15 x 304;
+// each adds at most 7 empty entries to each of its at most two list windows
+// (10 x 5 x 30 nodes): fewer than LINK_PAD in all.
+static_assert(15 * 304 * 2 * 7 <= LINK_PAD, "empty link entries fit");
 static ShellGrid shell_grid(const int ext[3], int np)
 {
     auto up = [](int a, int b) { return (a + b - 1) / b; };
-    ShellGrid g{up(ext[0], SHELL_X), up(ext[1], 22), up(ext[2], 22), 22, 22};
-    if ((long long)np * g.nx * g.ny * g.nz < 2 * 152) g = ShellGrid{g.nx, up(ext[1], 10), up(ext[2], 5), 10, 5};
+    ShellGrid g{up(ext[0], SHELL_X), up(ext[1], SHELL_MAX), up(ext[2], SHELL_MAX), SHELL_MAX, SHELL_MAX, 1};
+    if ((long long)np * g.nx * g.ny * g.nz < 2 * 152) g = ShellGrid{g.nx, up(ext[1], 10), up(ext[2], 5), 10, 5, 8};
     return g;
 }
 
@@ -2193,6 +2268,13 @@ static void shell_extent(const Lat &L, double rmax, int ext[3])
     for (int k = 0; k < 3; k++) ext[k] = std::max(ext[k], e < n[k] ? (int)e : n[k]);
 }
 
+static ShellGrid lattice_grid(const Lat &L, const Parts &P)
+{
+    int ext[3] = {1, 1, 1};
+    shell_extent(L, P.rmax, ext);
+    return shell_grid(ext, P.n);
+}
+
 template <class S, bool DENSE>
 static void shell_fill_launch(unsigned ctas, const Lat &L, const Parts &P, const ShellGrid &g, const void *f, float *rho,
                               float *psi, const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
@@ -2203,18 +2285,30 @@ static void shell_fill_launch(unsigned ctas, const Lat &L, const Parts &P, const
 void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
                        const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
 {
-    ShellGrid g{0, 0, 0, 1, 1};
-    if (P.n > 0) {
-        int ext[3] = {1, 1, 1};
-        shell_extent(L, P.rmax, ext);
-        g = shell_grid(ext, P.n);
-    }
+    const ShellGrid g = P.n > 0 ? lattice_grid(L, P) : ShellGrid{0, 0, 0, 1, 1, 1};
     const long long ctas = (long long)P.n * g.nx * g.ny * g.nz + wall_tiles(L);
     if (ctas == 0) return;
     if (dense)
         LBE_DISPATCH(storage, (shell_fill_launch<S, true>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
     else
         LBE_DISPATCH(storage, (shell_fill_launch<S, false>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
+}
+
+void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
+                 const Parts &P, void *fout, cudaStream_t s)
+{
+    if (P.n == 0 || !ll.ent) return;
+    int blocks = (L.N + 255) / 256;
+    if (blocks > 8 * 152) blocks = 8 * 152;
+    const int group = lattice_grid(L, P).pad == 8 ? 8 : 32;
+    LBE_DISPATCH(storage, (k_link<S><<<blocks, 256, 0, s>>>(L, ll, rho, owner, P, (typename S::P *)fout, group)));
+}
+
+void launch_link_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, cudaStream_t s)
+{
+    dim3 grid(LINK_BATCH_CTAS, B.nbox);
+    const int group = shell_grid(ext, total_parts).pad == 8 ? 8 : 32;
+    LBE_DISPATCH(storage, (k_link_batch<S><<<grid, 256, 0, s>>>(B, group)));
 }
 
 int batch_wall_tiles(const Lat &L) { return wall_tiles(L); }
@@ -2224,7 +2318,7 @@ void launch_begin_batch(const BatchIndex &B, cudaStream_t s) { k_begin_batch<<<1
 void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, int total_walls,
                         cudaStream_t s)
 {
-    const ShellGrid g = total_parts > 0 ? shell_grid(ext, total_parts) : ShellGrid{0, 0, 0, 1, 1};
+    const ShellGrid g = total_parts > 0 ? shell_grid(ext, total_parts) : ShellGrid{0, 0, 0, 1, 1, 1};
     const long long ctas = (long long)total_parts * g.nx * g.ny * g.nz + total_walls;
     if (ctas == 0) return;
     LBE_DISPATCH(storage, (k_shell_batch<S><<<(unsigned)ctas, PT, 0, s>>>(B, g, total_parts)));
