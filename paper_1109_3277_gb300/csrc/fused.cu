@@ -56,7 +56,7 @@ __device__ __forceinline__ int wrapc(int v, int n)
 // (any τ) or not (τ = 1), and SELF (the box holds
 // the tile and a one-node halo, whose densities the kernel forms itself) or
 // not (the box holds the tile; ψ of every ring entry comes from memory).
-template <class S, int TY, bool GEN, bool SELF>
+template <class S, int TY, bool GEN, bool SELF, bool TMA>
 struct Cfg {
     using P = typename S::P;
     static constexpr int NT = TX * TY;
@@ -64,7 +64,7 @@ struct Cfg {
     static constexpr int PADX = SELF ? 16 / E : 0;    // x margin of the box: 16 bytes
     static constexpr int BX = TX + 2 * PADX, BY = SELF ? TY + 2 : TY;
     static constexpr int HX = TX + 2, HY = TY + 2, HN = HX * HY, NHALO = HN - NT;
-    static constexpr size_t plane = (size_t)Q * BY * BX * E;        // bytes of one box
+    static constexpr size_t plane = TMA ? (size_t)Q * BY * BX * E : 0;  // bytes of one box
     static constexpr size_t pstride = (plane + 127) / 128 * 128;    // stages 128-byte aligned
     // CTAs per SM the kernel is compiled for: what shared memory allows
     // (228 KB per SM, about 1 KB of it reserved per CTA), capped so that a
@@ -77,7 +77,7 @@ struct Cfg {
         4 * HN * sizeof(float2) + MSLOTS * HY * sizeof(unsigned long long) + twords + 128 + 1024;
     static constexpr int ctas_for(int nst)
     {
-        const int m = (int)((228 * 1024) / (nst * pstride + nst * 8 + other));
+        const int m = (int)((228 * 1024) / (nst * pstride + nst * 8 + other));  // without TMA nothing is staged
         return m < by_regs ? (m > 0 ? m : 1) : by_regs;
     }
     // stage buffers: any τ with SELF re-reads plane z's box one iteration
@@ -88,7 +88,7 @@ struct Cfg {
     // three CTAs it leaves room for cover the copy (two boxes: one CTA of
     // eight warps per SM).  Without SELF a third buffer lets the copies run
     // two planes ahead where it costs no CTA per SM
-    static constexpr bool RELAX_STAGE = GEN && SELF && E == 4;
+    static constexpr bool RELAX_STAGE = GEN && SELF && TMA && E == 4;
     static constexpr int NST = RELAX_STAGE ? 3 : (SELF ? (E == 8 ? 1 : 2) : (ctas_for(3) >= ctas_for(2) ? 3 : 2));
     static constexpr int CTAS = ctas_for(NST);
     // dynamic shared memory (bytes from a 128-byte aligned base)
@@ -408,11 +408,11 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                                            const CUtensorMap *tmap, int bx, int by, int bz, int wait_limit,
                                            unsigned char *smem)
 {
-    using C = Cfg<S, TY, GEN, SELF>;
+    using C = Cfg<S, TY, GEN, SELF, TMA>;
     using P = typename S::P;
     constexpr int HX = C::HX, HN = C::HN, BX = C::BX, BY = C::BY, NST = C::NST;
     constexpr size_t PSTR = C::pstride / sizeof(P);  // pairs from one stage to the next
-    constexpr int BXY = SELF && !TMA ? HN : BX * BY;  // pairs from one direction of a stage to the next
+    constexpr int BXY = BX * BY;  // pairs from one direction of a stage to the next
     const P *stage = reinterpret_cast<const P *>(smem + C::stage);
     float2 *sps = reinterpret_cast<float2 *>(smem + C::sps);                                // [slot][e]
     unsigned long long *smask = reinterpret_cast<unsigned long long *>(smem + C::smask);   // [slot][ey]
@@ -436,7 +436,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         e.ring = ey * HX + ex;
         const int lx = x0 - 1 + ex, ly = y0 - 1 + ey;
         if (SELF) {
-            e.st = TMA ? ey * BX + ex - 1 + C::PADX : e.ring;
+            e.st = ey * BX + ex - 1 + C::PADX;
             e.inlat = TMA && lx >= 0 && lx < L.nx && ly >= 0 && ly < L.ny;
         } else {  // only the own entries of active nodes are in the box
             e.st = (ey - 1) * BX + ex - 1;
@@ -783,21 +783,11 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         __syncthreads();
         // plane copies: issued after the barrier of iteration k is box k +
         // NST - LAG (with LAG the collision re-reads the box one iteration
-        // after its densities); a thread without TMA copies its own entries
-        // (never read by another) for k + 1 once it has taken in plane k
+        // after its densities).  Without TMA the entries are read from global
+        // memory (staging them by cp.async, 19 copies a thread, cost more
+        // instructions than the latency it hid: 201 x 180 x 160 f16 457 us a
+        // step against 439)
         constexpr int LAG = C::RELAX_STAGE ? 2 : 0;
-        auto self_copy = [&](int k, int b) {
-            const int p = zb - 1 + k;
-            if (!pvalid(p)) return;
-            const size_t g = (size_t)nxy * gz_of(p);
-            P *d = const_cast<P *>(stage) + (size_t)b * PSTR;
-#pragma unroll
-            for (int i = 0; i < Q; i++) cp_async<sizeof(P)>(d + i * BXY + own.st, fin + pidx(L, i, (long long)(own.xy + g)));
-            if (has_halo)
-#pragma unroll
-                for (int i = 0; i < Q; i++)
-                    cp_async<sizeof(P)>(d + i * BXY + hal.st, fin + pidx(L, i, (long long)(hal.xy + g)));
-        };
         // ψ of the solid entries of plane k straight into the ring, in flight
         // until the plane is taken in
         auto solid_psi = [&](int k, const Ent &e, uint8_t t) {
@@ -808,13 +798,9 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             cp_async<4>(&d->x, psi + (size_t)L.N + n);
             cp_async<4>(&d->y, psi + n);
         };
-        if (TMA) {
 #pragma unroll
-            for (int q = 0; q < NST; q++)
-                if (q < kmax) issue(q, q);
-        } else {
-            self_copy(0, 0);
-        }
+        for (int q = 0; q < NST; q++)
+            if (q < kmax) issue(q, q);
         uint8_t t_own = load_type(0, own), t_hal = has_halo ? load_type(0, hal) : WALL;
         solid_psi(0, own, t_own);
         if (has_halo) solid_psi(0, hal, t_hal);
@@ -843,7 +829,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                 };
                 unsigned long long *mrows = smask + (k & MS) * C::HY;
                 if (t_own == FLUID && pv) {
-                    if (!TMA || own.inlat) {
+                    if (own.inlat) {
                         mnext = moments([&](int i) { return S::raw2(sb[i * BXY + own.st]); });
                     } else {
                         const size_t n = own.xy + gbase;
@@ -858,7 +844,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                         atomicOr(&mrows[hal.ey], 1ull << hal.ex);
                     } else if (pv) {
                         float2 dr;
-                        if (!TMA || hal.inlat) {
+                        if (hal.inlat) {
                             dr = density_sum([&](int i) { return S::raw2(sb[i * BXY + hal.st]); });
                         } else {
                             const size_t n = hal.xy + gbase;
@@ -868,7 +854,6 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                     }
                 }
             }
-            if (!TMA && k + 1 < kmax) self_copy(k + 1, b_next);
             if (__syncthreads_or(late)) {
                 ok = false;
                 break;
@@ -912,7 +897,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
 }
 
 template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32>
-__global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF>::CTAS))
+__global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
     k_fused(Lat L, const typename S::P *__restrict__ fin, typename S::P *__restrict__ fout,
             const float *__restrict__ psi, const uint8_t *__restrict__ type, int zc, FusedOfs ofs,
             const __grid_constant__ CUtensorMap tmap, int wait_limit)
@@ -931,7 +916,7 @@ __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF>::CTAS))
 constexpr int BATCH_TY = FUSED_TY_BATCH;
 
 template <class S, bool GEN>
-__global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true>::CTAS)) k_fused_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true, true>::CTAS)) k_fused_batch(BatchIndex B, int total)
 {
     constexpr int NT = TX * BATCH_TY;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -991,12 +976,15 @@ int fused_zchunk(const Lat &L, int ty, int es, bool self, double share)
     // 8 planes, 652 at 16, 805 at 48; f32 964 at 4, 1095 at 16.  With ψ from
     // memory (256^3 bijel, f16) 564 at 16, 601 at 64.
     const long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
-    const int cap = self ? (es == 4 ? 4 : 8) : 16, slots = 3 * 8 / ty;
+    const bool tma = (L.nx * 2 * es) % 16 == 0;
+    const int cap = !self ? 16 : (!tma ? 12 : (es == 4 ? (ty == 4 ? 5 : 4) : 8));
+    const int slots = (fused_tau1(L) && fused_rel32(L) ? 3 : 2) * 8 / ty;  // CTAs an SM takes
+    const double full = 1.7 + 0.9 * slots * ty / 8;
     int best = 1;
     double bt = 1e30;
     for (int zc = 1; zc <= L.nz && zc <= cap; zc++) {
         const double ctas = std::ceil(cols * std::ceil((double)L.nz / zc) / (152 * share));
-        const double t = (zc + 3) * (ctas <= slots ? 1.7 + 0.9 * ctas * ty / 8 : 4.4 * ctas / slots);
+        const double t = (zc + 3) * (ctas <= slots ? 1.7 + 0.9 * ctas * ty / 8 : full * ctas / slots);
         if (t < bt * 0.999) {
             bt = t;
             best = zc;
@@ -1061,7 +1049,7 @@ template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32>
 static void launch_cfg(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
                        const CUtensorMap &tm, int zc, int wait_limit, cudaStream_t s)
 {
-    using C = Cfg<S, TY, GEN, SELF>;
+    using C = Cfg<S, TY, GEN, SELF, TMA>;
     using P = typename S::P;
     auto kern = k_fused<S, TY, GEN, SELF, TMA, R32>;
     static bool configured = false;  // the attribute is per function and process
@@ -1104,16 +1092,21 @@ static void launch_fused_t(const Lat &L, const void *fin, void *fout, const floa
     }
 }
 
-int fused_rows(const Lat &L, int ty_request, bool tma)
+int fused_rows(const Lat &L, int ty_request, bool tma, int storage, bool self)
 {
-    // only the τ = 1 configurations with TMA come in two heights
-    return (ty_request == 4 && tma && fused_tau1(L) && fused_rel32(L)) ? 4 : 8;
+    // only the τ = 1 configurations with TMA come in two heights.  By
+    // default (request 0) FP32 with ψ on chip takes 4 rows: five CTAs of four
+    // warps fit an SM against three of eight, and one that waits idles fewer
+    // warps (256^3 909 us against 961, 128^3 133 against 140, 64^3 22.6
+    // against 24.5)
+    if (!tma || !fused_tau1(L) || !fused_rel32(L)) return 8;
+    return ty_request == 4 || (ty_request == 0 && self && storage == LBE_STORE_F32) ? 4 : 8;
 }
 
 void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
                   const CUtensorMap *tmap, cudaStream_t s, int zc, int ty, int wait_limit, bool self)
 {
-    const int rows = fused_rows(L, ty, tmap != nullptr);
+    const int rows = fused_rows(L, ty, tmap != nullptr, storage, self);
     if (zc <= 0) zc = fused_zchunk(L, rows, storage == LBE_STORE_F32 ? 4 : 2, self, 1.0);
     if (zc > L.nz) zc = L.nz;
     if (self)
@@ -1128,7 +1121,7 @@ static void batch_configure()
     static bool configured = false;  // the attribute is per function and process
     if (!configured) {
         cudaFuncSetAttribute(k_fused_batch<S, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Cfg<S, BATCH_TY, GEN, true>::bytes);
+                             (int)Cfg<S, BATCH_TY, GEN, true, true>::bytes);
         configured = true;
     }
 }
@@ -1136,7 +1129,7 @@ static void batch_configure()
 template <class S, bool GEN>
 static void launch_fused_batch_t(const BatchIndex &B, int total, int ctas, cudaStream_t s)
 {
-    using C = Cfg<S, BATCH_TY, GEN, true>;
+    using C = Cfg<S, BATCH_TY, GEN, true, true>;
     batch_configure<S, GEN>();
     k_fused_batch<S, GEN><<<ctas < total ? ctas : total, C::NT, C::bytes, s>>>(B, total);
 }
@@ -1150,7 +1143,7 @@ static int batch_occupancy()
     int n = 0;
     batch_configure<S, GEN>();
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S, GEN>, TX * BATCH_TY,
-                                                  Cfg<S, BATCH_TY, GEN, true>::bytes);
+                                                  Cfg<S, BATCH_TY, GEN, true, true>::bytes);
     return n > 0 ? n : 1;
 }
 

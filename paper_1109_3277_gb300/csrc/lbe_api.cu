@@ -47,7 +47,7 @@ struct lbe_ctx {
     // graphs keyed by (cur, ocur)
     cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
     int zc_tuned = 0;  // fused-kernel z chunk chosen by lbe_autotune (0: heuristic)
-    int ty_tuned = 8;  // fused-kernel tile rows chosen by lbe_autotune
+    int ty_tuned = 0;  // fused-kernel tile rows chosen by lbe_autotune (0: the default)
     int wait_limit = FUSED_WAIT_LIMIT;  // tries of each bounded wait for a box copy
     // profiling
     bool profiling = false;
@@ -222,7 +222,8 @@ bool fused_self(const lbe_ctx *c) { return 50.0 * c->area < (double)c->L.N; }
 const CUtensorMap *fused_map(const lbe_ctx *c, int buf, int ty)
 {
     if (!c->tma) return nullptr;
-    return &c->tmap[fused_self(c) ? 1 : 0][fused_rows(c->L, ty, true) == 4 ? 1 : 0][buf];
+    const bool self = fused_self(c);
+    return &c->tmap[self ? 1 : 0][fused_rows(c->L, ty, true, c->d.storage, self) == 4 ? 1 : 0][buf];
 }
 
 // Enqueue one time step (no host synchronisation).
@@ -845,15 +846,15 @@ lbe_status lbe_autotune(lbe_ctx *c, int32_t *chosen_zc)
         if (zc + zc / 2 < L.nz) zcs.push_back(zc + zc / 2);
     }
     zcs.push_back(L.nz);
+    const bool self = fused_self(c);
     std::vector<int> tys = {8};
-    if (fused_rows(L, 4, c->tma) == 4) tys.push_back(4);
+    if (fused_rows(L, 4, c->tma, c->d.storage, self) == 4) tys.push_back(4);
     cudaEvent_t e0, e1;
     CK(c, cudaEventCreate(&e0));
     CK(c, cudaEventCreate(&e1));
     void *fin = c->f[c->cur], *fout = c->f[1 - c->cur];
     // ψ of the solid nodes, as the step's shell fill gives them
     c->P.n = c->np;
-    const bool self = fused_self(c);
     if (!self) launch_rho(c->d.storage, L, fin, c->type, c->rho, c->psi, c->stream);
     launch_shell_fill(c->d.storage, L, c->P, !self, fin, c->rho, c->psi, c->type, c->owner[c->ocur],
                       LinkList{nullptr, nullptr, 0}, c->stream);
@@ -918,7 +919,7 @@ lbe_status lbe_get_tile(const lbe_ctx *c, int32_t *rows, int32_t *zc)
         *zc = 0;
         return LBE_OK;
     }
-    *rows = fused_rows(c->L, c->ty_tuned, c->tma);
+    *rows = fused_rows(c->L, c->ty_tuned, c->tma, c->d.storage, fused_self(c));
     *zc = c->zc_tuned > 0 ? c->zc_tuned : fused_zchunk(c->L, *rows, (int)c->esize, fused_self(c), 1.0);
     return LBE_OK;
 }

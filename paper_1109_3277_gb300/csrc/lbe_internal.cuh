@@ -403,7 +403,7 @@ void launch_flip_batch(const BatchIndex &B, cudaStream_t s);
 // ---- launchers (fused.cu) -------------------------------------------------
 // The fused kernel's tiles are 32 nodes wide and 4 or 8 rows high; zc is the
 // z chunk in planes (0: the default for the lattice), ty the requested tile
-// height (4 or 8; configurations without a 4-row variant take 8), and
+// height (4 or 8, 0 the default; configurations without a 4-row variant take 8), and
 // wait_limit the tries of each bounded wait for a box copy.
 constexpr int FUSED_TX = 32, FUSED_TY_BATCH = 8;
 constexpr int FUSED_WAIT_LIMIT = 1 << 22;
@@ -415,8 +415,9 @@ void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const 
 // The default z chunk for tiles of ty rows, populations of es bytes, and a
 // lattice that gets the given share of the GPU (1, or less in a batch).
 int fused_zchunk(const Lat &L, int ty, int es, bool self, double share);
-// The tile height launch_fused takes for a request (4 only where built).
-int fused_rows(const Lat &L, int ty_request, bool tma);
+// The tile height launch_fused takes for a request (4 or 8, 0 for the default;
+// 4 only where built).
+int fused_rows(const Lat &L, int ty_request, bool tma, int storage, bool self);
 bool fused_tau1(const Lat &L);
 // Tensor map of one population buffer for the fused kernel's box copies
 // (tile plus a one-node halo, x widened to 16-byte boundaries: 40 x (ty+2) x
