@@ -148,8 +148,8 @@ void free_all(lbe_ctx *c)
     cudaFree(c->x32);
     cudaFree(c->ppart);
     cudaFree(c->geo);
-    cudaFree(c->cells.count);
-    cudaFree(c->cells.idx);
+    cudaFree(c->cells.head);
+    cudaFree(c->cells.next);
     cudaFree(c->ll.ent);
     cudaFree(c->ll.count);
     if (c->L.err) cudaFree(c->L.err);
@@ -307,32 +307,30 @@ lbe_status build_cells(lbe_ctx *c, const std::vector<double> &blk, int cap, int 
         cinv[k] = (float)((double)n / dim[k]);
         ncell *= n;
     }
-    // count | start | fill in one buffer, idx | cid in another; the old
-    // buffers go only once the new ones exist
-    const size_t b0 = (size_t)(3 * ncell + 1) * sizeof(int), b1 = (size_t)2 * cap * sizeof(int);
-    int *ncount = nullptr, *nidx = nullptr;
-    cudaError_t e = lib_malloc((void **)&ncount, b0);
+    // head in one buffer, next | cid in another; the old buffers go only once
+    // the new ones exist
+    const size_t b0 = (size_t)ncell * sizeof(int), b1 = (size_t)2 * cap * sizeof(int);
+    int *nhead = nullptr, *nnext = nullptr;
+    cudaError_t e = lib_malloc((void **)&nhead, b0);
     if (e != cudaSuccess) return cuda_fail(c, e, "add_particles: cudaMalloc(cells)");
-    e = lib_malloc((void **)&nidx, b1);
+    e = lib_malloc((void **)&nnext, b1);
     if (e != cudaSuccess) {
-        cudaFree(ncount);
+        cudaFree(nhead);
         return cuda_fail(c, e, "add_particles: cudaMalloc(cells)");
     }
-    if (C.count) {
-        cudaFree(C.count);
-        cudaFree(C.idx);
+    if (C.head) {
+        cudaFree(C.head);
+        cudaFree(C.next);
         c->bytes -= c->cells_bytes;
     }
-    C.count = ncount;
-    C.idx = nidx;
+    C.head = nhead;
+    C.next = nnext;
     C.ncell = (int)ncell;
     for (int k = 0; k < 3; k++) {
         C.n[k] = cn[k];
         C.inv[k] = cinv[k];
     }
-    C.start = C.count + ncell;
-    C.fill = C.start + ncell + 1;
-    C.cid = C.idx + cap;
+    C.cid = C.next + cap;
     c->cells_bytes = b0 + b1;
     c->bytes += c->cells_bytes;
     return LBE_OK;
@@ -785,8 +783,8 @@ int32_t lbe_kernels_per_step(const lbe_ctx *c)
         k = 1 + (c->np > 0 || c->d.walls_z ? 1 : 0) + (fused_self(c) ? 0 : 1);
     if (c->np > 0) {
         // links, pairs, the update (with the geometry of the new coverage);
-        // from pairs_by_cells on the cell list (count, prefix, fill)
-        k += 3 + (pairs_by_cells(c->np) ? 3 : 0);
+        // with many particles the cell lists
+        k += 3 + (pairs_by_cells(c->np) ? 1 : 0);
         if (c->d.particle_mode != LBE_PARTICLES_STATIC) k += 3;  // claim, transition, reset
     }
     return k;

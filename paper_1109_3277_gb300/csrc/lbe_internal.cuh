@@ -304,10 +304,8 @@ struct Cells {
     int n[3];          // cells per axis
     float inv[3];      // cells per lattice unit
     int ncell;
-    int *count;        // [ncell] particles per cell
-    int *start;        // [ncell + 1] exclusive prefix
-    int *fill;         // [ncell] fill cursor
-    int *idx;          // [cap] particle indices by cell
+    int *head;         // [ncell] first particle of each cell, -1 for none
+    int *next;         // [cap] next particle of the same cell, -1 at the end
     int *cid;          // [cap] cell of each particle
 };
 
@@ -454,8 +452,8 @@ void launch_links(int storage, const Lat &L, const Parts &P, void *fnew, const f
 void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
                  const Parts &P, void *fout, cudaStream_t s);
 void launch_pairs(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, cudaStream_t s);
-// Whether the pair forces of np particles take the cell list (three more
-// kernels) or a loop over all partners.
+// Whether the pair forces of np particles take the cell lists (one more
+// kernel) or a loop over all partners.
 bool pairs_by_cells(int np);
 // The update of the particles and, unless they are static, the geometry of
 // their new coverage; links (may be null): the link list's counter, set to 0.

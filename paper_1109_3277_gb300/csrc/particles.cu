@@ -458,15 +458,23 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
     PGeom2 &G = reinterpret_cast<PGeom2 *>(P.geo)[p];
     constexpr int GW = (int)(sizeof(PGeom) / 8);
     static_assert(sizeof(PGeom) % 8 == 0, "PGeom is copied in 8-byte words");
-    auto copy_now = [&] {  // old_ = now
+    // old_ = now: all loads, then all stores (a load after a store that may
+    // alias it waits: one round trip to memory instead of eleven)
+    auto copy_now = [&] {
         const double *src = reinterpret_cast<const double *>(&G.now);
         double *dst = reinterpret_cast<double *>(&G.old_);
+        double v[(GW + 3) / 4];
+#pragma unroll
+        for (int w = 0; w < (GW + 3) / 4; w++) v[w] = lane + 4 * w < GW ? src[lane + 4 * w] : 0.0;
+        __syncwarp();
         if (act)
-            for (int w = lane; w < GW; w += 4) dst[w] = src[w];
+#pragma unroll
+            for (int w = 0; w < (GW + 3) / 4; w++)
+                if (lane + 4 * w < GW) dst[lane + 4 * w] = v[w];
         __syncwarp();
     };
+    const double rp = P.rp[p], ro = P.ro[p], lo_was = G.now.lo[k], hi_was = G.now.hi[k];
     if (!first) copy_now();
-    const double rp = P.rp[p], ro = P.ro[p];
     double row[3], col[3];
     quad_rot(k, q, row, col);
     const double h = sqrt(rp * rp * row[0] * row[0] + ro * ro * (row[1] * row[1] + row[2] * row[2]));
@@ -499,7 +507,7 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
     double lu, hu;
     box_axis(Xu, h, lu, hu);
     const bool eu = quad_empty(lu, hu);
-    double lo0 = first ? lo : G.old_.lo[k], hi0 = first ? hi : G.old_.hi[k];
+    double lo0 = first ? lo : lo_was, hi0 = first ? hi : hi_was;
     const bool e0 = quad_empty(lo0, hi0);
     if (e0) {
         lo0 = lu;
@@ -730,8 +738,8 @@ struct LinkWarp {
 // The links of up to 32 list entries (e = (node, mask of fluid neighbours)
 // per lane; mask 0 for a lane without an entry).  The entries' links are
 // laid out direction by direction, so that lanes taking neighbouring links
-// touch the same slot array at neighbouring nodes, and handed out 32 at a
-// time: every lane carries one link per round, and the loads of a round are
+// touch the same slot array at neighbouring nodes, and handed out 64 at a
+// time: every lane carries two links per round, and the loads of a round are
 // all in flight together.  What belongs to the entry (its place, the arm from
 // the particle) is formed once by the entry's lane.  Where all entries are of
 // one particle (most warps), each lane adds up its own terms over the rounds
@@ -799,21 +807,26 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, const float 
     float4 V = K32[2 * p0], W = K32[2 * p0 + 1];
     unsigned long long sum[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
     __syncwarp();
-    for (int k0 = 0; k0 < total; k0 += 32) {
-        const int k = k0 + lane;
-        const bool act = k < total;
-        const int d = act ? w.desc[k] : 0;
-        const int src = d & 31, j = act ? d >> 5 : 1;
-        const int sn = __shfl_sync(full, s, src), pn = __shfl_sync(full, p, src);
-        const float ex = __shfl_sync(full, dx, src), ey = __shfl_sync(full, dy, src), ez = __shfl_sync(full, dz, src);
-        const unsigned fc = __shfl_sync(full, face, src);
-        unsigned long long acc[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-        if (act) {
-            if (!uniform) {
-                V = K32[2 * pn];
-                W = K32[2 * pn + 1];
-            }
-            const int cxj = cdir(CXP, j), cyj = cdir(CYP, j), czj = cdir(CZP, j);
+    // two links a lane per round: the loads of both are in flight together
+    constexpr int U = 2;
+    for (int k0 = 0; k0 < total; k0 += 32 * U) {
+        int j[U], pn[U];
+        float rx[U], ry[U], rz[U];
+        typename S::P *q[U], raw[U];
+        float2 rho_y[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = k0 + 32 * u + lane;
+            const int d = k < total ? w.desc[k] : 0;
+            const int src = d & 31;
+            j[u] = d >> 5;  // 0: no link
+            const int sn = __shfl_sync(full, s, src);
+            pn[u] = __shfl_sync(full, p, src);
+            const float ex = __shfl_sync(full, dx, src), ey = __shfl_sync(full, dy, src),
+                        ez = __shfl_sync(full, dz, src);
+            const unsigned fc = __shfl_sync(full, face, src);
+            if (!j[u]) continue;
+            const int cxj = cdir(CXP, j[u]), cyj = cdir(CYP, j[u]), czj = cdir(CZP, j[u]);
             // the fluid node s + c_j, around the periodic faces
             int yf = sn + cxj + L.nx * (cyj + L.ny * czj);
             if (cxj > 0 && (fc & 1u)) yf -= L.nx;
@@ -822,39 +835,53 @@ __device__ __forceinline__ void link_entries(const Lat &L, uint2 e, const float 
             if (cyj < 0 && (fc & 8u)) yf += L.nx * L.ny;
             if (czj > 0 && (fc & 16u)) yf -= L.N;
             if (czj < 0 && (fc & 32u)) yf += L.N;
-            const float fcx = (float)cxj, fcy = (float)cyj, fcz = (float)czj;
-            const float rx = ex + 0.5f * fcx, ry = ey + 0.5f * fcy, rz = ez + 0.5f * fcz;
-            // surface velocity V + ω × r_b at the link midpoint
-            const float usx = __fsub_rn(__fmaf_rn(W.y, rz, V.x), __fmul_rn(W.z, ry));
-            const float usy = __fsub_rn(__fmaf_rn(W.z, rx, V.y), __fmul_rn(W.x, rz));
-            const float usz = __fsub_rn(__fmaf_rn(W.x, ry, V.z), __fmul_rn(W.y, rx));
-            // u_surf·c_i with c_i = -c_j
-            const float uci = -__fadd_rn(__fadd_rn(usx * fcx, usy * fcy), usz * fcz);
-            const float w6 = j < 7 ? -6.f / 18.f : -6.f / 36.f;
+            rx[u] = ex + 0.5f * (float)cxj;
+            ry[u] = ey + 0.5f * (float)cyj;
+            rz[u] = ez + 0.5f * (float)czj;
             // both components of slot j of the fluid node: one pair access
-            typename S::P *q = fout + pidx(L, j, yf);
-            const float2 fs = ld2f<S>(fout, L, j, yf);
-            const float2 ry2 = __ldg(reinterpret_cast<const float2 *>(rho) + yf);
-            const float C0 = __fmul_rn(__fmul_rn(w6, ry2.x), uci);
-            const float C1 = __fmul_rn(__fmul_rn(w6, ry2.y), uci);
-            *q = S::enc2(make_float2(__fadd_rn(fs.x, C0) - L.base[0][j], __fadd_rn(fs.y, C1) - L.base[1][j]));
-            float a = 0.f;
-            a = __fadd_rn(a, __fmaf_rn(2.f, fs.x, C0));
-            a = __fadd_rn(a, __fmaf_rn(2.f, fs.y, C1));
-            // F = a c_i = -a c_j
-            const float Fx = -a * fcx, Fy = -a * fcy, Fz = -a * fcz;
-            acc[0] = to_fixed(Fx);
-            acc[1] = to_fixed(Fy);
-            acc[2] = to_fixed(Fz);
-            acc[3] = to_fixed(__fsub_rn(__fmul_rn(ry, Fz), __fmul_rn(rz, Fy)));
-            acc[4] = to_fixed(__fsub_rn(__fmul_rn(rz, Fx), __fmul_rn(rx, Fz)));
-            acc[5] = to_fixed(__fsub_rn(__fmul_rn(rx, Fy), __fmul_rn(ry, Fx)));
+            q[u] = fout + pidx(L, j[u], yf);
+            raw[u] = *q[u];
+            rho_y[u] = __ldg(reinterpret_cast<const float2 *>(rho) + yf);
         }
-        if (uniform) {
 #pragma unroll
-            for (int c = 0; c < 6; c++) sum[c] += acc[c];
-        } else {
-            warp_add_fix(act ? pn : -1, acc, fix);
+        for (int u = 0; u < U; u++) {
+            unsigned long long acc[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+            if (j[u]) {
+                if (!uniform) {
+                    V = K32[2 * pn[u]];
+                    W = K32[2 * pn[u] + 1];
+                }
+                const float fcx = (float)cdir(CXP, j[u]), fcy = (float)cdir(CYP, j[u]), fcz = (float)cdir(CZP, j[u]);
+                // surface velocity V + ω × r_b at the link midpoint
+                const float usx = __fsub_rn(__fmaf_rn(W.y, rz[u], V.x), __fmul_rn(W.z, ry[u]));
+                const float usy = __fsub_rn(__fmaf_rn(W.z, rx[u], V.y), __fmul_rn(W.x, rz[u]));
+                const float usz = __fsub_rn(__fmaf_rn(W.x, ry[u], V.z), __fmul_rn(W.y, rx[u]));
+                // u_surf·c_i with c_i = -c_j
+                const float uci = -__fadd_rn(__fadd_rn(usx * fcx, usy * fcy), usz * fcz);
+                const float w6 = j[u] < 7 ? -6.f / 18.f : -6.f / 36.f;
+                const float2 base = make_float2(L.base[0][j[u]], L.base[1][j[u]]), st = S::raw2(raw[u]);
+                const float2 fs = make_float2(base.x + st.x, base.y + st.y);
+                const float C0 = __fmul_rn(__fmul_rn(w6, rho_y[u].x), uci);
+                const float C1 = __fmul_rn(__fmul_rn(w6, rho_y[u].y), uci);
+                *q[u] = S::enc2(make_float2(__fadd_rn(fs.x, C0) - base.x, __fadd_rn(fs.y, C1) - base.y));
+                float a = 0.f;
+                a = __fadd_rn(a, __fmaf_rn(2.f, fs.x, C0));
+                a = __fadd_rn(a, __fmaf_rn(2.f, fs.y, C1));
+                // F = a c_i = -a c_j
+                const float Fx = -a * fcx, Fy = -a * fcy, Fz = -a * fcz;
+                acc[0] = to_fixed(Fx);
+                acc[1] = to_fixed(Fy);
+                acc[2] = to_fixed(Fz);
+                acc[3] = to_fixed(__fsub_rn(__fmul_rn(ry[u], Fz), __fmul_rn(rz[u], Fy)));
+                acc[4] = to_fixed(__fsub_rn(__fmul_rn(rz[u], Fx), __fmul_rn(rx[u], Fz)));
+                acc[5] = to_fixed(__fsub_rn(__fmul_rn(rx[u], Fy), __fmul_rn(ry[u], Fx)));
+            }
+            if (uniform) {
+#pragma unroll
+                for (int c = 0; c < 6; c++) sum[c] += acc[c];
+            } else {
+                warp_add_fix(j[u] ? pn[u] : -1, acc, fix);
+            }
         }
     }
     if (uniform) {
@@ -990,8 +1017,7 @@ __device__ __forceinline__ bool near_pair(float4 me, float4 o, const float nl[3]
 // of the partners' indices, one component per lane, which gives the sums of
 // a plain loop bit for bit.  525
 // particles (150 x 141 x 133, 10 %): 81 us with one lane per particle, 34
-// now; 25,033: 127 and 175 us, where the other lanes' work had filled the
-// warps (1.7 % of that step).
+// now; 25,033: 127 us with one lane, 105 now.
 //
 // Up to PAIRS_SCAN_MAX particles the loop over all partners replaces the
 // cell list: its three kernels and the clearing cost about 10 us however few
@@ -1006,6 +1032,7 @@ struct PairGroup {
     int cand[CAND_MAX];    // partners waiting for evaluation
     int sorted[CAND_MAX];
     double term[PG][9];    // Hertz force and torque, lubrication force
+    int count;
 };
 
 // The Hertz and lubrication (Eq. 9 with 2R -> σ, R^2 -> (σ/2)^2, only for
@@ -1107,14 +1134,16 @@ __device__ __forceinline__ void pairs_store(const Parts &P, int i, double acc)
 }
 
 // ---------------------------------------------------------------- cells
-// Per step: count the particles of each cell, exclusive prefix over the
-// cells (one CTA), place each particle's index, then each particle gathers
-// the candidates of the 27 cells around its own (each cell once when an
-// axis has fewer than 3 cells), keeps those the FP32 prefilter passes, and
-// sums the pair terms in increasing partner index: the same terms in the
-// same order as a loop over all partners, so the sums do not depend on the
-// order the cells were filled in.  Lattices of at most PAIRS_SCAN_MAX
-// particles take the loop over all partners instead.
+// Per step every particle enters the list of its cell (head[c], then next[i];
+// the order does not matter).  A particle's lanes then walk the lists of the
+// 27 cells around its own (each cell once when an axis has fewer than 3
+// cells), one cell a lane, keep the partners the FP32 prefilter passes, sort
+// them, and sum the pair terms in increasing partner index: the same terms in
+// the same order as a loop over all partners.  Lattices of at most
+// PAIRS_SCAN_MAX particles take that loop instead.  A compact list (count,
+// prefix over the cells, fill) took three kernels, 45 us with 38 in the prefix
+// at 24,389 cells, and 167 us for a walk one cell after the other; the lists
+// take 4 and 105 (25,033 particles; 2,344: 12 + 34 -> 4 + 24).
 
 __device__ __forceinline__ int cell_axis(float x, float n, float inv, int nc, bool periodic)
 {
@@ -1123,7 +1152,7 @@ __device__ __forceinline__ int cell_axis(float x, float n, float inv, int nc, bo
     return c < 0 ? 0 : (c >= nc ? nc - 1 : c);
 }
 
-__global__ void k_cell_count(Lat L, Parts P, Cells C)
+__global__ void k_cell_lists(Lat L, Parts P, Cells C)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.n) return;
@@ -1133,42 +1162,7 @@ __global__ void k_cell_count(Lat L, Parts P, Cells C)
     const int cz_ = cell_axis(x.z, (float)L.nz, C.inv[2], C.n[2], !L.walls);
     const int c = cx_ + C.n[0] * (cy_ + C.n[1] * cz_);
     C.cid[i] = c;
-    atomicAdd(&C.count[c], 1);
-}
-
-// Exclusive prefix of the cell counts; one CTA of 1024 threads, each over a
-// contiguous run of cells.
-__global__ void __launch_bounds__(1024) k_cell_scan(Cells C)
-{
-    __shared__ int part[1024];
-    const int t = threadIdx.x;
-    const int per = (C.ncell + 1023) / 1024;
-    const int c0 = min(t * per, C.ncell), c1 = min(c0 + per, C.ncell);
-    int s = 0;
-    for (int c = c0; c < c1; c++) s += C.count[c];
-    part[t] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {  // inclusive scan of the run sums
-        const int v = t >= off ? part[t - off] : 0;
-        __syncthreads();
-        part[t] += v;
-        __syncthreads();
-    }
-    int run = t > 0 ? part[t - 1] : 0;
-    for (int c = c0; c < c1; c++) {
-        C.start[c] = run;
-        C.fill[c] = 0;
-        run += C.count[c];
-    }
-    if (t == 1023) C.start[C.ncell] = part[1023];
-}
-
-__global__ void k_cell_fill(Parts P, Cells C)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n) return;
-    const int c = C.cid[i];
-    C.idx[C.start[c] + atomicAdd(&C.fill[c], 1)] = i;
+    C.next[i] = atomicExch(&C.head[c], i);
 }
 
 __device__ __forceinline__ double pairs_cells(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, int i,
@@ -1179,44 +1173,54 @@ __device__ __forceinline__ double pairs_cells(const Lat &L, const Parts &P, cons
     const float inv[3] = {1.f / nl[0], 1.f / nl[1], 1.f / nl[2]};
     const bool per_z = !L.walls;
     const float extra = (float)pp.lub_cut + 0.05f;
-    int nc = 0;
     const int c0 = C.cid[i];
     const int ci[3] = {c0 % C.n[0], (c0 / C.n[0]) % C.n[1], c0 / (C.n[0] * C.n[1])};
-    int lo[3], hi[3];
+    int lo[3], ext[3];
+#pragma unroll
     for (int k = 0; k < 3; k++) {
-        if (C.n[k] < 3) {  // every cell of the axis once
-            lo[k] = 0;
-            hi[k] = C.n[k] - 1;
-        } else {
-            lo[k] = ci[k] - 1;
-            hi[k] = ci[k] + 1;
-        }
+        lo[k] = C.n[k] < 3 ? 0 : ci[k] - 1;  // every cell of a short axis once
+        ext[k] = C.n[k] < 3 ? C.n[k] : 3;
     }
-    for (int dz = lo[2]; dz <= hi[2]; dz++) {
-        int z = dz;
-        if (C.n[2] >= 3) {
-            if (per_z)
-                z = (z + C.n[2]) % C.n[2];
-            else if (z < 0 || z >= C.n[2])
-                continue;
+    if (l == 0) g.count = 0;
+    __syncwarp(m);
+    // up to four lists a lane, walked side by side so that their loads are in
+    // flight together
+    constexpr int NQ = (27 + PG - 1) / PG;
+    int jq[NQ];
+#pragma unroll
+    for (int u = 0; u < NQ; u++) {
+        const int q = l + PG * u;
+        int x = lo[0] + q % ext[0], y = lo[1] + q / ext[0] % ext[1], z = lo[2] + q / (ext[0] * ext[1]);
+        x = x < 0 ? x + C.n[0] : (x >= C.n[0] ? x - C.n[0] : x);
+        y = y < 0 ? y + C.n[1] : (y >= C.n[1] ? y - C.n[1] : y);
+        if (per_z) z = z < 0 ? z + C.n[2] : (z >= C.n[2] ? z - C.n[2] : z);
+        const bool in = q < ext[0] * ext[1] * ext[2] && z >= 0 && z < C.n[2];
+        jq[u] = in ? C.head[x + C.n[0] * (y + C.n[1] * z)] : -1;
+    }
+    for (;;) {
+        float4 o[NQ];
+        int nx[NQ];
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < NQ; u++) {
+            const int j = max(jq[u], 0);
+            any = any || jq[u] >= 0;
+            o[u] = P.X32[j];
+            nx[u] = C.next[j];
         }
-        for (int dy = lo[1]; dy <= hi[1]; dy++) {
-            const int y = C.n[1] >= 3 ? (dy + C.n[1]) % C.n[1] : dy;
-            for (int dx = lo[0]; dx <= hi[0]; dx++) {
-                const int x = C.n[0] >= 3 ? (dx + C.n[0]) % C.n[0] : dx;
-                const int c = x + C.n[0] * (y + C.n[1] * z);
-                const int k1 = C.start[c + 1];
-                for (int k0 = C.start[c]; k0 < k1; k0 += PG) {
-                    const int j = k0 + l < k1 ? C.idx[k0 + l] : i;
-                    const bool near = j != i && near_pair(me, P.X32[j], nl, inv, per_z, extra);
-                    const unsigned b = (__ballot_sync(m, near) >> (threadIdx.x & 24)) & 0xFFu;
-                    const int at = nc + __popc(b & ((1u << l) - 1u));
-                    if (near && at < CAND_MAX) g.cand[at] = j;
-                    nc += __popc(b);
-                }
+        if (!any) break;
+#pragma unroll
+        for (int u = 0; u < NQ; u++) {
+            if (jq[u] < 0) continue;
+            if (jq[u] != i && near_pair(me, o[u], nl, inv, per_z, extra)) {
+                const int at = atomicAdd(&g.count, 1);
+                if (at < CAND_MAX) g.cand[at] = jq[u];
             }
+            jq[u] = nx[u];
         }
     }
+    __syncwarp(m);
+    const int nc = g.count;
     if (nc > CAND_MAX) return pairs_scan(L, P, pp, i, me, oi, g, m);  // very dense
     __syncwarp(m);
     for (int a = l; a < nc; a += PG) {  // by increasing partner index (all distinct)
@@ -2204,10 +2208,8 @@ void launch_pairs(const Lat &L, const Parts &P, const Pair &pp, const Cells &C, 
         k_pairs<false><<<bp, 128, 0, s>>>(L, P, pp, C);
         return;
     }
-    cudaMemsetAsync(C.count, 0, (size_t)C.ncell * sizeof(int), s);
-    k_cell_count<<<b, 128, 0, s>>>(L, P, C);
-    k_cell_scan<<<1, 1024, 0, s>>>(C);
-    k_cell_fill<<<b, 128, 0, s>>>(P, C);
+    cudaMemsetAsync(C.head, 0xFF, (size_t)C.ncell * sizeof(int), s);  // empty lists: -1
+    k_cell_lists<<<b, 128, 0, s>>>(L, P, C);
     k_pairs<true><<<bp, 128, 0, s>>>(L, P, pp, C);
 }
 
