@@ -89,9 +89,10 @@ void drop_graphs(lbe_ctx *c)
 }
 
 // Field offsets inside the particle buffer (doubles per particle).
-enum { OX = 0, OQ = 3, OV = 7, OW = 10, OXO = 13, OQO = 16, ORP = 20, ORO = 21, ODR = 22, OM = 23,
-       OIP = 24, OIQ = 25, OFL = 26, OTL = 29, OFP = 32, OTP = 35, OFE = 38, OTE = 41, OF = 44,
-       OT = 47, OFX = 50, PSTRIDE = 56 };
+// Those that lbe_read_particles returns (NREAD of them) come first.
+enum { OX = 0, OQ = 3, OV = 7, OW = 10, OF = 13, OT = 16, NREAD = 19,
+       OXO = 19, OQO = 22, ORP = 26, ORO = 27, ODR = 28, OM = 29, OIP = 30, OIQ = 31, OFL = 32, OTL = 35,
+       OFP = 38, OTP = 41, OFE = 44, OTE = 47, OFX = 50, PSTRIDE = 56 };
 
 void bind_parts(lbe_ctx *c)
 {
@@ -345,11 +346,13 @@ lbe_status check_async(lbe_ctx *c, const char *where)
 
 lbe_status sync(lbe_ctx *c, const char *where)
 {
-    cudaError_t e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, where);
+    // the status word behind the stream's work, and one wait for both
     unsigned status = 0;
-    if (c->L.status && cudaMemcpy(&status, c->L.status, sizeof status, cudaMemcpyDeviceToHost) == cudaSuccess &&
-        (status & 1u))
+    cudaError_t e = cudaSuccess;
+    if (c->L.status) e = cudaMemcpyAsync(&status, c->L.status, sizeof status, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, where);
+    if (status & 1u)
         return fail(c, LBE_ETIMEOUT, std::string(where) + ": a plane copy of the fused kernel did not complete");
 #ifdef LBE_CHECK
     unsigned long long bad = 0;
@@ -689,15 +692,30 @@ lbe_status lbe_read_particles(lbe_ctx *c, double *pos, double *quat, double *vel
 {
     if (!c) return LBE_EINVAL;
     cudaSetDevice(c->device);
-    lbe_status st = sync(c, "read_particles");
-    if (st != LBE_OK || c->np == 0) return st;
-    size_t cp = (size_t)c->cap;
+    if (c->np == 0) return sync(c, "read_particles");
+    const size_t cp = (size_t)c->cap;
     struct { double *dst; int off, k; } outs[] = {{pos, OX, 3}, {quat, OQ, 4}, {vel, OV, 3},
                                                   {omega, OW, 3}, {force, OF, 3}, {torque, OT, 3}};
+    // Few particles: all fields in one copy and one wait (a
+    // small copy costs about 9 us however few its bytes; seven of them and two
+    // waits were 75 us of a 163 us step and read of one ellipsoid).
+    constexpr size_t SMALL = 128;
+    if (cp <= SMALL) {
+        double all[NREAD * SMALL];
+        CK(c, cudaMemcpyAsync(all, c->pbuf, NREAD * cp * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        const lbe_status st = sync(c, "read_particles");
+        if (st != LBE_OK) return st;
+        for (auto &o : outs)
+            if (o.dst) std::memcpy(o.dst, all + o.off * cp, (size_t)o.k * c->np * sizeof(double));
+        return LBE_OK;
+    }
+    const lbe_status st = sync(c, "read_particles");
+    if (st != LBE_OK) return st;
     for (auto &o : outs)
         if (o.dst)
-            CK(c, cudaMemcpy(o.dst, c->pbuf + (size_t)o.off * cp, (size_t)o.k * c->np * sizeof(double),
-                             cudaMemcpyDeviceToHost));
+            CK(c, cudaMemcpyAsync(o.dst, c->pbuf + (size_t)o.off * cp, (size_t)o.k * c->np * sizeof(double),
+                                  cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
     return LBE_OK;
 }
 
