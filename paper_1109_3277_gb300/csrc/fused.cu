@@ -400,8 +400,10 @@ constexpr int WAIT_LIMIT = FUSED_WAIT_LIMIT;
 // false.  A negative wait_limit makes every wait one that nothing completes
 // (tests).  SELF: ψ of fluid nodes is formed here from the densities of the
 // box; otherwise psi holds ψ of every node (the density kernel's and the
-// shell fill's), and the box holds the tile only.
-template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32>
+// shell fill's), and the box holds the tile only.  SOLIDS = false (with SELF):
+// a periodic lattice without particles, which needs no node types, no row
+// masks and no reflections.
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
 __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__restrict__ fin,
                                            typename S::P *__restrict__ fout, const float *__restrict__ psi,
                                            const uint8_t *__restrict__ type, int zc, const FusedOfs &ofs,
@@ -420,11 +422,14 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const int x0 = bx * TX, y0 = by * TY;
     const int zb = bz * zc, ze = min(zb + zc, L.nz);
-    // wait_limit < 0 (tests of the timeout path): every wait for a box is
-    // for the barrier's next phase, which no copy completes, with |limit|
-    // tries; the cleanup below still waits for the copies in flight
-    const unsigned unreachable = wait_limit < 0 ? 1u : 0u;
-    const int limit = wait_limit < 0 ? -wait_limit : wait_limit;
+    // wait_limit < 0 (tests of the timeout path): each wait for a box is
+    // followed by one, of |limit| tries, for the barrier's next phase, which no
+    // copy completes.  (The next phase alone will not do: its parity is also
+    // that of the phase before the first, which counts as complete until the
+    // first copy has landed, so the wait would pass and the box's barrier be
+    // armed a second time.)
+    const bool unreachable = wait_limit < 0;
+    const int limit = unreachable ? -wait_limit : wait_limit;
     const int nxy = L.nx * L.ny;
     const int gx = x0 + tx, gy = y0 + ty;
     const bool active = gx < L.nx && gy < L.ny;
@@ -458,10 +463,18 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
     // entries go into ring slot k & 3, and plane zb - 2 + k (k >= 2) is
     // collided
     const int kmax = ze - zb + 2;
-    auto pvalid = [&](int p) { return !L.walls || (p >= 0 && p < L.nz); };
+    auto pvalid = [&](int p) { return !SOLIDS || !L.walls || (p >= 0 && p < L.nz); };
     auto gz_of = [&](int p) { return p < 0 ? p + L.nz : (p >= L.nz ? p - L.nz : p); };  // p in [-1, nz]
     // per stage buffer: boxes issued (thread 0) and waited for (every thread)
     Counts<NST> issued{}, waited{};
+    // wait for the box of buffer b; false if it ran out
+    auto arrived = [&](int b) {
+        const unsigned par = (unsigned)(waited.get(b) & 1);
+        bool in = mbar_wait(&bar[b], par, unreachable ? WAIT_LIMIT : limit);
+        if (unreachable && in) in = mbar_wait(&bar[b], par ^ 1u, limit);
+        if (in) waited.inc(b);
+        return in;
+    };
     auto issue = [&](int k, int b) {
         if (!TMA || tid != 0) return;
         const int p = zb - 1 + k;
@@ -475,6 +488,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
 
     // node type of entry e of iteration k's plane
     auto load_type = [&](int k, const Ent &e) -> uint8_t {
+        if (!SOLIDS) return FLUID;
         const int p = zb - 1 + k;
         if (!pvalid(p)) return WALL;
         return type[e.xy + (size_t)nxy * gz_of(p)];
@@ -488,7 +502,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         const float2 *pl[3] = {sps + (j & 3) * HN, sps + ((j + 1) & 3) * HN, sps + ((j + 2) & 3) * HN};
         const unsigned long long *ml[3] = {smask + (j & M) * C::HY, smask + ((j + 1) & M) * C::HY,
                                            smask + ((j + 2) & M) * C::HY};
-        const bool solid_own = (ml[1][ty + 1] >> (tx + 1)) & 1ull;
+        const bool solid_own = SOLIDS && (ml[1][ty + 1] >> (tx + 1)) & 1ull;
         const int n = gx + L.nx * gy + nxy * z;
         if (active && !solid_own) {
             const Mom mcur = mom_of();
@@ -523,6 +537,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             // its fixed offset; mode 1 (solid neighbours) reflects where
             // the neighbour is solid; mode 2 also wraps the push offsets
             unsigned long long mrow = 0ull;
+            if (SOLIDS)
 #pragma unroll
             for (int dz = 0; dz < 3; dz++)
 #pragma unroll
@@ -537,7 +552,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                 // bit (cx+1) + 3 (cy+1) + 9 (cz+1): neighbour is solid
                 uint32_t nb27 = 0;
                 int wx[2] = {0, 0}, wy[2] = {0, 0}, wz[2] = {0, 0};
-                if (MODE >= 1) {
+                if (SOLIDS && MODE >= 1) {
 #pragma unroll
                     for (int dz = 0; dz < 3; dz++)
 #pragma unroll
@@ -576,7 +591,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                             dst[ofs.push[i]] = v;
                     } else {
                         const int bit = (cx(i) + 1) + 3 * ((cy(i) + 1) + 3 * (cz(i) + 1));
-                        const bool sol = (nb27 >> bit) & 1u;
+                        const bool sol = SOLIDS && ((nb27 >> bit) & 1u);
                         const int corr = (cx(i) > 0 ? wx[0] : (cx(i) < 0 ? wx[1] : 0)) +
                                          (cy(i) > 0 ? wy[0] : (cy(i) < 0 ? wy[1] : 0)) +
                                          (cz(i) > 0 ? wz[0] : (cz(i) < 0 ? wz[1] : 0));
@@ -632,11 +647,11 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             };
             if (inner && mrow == 0ull)
                 collide(std::integral_constant<int, 0>{});
-            else if (inner)
+            else if (SOLIDS && inner)
                 collide(std::integral_constant<int, 1>{});
             else
                 collide(std::integral_constant<int, 2>{});
-        } else if (active) {
+        } else if (SOLIDS && active) {
             // A solid node's populations are never read (a node that a
             // particle uncovers gets f^eq in all slots), but writing them
             // keeps every sector of the output fully written: a partly
@@ -750,10 +765,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             const int kn = j + 3;  // ring index of plane z + 2
             if (kn < kmax) ring_fetch(kn, kn & 3);
             bool late = false;
-            if (TMA) {
-                late = !mbar_wait(&bar[b], (unsigned)(waited.get(b) & 1) ^ unreachable, limit);
-                if (!late) waited.inc(b);
-            }
+            if (TMA) late = !arrived(b);
             // a copy that never arrived leaves stale shared data: the
             // collision then stores garbage (at valid addresses), and the
             // step is reported as timed out
@@ -779,7 +791,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         // barrier that follows its last reader; the row masks have eight
         // slots, cleared two iterations before they are filled.
         constexpr int MS = C::MSLOTS - 1;
-        if (tid < C::HY) smask[tid] = smask[C::HY + tid] = 0ull;  // slots 0 and 1
+        if (SOLIDS && tid < C::HY) smask[tid] = smask[C::HY + tid] = 0ull;  // slots 0 and 1
         __syncthreads();
         // plane copies: issued after the barrier of iteration k is box k +
         // NST - LAG (with LAG the collision re-reads the box one iteration
@@ -792,7 +804,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         // until the plane is taken in
         auto solid_psi = [&](int k, const Ent &e, uint8_t t) {
             const int p = zb - 1 + k;
-            if (t == FLUID || !pvalid(p)) return;
+            if (!SOLIDS || t == FLUID || !pvalid(p)) return;
             const size_t n = e.xy + (size_t)nxy * gz_of(p);
             float2 *d = sps + (k & 3) * HN + e.ring;  // (ψ_b, ψ_r): the partner first
             cp_async<4>(&d->x, psi + (size_t)L.N + n);
@@ -813,11 +825,8 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             const int p = zb - 1 + k;
             const bool pv = pvalid(p);
             bool late = false;
-            if (TMA && pv) {
-                late = !mbar_wait(&bar[b_cur], (unsigned)(waited.get(b_cur) & 1) ^ unreachable, limit);
-                if (!late) waited.inc(b_cur);
-            }
-            asm volatile("cp.async.wait_all;" ::: "memory");
+            if (TMA && pv) late = !arrived(b_cur);
+            if (SOLIDS) asm volatile("cp.async.wait_all;" ::: "memory");
             // this plane's entries into ring slot k & 3: ψ of fluid nodes,
             // solid bits; the own node's moments
             {
@@ -837,7 +846,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
                     }
                     put_psi(own, mnext.dr);
                 }
-                const unsigned so = __ballot_sync(0xffffffffu, t_own != FLUID);
+                const unsigned so = SOLIDS ? __ballot_sync(0xffffffffu, t_own != FLUID) : 0u;
                 if (tx == 0 && so) atomicOr(&mrows[own.ey], (unsigned long long)so << 1);
                 if (has_halo) {
                     if (t_hal != FLUID) {
@@ -860,7 +869,7 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
             }
             // refill, the next plane's solid ψ, the types of the one after it
             if (TMA && k >= LAG && k + NST - LAG < kmax) issue(k + NST - LAG, LAG == 0 ? b_cur : (b_cur + NST - LAG) % NST);
-            if (tid < C::HY) smask[((k + 2) & MS) * C::HY + tid] = 0ull;
+            if (SOLIDS && tid < C::HY) smask[((k + 2) & MS) * C::HY + tid] = 0ull;
             if (k + 1 < kmax) {
                 t_own = tn_own;
                 t_hal = tn_hal;
@@ -896,14 +905,14 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
     return ok;
 }
 
-template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32>
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
 __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
     k_fused(Lat L, const typename S::P *__restrict__ fin, typename S::P *__restrict__ fout,
             const float *__restrict__ psi, const uint8_t *__restrict__ type, int zc, FusedOfs ofs,
             const __grid_constant__ CUtensorMap tmap, int wait_limit)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    fused_tile<S, TY, GEN, SELF, TMA, R32>(L, fin, fout, psi, type, zc, ofs, &tmap, blockIdx.x, blockIdx.y,
+    fused_tile<S, TY, GEN, SELF, TMA, R32, SOLIDS>(L, fin, fout, psi, type, zc, ofs, &tmap, blockIdx.x, blockIdx.y,
                                            blockIdx.z, wait_limit, align128(smem_raw));
 }
 
@@ -939,10 +948,10 @@ __global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true, tru
         using P = typename S::P;
         bool ok;
         if (sb.tma)
-            ok = fused_tile<S, BATCH_TY, GEN, true, true, !GEN>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
+            ok = fused_tile<S, BATCH_TY, GEN, true, true, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
                                                           sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         else
-            ok = fused_tile<S, BATCH_TY, GEN, true, false, !GEN>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
+            ok = fused_tile<S, BATCH_TY, GEN, true, false, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
                                                            sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         if (!ok) break;
         __syncthreads();
@@ -1045,13 +1054,13 @@ bool fused_rel32(const Lat &L)
     return !L.wide && (long long)Q * L.S + 2LL * L.N + (long long)L.nx * L.ny + L.nx + 1 < (1LL << 32);
 }
 
-template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32>
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
 static void launch_cfg(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
                        const CUtensorMap &tm, int zc, int wait_limit, cudaStream_t s)
 {
     using C = Cfg<S, TY, GEN, SELF, TMA>;
     using P = typename S::P;
-    auto kern = k_fused<S, TY, GEN, SELF, TMA, R32>;
+    auto kern = k_fused<S, TY, GEN, SELF, TMA, R32, SOLIDS>;
     static bool configured = false;  // the attribute is per function and process
     if (!configured) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes);
@@ -1061,11 +1070,11 @@ static void launch_cfg(const Lat &L, const void *fin, void *fout, const float *p
     kern<<<grid, C::NT, C::bytes, s>>>(L, (const P *)fin, (P *)fout, psi, type, zc, fused_offsets(L), tm, wait_limit);
 }
 
-// Configurations built, each with ψ formed in the kernel (SELF) or from
-// memory: τ = 1 with 32-bit offsets at 4 or 8 rows per tile (TMA) or 8
+// Configurations built, each with ψ formed in the kernel (SELF; also without
+// SOLIDS) or from memory: τ = 1 with 32-bit offsets at 4 or 8 rows per tile (TMA) or 8
 // (loads); any τ with 32- or 64-bit offsets at 8 rows (also taken by τ = 1
 // lattices that need 64-bit offsets: same results).
-template <class S, bool SELF>
+template <class S, bool SELF, bool SOLIDS>
 static void launch_fused_t(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
                            const CUtensorMap *tmap, cudaStream_t s, int zc, int ty, int wait_limit)
 {
@@ -1074,21 +1083,21 @@ static void launch_fused_t(const Lat &L, const void *fin, void *fout, const floa
     const bool r32 = fused_rel32(L), tau1 = fused_tau1(L) && r32;
     if (tau1) {
         if (tmap && ty == 4)
-            launch_cfg<S, 4, false, SELF, true, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 4, false, SELF, true, true, SOLIDS>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
         else if (tmap)
-            launch_cfg<S, 8, false, SELF, true, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, false, SELF, true, true, SOLIDS>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
         else
-            launch_cfg<S, 8, false, SELF, false, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, false, SELF, false, true, SOLIDS>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
     } else if (r32) {
         if (tmap)
-            launch_cfg<S, 8, true, SELF, true, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, true, SELF, true, true, SOLIDS>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
         else
-            launch_cfg<S, 8, true, SELF, false, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, true, SELF, false, true, SOLIDS>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
     } else {
         if (tmap)
-            launch_cfg<S, 8, true, SELF, true, false>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, true, SELF, true, false, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
         else
-            launch_cfg<S, 8, true, SELF, false, false>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
+            launch_cfg<S, 8, true, SELF, false, false, true>(L, fin, fout, psi, type, tm, zc, wait_limit, s);
     }
 }
 
@@ -1109,10 +1118,13 @@ void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const 
     const int rows = fused_rows(L, ty, tmap != nullptr, storage, self);
     if (zc <= 0) zc = fused_zchunk(L, rows, storage == LBE_STORE_F32 ? 4 : 2, self, 1.0);
     if (zc > L.nz) zc = L.nz;
-    if (self)
-        LBE_DISPATCH(storage, (launch_fused_t<S, true>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
+    const bool solids = L.walls || L.np > 0;
+    if (self && !solids)
+        LBE_DISPATCH(storage, (launch_fused_t<S, true, false>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
+    else if (self)
+        LBE_DISPATCH(storage, (launch_fused_t<S, true, true>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
     else
-        LBE_DISPATCH(storage, (launch_fused_t<S, false>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
+        LBE_DISPATCH(storage, (launch_fused_t<S, false, true>(L, fin, fout, psi, type, tmap, s, zc, rows, wait_limit)));
 }
 
 template <class S, bool GEN>
