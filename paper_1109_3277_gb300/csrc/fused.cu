@@ -922,12 +922,14 @@ __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
 // boxes hold few particles each.  GEN: some box needs any τ or
 // 64-bit offsets (it stores exactly what the τ = 1 configuration stores: τ =
 // 1 takes f^eq in the relaxation); otherwise all are τ = 1 with 32-bit offsets.
-constexpr int BATCH_TY = FUSED_TY_BATCH;
+template <class S, bool GEN>
+constexpr int BATCH_TY = fused_batch_rows(sizeof(typename S::T) == 4 ? LBE_STORE_F32 : LBE_STORE_F16_OFS, GEN);
 
 template <class S, bool GEN>
-__global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true, true>::CTAS)) k_fused_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(TX *BATCH_TY<S, GEN>, (Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::CTAS))
+    k_fused_batch(BatchIndex B, int total)
 {
-    constexpr int NT = TX * BATCH_TY;
+    constexpr int TY = BATCH_TY<S, GEN>, NT = TX * TY;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = align128(smem_raw);
     __shared__ int s_tile;
@@ -948,10 +950,10 @@ __global__ void __launch_bounds__(TX *BATCH_TY, (Cfg<S, BATCH_TY, GEN, true, tru
         using P = typename S::P;
         bool ok;
         if (sb.tma)
-            ok = fused_tile<S, BATCH_TY, GEN, true, true, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
+            ok = fused_tile<S, TY, GEN, true, true, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
                                                           sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         else
-            ok = fused_tile<S, BATCH_TY, GEN, true, false, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
+            ok = fused_tile<S, TY, GEN, true, false, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
                                                            sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         if (!ok) break;
         __syncthreads();
@@ -986,7 +988,7 @@ int fused_zchunk(const Lat &L, int ty, int es, bool self, double share)
     // memory (256^3 bijel, f16) 564 at 16, 601 at 64.
     const long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
     const bool tma = (L.nx * 2 * es) % 16 == 0;
-    const int cap = !self ? 16 : (!tma ? 12 : (es == 4 ? (ty == 4 ? 5 : 4) : 8));
+    const int cap = !self ? 16 : (!tma ? 12 : (es == 4 ? (ty == 4 ? 5 : 4) : (ty == 4 ? 6 : 8)));
     const int slots = (fused_tau1(L) && fused_rel32(L) ? 3 : 2) * 8 / ty;  // CTAs an SM takes
     const double full = 1.7 + 0.9 * slots * ty / 8;
     int best = 1;
@@ -1103,13 +1105,15 @@ static void launch_fused_t(const Lat &L, const void *fin, void *fout, const floa
 
 int fused_rows(const Lat &L, int ty_request, bool tma, int storage, bool self)
 {
-    // only the τ = 1 configurations with TMA come in two heights.  By
-    // default (request 0) FP32 with ψ on chip takes 4 rows: five CTAs of four
-    // warps fit an SM against three of eight, and one that waits idles fewer
-    // warps (256^3 909 us against 961, 128^3 133 against 140, 64^3 22.6
-    // against 24.5)
+    // only the τ = 1 configurations with TMA come in two heights.  By default
+    // (request 0) those with ψ on chip take 4 rows in FP32 and, without solid
+    // nodes, at 16 bit: more and smaller CTAs fit an SM, and one that waits
+    // idles fewer warps (f32 256^3 909 us against 961, 128^3 133 against 140,
+    // 64^3 22.6 against 24.5; f16 without solid nodes 256^3 517 against 543,
+    // 128^3 82 against 86; with them 598 against 600)
     if (!tma || !fused_tau1(L) || !fused_rel32(L)) return 8;
-    return ty_request == 4 || (ty_request == 0 && self && storage == LBE_STORE_F32) ? 4 : 8;
+    const bool few = self && (storage == LBE_STORE_F32 || !(L.walls || L.np > 0));
+    return ty_request == 4 || (ty_request == 0 && few) ? 4 : 8;
 }
 
 void launch_fused(int storage, const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
@@ -1133,7 +1137,7 @@ static void batch_configure()
     static bool configured = false;  // the attribute is per function and process
     if (!configured) {
         cudaFuncSetAttribute(k_fused_batch<S, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Cfg<S, BATCH_TY, GEN, true, true>::bytes);
+                             (int)Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::bytes);
         configured = true;
     }
 }
@@ -1141,7 +1145,7 @@ static void batch_configure()
 template <class S, bool GEN>
 static void launch_fused_batch_t(const BatchIndex &B, int total, int ctas, cudaStream_t s)
 {
-    using C = Cfg<S, BATCH_TY, GEN, true, true>;
+    using C = Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>;
     batch_configure<S, GEN>();
     k_fused_batch<S, GEN><<<ctas < total ? ctas : total, C::NT, C::bytes, s>>>(B, total);
 }
@@ -1154,8 +1158,8 @@ static int batch_occupancy()
 {
     int n = 0;
     batch_configure<S, GEN>();
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S, GEN>, TX * BATCH_TY,
-                                                  Cfg<S, BATCH_TY, GEN, true, true>::bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S, GEN>, TX * BATCH_TY<S, GEN>,
+                                                  Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::bytes);
     return n > 0 ? n : 1;
 }
 

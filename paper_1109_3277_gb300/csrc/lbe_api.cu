@@ -44,8 +44,9 @@ struct lbe_ctx {
     Cells cells{};   // pair-force cell list (with the particles)
     size_t cells_bytes = 0;
     LinkList ll{nullptr, nullptr, 0};  // link nodes of the step (allocated with the first particles)
-    // graphs keyed by (cur, ocur)
-    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    // graphs of one step and of two, keyed by (cur, ocur)
+    cudaGraphExec_t graph[2][4] = {};
+    int odd_steps = 0;  // single steps launched since the graphs were dropped
     int zc_tuned = 0;  // fused-kernel z chunk chosen by lbe_autotune (0: heuristic)
     int ty_tuned = 0;  // fused-kernel tile rows chosen by lbe_autotune (0: the default)
     int wait_limit = FUSED_WAIT_LIMIT;  // tries of each bounded wait for a box copy
@@ -81,11 +82,13 @@ size_t storage_size(int s) { return s == LBE_STORE_F32 ? 4 : 2; }
 
 void drop_graphs(lbe_ctx *c)
 {
-    for (auto &g : c->graph)
-        if (g) {
-            cudaGraphExecDestroy(g);
-            g = nullptr;
-        }
+    for (auto &gs : c->graph)
+        for (auto &g : gs)
+            if (g) {
+                cudaGraphExecDestroy(g);
+                g = nullptr;
+            }
+    c->odd_steps = 0;
 }
 
 // Field offsets inside the particle buffer (doubles per particle).
@@ -637,26 +640,46 @@ lbe_status lbe_step(lbe_ctx *c, int32_t nsteps)
         for (int k = 0; k < nsteps; k++) enqueue_step(c);
         return check_async(c, "step");
     }
-    int pairs = nsteps / 2;
-    if (pairs > 0) {
-        int key = c->cur * 2 + c->ocur;
-        if (!c->graph[key]) {
-            int cur0 = c->cur, ocur0 = c->ocur;
+    // Pairs of steps replay a captured graph.  On the library's own stream
+    // (which no caller can be capturing) so does a single step once they are
+    // taken repeatedly: one launch instead of one per kernel.
+    constexpr int CAPTURE_AFTER = 16;
+    auto replay = [&](int steps, int times) -> lbe_status {
+        const int key = c->cur * 2 + c->ocur;
+        cudaGraphExec_t &exec = c->graph[steps - 1][key];
+        const int cur0 = c->cur, ocur0 = c->ocur;
+        if (!exec) {
             cudaGraph_t g;
             CK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-            enqueue_step(c);
-            enqueue_step(c);
+            for (int k = 0; k < steps; k++) enqueue_step(c);
             cudaError_t e = cudaStreamEndCapture(c->stream, &g);
             c->cur = cur0;
             c->ocur = ocur0;
             if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
-            e = cudaGraphInstantiate(&c->graph[key], g, 0);
+            e = cudaGraphInstantiate(&exec, g, 0);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) return cuda_fail(c, e, "cudaGraphInstantiate");
         }
-        for (int k = 0; k < pairs; k++) CK(c, cudaGraphLaunch(c->graph[key], c->stream));
+        for (int k = 0; k < times; k++) CK(c, cudaGraphLaunch(exec, c->stream));
+        if (steps & 1) {  // as enqueue_step leaves the parities
+            c->cur = 1 - cur0;
+            if (c->np > 0 && c->d.particle_mode != LBE_PARTICLES_STATIC) c->ocur = 1 - ocur0;
+        }
+        return LBE_OK;
+    };
+    if (nsteps / 2 > 0) {
+        const lbe_status st = replay(2, nsteps / 2);
+        if (st != LBE_OK) return st;
     }
-    if (nsteps & 1) enqueue_step(c);
+    if (nsteps & 1) {
+        if (!c->own_stream || c->odd_steps < CAPTURE_AFTER) {
+            c->odd_steps++;
+            enqueue_step(c);
+        } else {
+            const lbe_status st = replay(1, 1);
+            if (st != LBE_OK) return st;
+        }
+    }
     return check_async(c, "step");
 }
 
@@ -967,7 +990,7 @@ struct lbe_batch {
     cudaEvent_t done = nullptr;       // end of the last batched launch
     std::vector<cudaEvent_t> mev;     // per member: its stream's last work
     BoxDev *d_box = nullptr;
-    int *d_idx = nullptr;             // tile0 | node0 | part0 | par | counter
+    int *d_idx = nullptr;             // tile0 | part0 | wall0 | par | counter | pbox
     BatchIndex idx{};
     int total_tiles = 0, total_parts = 0, total_walls = 0;
     int ext[3] = {1, 1, 1};           // bound of the particle boxes
@@ -1064,18 +1087,24 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
     }
     std::vector<BoxDev> box(n);
     double nodes = 0.0;
-    for (lbe_ctx *c : b->members) nodes += (double)c->L.N;
-    std::vector<int> idx(3 * (n + 1) + 2 * n + 1, 0);
-    int *tile0 = idx.data(), *part0 = tile0 + (n + 1), *wall0 = part0 + (n + 1), *par = wall0 + (n + 1);
+    for (lbe_ctx *c : b->members) {
+        nodes += (double)c->L.N;
+        if (!fused_tau1(c->L) || !fused_rel32(c->L)) b->general = true;
+    }
+    const int rows = fused_batch_rows(b->storage, b->general);
+    int np_all = 0;
+    for (lbe_ctx *c : b->members) np_all += c->np;
+    std::vector<int> idx(3 * (n + 1) + 2 * n + 1 + np_all, 0);
+    int *tile0 = idx.data(), *part0 = tile0 + (n + 1), *wall0 = part0 + (n + 1), *par = wall0 + (n + 1), *pbox = par + 2 * n + 1;
     for (int k = 0; k < n; k++) {
         lbe_ctx *c = b->members[k];
         BoxDev &d = box[k];
         d.L = c->L;
         d.ofs = fused_offsets(c->L);
         d.tma = c->tma ? 1 : 0;
-        if (c->tma) {  // the batched kernel's tiles have FUSED_TY_BATCH = 8 rows
-            d.tmap[0] = c->tmap[1][0][0];  // ψ formed in the kernel
-            d.tmap[1] = c->tmap[1][0][1];
+        if (c->tma) {
+            d.tmap[0] = c->tmap[1][rows == 4 ? 1 : 0][0];  // ψ formed in the kernel
+            d.tmap[1] = c->tmap[1][rows == 4 ? 1 : 0][1];
         }
         d.f[0] = c->f[0];
         d.f[1] = c->f[1];
@@ -1090,15 +1119,15 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         d.mode = c->d.particle_mode;
         d.links = c->np > 0 ? c->ll : LinkList{nullptr, nullptr, 0};
         d.zc = c->zc_tuned > 0 ? c->zc_tuned
-                               : fused_zchunk(c->L, FUSED_TY_BATCH, (int)c->esize, true, (double)c->L.N / nodes);
+                               : fused_zchunk(c->L, rows, (int)c->esize, true, (double)c->L.N / nodes);
         d.ntx = (c->L.nx + FUSED_TX - 1) / FUSED_TX;
-        d.nty = (c->L.ny + FUSED_TY_BATCH - 1) / FUSED_TY_BATCH;
+        d.nty = (c->L.ny + rows - 1) / rows;
         d.nzc = (c->L.nz + d.zc - 1) / d.zc;
         tile0[k + 1] = tile0[k] + d.ntx * d.nty * d.nzc;
         part0[k + 1] = part0[k] + c->np;
+        std::fill(pbox + part0[k], pbox + part0[k + 1], k);
         wall0[k + 1] = wall0[k] + batch_wall_tiles(c->L);
         batch_shell_extent(c->L, d.P, b->ext);
-        if (!fused_tau1(c->L) || !fused_rel32(c->L)) b->general = true;
         par[2 * k] = c->cur;
         par[2 * k + 1] = c->ocur;
     }
@@ -1123,6 +1152,7 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
     b->idx.wall0 = b->d_idx + 2 * (n + 1);
     b->idx.par = b->d_idx + 3 * (n + 1);
     b->idx.counter = b->idx.par + 2 * n;
+    b->idx.pbox = b->idx.counter + 1;
     b->ctas_per_sm = fused_batch_ctas_per_sm(b->storage, b->general);
     // link lists start empty; the last kernel of each batched step empties them
     for (lbe_ctx *c : b->members)

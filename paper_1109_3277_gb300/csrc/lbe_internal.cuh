@@ -355,6 +355,7 @@ struct BatchIndex {
     const int *tile0, *part0, *wall0;   // [nbox + 1]
     int *par;                           // [2 nbox]: cur, ocur
     int *counter;                       // persistent tile queue of the fused kernel
+    const int *pbox;                    // box of each particle
 };
 
 // ---- launchers (fluid.cu) -------------------------------------------------
@@ -403,7 +404,9 @@ void launch_flip_batch(const BatchIndex &B, cudaStream_t s);
 // z chunk in planes (0: the default for the lattice), ty the requested tile
 // height (4 or 8, 0 the default; configurations without a 4-row variant take 8), and
 // wait_limit the tries of each bounded wait for a box copy.
-constexpr int FUSED_TX = 32, FUSED_TY_BATCH = 8;
+constexpr int FUSED_TX = 32;
+// Tile rows of the batched kernel (general: see launch_fused_batch).
+constexpr int fused_batch_rows(int storage, bool general) { return storage == LBE_STORE_F32 && !general ? 4 : 8; }
 constexpr int FUSED_WAIT_LIMIT = 1 << 22;
 // self: the kernel forms ψ of fluid nodes from the densities of the tile
 // and a one-node halo (psi then holds ψ of solid nodes only); otherwise psi

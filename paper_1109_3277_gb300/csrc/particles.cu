@@ -400,12 +400,16 @@ __device__ __forceinline__ void quad_rot(int k, const double q[4], double row[3]
     order3(k, d, m_(2.0, a_(ab, wc)), m_(2.0, s_(ac, wb)), col);
 }
 
-// Axis k of box_of for centre X and half-extent h.
-__device__ __forceinline__ void box_axis(double X, double h, double &lo, double &hi)
+// Axis k of box_of for centre Xi + Xf and half-extent h, in FP32 (the box is
+// a node wider than the ellipsoid on each side; the FP32 error is below 1e-3
+// of a node up to half-extents of 1e4).
+__device__ __forceinline__ void box_axis(double X, float h, double &fl, double &lo, double &hi)
 {
-    lo = floor(X - h) - 1.0;
-    hi = ceil(X + h) + 1.0;
-    if (!(lo <= hi) || !(fabs(X) < 1e9) || !(h < 1e9)) {
+    fl = floor(X);
+    const float Xf = (float)(X - fl);
+    lo = fl + (double)(floorf(Xf - h) - 1.f);
+    hi = fl + (double)(ceilf(Xf + h) + 1.f);
+    if (!(lo <= hi) || !(fabs(X) < 1e9) || !(h < 1e9f)) {
         lo = 1.0;
         hi = 0.0;
     }
@@ -477,12 +481,13 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
     if (!first) copy_now();
     double row[3], col[3];
     quad_rot(k, q, row, col);
-    const double h = sqrt(rp * rp * row[0] * row[0] + ro * ro * (row[1] * row[1] + row[2] * row[2]));
-    double lo, hi;
-    box_axis(X, h, lo, hi);
+    const float r0 = (float)row[0], r1 = (float)row[1], r2 = (float)row[2], rpf = (float)rp, rof = (float)ro;
+    // a little wide, for the FP32 rounding
+    const float h = 1.00001f * sqrtf(rpf * rpf * r0 * r0 + rof * rof * (r1 * r1 + r2 * r2));
+    double fl, flu, lo, hi;
+    box_axis(X, h, fl, lo, hi);
     const bool empty = quad_empty(lo, hi);
     quad_box(L, k, wr, empty, lo, hi, G.now.box);
-    const double fl = floor(X);
     if (wr) {
         for (int j = 0; j < 3; j++) {
             G.now.g.R[k][j] = row[j];
@@ -505,7 +510,7 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
     // the new centre next to the old one, and the union of the two boxes
     const double Xu = Xold + pair_disp(L, k, Xold, X);
     double lu, hu;
-    box_axis(Xu, h, lu, hu);
+    box_axis(Xu, h, flu, lu, hu);
     const bool eu = quad_empty(lu, hu);
     double lo0 = first ? lo : lo_was, hi0 = first ? hi : hi_was;
     const bool e0 = quad_empty(lo0, hi0);
@@ -517,7 +522,6 @@ __device__ __forceinline__ void geom_quad(const Lat &L, const Parts &P, int p, b
         hi0 = fmax(hi0, hu);
     }
     quad_box(L, k, wr, e0 && eu, lo0, hi0, G.uni);
-    const double flu = floor(Xu);
     if (wr) {
         G.Xui[k] = eu ? 0 : (int)flu;
         G.Xuf[k] = eu ? NAN : (float)(Xu - flu);
@@ -1020,9 +1024,8 @@ __device__ __forceinline__ bool near_pair(float4 me, float4 o, const float nl[3]
 // now; 25,033: 127 us with one lane, 105 now.
 //
 // Up to PAIRS_SCAN_MAX particles the loop over all partners replaces the
-// cell list: its three kernels and the clearing cost about 10 us however few
-// the particles (1 particle: 18 -> 4 us; 40: 38 -> 17 us), and 256 prefilter
-// rounds of eight stay below that.
+// cell lists: at 10 % volume fraction it takes 15 us for 60 particles, 20 for
+// 130 and 26 for 250, against 31 + 3 for 300 with the lists and a memset.
 constexpr int PAIRS_SCAN_MAX = 256;
 constexpr int PG = 8;                  // lanes per particle
 constexpr int PAIR_GROUPS = 128 / PG;  // particles per CTA
@@ -1345,8 +1348,10 @@ __device__ __forceinline__ void integrate_quad(const Lat &L, const Parts &P, int
         o += lane == 1 || lane == 2 ? t2 : -t2;
         o += lane >= 2 ? t3 : -t3;
         const double o0 = quad(o, 0), o1 = quad(o, 1), o2 = quad(o, 2), o3 = quad(o, 3);
-        const double nn = sqrt(o0 * o0 + o1 * o1 + o2 * o2 + o3 * o3);
-        const double qn = o / nn;
+        // o / |o|: the product of two unit quaternions is off by rounding only,
+        // and 1.5 - x / 2 is 1 / sqrt(x) to 3/8 (x - 1)^2
+        const double n2 = o0 * o0 + o1 * o1 + o2 * o2 + o3 * o3;
+        const double qn = fabs(n2 - 1.0) < 1e-9 ? o * (1.5 - 0.5 * n2) : o / sqrt(n2);
         if (moves) P.q[4 * p + lane] = qn;
 #pragma unroll
         for (int j = 0; j < 4; j++) q[j] = quad(qn, j);
@@ -2033,7 +2038,7 @@ __global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, 
     const bool part = c < parts * nt;
     const int g = part ? c / nt : c - parts * nt;
     const int *off = part ? B.part0 : B.wall0;
-    const int b = find_box(off, B.nbox, g);
+    const int b = part ? B.pbox[g] : find_box(B.wall0, B.nbox, g);
     const BoxDev &bx = B.box[b];
     const int cur = B.par[2 * b], ocur = B.par[2 * b + 1];
     const typename S::P *f = (const typename S::P *)bx.f[cur];
@@ -2046,7 +2051,7 @@ __global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, 
 __global__ void __launch_bounds__(PT) k_claim_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     if (bx.mode == LBE_PARTICLES_STATIC) return;
     claim_body(bx.L, bx.P, g - B.part0[b], bx.owner[1 - B.par[2 * b + 1]]);
@@ -2056,7 +2061,7 @@ template <class S>
 __global__ void __launch_bounds__(PT) k_transition_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     if (bx.mode == LBE_PARTICLES_STATIC) return;
     const int cur = B.par[2 * b], ocur = B.par[2 * b + 1];
@@ -2067,7 +2072,7 @@ __global__ void __launch_bounds__(PT) k_transition_batch(BatchIndex B, int total
 __global__ void __launch_bounds__(PT) k_reset_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     if (bx.mode == LBE_PARTICLES_STATIC) return;
     reset_body(bx.L, bx.P, g - B.part0[b], 1, bx.owner[B.par[2 * b + 1]]);
@@ -2077,7 +2082,7 @@ __global__ void __launch_bounds__(128) k_geom_batch(BatchIndex B, int total)
 {
     bool act;
     const int g = quad_particle(total, act);
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     // the quads of a warp may belong to boxes of either kind: all take part
     geom_body(bx.L, bx.P, g - B.part0[b], act && bx.mode != LBE_PARTICLES_STATIC, false);
@@ -2087,7 +2092,7 @@ __global__ void __launch_bounds__(128) k_integrate_batch(BatchIndex B, int total
 {
     bool act;
     const int g = quad_particle(total, act);
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     double X, Xold, q[4];
     integrate_quad(bx.L, bx.P, bx.mode, g - B.part0[b], act, X, Xold, q);
@@ -2100,7 +2105,7 @@ __global__ void __launch_bounds__(128) k_pairs_batch(BatchIndex B, int total)
     __shared__ PairGroup gr[PAIR_GROUPS];
     const int g = (blockIdx.x * 128 + threadIdx.x) / PG;
     if (g >= total) return;
-    const int b = find_box(B.part0, B.nbox, g);
+    const int b = B.pbox[g];
     const BoxDev &bx = B.box[b];
     pairs_body(bx.L, bx.P, bx.pair, nullptr, g - B.part0[b], gr[threadIdx.x / PG]);
 }
@@ -2261,11 +2266,11 @@ static ShellGrid shell_grid(const int ext[3], int np)
     return g;
 }
 
-// An upper bound of a particle box's extent (box_axis: 2 h + 5 nodes at
-// most, h <= rmax).
+// An upper bound of a particle box's extent (box_axis: fewer than 2 h + 5
+// nodes, with h at most 1.00002 rmax).
 static void shell_extent(const Lat &L, double rmax, int ext[3])
 {
-    const double e = std::floor(2.0 * rmax) + 5.0;
+    const double e = std::floor(2.0001 * rmax) + 5.0;
     const int n[3] = {L.nx, L.ny, L.nz};
     for (int k = 0; k < 3; k++) ext[k] = std::max(ext[k], e < n[k] ? (int)e : n[k]);
 }
