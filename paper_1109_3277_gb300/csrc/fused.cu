@@ -129,13 +129,10 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src)
                  : "memory");
 }
 
-// The first 128-byte aligned byte at or after p.  The result is a generic
-// address (rounded through an integer), so the compiler issues generic
-// loads for the box, ring and mask reads: measured faster for this kernel
-// than shared-memory instructions, which stall on their issue queue.
+// The first 128-byte aligned byte at or after p, of shared memory.
 __device__ __forceinline__ unsigned char *align128(unsigned char *p)
 {
-    return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(p) + 127) & ~uintptr_t(127));
+    return p + ((128u - ((unsigned)__cvta_generic_to_shared(p) & 127u)) & 127u);
 }
 
 // ---- TMA and mbarrier (PTX) -------------------------------------------------

@@ -47,6 +47,11 @@ struct lbe_ctx {
     // graphs of one step and of two, keyed by (cur, ocur)
     cudaGraphExec_t graph[2][4] = {};
     int odd_steps = 0;  // single steps launched since the graphs were dropped
+    // branch of a captured step beside the fluid's kernels (created at the
+    // first capture with particles): its stream, and the events that order
+    // the two
+    cudaStream_t side = nullptr;
+    cudaEvent_t forked = nullptr, joined = nullptr;
     int zc_tuned = 0;  // fused-kernel z chunk chosen by lbe_autotune (0: heuristic)
     int ty_tuned = 0;  // fused-kernel tile rows chosen by lbe_autotune (0: the default)
     int wait_limit = FUSED_WAIT_LIMIT;  // tries of each bounded wait for a box copy
@@ -158,6 +163,9 @@ void free_all(lbe_ctx *c)
     cudaFree(c->ll.count);
     if (c->L.err) cudaFree(c->L.err);
     cudaFree(c->L.status);
+    if (c->side) cudaStreamDestroy(c->side);
+    if (c->forked) cudaEventDestroy(c->forked);
+    if (c->joined) cudaEventDestroy(c->joined);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
 
@@ -230,14 +238,39 @@ const CUtensorMap *fused_map(const lbe_ctx *c, int buf, int ty)
     return &c->tmap[self ? 1 : 0][fused_rows(c->L, ty, true, c->d.storage, self) == 4 ? 1 : 0][buf];
 }
 
-// Enqueue one time step (no host synchronisation).
-void enqueue_step(lbe_ctx *c)
+// Work that follows on c->side runs after everything enqueued on c->stream
+// so far (fork), and work that follows on c->stream after that (join).
+void fork(lbe_ctx *c)
+{
+    cudaEventRecord(c->forked, c->stream);
+    cudaStreamWaitEvent(c->side, c->forked, 0);
+}
+void join(lbe_ctx *c)
+{
+    cudaEventRecord(c->joined, c->side);
+    cudaStreamWaitEvent(c->stream, c->joined, 0);
+}
+
+// Enqueue one time step (no host synchronisation).  branch (captured steps):
+// what does not depend on the fluid's kernels runs beside them.  The pair
+// forces need the particles' state of the last step only, so they run beside
+// the shell fill, the fused kernel and the links; the reset of the spare owner
+// map comes after the transition, and nothing reads or writes that map before
+// the next claim, so it runs on the branch ahead of the next step's pair
+// forces.  The update joins the branch, and so does the end of the captured
+// steps (the caller).
+void enqueue_step(lbe_ctx *c, bool branch = false)
 {
     cudaStream_t s = c->stream;
     const Lat &L = c->L;
     int st = c->d.storage;
     void *fin = c->f[c->cur], *fout = c->f[1 - c->cur];
     const bool two_pass = (c->d.flags & LBE_FLAG_TWO_PASS) != 0;
+    if (branch) {
+        c->P.n = c->np;
+        fork(c);
+        launch_pairs(L, c->P, c->pair, c->cells, c->side);
+    }
     if (two_pass) {
         launch_moments(st, L, fin, c->type, c->rho, c->psi, s);
         launch_shell(L, c->rho, c->psi, c->type, c->owner[c->ocur], c->P.drho, s);
@@ -275,13 +308,17 @@ void enqueue_step(lbe_ctx *c)
         else {
             launch_link(st, L, c->ll, c->rho, c->owner[c->ocur], c->P, fout, s);
         }
-        launch_pairs(L, c->P, c->pair, c->cells, s);
+        if (branch)
+            join(c);
+        else
+            launch_pairs(L, c->P, c->pair, c->cells, s);
         launch_integrate(L, c->P, c->d.particle_mode, c->ll.count, s);  // the list is empty between steps
         if (c->d.particle_mode != LBE_PARTICLES_STATIC) {
             uint32_t *oo = c->owner[c->ocur], *on = c->owner[1 - c->ocur];
             launch_claim(L, c->P, 0, on, s);
             launch_transition(st, L, c->P, fout, c->type, oo, on, 0, s);
-            launch_reset(L, c->P, 1, oo, s);
+            if (branch) fork(c);
+            launch_reset(L, c->P, 1, oo, branch ? c->side : s);
             c->ocur = 1 - c->ocur;
             launch_verify(L, c->type, on, s);
         }
@@ -644,14 +681,26 @@ lbe_status lbe_step(lbe_ctx *c, int32_t nsteps)
     // (which no caller can be capturing) so does a single step once they are
     // taken repeatedly: one launch instead of one per kernel.
     constexpr int CAPTURE_AFTER = 16;
+    // Branches pay while the kernels leave room on the GPU: 77 x 53 x 61 with 40
+    // particles 111 -> 87 us a step, 150 x 141 x 133 with 525 519 -> 459, 256^3
+    // 1,300 -> 1,285, but 512^3 8.9 -> 9.0 ms; a graph of a single step launches
+    // more slowly with them (87 -> 90 us with its read).
+    constexpr int BRANCH_MAX = 1 << 25;
     auto replay = [&](int steps, int times) -> lbe_status {
         const int key = c->cur * 2 + c->ocur;
         cudaGraphExec_t &exec = c->graph[steps - 1][key];
         const int cur0 = c->cur, ocur0 = c->ocur;
         if (!exec) {
+            const bool branch = steps > 1 && c->np > 0 && c->L.N <= BRANCH_MAX;
+            if (branch && !c->joined) {
+                if (!c->side) CK(c, cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+                if (!c->forked) CK(c, cudaEventCreateWithFlags(&c->forked, cudaEventDisableTiming));
+                CK(c, cudaEventCreateWithFlags(&c->joined, cudaEventDisableTiming));
+            }
             cudaGraph_t g;
             CK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-            for (int k = 0; k < steps; k++) enqueue_step(c);
+            for (int k = 0; k < steps; k++) enqueue_step(c, branch);
+            if (branch) join(c);
             cudaError_t e = cudaStreamEndCapture(c->stream, &g);
             c->cur = cur0;
             c->ocur = ocur0;

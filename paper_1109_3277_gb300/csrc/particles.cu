@@ -16,6 +16,11 @@ namespace lbe {
 namespace {
 
 constexpr int PT = 128;  // threads per per-particle CTA
+// Threads per particle of the claim and the reset, whose order does not
+// matter: with fewer particles than SMs a particle's rows spread over 16
+// warps.
+constexpr int PT_WIDE = 512;
+static int cover_threads(int np) { return np < 152 ? PT_WIDE : PT; }
 
 // Tiles of a particle's box in the shell fill: nx x ny x nz of them, of 30 x
 // tyi x tzi nodes; a tile's link entries are filled up to a multiple of pad.
@@ -1438,7 +1443,7 @@ __device__ __forceinline__ void claim_body(const Lat &L, const Parts &P, int p, 
     });
 }
 
-__global__ void __launch_bounds__(PT) k_claim(Lat L, Parts P, uint32_t *__restrict__ owner_new)
+__global__ void __launch_bounds__(PT_WIDE) k_claim(Lat L, Parts P, uint32_t *__restrict__ owner_new)
 {
     claim_body(L, P, blockIdx.x, owner_new);
 }
@@ -1666,7 +1671,7 @@ __device__ __forceinline__ void reset_body(const Lat &L, const Parts &P, int p, 
     });
 }
 
-__global__ void __launch_bounds__(PT) k_reset(Lat L, Parts P, int use_old, uint32_t *__restrict__ owner)
+__global__ void __launch_bounds__(PT_WIDE) k_reset(Lat L, Parts P, int use_old, uint32_t *__restrict__ owner)
 {
     reset_body(L, P, blockIdx.x, use_old, owner);
 }
@@ -2048,7 +2053,7 @@ __global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, 
         wall_tile<S>(bx.L, g - off[b], f, bx.psi, bx.type, sm);
 }
 
-__global__ void __launch_bounds__(PT) k_claim_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(PT_WIDE) k_claim_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
     const int b = B.pbox[g];
@@ -2069,7 +2074,7 @@ __global__ void __launch_bounds__(PT) k_transition_batch(BatchIndex B, int total
                        bx.owner[1 - ocur], 0);
 }
 
-__global__ void __launch_bounds__(PT) k_reset_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(PT_WIDE) k_reset_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
     const int b = B.pbox[g];
@@ -2162,12 +2167,12 @@ void launch_geom_batch(const BatchIndex &B, int total, cudaStream_t s)
 
 void launch_claim_batch(const BatchIndex &B, int total, cudaStream_t s)
 {
-    if (total > 0) k_claim_batch<<<total, PT, 0, s>>>(B, total);
+    if (total > 0) k_claim_batch<<<total, cover_threads(total), 0, s>>>(B, total);
 }
 
 void launch_reset_batch(const BatchIndex &B, int total, cudaStream_t s)
 {
-    if (total > 0) k_reset_batch<<<total, PT, 0, s>>>(B, total);
+    if (total > 0) k_reset_batch<<<total, cover_threads(total), 0, s>>>(B, total);
 }
 
 void launch_batch_quat(const BatchIndex &B, double *out, cudaStream_t s)
@@ -2235,7 +2240,7 @@ void launch_integrate(const Lat &L, const Parts &P, int mode, int *links, cudaSt
 void launch_claim(const Lat &L, const Parts &P, int, uint32_t *owner_new, cudaStream_t s)
 {
     if (P.n == 0) return;
-    k_claim<<<P.n, PT, 0, s>>>(L, P, owner_new);
+    k_claim<<<P.n, cover_threads(P.n), 0, s>>>(L, P, owner_new);
 }
 
 void launch_transition(int storage, const Lat &L, const Parts &P, void *f, uint8_t *type,
@@ -2339,7 +2344,7 @@ void batch_shell_extent(const Lat &L, const Parts &P, int ext[3])
 void launch_reset(const Lat &L, const Parts &P, int use_old, uint32_t *owner, cudaStream_t s)
 {
     if (P.n == 0) return;
-    k_reset<<<P.n, PT, 0, s>>>(L, P, use_old, owner);
+    k_reset<<<P.n, cover_threads(P.n), 0, s>>>(L, P, use_old, owner);
 }
 
 }  // namespace lbe
