@@ -16,9 +16,9 @@ namespace lbe {
 namespace {
 
 constexpr int PT = 128;  // threads per per-particle CTA
-// Threads per particle of the claim and the reset, whose order does not
-// matter: with fewer particles than SMs a particle's rows spread over 16
-// warps.
+// Threads per particle of the claim, the transition and the reset: with fewer
+// particles than SMs a particle's rows spread over 16 warps (one ellipsoid
+// (12, 6): 5.3, 5.2 and 4.8 us against 9.0, 8.6 and 7.6 with four).
 constexpr int PT_WIDE = 512;
 static int cover_threads(int np) { return np < 152 ? PT_WIDE : PT; }
 
@@ -297,16 +297,17 @@ __device__ __forceinline__ RowSpan span_of(const Geo &g, const int Xi[3], const 
 }
 
 // Rows of a box that is no whole period along any axis, 32 at a time per
-// warp (one a lane): f(valid, u1, u2) is called by whole warps.
+// warp (one a lane): f(chunk, valid, u1, u2) is called by whole warps, chunk
+// counting the 32s.
 template <class F>
 __device__ __forceinline__ void for_rows(const Box &b, F f)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int rows = b.ext[1] * b.ext[2];
-    for (int r0 = warp * 32; r0 < rows; r0 += nw * 32) {
-        const int r = r0 + lane;
+    for (int c = warp; c * 32 < rows; c += nw) {
+        const int r = c * 32 + lane;
         const bool valid = r < rows;
-        f(valid, b.lo[1] + (valid ? r % b.ext[1] : 0), b.lo[2] + (valid ? r / b.ext[1] : 0));
+        f(c, valid, b.lo[1] + (valid ? r % b.ext[1] : 0), b.lo[2] + (valid ? r / b.ext[1] : 0));
     }
 }
 
@@ -337,12 +338,12 @@ template <class F>
 __device__ __forceinline__ void for_box(const Box &b, F f)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k0 = warp * 32; k0 < b.count; k0 += nw * 32) {
-        const int k = k0 + lane;
+    for (int c = warp; c * 32 < b.count; c += nw) {
+        const int k = c * 32 + lane;
         const bool valid = k < b.count;
         const int kk = valid ? k : 0;
         const int t = kk / b.ext[0];
-        f(valid, b.lo[0] + kk % b.ext[0], b.lo[1] + t % b.ext[1], b.lo[2] + t / b.ext[1]);
+        f(c, valid, b.lo[0] + kk % b.ext[0], b.lo[1] + t % b.ext[1], b.lo[2] + t / b.ext[1]);
     }
 }
 
@@ -1400,7 +1401,7 @@ __device__ __forceinline__ void claim_body(const Lat &L, const Parts &P, int p, 
     const PGeom &G = reinterpret_cast<const PGeom2 *>(P.geo)[p].now;
     const Box &box = G.box;
     if (box_full(box)) {
-        for_box(box, [&](bool valid, int ux, int u1, int u2) {
+        for_box(box, [&](int, bool valid, int ux, int u1, int u2) {
             if (!valid) return;
             const int u[3] = {ux, u1, u2};
             const int x = wrapi(ux, L.nx), y = wrapi(u1, L.ny), z = wrapi(u2, L.nz);
@@ -1422,7 +1423,7 @@ __device__ __forceinline__ void claim_body(const Lat &L, const Parts &P, int p, 
         });
         return;
     }
-    for_rows(box, [&](bool valid, int u1, int u2) {
+    for_rows(box, [&](int, bool valid, int u1, int u2) {
         int a = 1, b = 0;
         if (valid && !is_wall_z(L, wrapi(u2, L.nz))) {
             const RowSpan r = span_of(G.g, G.Xi, G.Xf, box, u1, u2);
@@ -1465,8 +1466,8 @@ __global__ void __launch_bounds__(PT_WIDE) k_claim(Lat L, Parts P, uint32_t *__r
 // The fill or empty of a changed node is the work of a whole warp (one
 // direction, or one neighbour's populations, per lane).  512^3 Pickering:
 // 731 us when every candidate's two owners were read and one lane did each
-// change, 501 now; 40 dragged particles, of which some change every step:
-// 67 and 22 us.
+// change, 198 now; 40 dragged particles, of which some change every step:
+// 67 and 17 us.
 
 // What a particle takes over with (o == NONE, covered) or gives to (w ==
 // NONE, uncovered) node (x, y, z): momentum mom.  Called by a whole warp.
@@ -1552,15 +1553,19 @@ __device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, in
                                                 const uint32_t *__restrict__ own_new, int placement)
 {
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __shared__ double part[PT / 32][6];
+    const int lane = threadIdx.x & 31;
+    // the sums of the chunks c = k mod CHUNKS, each in the order of its chunks,
+    // whatever warp takes them: the totals do not depend on the threads
+    constexpr int CHUNKS = PT_WIDE / 32;
+    __shared__ double part[CHUNKS][6];
+    for (int k = threadIdx.x; k < CHUNKS * 6; k += blockDim.x) part[k / 6][k % 6] = 0.0;
+    __syncthreads();
     const PGeom2 &G2 = reinterpret_cast<const PGeom2 *>(P.geo)[p];
     const Box &box = G2.uni;
-    double acc[6] = {0, 0, 0, 0, 0, 0};  // the same on every lane
     bool any = false;
     // one node a lane (cand: it has one): the changed ones go through
     // change_node one after the other
-    auto visit = [&](bool cand, int ux, int u1, int u2) {
+    auto visit = [&](int chunk, bool cand, int ux, int u1, int u2) {
         int x = 0, y = 0, z = 0;
         uint32_t o = NONE, w = NONE;
         if (cand) {
@@ -1579,17 +1584,24 @@ __device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, in
         }
         unsigned m = __ballot_sync(full, o != w);
         if (placement) return;
+        if (!m) return;
+        any = true;
+        double acc[6];  // the same on every lane
+        for (int k = 0; k < 6; k++) acc[k] = part[chunk % CHUNKS][k];
         for (; m; m &= m - 1) {
             const int src = __ffs(m) - 1;
             change_node<S>(L, P, p, f, __shfl_sync(full, x, src), __shfl_sync(full, y, src), __shfl_sync(full, z, src),
                            __shfl_sync(full, (int)(o == NONE), src) != 0, own_old, own_new, acc);
-            any = true;
         }
+        __syncwarp();
+        if (lane == 0)
+            for (int k = 0; k < 6; k++) part[chunk % CHUNKS][k] = acc[k];
+        __syncwarp();
     };
     if (box_full(box)) {
         for_box(box, visit);
     } else {
-        for_rows(box, [&](bool valid, int u1, int u2) {
+        for_rows(box, [&](int chunk, bool valid, int u1, int u2) {
             int a = 1, b = 0, ca = 1, cb = 0;  // nodes [a, b] but for [ca, cb]
             if (valid) {
                 const RowSpan s0 = span_of(G2.old_.g, G2.old_.Xi, G2.old_.Xf, box, u1, u2);
@@ -1611,31 +1623,26 @@ __device__ __forceinline__ void transition_body(const Lat &L, const Parts &P, in
             }
             if (a == ca && ca <= cb) a = cb + 1;
             while (__any_sync(full, a <= b)) {
-                visit(a <= b, a, u1, u2);
+                visit(chunk, a <= b, a, u1, u2);
                 if (++a == ca && ca <= cb) a = cb + 1;
             }
         });
     }
     if (placement) return;
-    if (!__syncthreads_or(any)) {
-        if (threadIdx.x < 3) {
-            P.Fpend[3 * p + threadIdx.x] = 0.0;
-            P.Tpend[3 * p + threadIdx.x] = 0.0;
-        }
-        return;
-    }
-    if (lane == 0)
-        for (int k = 0; k < 6; k++) part[warp][k] = acc[k];
-    __syncthreads();
+    any = __syncthreads_or(any);
     if (threadIdx.x < 6) {
         double a = 0.0;
-        for (int w = 0; w < PT / 32; w++) a += part[w][threadIdx.x];
+        if (any)
+            for (int c = 0; c < CHUNKS; c++) a += part[c][threadIdx.x];
         (threadIdx.x < 3 ? P.Fpend + 3 * p + threadIdx.x : P.Tpend + 3 * p + threadIdx.x - 3)[0] = a;
     }
 }
 
-template <class S>
-__global__ void __launch_bounds__(PT) k_transition(Lat L, Parts P, typename S::P *f, uint8_t *type,
+// T threads per CTA.  With many particles eight CTAs per SM (64 registers)
+// hide the latency of the row bounds (25,033: 198 us against 281 with 96
+// registers); the rare changes spill.
+template <class S, int T>
+__global__ void __launch_bounds__(T, T == PT ? 8 : 1) k_transition(Lat L, Parts P, typename S::P *f, uint8_t *type,
                                                    const uint32_t *__restrict__ own_old,
                                                    const uint32_t *__restrict__ own_new, int placement)
 {
@@ -1655,14 +1662,14 @@ __device__ __forceinline__ void reset_body(const Lat &L, const Parts &P, int p, 
     const PGeom2 &G2 = reinterpret_cast<const PGeom2 *>(P.geo)[p];
     const PGeom &G = use_old ? G2.old_ : G2.now;
     if (box_full(G.box)) {
-        for_box(G.box, [&](bool valid, int ux, int u1, int u2) {
+        for_box(G.box, [&](int, bool valid, int ux, int u1, int u2) {
             if (!valid) return;
             const int n = wrapi(ux, L.nx) + L.nx * (wrapi(u1, L.ny) + L.ny * wrapi(u2, L.nz));
             if (idx_ok(L, n, L.N, 7)) owner[n] = NONE;
         });
         return;
     }
-    for_rows(G.box, [&](bool valid, int u1, int u2) {
+    for_rows(G.box, [&](int, bool valid, int u1, int u2) {
         int a = 1, b = 0;
         if (valid) row_span(G.g, G.Xi, G.Xf, G.box, u1, u2, a, b);
         fill_rows(L, a, b, u1, u2, [&](int n) {
@@ -1696,9 +1703,9 @@ __global__ void __launch_bounds__(PT_WIDE) k_reset(Lat L, Parts P, int use_old, 
 // the pass's 225; it pays where particles are few (dense_rho).
 //
 // Tiles: with many particles 22 x 22 rows (an ellipsoid of reach 8 is one
-// tile); with few, 10 x 5 rows, so that one particle spreads over several
-// SMs (the halo rows are then 68 % more rows, which costs less than idle
-// SMs).  Results do not depend on the tiling.
+// tile); with few, 10 x 5 rows, and with fewer than 64 such tiles 8 x 2, so
+// that one particle spreads over many SMs (the halo rows are then 68 % or 150
+// % more rows, which costs less than idle SMs).  Results do not depend on the tiling.
 //
 // A tile's link entries go into the list as one contiguous segment in row
 // order (one reservation, while the densities come in), so that the link
@@ -2063,7 +2070,7 @@ __global__ void __launch_bounds__(PT_WIDE) k_claim_batch(BatchIndex B, int total
 }
 
 template <class S>
-__global__ void __launch_bounds__(PT) k_transition_batch(BatchIndex B, int total)
+__global__ void __launch_bounds__(PT_WIDE) k_transition_batch(BatchIndex B, int total)
 {
     const int g = blockIdx.x;
     const int b = B.pbox[g];
@@ -2248,26 +2255,32 @@ void launch_transition(int storage, const Lat &L, const Parts &P, void *f, uint8
                        cudaStream_t s)
 {
     if (P.n == 0) return;
-    LBE_DISPATCH(storage, (k_transition<S><<<P.n, PT, 0, s>>>(L, P, (typename S::P *)f, type, owner_old,
-                                                               owner_new, placement)));
+    if (cover_threads(P.n) == PT)
+        LBE_DISPATCH(storage, (k_transition<S, PT><<<P.n, PT, 0, s>>>(L, P, (typename S::P *)f, type, owner_old, owner_new,
+                                                                      placement)));
+    else
+        LBE_DISPATCH(storage, (k_transition<S, PT_WIDE><<<P.n, PT_WIDE, 0, s>>>(L, P, (typename S::P *)f, type, owner_old,
+                                                                                owner_new, placement)));
 }
 
 void launch_transition_batch(int storage, const BatchIndex &B, int total, cudaStream_t s)
 {
     if (total == 0) return;
-    LBE_DISPATCH(storage, (k_transition_batch<S><<<total, PT, 0, s>>>(B, total)));
+    LBE_DISPATCH(storage, (k_transition_batch<S><<<total, cover_threads(total), 0, s>>>(B, total)));
 }
 
 // Tiles for np particles in boxes of at most ext nodes a side.  The small
-// tiles are at most 15 times as many as the large ones, fewer than 15 x 304;
-// each adds at most 7 empty entries to each of its at most two list windows
-// (10 x 5 x 30 nodes): fewer than LINK_PAD in all.
+// tiles are at most 15 times as many as the large ones, fewer than 15 x 304
+// (the smallest at most 6 times 64); each adds at most 7 empty entries to each
+// of its at most two list windows (10 x 5 x 30 nodes): fewer than LINK_PAD in
+// all.
 static_assert(15 * 304 * 2 * 7 <= LINK_PAD, "empty link entries fit");
 static ShellGrid shell_grid(const int ext[3], int np)
 {
     auto up = [](int a, int b) { return (a + b - 1) / b; };
     ShellGrid g{up(ext[0], SHELL_X), up(ext[1], SHELL_MAX), up(ext[2], SHELL_MAX), SHELL_MAX, SHELL_MAX, 1};
     if ((long long)np * g.nx * g.ny * g.nz < 2 * 152) g = ShellGrid{g.nx, up(ext[1], 10), up(ext[2], 5), 10, 5, 8};
+    if (g.pad == 8 && (long long)np * g.nx * g.ny * g.nz < 64) g = ShellGrid{g.nx, up(ext[1], 8), up(ext[2], 2), 8, 2, 8};
     return g;
 }
 
