@@ -1,0 +1,127 @@
+"""The step's kernels at the sizes where their work splits change: tile edges
+of the shell fill, the two sources of densities, the pair forces with and
+without cell lists, the wide and the narrow coverage kernels, tile heights
+and z chunks of the fused kernel, and captured single steps.
+
+One step from random populations agrees with the FP64 oracle to 2e-6 on
+populations of order 0.03 (a few FP32 ulps of the largest intermediate);
+forces to 1e-5 of their largest (sums of FP32 link terms).  Where two splits of
+the same work are compared, they agree bit for bit."""
+import numpy as np
+import pytest
+
+from oracle import lbref
+from paper_1109_3277_gb300 import lbe
+from paper_1109_3277_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TOL_F, TOL_FORCE = 2e-6, 1e-5
+
+
+def _one_step(shape, part, walls=False, mode="static", steps=1):
+    """The library and the oracle after `steps` steps from random populations."""
+    nx, ny, nz = shape
+    f0 = W.random_populations(shape, seed=61)
+    kw = dict(walls_z=walls, g_br=0.1)
+    g = lbe.Lattice(shape, np.full((2, nz, ny, nx), 0.5), particle_mode=mode, **kw)
+    r = lbref.Lattice(shape, np.full((2, nz, ny, nx), 0.5), particle_mode=lbe.MODES[mode], **kw)
+    n = len(part["pos"])
+    rp, ro, dr = (np.broadcast_to(part[k], (n,)).astype(float) for k in ("r_par", "r_perp", "delta_rho"))
+    for L in (g, r):
+        L.add_particles(part["pos"], part["quat"], rp, ro, dr, vel=part.get("vel"), omega=part.get("omega"))
+        L.set_populations(f0)
+        L.step(steps)
+    return g, r
+
+
+def _agree(g, r):
+    _, _, tg = g.read_fields()
+    _, _, tr = r.read_fields()
+    assert np.array_equal(tg, tr)
+    fl = tr == 0
+    assert np.max(np.abs(g.get_populations()[:, :, fl] - r.get_populations()[:, :, fl])) < TOL_F
+    pg, pr = g.read_particles(), r.read_particles()
+    for k in ("force", "torque"):
+        assert np.max(np.abs(pg[k] - pr[k])) < TOL_FORCE * max(1.0, np.abs(pr[k]).max()), k
+
+
+# Boxes of one particle: 8 x 2 rows, 10 x 5 rows, one and two x tiles (30
+# nodes), rows across the large tile's edge (22); a box that is a whole period
+# of the lattice.
+@pytest.mark.parametrize("shape,r_par,r_perp,tilt", [((20, 22, 24), 2.3, 2.1, 0.3),
+                                                     ((24, 26, 40), 12.4, 3.2, 0.1),
+                                                     ((48, 24, 24), 13.6, 4.0, 1.5),
+                                                     ((44, 44, 44), 9.3, 8.7, 0.8),
+                                                     ((14, 30, 26), 5.2, 4.9, 1.1)])
+@pytest.mark.parametrize("walls", [False, True])
+def test_shell_tiles_of_one_particle(shape, r_par, r_perp, tilt, walls):
+    part = dict(pos=[[shape[0] / 2 - 0.3, shape[1] / 2 + 0.2, shape[2] / 2 + 0.1]],
+                quat=[W.axis_tilt_quaternion(tilt, 0.4)], r_par=r_par, r_perp=r_perp, delta_rho=0.07,
+                vel=[[0.01, -0.02, 0.005]], omega=[[0.003, 0.002, -0.004]])
+    _agree(*_one_step(shape, part, walls))
+
+
+# 5 and 40 small particles take small tiles, 320 the large ones with the
+# 128-thread coverage and narrow link groups; 255 to 257 straddle the cell
+# lists' threshold.  From 40 on the density pass runs.
+@pytest.mark.parametrize("count", [5, 40, 255, 256, 257, 320])
+def test_many_particles_one_step(count):
+    shape = (56, 52, 50)
+    pos, quat = W.place_ellipsoids(shape, count, 3.0, 1.5, seed=62, margin=0.6)
+    assert len(pos) == count
+    part = dict(pos=pos, quat=quat, r_par=3.0, r_perp=1.5, delta_rho=-0.05,
+                vel=W.uniform(63, (count, 3), lo=-2e-3, hi=2e-3), omega=W.uniform(64, (count, 3), lo=-2e-3, hi=2e-3))
+    _agree(*_one_step(shape, part, mode="free"))
+
+
+@pytest.mark.parametrize("count", [1, 151, 152])
+def test_driven_particles_change_the_same_nodes(count):
+    """Particles driven by up to 0.2 nodes a step for 8 steps: every covered
+    and uncovered node is the oracle's, with 16 and with 4 warps a particle."""
+    shape = (48, 46, 44)
+    pos, quat = W.place_ellipsoids(shape, count, 3.0, 2.0, seed=65, margin=1.0)
+    part = dict(pos=pos, quat=quat, r_par=3.0, r_perp=2.0, delta_rho=0.0,
+                vel=W.uniform(66, (len(pos), 3), lo=-0.2, hi=0.2), omega=W.uniform(67, (len(pos), 3), lo=-0.05, hi=0.05))
+    assert len(pos) == count
+    g, r = _one_step(shape, part, mode="prescribed", steps=8)
+    assert np.array_equal(g.read_fields()[2], r.read_fields()[2])
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("shape,walls,count", [((64, 20, 18), False, 0), ((64, 20, 18), True, 0), ((45, 20, 18), False, 0),
+                                               ((64, 36, 30), False, 2), ((64, 36, 30), False, 20)])
+def test_tiles_and_chunks_give_identical_results(shape, walls, count, storage):
+    """Tile heights and z chunks (1 to beyond the lattice) split the same work:
+    with and without solid nodes, tensor copies (nx = 45: none at 16 bit), and
+    the density pass (20 particles)."""
+    pos, quat = W.place_ellipsoids(shape, count, 4.0, 3.0, seed=68)
+    out = []
+    for rows, zc in ((None, 0), (8, 1), (8, 7), (4, 2), (4, 100)):
+        nx, ny, nz = shape
+        g = lbe.Lattice(shape, W.random_phases(shape, 0.5, seed=69), walls_z=walls, g_br=0.1, storage=storage)
+        if count:
+            g.add_particles(pos, quat, 4.0, 3.0, 0.05)
+        if rows:
+            g.set_tile(rows, zc)
+        g.step(7)
+        out.append(g.get_populations())
+    for f in out[1:]:
+        assert np.array_equal(out[0], f)
+
+
+@pytest.mark.parametrize("mode,count", [("free", 1), ("free", 30), ("static", 2)])
+def test_single_steps_replayed_equal_pairs_of_steps(mode, count):
+    """40 single steps (direct, then a captured graph) and 40 at once (captured
+    pairs, with the pair forces and the owner map's reset on a branch)."""
+    shape = (40, 36, 34)
+    pos, quat = W.place_ellipsoids(shape, count, 3.0, 2.0, seed=70)
+    a, b = [], []
+    for steps, out in (([1] * 40, a), ([40], b)):
+        g = lbe.Lattice(shape, W.random_phases(shape, 0.5, seed=71), g_br=0.1, particle_mode=mode)
+        g.add_particles(pos, quat, 3.0, 2.0, 0.05, vel=np.full((count, 3), 0.004))
+        for n in steps:
+            g.step(n)
+        out += [g.get_populations(), g.read_fields()[2]] + [g.read_particles()[k] for k in ("pos", "quat", "force")]
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
