@@ -197,14 +197,14 @@ LBE_API lbe_status lbe_mass_noalloc(const void *f, int32_t storage, const uint8_
 
 /* Pick the fused kernel's tile height and z-chunk length for this lattice
  * by timing the candidates (heights 8 and, where built, 4, times chunks
- * 4, 8, 16, ... and the full height) with CUDA events on the current state
+ * 2, 3, 4, 6, 8, 12, ... and the full height) with CUDA events on the current state
  * (which is not changed); later steps use the fastest.  *chosen_zc (may be
  * NULL) receives the chunk; lbe_get_tile gives both. */
 LBE_API lbe_status lbe_autotune(lbe_ctx *c, int32_t *chosen_zc);
 
 /* Set the fused kernel's z-chunk length (planes per CTA; 0 restores the
- * default, sized for about 16 waves of CTAs).  A chunk longer than the
- * lattice is clipped.  Only the order in which tiles run depends on it,
+ * default, which follows the number of CTAs and the storage).  A chunk longer
+ * than the lattice is clipped.  Only the order in which tiles run depends on it,
  * never a result.  Synchronises first (and returns a pending error of
  * earlier steps).  LBE_EINVAL for a negative length. */
 LBE_API lbe_status lbe_set_zchunk(lbe_ctx *c, int32_t zc);
@@ -251,8 +251,8 @@ LBE_API void lbe_fail_allocations(int32_t after);
  * batch exists; the batch does not own them.  After lbe_batch_step the
  * members are read with the usual calls.  Every member's populations and
  * particles are bit-identical to those of stepping it alone with lbe_step,
- * whatever else is in the batch.  The pair forces run one thread per
- * particle over the member's particles, so members are limited to
+ * whatever else is in the batch.  The pair forces loop over all of the
+ * member's particles, so members are limited to
  * LBE_BATCH_MAX_PARTICLES particles each (LBE_EINVAL beyond). */
 #define LBE_BATCH_MAX_PARTICLES 4096
 typedef struct lbe_batch lbe_batch;

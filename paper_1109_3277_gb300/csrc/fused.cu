@@ -10,23 +10,26 @@
 // per-row bitmask of solid nodes of the tile and a one-node halo go into a
 // four-slot ring of planes; the collision of plane z reads planes z-1, z
 // and z+1 of it.  Two configurations fill the ring:
-//  - ψ formed on chip (lattices with no or few particles, batches): the box also holds a
-//    one-node halo (x widened to 16-byte boundaries), and each thread sums
-//    the densities of its node and of at most one halo node, so ψ of the
-//    tile and its halo comes from the stage; halo nodes beyond the lattice
-//    edge wrap around and are read from global memory.  Solid nodes (walls)
-//    take their ψ from the shell fill.
+//  - ψ formed on chip (lattices with no or few particles, batches): the box
+//    also holds a one-node halo (x widened to 16-byte boundaries), and each
+//    thread sums the densities of its node and of at most one halo node, so ψ
+//    of the tile and its halo comes from the stage; halo nodes beyond the
+//    lattice edge wrap around and are read from global memory.  Solid nodes
+//    take their ψ from the shell fill; a variant for lattices without any
+//    has neither types nor masks.
 //  - ψ from memory (lattices with many particles): the density pass and the
 //    shell fill have written ψ of every node a fluid node sees.  The ring
 //    entries of plane z + 2 arrive by asynchronous copies issued before the
 //    collision of plane z and waited for after it.
 //
 // With τ = 1 for both components the post-collision populations are the
-// equilibria, so a node's populations are needed only for its moments:
-// with ψ formed on chip two stages suffice, while other τ keep three and
-// re-read the node's populations at the collision.  With ψ from memory a
-// third stage (copies two planes ahead) is kept where it costs no CTA per
-// SM.
+// equilibria, so a node's populations are needed only for its moments, and
+// with ψ formed on chip a stage is free as soon as they are taken: two stages
+// at 16 bit, one in FP32.  Other τ re-read the node's populations at the
+// collision, at 16 bit from a third stage, in FP32 from L2.  With ψ from
+// memory a third stage (copies two planes ahead) is kept where it costs no
+// CTA per SM.  Lattices whose rows are no multiple of 16 bytes have no tensor
+// copies: their entries are read from global memory.
 //
 // Populations streaming into a wall or particle node are reflected into the
 // opposite slot of their own node (halfway bounce-back).  For particle

@@ -3,9 +3,11 @@
 // Hertz / Berne–Pechukas and lubrication pair forces (Eq. 6-9), the
 // Newton–Euler update, and the node coverage with fill and empty.
 //
-// Per-particle work runs one CTA per particle over the particle's bounding
-// box; per-particle sums are FP64 and reduced in a fixed order, so results
-// are bit-reproducible run to run.
+// The coverage kernels run a CTA per particle over the rows of its bounding
+// box, the shell fill one or more tiles of that box, the update four lanes and
+// the pair forces eight lanes per particle.  Sums are 64-bit fixed point or
+// FP64 in an order that does not depend on the split of the work, so results
+// are bit-reproducible run to run, alone and in a batch.
 #include <algorithm>
 #include <cmath>
 
