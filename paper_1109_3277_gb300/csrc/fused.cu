@@ -38,6 +38,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -905,15 +906,25 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
     return ok;
 }
 
-template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
+// BANDS: grid z counts the z chunks of one band of tile rows after the other.
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS, bool BANDS>
 __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
     k_fused(Lat L, const typename S::P *__restrict__ fin, typename S::P *__restrict__ fout,
             const float *__restrict__ psi, const uint8_t *__restrict__ type, int zc, FusedOfs ofs,
-            const __grid_constant__ CUtensorMap tmap, int wait_limit)
+            const __grid_constant__ CUtensorMap tmap, int wait_limit, unsigned nzc, unsigned zmul)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    fused_tile<S, TY, GEN, SELF, TMA, R32, SOLIDS>(L, fin, fout, psi, type, zc, ofs, &tmap, blockIdx.x, blockIdx.y,
-                                           blockIdx.z, wait_limit, align128(smem_raw));
+    int by = blockIdx.y, bz = blockIdx.z;
+    if (BANDS) {
+        // blockIdx.z / nzc by its reciprocal: a division would take the tile's
+        // coordinates out of the uniform registers
+        const unsigned band = __umulhi(blockIdx.z, zmul);
+        by += band * gridDim.y;
+        bz -= band * nzc;
+        if (by * TY >= L.ny) return;
+    }
+    fused_tile<S, TY, GEN, SELF, TMA, R32, SOLIDS>(L, fin, fout, psi, type, zc, ofs, &tmap, blockIdx.x, by, bz,
+                                                   wait_limit, align128(smem_raw));
 }
 
 // Persistent multi-lattice variant: CTAs take tiles of all boxes of a batch
@@ -984,12 +995,17 @@ int fused_zchunk(const Lat &L, int ty, int es, bool self, double share)
     // planes 25 us, 16 planes 53.  With ψ formed on chip, chunks of more than
     // 8 planes (FP32: 4) let the halo rows of the next chunk and the next
     // rows of tiles leave L2 before they are read again: 256^3 f16 598 us at
-    // 8 planes, 652 at 16, 805 at 48; f32 964 at 4, 1095 at 16.  With ψ from
-    // memory (256^3 bijel, f16) 564 at 16, 601 at 64.
+    // 8 planes, 652 at 16, 805 at 48; f32 964 at 4, 1095 at 16.  With any
+    // τ at 16 bit, whose collision takes longer, the halo planes that longer
+    // chunks save are worth more: 256^3 f16 676 at 12 against 710 at 8 and 688
+    // at 16.  With ψ from memory (256^3 bijel, f16) 564 at 16, 601 at 64.
     const long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
     const bool tma = (L.nx * 2 * es) % 16 == 0;
-    const int cap = !self ? 16 : (!tma ? 12 : (es == 4 ? (ty == 4 ? 5 : 4) : (ty == 4 ? 6 : 8)));
-    const int slots = (fused_tau1(L) && fused_rel32(L) ? 3 : 2) * 8 / ty;  // CTAs an SM takes
+    const bool gen = !(fused_tau1(L) && fused_rel32(L));
+    const int cap = !self ? 16
+                    : !tma || (es == 2 && gen) ? 12
+                    : es == 4 ? (ty == 4 ? 5 : 4) : (ty == 4 ? 6 : 8);
+    const int slots = (gen ? 2 : 3) * 8 / ty;  // CTAs an SM takes
     const double full = 1.7 + 0.9 * slots * ty / 8;
     int best = 1;
     double bt = 1e30;
@@ -1056,20 +1072,50 @@ bool fused_rel32(const Lat &L)
     return !L.wide && (long long)Q * L.S + 2LL * L.N + (long long)L.nx * L.ny + L.nx + 1 < (1LL << 32);
 }
 
-template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
-static void launch_cfg(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
-                       const CUtensorMap &tm, int zc, int wait_limit, cudaStream_t s)
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS, bool BANDS>
+static void launch_bands(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
+                         const CUtensorMap &tm, int zc, int bands, int wait_limit, cudaStream_t s)
 {
     using C = Cfg<S, TY, GEN, SELF, TMA>;
     using P = typename S::P;
-    auto kern = k_fused<S, TY, GEN, SELF, TMA, R32, SOLIDS>;
+    auto kern = k_fused<S, TY, GEN, SELF, TMA, R32, SOLIDS, BANDS>;
     static bool configured = false;  // the attribute is per function and process
     if (!configured) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes);
         configured = true;
     }
-    dim3 grid((L.nx + TX - 1) / TX, (L.ny + TY - 1) / TY, (L.nz + zc - 1) / zc);
-    kern<<<grid, C::NT, C::bytes, s>>>(L, (const P *)fin, (P *)fout, psi, type, zc, fused_offsets(L), tm, wait_limit);
+    const unsigned nty = (L.ny + TY - 1) / TY, nzc = (L.nz + zc - 1) / zc;
+    const unsigned zmul = bands > 1 ? 0xffffffffu / nzc + 1u : 0u;  // exact: nzc > 1, nzc * bands < 2^16
+    dim3 grid((L.nx + TX - 1) / TX, (nty + bands - 1) / bands, nzc * bands);
+    kern<<<grid, C::NT, C::bytes, s>>>(L, (const P *)fin, (P *)fout, psi, type, zc, fused_offsets(L), tm, wait_limit, nzc,
+                                       zmul);
+}
+
+template <class S, int TY, bool GEN, bool SELF, bool TMA, bool R32, bool SOLIDS>
+static void launch_cfg(const Lat &L, const void *fin, void *fout, const float *psi, const uint8_t *type,
+                       const CUtensorMap &tm, int zc, int wait_limit, cudaStream_t s)
+{
+    // A chunk reads again the last planes of the chunk below it.  They are
+    // still in L2 (128 MB) if the reads and writes of one layer of chunks fit,
+    // so wider layers are split into bands of 16 or more tile rows and each
+    // band goes through all of z first: f16 512^3 3.76 ms against 4.09 (bands
+    // of 32 tiles of 4 rows; 64: 3.95, 16: 3.81), f32 512^3 6.54 against 7.41,
+    // f16 384^3 1.62 against 1.69, f32 320^3 1.65 against 1.70.  With ψ from
+    // memory only ψ is read twice: a split gains nothing at 301 MB a layer
+    // (352^3) and 1.7 % at 637 (512^3).  Any τ: 1 to 2 %, not built.
+    if constexpr (!GEN && TMA) {
+        constexpr size_t pair = sizeof(typename S::P);
+        const double layer = (double)L.nx * L.ny * zc * 2 * Q * pair, fits = SELF ? 100e6 : 512e6;
+        const int nty = (L.ny + TY - 1) / TY, nzc = (L.nz + zc - 1) / zc;
+        const int most = nzc > 1 ? std::min(65535 / nzc, nty / 16) : 1;
+        const int bands = (int)std::min<double>(most, std::ceil(layer / fits));
+        if (bands > 1) {
+            launch_bands<S, TY, GEN, SELF, TMA, R32, SOLIDS, true>(L, fin, fout, psi, type, tm, zc, bands, wait_limit,
+                                                                   s);
+            return;
+        }
+    }
+    launch_bands<S, TY, GEN, SELF, TMA, R32, SOLIDS, false>(L, fin, fout, psi, type, tm, zc, 1, wait_limit, s);
 }
 
 // Configurations built, each with ψ formed in the kernel (SELF; also without

@@ -110,6 +110,28 @@ def test_tiles_and_chunks_give_identical_results(shape, walls, count, storage):
         assert np.array_equal(out[0], f)
 
 
+@pytest.mark.parametrize("nz,walls,count,storage,thick", [(30, False, 0, "f16", 24), (30, True, 0, "f32", 24),
+                                                          (30, False, 1, "bf16", 24), (64, False, 700, "f16", 62)])
+def test_bands_of_tiles_give_identical_results(nz, walls, count, storage, thick):
+    """Layers of chunks too large for L2 go in bands of tile rows (35 rows of 8
+    nodes as 18 and 17, 70 of 4 in up to four bands), as thin chunks do in one;
+    with ψ on chip and (700 particles) from memory."""
+    shape = (200, 277, nz)
+    pos, quat = W.place_ellipsoids(shape, count, 4.0, 3.0, seed=72)
+    rho0 = W.random_phases(shape, 0.5, seed=73)
+    out = []
+    for rows, zc in ((8, 2), (8, thick), (4, thick)):
+        g = lbe.Lattice(shape, rho0, walls_z=walls, g_br=0.1, storage=storage)
+        if count:
+            g.add_particles(pos, quat, 4.0, 3.0, 0.05)
+        g.set_tile(rows, zc)
+        g.step(3)
+        out.append(g.get_populations())
+        g.close()
+    for f in out[1:]:
+        assert np.array_equal(out[0], f)
+
+
 @pytest.mark.parametrize("mode,count", [("free", 1), ("free", 30), ("static", 2)])
 def test_single_steps_replayed_equal_pairs_of_steps(mode, count):
     """40 single steps (direct, then a captured graph) and 40 at once (captured
