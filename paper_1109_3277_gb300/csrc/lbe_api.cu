@@ -328,54 +328,42 @@ void enqueue_step(lbe_ctx *c, bool branch = false)
 
 // Cell list for the pair forces: cells of edge >= the largest pair reach
 // (2 max radius + Δc + the prefilter's margin), at least 2 nodes a side.
-// (np particles of the block blk laid out for capacity cap; on failure the
-// context keeps its old cells)
-lbe_status build_cells(lbe_ctx *c, const std::vector<double> &blk, int cap, int np)
+// (np particles of the block blk laid out for capacity cap; the geometry only)
+Cells cell_grid(const lbe_ctx *c, const std::vector<double> &blk, int cap, int np)
 {
     double rmax = 0.0;
     for (int p = 0; p < np; p++)
         rmax = std::fmax(rmax, std::fmax(blk[(size_t)ORP * cap + p], blk[(size_t)ORO * cap + p]));
     const double reach = 2.0 * rmax + c->pair.lub_cut + 0.1;
-    Cells &C = c->cells;
+    Cells C{};
     const int dim[3] = {c->L.nx, c->L.ny, c->L.nz};
-    long long ncell = 1;
-    int cn[3];
-    float cinv[3];
+    C.ncell = 1;
     for (int k = 0; k < 3; k++) {
-        int n = (int)std::floor(dim[k] / reach);
-        n = std::max(1, std::min(n, dim[k] / 2));
-        cn[k] = n;
-        cinv[k] = (float)((double)n / dim[k]);
-        ncell *= n;
+        const int n = std::max(1, std::min((int)std::floor(dim[k] / reach), dim[k] / 2));
+        C.n[k] = n;
+        C.inv[k] = (float)((double)n / dim[k]);
+        C.ncell *= n;
     }
-    // head in one buffer, next | cid in another; the old buffers go only once
-    // the new ones exist
-    const size_t b0 = (size_t)ncell * sizeof(int), b1 = (size_t)2 * cap * sizeof(int);
-    int *nhead = nullptr, *nnext = nullptr;
-    cudaError_t e = lib_malloc((void **)&nhead, b0);
-    if (e != cudaSuccess) return cuda_fail(c, e, "add_particles: cudaMalloc(cells)");
-    e = lib_malloc((void **)&nnext, b1);
-    if (e != cudaSuccess) {
-        cudaFree(nhead);
-        return cuda_fail(c, e, "add_particles: cudaMalloc(cells)");
-    }
-    if (C.head) {
-        cudaFree(C.head);
-        cudaFree(C.next);
-        c->bytes -= c->cells_bytes;
-    }
-    C.head = nhead;
-    C.next = nnext;
-    C.ncell = (int)ncell;
-    for (int k = 0; k < 3; k++) {
-        C.n[k] = cn[k];
-        C.inv[k] = cinv[k];
-    }
-    C.cid = C.next + cap;
-    c->cells_bytes = b0 + b1;
-    c->bytes += c->cells_bytes;
-    return LBE_OK;
+    return C;
 }
+
+// Device buffers of a call that may still fail: freed at its end unless kept.
+struct Pending {
+    void *held[8];
+    int n = 0;
+    template <class T>
+    cudaError_t alloc(T **p, size_t bytes)
+    {
+        const cudaError_t e = lib_malloc((void **)p, bytes);
+        if (e == cudaSuccess) held[n++] = *p;
+        return e;
+    }
+    void keep() { n = 0; }
+    ~Pending()
+    {
+        while (n > 0) cudaFree(held[--n]);
+    }
+};
 
 lbe_status check_async(lbe_ctx *c, const char *where)
 {
@@ -592,58 +580,60 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
         x32[ncap + 2 * p + 1] = make_float4((float)blk[OW * cp + 3 * p], (float)blk[OW * cp + 3 * p + 1],
                                             (float)blk[OW * cp + 3 * p + 2], 0.f);
     }
-    if (!c->ll.ent) {
+    // Every allocation comes before the first buffer is replaced: a failed call
+    // leaves the lattice, and the graphs captured of its steps, as they were.
+    Pending fresh;
+    cudaError_t e = cudaSuccess;
+    LinkList nll = c->ll;
+    const size_t cap_ll = (size_t)c->L.N + LINK_PAD;
+    const bool first = !nll.ent;
+    if (first) {
         // a particle node enters the link list at most once per step, and
         // LINK_PAD bounds the empty entries
-        const size_t cap_ll = (size_t)c->L.N + LINK_PAD;
-        uint2 *ent = nullptr;
-        int *cnt = nullptr;
-        CK(c, lib_malloc((void **)&ent, cap_ll * sizeof(uint2)));
-        cudaError_t e = lib_malloc((void **)&cnt, sizeof(int));
-        if (e != cudaSuccess) {
-            cudaFree(ent);
-            return cuda_fail(c, e, "add_particles: cudaMalloc(link list)");
-        }
-        CK(c, cudaMemset(cnt, 0, sizeof(int)));
-        c->ll.ent = ent;
-        c->ll.count = cnt;
-        c->ll.cap = (int)std::min<size_t>(cap_ll, INT32_MAX);
+        e = fresh.alloc(&nll.ent, cap_ll * sizeof(uint2));
+        if (e == cudaSuccess) e = fresh.alloc(&nll.count, sizeof(int));
+        if (e == cudaSuccess) e = cudaMemset(nll.count, 0, sizeof(int));
+        nll.cap = (int)std::min<size_t>(cap_ll, INT32_MAX);
+    }
+    Cells ncells = cell_grid(c, blk, ncap, np);  // head in one buffer, next | cid in another
+    const size_t cells_bytes = (size_t)ncells.ncell * sizeof(int) + (size_t)2 * ncap * sizeof(int);
+    if (e == cudaSuccess) e = fresh.alloc(&ncells.head, (size_t)ncells.ncell * sizeof(int));
+    if (e == cudaSuccess) e = fresh.alloc(&ncells.next, (size_t)2 * ncap * sizeof(int));
+    double *nb = nullptr, *npp = nullptr;
+    float4 *nx32 = nullptr;
+    void *ngeo = nullptr;
+    if (ncap != cap) {
+        if (e == cudaSuccess) e = fresh.alloc(&nb, blk.size() * sizeof(double));
+        if (e == cudaSuccess) e = fresh.alloc(&nx32, x32.size() * sizeof(float4));
+        if (e == cudaSuccess) e = fresh.alloc(&npp, (size_t)6 * ncap * sizeof(double));
+        if (e == cudaSuccess) e = fresh.alloc(&ngeo, (size_t)ncap * geom_bytes_per_particle());
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "add_particles: cudaMalloc");
+    fresh.keep();
+    drop_graphs(c);
+    if (first) {
+        c->ll = nll;
         c->bytes += cap_ll * sizeof(uint2) + sizeof(int);
     }
-    {
-        lbe_status cst = build_cells(c, blk, ncap, np);
-        if (cst != LBE_OK) return cst;
-    }
+    cudaFree(c->cells.head);
+    cudaFree(c->cells.next);
+    ncells.cid = ncells.next + ncap;
+    c->cells = ncells;
+    c->bytes += cells_bytes - c->cells_bytes;
+    c->cells_bytes = cells_bytes;
     if (ncap != cap) {
-        double *nb = nullptr;
-        float4 *nx32 = nullptr;
-        double *npp = nullptr;
-        void *ngeo = nullptr;
-        CK(c, lib_malloc((void **)&nb, blk.size() * sizeof(double)));
-        cudaError_t e = lib_malloc((void **)&nx32, x32.size() * sizeof(float4));
-        if (e == cudaSuccess) e = lib_malloc((void **)&npp, (size_t)6 * ncap * sizeof(double));
-        if (e == cudaSuccess) e = lib_malloc(&ngeo, (size_t)ncap * geom_bytes_per_particle());
-        if (e != cudaSuccess) {
-            cudaFree(nb);
-            cudaFree(nx32);
-            cudaFree(npp);
-            return cuda_fail(c, e, "add_particles: cudaMalloc");
-        }
         const size_t per_cap = PSTRIDE * sizeof(double) + 3 * sizeof(float4) + 6 * sizeof(double) +
                                geom_bytes_per_particle();
-        if (c->pbuf) {
-            cudaFree(c->pbuf);
-            cudaFree(c->x32);
-            cudaFree(c->ppart);
-            cudaFree(c->geo);
-            c->bytes -= (size_t)cap * per_cap;
-        }
+        cudaFree(c->pbuf);
+        cudaFree(c->x32);
+        cudaFree(c->ppart);
+        cudaFree(c->geo);
         c->pbuf = nb;
         c->x32 = nx32;
         c->ppart = npp;
         c->geo = ngeo;
         c->cap = ncap;
-        c->bytes += (size_t)ncap * per_cap;
+        c->bytes += (size_t)(ncap - cap) * per_cap;
     }
     CK(c, cudaMemcpy(c->pbuf, blk.data(), blk.size() * sizeof(double), cudaMemcpyHostToDevice));
     CK(c, cudaMemcpy(c->x32, x32.data(), x32.size() * sizeof(float4), cudaMemcpyHostToDevice));
@@ -657,7 +647,6 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
         c->area += 4.0 * M_PI * std::sqrt((rp * rp * ro * ro * 2.0 + ro * ro * ro * ro) / 3.0);
     }
     bind_parts(c);
-    drop_graphs(c);
     cudaStream_t s = c->stream;
     uint32_t *oo = c->owner[c->ocur], *on = c->owner[1 - c->ocur];
     launch_geom(c->L, c->P, s);

@@ -91,6 +91,57 @@ def test_allocation_failures_keep_nothing():
     assert free0 - _free_bytes() < (8 << 20)
 
 
+def test_failed_add_leaves_a_stepped_lattice_as_it_was():
+    """A lattice of 300 particles with captured graphs of one step and of two
+    (the pair forces by cell lists) whose next add_particles fails at each of
+    its allocations in turn: it steps on like a twin that was never asked, and
+    so it does once the call succeeds on both."""
+    shape = (72, 70, 68)
+    pos, quat = W.place_ellipsoids(shape, 400, 2.5, 2.0, seed=75, margin=0.8)
+    assert len(pos) == 400
+    rho0 = W.random_phases(shape, 0.5, seed=76)
+
+    def make():
+        g = lbe.Lattice(shape, rho0, g_br=0.1, device=0)
+        g.add_particles(pos[:300], quat[:300], 2.5, 2.0, 0.05)
+        g.step(4)
+        for _ in range(24):  # single steps replay a graph after 16
+            g.step(1)
+        return g
+
+    def same(a, b):
+        x, y = a.read_particles(), b.read_particles()
+        return np.array_equal(a.get_populations(), b.get_populations()) and all(np.array_equal(x[k], y[k]) for k in x)
+
+    a, b = make(), make()
+    failures = 0
+    for k in range(12):
+        bytes0 = a.device_bytes()
+        lbe.fail_allocations(k)
+        try:
+            a.add_particles(pos[300:], quat[300:], 2.5, 2.0, 0.05)
+            added = True
+        except lbe.LbeError as e:
+            assert e.status == ENOMEM
+            added = False
+        lbe.fail_allocations(-1)
+        if added:
+            break
+        failures += 1
+        assert a.device_bytes() == bytes0 and a.kernels_per_step() == b.kernels_per_step()
+        for g in (a, b):
+            g.step(2)
+            g.step(1)
+        assert same(a, b), k
+    assert added and failures == 6  # cells (2), state, FP32 copies, pair sums, geometry
+    b.add_particles(pos[300:], quat[300:], 2.5, 2.0, 0.05)
+    for g in (a, b):
+        g.step(5)
+    assert same(a, b)
+    a.close()
+    b.close()
+
+
 def test_server_request_failing_allocation_is_reported():
     w = W.adsorption_request(7, 0, edge_range=(32, 36))
     p = w.particles
