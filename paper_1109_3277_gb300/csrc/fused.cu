@@ -669,7 +669,10 @@ __device__ __forceinline__ bool fused_tile(const Lat &L, const typename S::P *__
         }
     };
 
-    if (tid == 0) {
+    // Barriers only where copies complete on them: a batch's CTA takes tiles of
+    // both kinds, and a barrier left by a tile without copies would lie inside
+    // the stage of the next tile with them.
+    if (TMA && tid == 0) {
 #pragma unroll
         for (int b = 0; b < NST; b++) mbar_init(&bar[b], 1);
         fence_barrier_init();

@@ -129,6 +129,28 @@ def test_odd_steps_and_interleaving_with_member_steps():
     assert _equal(_state(a), _state(b))
 
 
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_batch_mixing_rows_with_and_without_tensor_copies(storage):
+    """Edges 96 (rows of whole 16 bytes: tensor copies) and 81 (none) at tau = 1,
+    with more tiles than the GPU takes at once, so that a CTA goes from tiles
+    of one kind to the other, whose shared memory is laid out differently."""
+    def make():
+        out = []
+        for n in (96, 81):
+            shape = (n, n, n)
+            out.append(lbe.Lattice(shape, W.random_phases(shape, 0.5, seed=n), g_br=0.1, storage=storage))
+        return out
+
+    alone, mixed = make(), make()
+    batch = lbe.Batch(mixed)
+    for g in alone:
+        g.step(9)
+    batch.step(9)
+    for a, b in zip(alone, mixed):
+        assert np.array_equal(a.get_populations(), b.get_populations())
+    batch.close()
+
+
 def test_batch_without_particles():
     a = [_spinodal(), _spinodal()]
     b = [_spinodal(), _spinodal()]
