@@ -1297,7 +1297,9 @@ lbe_status lbe_batch_first_quat(lbe_batch *b, double *quat_out)
 int32_t lbe_batch_kernels_per_step(const lbe_batch *b)
 {
     if (!b) return 0;
-    return b->total_parts > 0 ? 11 : 4;
+    // the queue's reset, the fused kernel and the parity flip; the shell fill
+    // where there are solid nodes; seven particle kernels
+    return 3 + (b->total_parts > 0 || b->total_walls > 0 ? 1 : 0) + (b->total_parts > 0 ? 7 : 0);
 }
 
 void lbe_batch_destroy(lbe_batch *b)

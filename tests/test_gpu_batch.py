@@ -155,12 +155,15 @@ def test_batch_without_particles():
     a = [_spinodal(), _spinodal()]
     b = [_spinodal(), _spinodal()]
     batch = lbe.Batch(b)
-    assert batch.kernels_per_step() == 4
+    assert batch.kernels_per_step() == 3  # queue reset, fused kernel, parity flip
     for g in a:
         g.step(11)
     batch.step(11)
     for x, y in zip(a, b):
         assert _equal(_state(x), _state(y))
+    shape = (24, 20, 16)
+    walled = lbe.Lattice(shape, W.uniform_mixture(shape, 0.7, 0.01, seed=22), walls_z=True, g_br=0.1)
+    assert lbe.Batch([walled]).kernels_per_step() == 4  # and the shell fill of the wall planes
 
 
 def test_autotuners_keep_results_bit_identical():
