@@ -886,7 +886,9 @@ size_t lbe_footprint(const lbe_lattice_desc *d, int32_t nparticles)
         const size_t cap = nparticles < 64 ? 64 : (size_t)nparticles + nparticles / 4;
         b += cap * (PSTRIDE * sizeof(double) + 3 * sizeof(float4) + 6 * sizeof(double) + 2 * sizeof(int) +
                     geom_bytes_per_particle());
-        b += (3 * (N / 8) + 1) * sizeof(int);  // cells (at least 2 nodes a side)
+        size_t cells = 1;  // heads of the pair cells: at least 2 nodes a side, where there are two
+        for (const int k : {d->nx, d->ny, d->nz}) cells *= (size_t)std::max(1, k / 2);
+        b += cells * sizeof(int);
         b += (N + LINK_PAD) * sizeof(uint2) + sizeof(int);  // link list
     }
     return b;

@@ -104,3 +104,16 @@ def test_footprint_arithmetic():
     assert with_p - f16 >= N * 8
     assert lbe.footprint((0, 36, 30)) == 0
     assert lbe.footprint(shape, storage=9) == 0
+
+
+def test_footprint_counts_the_particles_arrays():
+    """What particles add: the link list (8 bytes a node and 65,536 more entries,
+    and its counter), one cell head per 2 nodes along each axis (one along an
+    axis of a single node), and arrays that do not depend on the shape."""
+    from paper_1109_3277_gb300 import lbe
+    fixed = set()
+    for nx, ny, nz in ((40, 36, 30), (41, 37, 31), (1, 64, 64), (1, 1, 500), (1, 1, 1), (3, 2, 5)):
+        cells = max(1, nx // 2) * max(1, ny // 2) * max(1, nz // 2)
+        more = lbe.footprint((nx, ny, nz), 10) - lbe.footprint((nx, ny, nz))
+        fixed.add(more - 8 * (nx * ny * nz + 65536) - 4 - 4 * cells)
+    assert len(fixed) == 1
