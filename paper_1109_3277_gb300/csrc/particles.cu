@@ -30,6 +30,12 @@ struct ShellGrid {
     int nx, ny, nz, tyi, tzi, pad;
 };
 
+// The particles [first, first + parts) whose tiles a launch of the shell fill
+// takes.
+struct ShellRange {
+    int first, parts;
+};
+
 // ---------------------------------------------------------- geometry (FP64)
 // The inside test is written with explicit round-to-nearest intrinsics so
 // that no multiply-add is contracted: the quadric is evaluated in a fixed
@@ -2023,16 +2029,16 @@ __device__ void wall_tile(const Lat &L, int tile, const typename S::P *__restric
     }
 }
 
-// The tiles of all particles, then those of the walls.
+// The tiles of a range of the particles, then those of the walls.
 template <class S, bool DENSE>
 __global__ void __launch_bounds__(PT) k_shell_fill(Lat L, Parts P, ShellGrid sg, const typename S::P *__restrict__ f,
                                                    float *rho, float *__restrict__ psi, const uint8_t *__restrict__ type,
-                                                   const uint32_t *__restrict__ owner, LinkList ll)
+                                                   const uint32_t *__restrict__ owner, LinkList ll, ShellRange range)
 {
     __shared__ ShellTile sm;
-    const int nt = sg.nx * sg.ny * sg.nz, npt = P.n * nt, c = blockIdx.x;
+    const int nt = sg.nx * sg.ny * sg.nz, npt = range.parts * nt, c = blockIdx.x;
     if (c < npt)
-        shell_tile<S, DENSE>(L, P, c / nt, c % nt, sg, f, rho, psi, type, owner, ll, sm);
+        shell_tile<S, DENSE>(L, P, range.first + c / nt, c % nt, sg, f, rho, psi, type, owner, ll, sm);
     else
         wall_tile<S>(L, c - npt, f, psi, type, sm);
 }
@@ -2045,12 +2051,12 @@ __global__ void __launch_bounds__(PT) k_shell_fill(Lat L, Parts P, ShellGrid sg,
 __global__ void k_begin_batch(BatchIndex B) { *B.counter = 0; }
 
 template <class S>
-__global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, int parts)
+__global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, ShellRange range)
 {
     __shared__ ShellTile sm;
     const int nt = sg.nx * sg.ny * sg.nz, c = blockIdx.x;
-    const bool part = c < parts * nt;
-    const int g = part ? c / nt : c - parts * nt;
+    const bool part = c < range.parts * nt;
+    const int g = part ? range.first + c / nt : c - range.parts * nt;
     const int *off = part ? B.part0 : B.wall0;
     const int b = part ? B.pbox[g] : find_box(B.wall0, B.nbox, g);
     const BoxDev &bx = B.box[b];
@@ -2302,23 +2308,45 @@ static ShellGrid lattice_grid(const Lat &L, const Parts &P)
     return shell_grid(ext, P.n);
 }
 
-template <class S, bool DENSE>
-static void shell_fill_launch(unsigned ctas, const Lat &L, const Parts &P, const ShellGrid &g, const void *f, float *rho,
-                              float *psi, const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
+// The launches of a shell fill: every particle has as many tiles as the
+// largest one, whose product with the particles may exceed a grid (a radius
+// of 250 among 240,000 small particles), so the particles go in ranges of
+// SHELL_CTAS tiles at most; the walls' tiles go with the last.
+#ifdef LBE_CHECK
+constexpr int SHELL_CTAS = 32;  // several launches in small cases
+#else
+constexpr int SHELL_CTAS = 1 << 30;
+#endif
+template <class F>
+static void shell_ranges(const ShellGrid &g, int np, int walls, F launch)
 {
-    k_shell_fill<S, DENSE><<<ctas, PT, 0, s>>>(L, P, g, (const typename S::P *)f, rho, psi, type, owner, ll);
+    const int nt = g.nx * g.ny * g.nz, most = std::max(1, SHELL_CTAS / std::max(nt, 1));
+    int first = 0;
+    do {
+        const int parts = std::min(np - first, most);
+        const unsigned ctas = (unsigned)(parts * nt + (first + parts == np ? walls : 0));
+        if (ctas) launch(ctas, ShellRange{first, parts});
+        first += parts;
+    } while (first < np);
+}
+
+template <class S, bool DENSE>
+static void shell_fill_launch(const Lat &L, const Parts &P, const ShellGrid &g, const void *f, float *rho, float *psi,
+                              const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
+{
+    shell_ranges(g, P.n, wall_tiles(L), [&](unsigned ctas, ShellRange range) {
+        k_shell_fill<S, DENSE><<<ctas, PT, 0, s>>>(L, P, g, (const typename S::P *)f, rho, psi, type, owner, ll, range);
+    });
 }
 
 void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
                        const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
 {
     const ShellGrid g = P.n > 0 ? lattice_grid(L, P) : ShellGrid{0, 0, 0, 1, 1, 1};
-    const long long ctas = (long long)P.n * g.nx * g.ny * g.nz + wall_tiles(L);
-    if (ctas == 0) return;
     if (dense)
-        LBE_DISPATCH(storage, (shell_fill_launch<S, true>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
+        LBE_DISPATCH(storage, (shell_fill_launch<S, true>(L, P, g, f, rho, psi, type, owner, ll, s)));
     else
-        LBE_DISPATCH(storage, (shell_fill_launch<S, false>((unsigned)ctas, L, P, g, f, rho, psi, type, owner, ll, s)));
+        LBE_DISPATCH(storage, (shell_fill_launch<S, false>(L, P, g, f, rho, psi, type, owner, ll, s)));
 }
 
 void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,
@@ -2346,9 +2374,9 @@ void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int 
                         cudaStream_t s)
 {
     const ShellGrid g = total_parts > 0 ? shell_grid(ext, total_parts) : ShellGrid{0, 0, 0, 1, 1, 1};
-    const long long ctas = (long long)total_parts * g.nx * g.ny * g.nz + total_walls;
-    if (ctas == 0) return;
-    LBE_DISPATCH(storage, (k_shell_batch<S><<<(unsigned)ctas, PT, 0, s>>>(B, g, total_parts)));
+    shell_ranges(g, total_parts, total_walls, [&](unsigned ctas, ShellRange range) {
+        LBE_DISPATCH(storage, (k_shell_batch<S><<<ctas, PT, 0, s>>>(B, g, range)));
+    });
 }
 
 void batch_shell_extent(const Lat &L, const Parts &P, int ext[3])

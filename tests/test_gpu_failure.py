@@ -195,3 +195,51 @@ def test_bounds_checked_build_runs_clean():
                        timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
     assert "checked build ok" in r.stdout
+
+
+SPLIT_RUN = r"""
+import numpy as np
+import paper_1109_3277_gb300.lbe as lbe
+from oracle import lbref
+from paper_1109_3277_gb300 import workloads as W
+pairs = []
+for shape in ((40, 38, 36), (26, 24, 22)):
+    pos, quat = W.place_ellipsoids(shape, 6, 3.2, 2.0, seed=77, margin=1.0, periodic=(True, True, False))
+    assert len(pos) == 6
+    kw = dict(walls_z=True, g_br=0.1, rho_ref=(0.37, 0.37))
+    rho0 = W.random_phases(shape, 0.5, seed=78)
+    vel = W.uniform(79, (6, 3), lo=-0.05, hi=0.05)
+    for n in range(2):  # alone and in a batch
+        g = lbe.Lattice(shape, rho0, device=0, particle_mode="prescribed", **kw)
+        r = lbref.Lattice(shape, rho0, particle_mode=2, **kw)
+        for L in (g, r):
+            L.add_particles(pos, quat, np.full(6, 3.2), np.full(6, 2.0), np.full(6, 0.05), vel=vel)
+        pairs.append((g, r))
+batch = lbe.Batch([pairs[1][0], pairs[3][0]])
+pairs[0][0].step(12)
+pairs[2][0].step(12)
+batch.step(12)
+for g, r in pairs:
+    r.step(12)
+    rg, _, tg = g.read_fields()
+    rr, _, tr = r.read_fields()
+    assert np.array_equal(tg, tr)
+    assert np.max(np.abs(rg - rr)) < 1e-5
+    # about 300 links a particle, each 2 f of a density that is off by 1e-5 at most
+    # (f <= rho / 18): 300 * 2 * 1e-5 / 18
+    pg, pr = g.read_particles(), r.read_particles()
+    assert np.max(np.abs(pg["force"] - pr["force"])) < 3.4e-4
+print("split shell fill ok")
+"""
+
+
+def test_shell_fill_in_several_launches():
+    """The checked build takes 32 tiles of the particles' boxes per launch of
+    the shell fill (the regular one 2^30): 6 particles of 12 tiles each and the
+    walls, alone (densities from the density pass, and summed in place) and in a
+    batch, against the oracle."""
+    from paper_1109_3277_gb300 import build as b
+    env = dict(os.environ, LBE_LIB=b.build(check=True))
+    r = subprocess.run([sys.executable, "-c", SPLIT_RUN], cwd=ROOT, env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert "split shell fill ok" in r.stdout
