@@ -99,8 +99,8 @@ void drop_graphs(lbe_ctx *c)
 // Field offsets inside the particle buffer (doubles per particle).
 // Those that lbe_read_particles returns (NREAD of them) come first.
 enum { OX = 0, OQ = 3, OV = 7, OW = 10, OF = 13, OT = 16, NREAD = 19,
-       OXO = 19, OQO = 22, ORP = 26, ORO = 27, ODR = 28, OM = 29, OIP = 30, OIQ = 31, OFL = 32, OTL = 35,
-       OFP = 38, OTP = 41, OFE = 44, OTE = 47, OFX = 50, PSTRIDE = 56 };
+       OXO = 19, ORP = 22, ORO = 23, ODR = 24, OM = 25, OIP = 26, OIQ = 27, OFL = 28, OTL = 31,
+       OFP = 34, OTP = 37, OFE = 40, OTE = 43, OFX = 46, PSTRIDE = 52 };
 
 void bind_parts(lbe_ctx *c)
 {
@@ -116,7 +116,6 @@ void bind_parts(lbe_ctx *c)
     P.V = at(OV);
     P.W = at(OW);
     P.Xold = at(OXO);
-    P.qold = at(OQO);
     P.rp = at(ORP);
     P.ro = at(ORO);
     P.drho = at(ODR);
@@ -524,7 +523,7 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
     }
     lbe_status st = sync(c, "add_particles");
     if (st != LBE_OK) return st;
-    static const int FIELDS[][2] = {{OX, 3},  {OQ, 4},  {OV, 3},  {OW, 3},  {OXO, 3}, {OQO, 4}, {ORP, 1},
+    static const int FIELDS[][2] = {{OX, 3},  {OQ, 4},  {OV, 3},  {OW, 3},  {OXO, 3}, {ORP, 1},
                                     {ORO, 1}, {ODR, 1}, {OM, 1},  {OIP, 1}, {OIQ, 1}, {OFL, 3}, {OTL, 3},
                                     {OFP, 3}, {OTP, 3}, {OFE, 3}, {OTE, 3}, {OF, 3},  {OT, 3},
                                     {OFX, 6}};
@@ -565,11 +564,9 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
         blk[OIP * cp + p] = 0.4 * M * ro * ro;
         blk[OIQ * cp + p] = 0.2 * M * (rp * rp + ro * ro);
     }
-    // placement does not move anything: old geometry = current geometry
-    for (int p = 0; p < np; p++) {
+    // placement does not move anything: old centre = current centre
+    for (int p = 0; p < np; p++)
         for (int j = 0; j < 3; j++) blk[OXO * cp + 3 * p + j] = blk[OX * cp + 3 * p + j];
-        for (int j = 0; j < 4; j++) blk[OQO * cp + 4 * p + j] = blk[OQ * cp + 4 * p + j];
-    }
     // FP32 copies: [0, ncap) position and reach, then velocity and ω pairs
     std::vector<float4> x32((size_t)3 * ncap, make_float4(0.f, 0.f, 0.f, 0.f));
     for (int p = 0; p < np; p++) {

@@ -228,7 +228,7 @@ __device__ __forceinline__ bool idx_ok(const Lat &, long long, long long, int) {
 struct Parts {
     int n;
     double *X, *q, *V, *W;          // position [3n], quaternion [4n], velocity, ω (lab)
-    double *Xold, *qold;            // geometry before the last update
+    double *Xold;                   // centre before the last update
     double *rp, *ro, *drho;         // radii, colour Δρ
     double *M, *Ipar, *Iperp;       // mass and body-frame inertia
     double *Flink, *Tlink;          // momentum exchange of the current step

@@ -1316,7 +1316,6 @@ __device__ __forceinline__ void integrate_quad(const Lat &L, const Parts &P, int
         P.Tlink[e] = 0.0;
         P.Xold[e] = X;
     }
-    if (act) P.qold[4 * p + lane] = qc;
 #pragma unroll
     for (int j = 0; j < 4; j++) q[j] = quad(qc, j);
     if (__all_sync(0xffffffffu, mode == LBE_PARTICLES_STATIC)) return;
