@@ -219,6 +219,13 @@ LBE_API lbe_status lbe_set_zchunk(lbe_ctx *c, int32_t zc);
 LBE_API lbe_status lbe_set_tile(lbe_ctx *c, int32_t rows, int32_t zc);
 LBE_API lbe_status lbe_get_tile(const lbe_ctx *c, int32_t *rows, int32_t *zc);
 
+/* How the shell fill divides the particles' boxes (for tests): tiles of 30 x
+ * rows[0] x rows[1] nodes, *tiles of them for every particle (all 0 without
+ * particles and with LBE_FLAG_TWO_PASS), and whether it takes the densities
+ * next to the particles from the density pass (*dense = 1) or sums them
+ * itself (0).  Results do not depend on either. */
+LBE_API lbe_status lbe_get_shell_tiles(const lbe_ctx *c, int32_t rows[2], int32_t *tiles, int32_t *dense);
+
 /* Failure detection of the fused kernel's copies: every wait for a plane's
  * box copy gives up after a bounded number of tries (a non-blocking look,
  * then about 2^22 tries by default, each of which may suspend the thread

@@ -1000,6 +1000,16 @@ lbe_status lbe_get_tile(const lbe_ctx *c, int32_t *rows, int32_t *zc)
     return LBE_OK;
 }
 
+lbe_status lbe_get_shell_tiles(const lbe_ctx *c, int32_t rows[2], int32_t *tiles, int32_t *dense)
+{
+    if (!c || !rows || !tiles || !dense) return LBE_EINVAL;
+    rows[0] = rows[1] = *tiles = *dense = 0;
+    if (c->np == 0 || (c->d.flags & LBE_FLAG_TWO_PASS)) return LBE_OK;
+    shell_tiles(c->L, c->P.rmax, c->np, rows, tiles);
+    *dense = fused_self(c) ? 0 : 1;
+    return LBE_OK;
+}
+
 void lbe_fail_allocations(int32_t after) { g_alloc_left.store(after < 0 ? -1 : after); }
 
 lbe_status lbe_set_wait_limit(lbe_ctx *c, int32_t tries, int32_t unreachable)

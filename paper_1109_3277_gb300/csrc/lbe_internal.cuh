@@ -450,6 +450,9 @@ __device__ __forceinline__ int find_box(const int *off, int nbox, int i)
 // rho for the link kernel.  No launch without particles and walls.
 void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
                        const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s);
+// Its tiles for np particles of radii up to rmax: rows along y and z, and
+// how many for every particle.
+void shell_tiles(const Lat &L, float rmax, int np, int rows[2], int *tiles);
 void launch_links(int storage, const Lat &L, const Parts &P, void *fnew, const float *rho,
                   const uint8_t *type, const uint32_t *owner, cudaStream_t s);
 void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho, const uint32_t *owner,

@@ -2300,11 +2300,19 @@ static void shell_extent(const Lat &L, double rmax, int ext[3])
     for (int k = 0; k < 3; k++) ext[k] = std::max(ext[k], e < n[k] ? (int)e : n[k]);
 }
 
-static ShellGrid lattice_grid(const Lat &L, const Parts &P)
+static ShellGrid lattice_grid(const Lat &L, float rmax, int np)
 {
     int ext[3] = {1, 1, 1};
-    shell_extent(L, P.rmax, ext);
-    return shell_grid(ext, P.n);
+    shell_extent(L, rmax, ext);
+    return shell_grid(ext, np);
+}
+
+void shell_tiles(const Lat &L, float rmax, int np, int rows[2], int *tiles)
+{
+    const ShellGrid g = lattice_grid(L, rmax, np);
+    rows[0] = g.tyi;
+    rows[1] = g.tzi;
+    *tiles = g.nx * g.ny * g.nz;
 }
 
 // The launches of a shell fill: every particle has as many tiles as the
@@ -2341,7 +2349,7 @@ static void shell_fill_launch(const Lat &L, const Parts &P, const ShellGrid &g, 
 void launch_shell_fill(int storage, const Lat &L, const Parts &P, bool dense, const void *f, float *rho, float *psi,
                        const uint8_t *type, const uint32_t *owner, const LinkList &ll, cudaStream_t s)
 {
-    const ShellGrid g = P.n > 0 ? lattice_grid(L, P) : ShellGrid{0, 0, 0, 1, 1, 1};
+    const ShellGrid g = P.n > 0 ? lattice_grid(L, P.rmax, P.n) : ShellGrid{0, 0, 0, 1, 1, 1};
     if (dense)
         LBE_DISPATCH(storage, (shell_fill_launch<S, true>(L, P, g, f, rho, psi, type, owner, ll, s)));
     else
@@ -2354,7 +2362,7 @@ void launch_link(int storage, const Lat &L, const LinkList &ll, const float *rho
     if (P.n == 0 || !ll.ent) return;
     int blocks = (L.N + 255) / 256;
     if (blocks > 8 * 152) blocks = 8 * 152;
-    const int group = lattice_grid(L, P).pad == 8 ? 8 : 32;
+    const int group = lattice_grid(L, P.rmax, P.n).pad == 8 ? 8 : 32;
     LBE_DISPATCH(storage, (k_link<S><<<blocks, 256, 0, s>>>(L, ll, rho, owner, P, (typename S::P *)fout, group)));
 }
 

@@ -71,6 +71,8 @@ SIGNATURES = {
     "lbe_set_zchunk": (ctypes.c_int, [_P, ctypes.c_int32]),
     "lbe_set_tile": (ctypes.c_int, [_P, ctypes.c_int32, ctypes.c_int32]),
     "lbe_get_tile": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
+    "lbe_get_shell_tiles": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32),
+                                           ctypes.POINTER(ctypes.c_int32)]),
     "lbe_set_wait_limit": (ctypes.c_int, [_P, ctypes.c_int32, ctypes.c_int32]),
     "lbe_fail_allocations": (None, [ctypes.c_int32]),
     "lbe_batch_create": (ctypes.c_int, [ctypes.POINTER(_P), ctypes.c_int32, ctypes.POINTER(_P)]),
@@ -249,6 +251,13 @@ class Lattice:
         r, z = ctypes.c_int32(), ctypes.c_int32()
         self._check(load().lbe_get_tile(self._ptr, ctypes.byref(r), ctypes.byref(z)), "get_tile")
         return r.value, z.value
+
+    def shell_tiles(self):
+        """(rows along y, rows along z, tiles per particle, whether the densities
+        come from the density pass) of the shell fill."""
+        rows, n, dense = (ctypes.c_int32 * 2)(), ctypes.c_int32(), ctypes.c_int32()
+        self._check(load().lbe_get_shell_tiles(self._ptr, rows, ctypes.byref(n), ctypes.byref(dense)), "get_shell_tiles")
+        return rows[0], rows[1], n.value, bool(dense.value)
 
     def set_wait_limit(self, tries, unreachable=False):
         """Tries of each bounded wait for a box copy (0: the default);

@@ -99,10 +99,10 @@ def test_static_particle_one_step():
 
 
 def test_large_particle_links_beyond_the_shell_buffer():
-    """A sphere of radius 14 has about 3,000 shell nodes, more than the
-    shell kernel collects per particle in shared memory (1,024): the rest
-    enter the link list directly.  One step of a moving static sphere
-    against the oracle: populations, and the momentum exchange."""
+    """A sphere of radius 14 has about 3,000 shell nodes, spread over many
+    small tiles of its box, whose segments of the link list are shared out
+    in groups of 8.  One step of a moving static sphere against the
+    oracle: populations, and the momentum exchange."""
     shape = (40, 40, 40)
     f0 = W.random_populations(shape, seed=29)
     g, r = _pair(shape, np.full((2, 40, 40, 40), 0.5), g_br=0.1, particle_mode="static")
