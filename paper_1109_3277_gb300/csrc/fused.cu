@@ -57,9 +57,11 @@ __device__ __forceinline__ int wrapc(int v, int n)
 }
 
 // Compile-time layout of one configuration: storage S, tile rows TY, GEN
-// (any τ) or not (τ = 1), and SELF (the box holds
+// (any τ) or not (τ = 1), SELF (the box holds
 // the tile and a one-node halo, whose densities the kernel forms itself) or
-// not (the box holds the tile; ψ of every ring entry comes from memory).
+// not (the box holds the tile; ψ of every ring entry comes from memory), and
+// TMA (boxes arrive by tensor copies) or not (no stage: entries are read from
+// global memory).
 template <class S, int TY, bool GEN, bool SELF, bool TMA>
 struct Cfg {
     using P = typename S::P;
@@ -932,10 +934,14 @@ __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
 
 // Persistent multi-lattice variant: CTAs take tiles of all boxes of a batch
 // from one queue (largest boxes first in the queue order set by the host);
-// the first tile of a CTA is its own index.  ψ is formed on chip: a batch's
-// boxes hold few particles each.  GEN: some box needs any τ or
-// 64-bit offsets (it stores exactly what the τ = 1 configuration stores: τ =
-// 1 takes f^eq in the relaxation); otherwise all are τ = 1 with 32-bit offsets.
+// the first tile of a CTA is its own index.  ψ is formed on chip in every
+// box, also in those whose particles cover so much that the lattice alone would
+// run the density pass: with a pass and a sweep for the shell over all boxes,
+// four of 64^3 with 10 % ellipsoids (f16) took 1,594 us a step, two of 128^3 with
+// 14 % 10,376; now 320 and 1,101 (links and coverage changed as well).  GEN: some
+// box needs any τ or 64-bit offsets (it stores exactly what the τ = 1
+// configuration stores: τ = 1 takes f^eq in the relaxation); otherwise all are
+// τ = 1 with 32-bit offsets.
 template <class S, bool GEN>
 constexpr int BATCH_TY = fused_batch_rows(sizeof(typename S::T) == 4 ? LBE_STORE_F32 : LBE_STORE_F16_OFS, GEN);
 
@@ -997,11 +1003,16 @@ int fused_zchunk(const Lat &L, int ty, int es, bool self, double share)
     // lattice gets) keeps small lattices from leaving SMs idle, e.g. 64^3: 4
     // planes 25 us, 16 planes 53.  With ψ formed on chip, chunks of more than
     // 8 planes (FP32: 4) let the halo rows of the next chunk and the next
-    // rows of tiles leave L2 before they are read again: 256^3 f16 598 us at
-    // 8 planes, 652 at 16, 805 at 48; f32 964 at 4, 1095 at 16.  With any
-    // τ at 16 bit, whose collision takes longer, the halo planes that longer
-    // chunks save are worth more: 256^3 f16 676 at 12 against 710 at 8 and 688
-    // at 16.  With ψ from memory (256^3 bijel, f16) 564 at 16, 601 at 64.
+    // rows of tiles leave L2 before they are read again.  The cap follows the
+    // kernel, hardly the plane: with 4 rows and no solid nodes f32 384^2 x 128
+    // takes 976 us at 5 planes and 1,436 at 16, 256^3 909 and 1,260, 192^3 383
+    // and 523, 128^3 130 and 160 (best 128, at 3); f16 256^3 516 at 6, 632 at 16,
+    // 128^3 79 and 95.  64^2 x 256 would gain from longer chunks (f32 75 at 5, 62
+    // at 12; f16 48 at 5, 45 at 12).  With any τ at 16 bit, whose collision takes
+    // longer, the halo planes that longer chunks save are worth more: 256^3 601
+    // at 12, 620 at 8, 609 at 16; in FP32 256^3 takes 1,054 at 4, 1,031 at 6 and
+    // 1,078 at 16, but 384^2 x 128 1,271 at 4 and 1,133 at 12.  With ψ from memory
+    // (256^3 bijel, f16) 564 at 16, 601 at 64.
     const long long cols = (long long)((L.nx + TX - 1) / TX) * ((L.ny + ty - 1) / ty);
     const bool tma = (L.nx * 2 * es) % 16 == 0;
     const bool gen = !(fused_tau1(L) && fused_rel32(L));

@@ -225,7 +225,12 @@ __global__ void k_set_types(Lat L, uint8_t *type)
 // us for 1.4 M of them), so the pass wins as soon as those are more than a
 // few percent of the lattice: 15 % oblate particles in 256^3 (f16) 786 + 100
 // us with the pass, 728 + 479 without.  Below, it saves the pass and a launch
-// (a single particle in 64^3 f32: 9 us of 55).
+// (a single particle in 64^3 f32: 9 us of 55).  Whole steps with ellipsoids
+// (8, 4), on chip against the pass, at 0.5, 1 and 2 times the line: 16 bit
+// 256^3 808 / 845, 909 / 894, 1132 / 1014 us, 384^3 2442 / 2619, 2752 / 2799, 3437
+// / 3163, 128^3 equal at 0.6 times.  FP32, whose pass reads twice the bytes,
+// crosses later: 128^3 at 1.4 times (222 / 229 at the line), 256^3 beyond 2
+// (1254 / 1405 and 1512 / 1538).
 bool fused_self(const lbe_ctx *c) { return 50.0 * c->area < (double)c->L.N; }
 
 // Tensor map of buffer `buf` for the fused kernel's mode and tile height
@@ -640,7 +645,8 @@ lbe_status lbe_add_particles(lbe_ctx *c, int32_t n, const double *pos, const dou
     for (int p = 0; p < np; p++) {
         const double rp = blk[ORP * cp + p], ro = blk[ORO * cp + p];
         c->rmax = std::fmax(c->rmax, std::fmax(rp, ro));
-        // mean of the squared radii of the three axes (at least the area)
+        // 4 pi times the root mean square of the products of two of the three
+        // semi-axes: at least the area
         c->area += 4.0 * M_PI * std::sqrt((rp * rp * ro * ro * 2.0 + ro * ro * ro * ro) / 3.0);
     }
     bind_parts(c);
@@ -669,8 +675,10 @@ lbe_status lbe_step(lbe_ctx *c, int32_t nsteps)
     constexpr int CAPTURE_AFTER = 16;
     // Branches pay while the kernels leave room on the GPU: 77 x 53 x 61 with 40
     // particles 111 -> 87 us a step, 150 x 141 x 133 with 525 519 -> 459, 256^3
-    // 1,300 -> 1,285, but 512^3 8.9 -> 9.0 ms; a graph of a single step launches
-    // more slowly with them (87 -> 90 us with its read).
+    // 1,300 -> 1,285, but 512^3 8.9 -> 9.0 ms.  From 192^3 to 448^3 (10 %
+    // ellipsoids, 16 bit and FP32) they are worth 0 to 0.7 %, so the line may lie
+    // anywhere there.  A graph of a single step launches more slowly with them
+    // (87 -> 90 us with its read).
     constexpr int BRANCH_MAX = 1 << 25;
     auto replay = [&](int steps, int times) -> lbe_status {
         const int key = c->cur * 2 + c->ocur;

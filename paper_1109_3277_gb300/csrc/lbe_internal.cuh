@@ -252,7 +252,7 @@ struct Parts {
 constexpr int LINK_PAD = 65536;
 struct LinkList {
     uint2 *ent;   // [cap]
-    int *count;   // entries this step (reset before the density kernel)
+    int *count;   // entries this step (set to 0 by the particles' update, or the end of a batched step)
     int cap;
 };
 

@@ -356,10 +356,11 @@ __device__ __forceinline__ void for_box(const Box &b, F f)
 }
 
 // ---- coverage geometry ----------------------------------------------------
-// The geometry the coverage kernels need of a particle, computed once per
-// step by one thread per particle (k_geom) instead of by every CTA: the
-// rotation and inverse squared radii, the centre the box was formed around
-// with its integer and FP32 parts, and the box.
+// The geometry the coverage kernels and the shell fill need of a particle,
+// computed once per update by the particle's four lanes (in the update's
+// kernel; at placement and in batches in one of its own) instead of by every
+// CTA: the rotation and inverse squared radii, the centre the box was formed
+// around with its integer and FP32 parts, and the box.
 struct PGeom {
     Geo g;
     double X[3];
@@ -939,7 +940,10 @@ __global__ void __launch_bounds__(256) k_link(Lat L, LinkList ll, const float *r
     link_list<S>(L, ll, rho, owner, P, fout, group, w[threadIdx.x >> 5]);
 }
 
-// Batched: blockIdx.y is the box; LINK_BATCH_CTAS CTAs per box.
+// Batched: blockIdx.y is the box; LINK_BATCH_CTAS CTAs per box.  With 4, 8, 16
+// and 32 a step of 7 boxes of one sphere (48 x 48 x 40 f32) takes 135, 131, 131
+// and 131 us, of 64 boxes of 32^3 307, 306, 311 and 314; only boxes of many
+// particles would gain from more (four of 96^3 with 100 each: 558, 461, 409, 394).
 constexpr int LINK_BATCH_CTAS = 8;
 
 template <class S>
@@ -1464,7 +1468,6 @@ __global__ void __launch_bounds__(PT_WIDE) k_claim(Lat L, Parts P, uint32_t *__r
 //    neighbours fluid before and after (ρ_ref if none); the particle loses
 //    that momentum;  both through the pending force/torque.
 // With placement != 0 (particles just added) nodes only change type.
-
 //
 // A node whose owner changes with p the lower of the two owners is inside
 // the particle's old ellipsoid or its new one but not both, so it lies in
@@ -1707,7 +1710,8 @@ __global__ void __launch_bounds__(PT_WIDE) k_reset(Lat L, Parts P, int use_old, 
 // pass but gathers 19 scattered 32-byte sectors per node (about 450 nodes per
 // (8, 4, 4) ellipsoid): at 15 % oblate ellipsoids in 256^3 (f16) that was 1.5
 // GB of DRAM traffic, more than the 1.3 GB of the pass, and 479 us against
-// the pass's 225; it pays where particles are few (dense_rho).
+// the pass's 225; it pays where particles are few (the host decides by their
+// surface, fused_self).
 //
 // Tiles: with many particles 22 x 22 rows (an ellipsoid of reach 8 is one
 // tile); with few, 10 x 5 rows, and with fewer than 64 such tiles 8 x 2, so
