@@ -1261,8 +1261,7 @@ lbe_status lbe_batch_autotune(lbe_batch *b, int32_t *chosen_ctas_per_sm)
     for (lbe_ctx *c : b->members)
         if (cudaStreamSynchronize(c->stream) != cudaSuccess) return LBE_ECUDA;
     // Persistent CTAs per SM for the batched fused kernel, timed on the
-    // fused kernel alone (it writes only the spare buffers; the link sums it
-    // accumulates are cleared afterwards).
+    // fused kernel alone, which writes only the spare buffers.
     const int maxc = fused_batch_ctas_per_sm(b->storage, b->general);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -1286,8 +1285,6 @@ lbe_status lbe_batch_autotune(lbe_batch *b, int32_t *chosen_ctas_per_sm)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    for (lbe_ctx *c : b->members)
-        if (c->np > 0) cudaMemsetAsync(c->P.fix, 0, (size_t)6 * c->np * sizeof(unsigned long long), b->stream);
     b->ctas_per_sm = best_c;
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
