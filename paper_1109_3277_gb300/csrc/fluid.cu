@@ -2,6 +2,8 @@
 // arXiv:1109.3277): moments, ψ, outer-shell fill with the colour rule,
 // Shan–Chen force (Eq. 3), shifted-velocity BGK collision (Eq. 2) and
 // streaming (Eq. 1) with halfway bounce-back, plus readers and mass sums.
+#include <algorithm>
+
 #include "lbe_internal.cuh"
 
 namespace lbe {
@@ -100,16 +102,37 @@ __global__ void __launch_bounds__(256) k_moments(Lat L, const typename S::P *__r
 // components of a direction.
 
 template <class S>
+__device__ __forceinline__ void rho_node(const Lat &L, const typename S::P *__restrict__ f,
+                                         const uint8_t *__restrict__ type, float *__restrict__ rho,
+                                         float *__restrict__ psi, long long n)
+{
+    if (type[n] != FLUID) return;
+    const float2 r = node_rho2<S>(f, L, n);
+    st_pair(rho, n, r);
+    psi[n] = 1.f - expf(-r.x);
+    psi[(size_t)L.N + n] = 1.f - expf(-r.y);
+}
+
+template <class S>
 __global__ void __launch_bounds__(256) k_rho(Lat L, const typename S::P *__restrict__ f,
                                              const uint8_t *__restrict__ type, float *__restrict__ rho,
                                              float *__restrict__ psi)
 {
     const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (n >= L.N || type[n] != FLUID) return;
-    const float2 r = node_rho2<S>(f, L, n);
-    st_pair(rho, n, r);
-    psi[n] = 1.f - expf(-r.x);
-    psi[(size_t)L.N + n] = 1.f - expf(-r.y);
+    if (n < L.N) rho_node<S>(L, f, type, rho, psi, n);
+}
+
+// All boxes of a batch: blockIdx.y is the box.  As the first kernel of the step
+// it also empties the fused kernel's tile queue.
+template <class S>
+__global__ void __launch_bounds__(256) k_rho_batch(BatchIndex B)
+{
+    const int b = blockIdx.y;
+    if (blockIdx.x == 0 && b == 0 && threadIdx.x == 0) *B.counter = 0;
+    const BoxDev &bx = B.box[b];
+    const typename S::P *f = (const typename S::P *)bx.f[B.par[2 * b]];
+    for (long long n = blockIdx.x * 256ll + threadIdx.x; n < bx.L.N; n += gridDim.x * 256ll)
+        rho_node<S>(bx.L, f, bx.type, bx.rho, bx.psi, n);
 }
 
 // Neighbour indexing on a 3D grid (x per thread, one y row and z plane per
@@ -470,6 +493,12 @@ void launch_rho(int storage, const Lat &L, const void *f, const uint8_t *type, f
 {
     LBE_DISPATCH(storage,
                  (k_rho<S><<<blocks_for(L.N, 256), 256, 0, s>>>(L, (const typename S::P *)f, type, rho, psi)));
+}
+
+void launch_rho_batch(const BatchIndex &B, int nodes_max, cudaStream_t s)
+{
+    const unsigned x = std::min((nodes_max - 1) / 256 + 1, 8 * 152);
+    k_rho_batch<StF32><<<dim3(x, B.nbox), 256, 0, s>>>(B);
 }
 
 void launch_shell(const Lat &L, const float *rho, float *psi, const uint8_t *type, const uint32_t *owner,

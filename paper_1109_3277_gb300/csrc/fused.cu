@@ -10,15 +10,15 @@
 // per-row bitmask of solid nodes of the tile and a one-node halo go into a
 // four-slot ring of planes; the collision of plane z reads planes z-1, z
 // and z+1 of it.  Two configurations fill the ring:
-//  - ψ formed on chip (lattices with no or few particles, batches): the box
-//    also holds a one-node halo (x widened to 16-byte boundaries), and each
+//  - ψ formed on chip (lattices with no or few particles, batches but those of
+//    any τ in FP32): the box also holds a one-node halo (x widened to 16-byte boundaries), and each
 //    thread sums the densities of its node and of at most one halo node, so ψ
 //    of the tile and its halo comes from the stage; halo nodes beyond the
 //    lattice edge wrap around and are read from global memory.  Solid nodes
 //    take their ψ from the shell fill; a variant for lattices without any
 //    has neither types nor masks.
-//  - ψ from memory (lattices with many particles): the density pass and the
-//    shell fill have written ψ of every node a fluid node sees.  The ring
+//  - ψ from memory (lattices with many particles, FP32 batches of any τ): the
+//    density pass and the shell fill have written ψ of every node a fluid node sees.  The ring
 //    entries of plane z + 2 arrive by asynchronous copies issued before the
 //    collision of plane z and waited for after it.
 //
@@ -934,9 +934,9 @@ __global__ void __launch_bounds__(TX *TY, (Cfg<S, TY, GEN, SELF, TMA>::CTAS))
 
 // Persistent multi-lattice variant: CTAs take tiles of all boxes of a batch
 // from one queue (largest boxes first in the queue order set by the host);
-// the first tile of a CTA is its own index.  ψ is formed on chip in every
-// box, also in those whose particles cover so much that the lattice alone would
-// run the density pass: with a pass and a sweep for the shell over all boxes,
+// the first tile of a CTA is its own index.  ψ is formed on chip but for the
+// general kernel in FP32 (fused_batch_self), also in boxes whose particles cover
+// so much that the lattice alone would run the density pass: with a pass and a sweep for the shell over all boxes,
 // four of 64^3 with 10 % ellipsoids (f16) took 1,594 us a step, two of 128^3 with
 // 14 % 10,376; now 320 and 1,101 (links and coverage changed as well).  GEN: some
 // box needs any τ or 64-bit offsets (it stores exactly what the τ = 1
@@ -946,10 +946,15 @@ template <class S, bool GEN>
 constexpr int BATCH_TY = fused_batch_rows(sizeof(typename S::T) == 4 ? LBE_STORE_F32 : LBE_STORE_F16_OFS, GEN);
 
 template <class S, bool GEN>
-__global__ void __launch_bounds__(TX *BATCH_TY<S, GEN>, (Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::CTAS))
-    k_fused_batch(BatchIndex B, int total)
+constexpr bool BATCH_SELF = fused_batch_self(sizeof(typename S::T) == 4 ? LBE_STORE_F32 : LBE_STORE_F16_OFS, GEN);
+template <class S, bool GEN>
+using BatchCfg = Cfg<S, BATCH_TY<S, GEN>, GEN, BATCH_SELF<S, GEN>, true>;
+
+template <class S, bool GEN>
+__global__ void __launch_bounds__(TX *BATCH_TY<S, GEN>, (BatchCfg<S, GEN>::CTAS)) k_fused_batch(BatchIndex B, int total)
 {
     constexpr int TY = BATCH_TY<S, GEN>, NT = TX * TY;
+    constexpr bool SELF = BATCH_SELF<S, GEN>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = align128(smem_raw);
     __shared__ int s_tile;
@@ -970,10 +975,10 @@ __global__ void __launch_bounds__(TX *BATCH_TY<S, GEN>, (Cfg<S, BATCH_TY<S, GEN>
         using P = typename S::P;
         bool ok;
         if (sb.tma)
-            ok = fused_tile<S, TY, GEN, true, true, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
+            ok = fused_tile<S, TY, GEN, SELF, true, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi, sb.type,
                                                           sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         else
-            ok = fused_tile<S, TY, GEN, true, false, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
+            ok = fused_tile<S, TY, GEN, SELF, false, !GEN, true>(sb.L, (const P *)sb.f[cur], (P *)sb.f[1 - cur], sb.psi,
                                                            sb.type, sb.zc, sb.ofs, tm, bx, by, bz, WAIT_LIMIT, smem);
         if (!ok) break;
         __syncthreads();
@@ -1197,7 +1202,7 @@ static void batch_configure()
     static bool configured = false;  // the attribute is per function and process
     if (!configured) {
         cudaFuncSetAttribute(k_fused_batch<S, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::bytes);
+                             (int)BatchCfg<S, GEN>::bytes);
         configured = true;
     }
 }
@@ -1205,7 +1210,7 @@ static void batch_configure()
 template <class S, bool GEN>
 static void launch_fused_batch_t(const BatchIndex &B, int total, int ctas, cudaStream_t s)
 {
-    using C = Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>;
+    using C = BatchCfg<S, GEN>;
     batch_configure<S, GEN>();
     k_fused_batch<S, GEN><<<ctas < total ? ctas : total, C::NT, C::bytes, s>>>(B, total);
 }
@@ -1219,7 +1224,7 @@ static int batch_occupancy()
     int n = 0;
     batch_configure<S, GEN>();
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused_batch<S, GEN>, TX * BATCH_TY<S, GEN>,
-                                                  Cfg<S, BATCH_TY<S, GEN>, GEN, true, true>::bytes);
+                                                  BatchCfg<S, GEN>::bytes);
     return n > 0 ? n : 1;
 }
 

@@ -1050,6 +1050,8 @@ struct lbe_batch {
     int total_tiles = 0, total_parts = 0, total_walls = 0;
     int ext[3] = {1, 1, 1};           // bound of the particle boxes
     bool general = false;             // some member is not τ = 1 with 32-bit offsets
+    bool dense = false;               // ψ from memory (fused_batch_self)
+    int nodes_max = 0;                // nodes of the largest box
     int ctas_per_sm = 0;
     cudaGraphExec_t graph = nullptr;
     std::string err;
@@ -1060,8 +1062,11 @@ namespace {
 void batch_enqueue_step(lbe_batch *b)
 {
     cudaStream_t s = b->stream;
-    launch_begin_batch(b->idx, s);
-    launch_shell_batch(b->storage, b->idx, b->ext, b->total_parts, b->total_walls, s);
+    if (b->dense)
+        launch_rho_batch(b->idx, b->nodes_max, s);
+    else
+        launch_begin_batch(b->idx, s);
+    launch_shell_batch(b->storage, b->idx, b->dense, b->ext, b->total_parts, b->total_walls, s);
     launch_fused_batch(b->storage, b->idx, b->total_tiles, 152 * b->ctas_per_sm, b->general, s);
     if (b->total_parts > 0) {
         launch_link_batch(b->storage, b->idx, b->ext, b->total_parts, s);
@@ -1146,6 +1151,8 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         nodes += (double)c->L.N;
         if (!fused_tau1(c->L) || !fused_rel32(c->L)) b->general = true;
     }
+    b->dense = !fused_batch_self(b->storage, b->general);
+    b->nodes_max = b->members[0]->L.N;
     const int rows = fused_batch_rows(b->storage, b->general);
     int np_all = 0;
     for (lbe_ctx *c : b->members) np_all += c->np;
@@ -1158,8 +1165,8 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         d.ofs = fused_offsets(c->L);
         d.tma = c->tma ? 1 : 0;
         if (c->tma) {
-            d.tmap[0] = c->tmap[1][rows == 4 ? 1 : 0][0];  // ψ formed in the kernel
-            d.tmap[1] = c->tmap[1][rows == 4 ? 1 : 0][1];
+            // boxes with a halo where ψ is formed in the kernel
+            for (int k2 = 0; k2 < 2; k2++) d.tmap[k2] = c->tmap[b->dense ? 0 : 1][rows == 4 ? 1 : 0][k2];
         }
         d.f[0] = c->f[0];
         d.f[1] = c->f[1];
@@ -1174,7 +1181,7 @@ lbe_status lbe_batch_create(lbe_ctx *const *members, int32_t n, lbe_batch **out)
         d.mode = c->d.particle_mode;
         d.links = c->np > 0 ? c->ll : LinkList{nullptr, nullptr, 0};
         d.zc = c->zc_tuned > 0 ? c->zc_tuned
-                               : fused_zchunk(c->L, rows, (int)c->esize, true, (double)c->L.N / nodes);
+                               : fused_zchunk(c->L, rows, (int)c->esize, !b->dense, (double)c->L.N / nodes);
         d.ntx = (c->L.nx + FUSED_TX - 1) / FUSED_TX;
         d.nty = (c->L.ny + rows - 1) / rows;
         d.nzc = (c->L.nz + d.zc - 1) / d.zc;
@@ -1311,8 +1318,9 @@ lbe_status lbe_batch_first_quat(lbe_batch *b, double *quat_out)
 int32_t lbe_batch_kernels_per_step(const lbe_batch *b)
 {
     if (!b) return 0;
-    // the queue's reset, the fused kernel and the parity flip; the shell fill
-    // where there are solid nodes; seven particle kernels
+    // the queue's reset (by the density pass, where there is one), the fused
+    // kernel and the parity flip; the shell fill where there are solid nodes;
+    // seven particle kernels
     return 3 + (b->total_parts > 0 || b->total_walls > 0 ? 1 : 0) + (b->total_parts > 0 ? 7 : 0);
 }
 

@@ -381,9 +381,12 @@ int mass_blocks();
 
 // ---- batched launchers (one launch steps every box of a batch) -------------
 void launch_begin_batch(const BatchIndex &B, cudaStream_t s);
+// The density pass over all boxes (FP32), in the place of launch_begin_batch;
+// nodes_max: of the largest box.
+void launch_rho_batch(const BatchIndex &B, int nodes_max, cudaStream_t s);
 // ext: bound of the particle boxes of all members (batch_shell_extent).
-void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, int total_walls,
-                        cudaStream_t s);
+void launch_shell_batch(int storage, const BatchIndex &B, bool dense, const int ext[3], int total_parts,
+                        int total_walls, cudaStream_t s);
 int batch_wall_tiles(const Lat &L);
 void batch_shell_extent(const Lat &L, const Parts &P, int ext[3]);
 // general: some member needs any-τ or 64-bit offsets.
@@ -407,6 +410,14 @@ void launch_flip_batch(const BatchIndex &B, cudaStream_t s);
 constexpr int FUSED_TX = 32;
 // Tile rows of the batched kernel (general: see launch_fused_batch).
 constexpr int fused_batch_rows(int storage, bool general) { return storage == LBE_STORE_F32 && !general ? 4 : 8; }
+// Whether the batched kernel forms ψ itself.  The general kernel in FP32 reads
+// it from memory, with a density pass over all boxes: formed on chip, its one
+// stage holds the next plane by the time of the relaxation, which then reads
+// the populations again from L2, with two CTAs an SM.  tau = (0.8, 1.2), us a
+// step, on chip / from memory: 1 box of 32^3 17.5 / 15.4, 8 of 48^3 122 / 88, 4 of
+// 64^3 125 / 94 (with one ellipsoid each 196 / 166), 1 of 96^3 100 / 81, 4 of 128^3
+// 744 / 616.
+constexpr bool fused_batch_self(int storage, bool general) { return storage != LBE_STORE_F32 || !general; }
 constexpr int FUSED_WAIT_LIMIT = 1 << 22;
 // self: the kernel forms ψ of fluid nodes from the densities of the tile
 // and a one-node halo (psi then holds ψ of solid nodes only); otherwise psi

@@ -2053,7 +2053,7 @@ __global__ void __launch_bounds__(PT) k_shell_fill(Lat L, Parts P, ShellGrid sg,
 // Start of a batched step: the fused kernel's tile queue is empty again.
 __global__ void k_begin_batch(BatchIndex B) { *B.counter = 0; }
 
-template <class S>
+template <class S, bool DENSE>
 __global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, ShellRange range)
 {
     __shared__ ShellTile sm;
@@ -2066,7 +2066,7 @@ __global__ void __launch_bounds__(PT) k_shell_batch(BatchIndex B, ShellGrid sg, 
     const int cur = B.par[2 * b], ocur = B.par[2 * b + 1];
     const typename S::P *f = (const typename S::P *)bx.f[cur];
     if (part)
-        shell_tile<S, false>(bx.L, bx.P, g - off[b], c % nt, sg, f, bx.rho, bx.psi, bx.type, bx.owner[ocur], bx.links, sm);
+        shell_tile<S, DENSE>(bx.L, bx.P, g - off[b], c % nt, sg, f, bx.rho, bx.psi, bx.type, bx.owner[ocur], bx.links, sm);
     else
         wall_tile<S>(bx.L, g - off[b], f, bx.psi, bx.type, sm);
 }
@@ -2381,12 +2381,15 @@ int batch_wall_tiles(const Lat &L) { return wall_tiles(L); }
 
 void launch_begin_batch(const BatchIndex &B, cudaStream_t s) { k_begin_batch<<<1, 1, 0, s>>>(B); }
 
-void launch_shell_batch(int storage, const BatchIndex &B, const int ext[3], int total_parts, int total_walls,
-                        cudaStream_t s)
+void launch_shell_batch(int storage, const BatchIndex &B, bool dense, const int ext[3], int total_parts,
+                        int total_walls, cudaStream_t s)
 {
     const ShellGrid g = total_parts > 0 ? shell_grid(ext, total_parts) : ShellGrid{0, 0, 0, 1, 1, 1};
     shell_ranges(g, total_parts, total_walls, [&](unsigned ctas, ShellRange range) {
-        LBE_DISPATCH(storage, (k_shell_batch<S><<<ctas, PT, 0, s>>>(B, g, range)));
+        if (dense)
+            k_shell_batch<StF32, true><<<ctas, PT, 0, s>>>(B, g, range);
+        else
+            LBE_DISPATCH(storage, (k_shell_batch<S, false><<<ctas, PT, 0, s>>>(B, g, range)));
     });
 }
 

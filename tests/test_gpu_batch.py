@@ -151,6 +151,34 @@ def test_batch_mixing_rows_with_and_without_tensor_copies(storage):
     batch.close()
 
 
+@pytest.mark.parametrize("walls", [False, True])
+def test_general_fp32_batch_reads_psi_from_memory(walls):
+    """Any tau in FP32: the density pass and the fused kernel that reads psi from
+    memory, over boxes with and without tensor copies (edges 32, 27), of one node
+    thickness, and with particles; alone the lattices form psi on chip."""
+    def make():
+        out = []
+        for shape, count in (((32, 40, 24), 0), ((27, 20, 18), 1), ((9, 1, 5), 0), ((36, 30, 33), 2)):
+            g = lbe.Lattice(shape, W.random_phases(shape, 0.5, seed=40), g_br=0.1, tau=(0.8, 1.2), walls_z=walls,
+                            particle_mode="prescribed")
+            if count:
+                pos = [[9.2, 9.7, 8.9], [22.3, 16.1, 20.4]][:count]
+                g.add_particles(pos, [W.axis_tilt_quaternion(0.6, 0.3)] * count, 4.0, 2.5, 0.05,
+                                vel=[[0.05, -0.03, 0.02]] * count)
+            out.append(g)
+        return out
+
+    alone, mixed = make(), make()
+    batch = lbe.Batch(mixed)
+    assert batch.kernels_per_step() == 11
+    for g in alone:
+        g.step(25)
+    batch.step(25)
+    for a, b in zip(alone, mixed):
+        assert _equal(_state(a), _state(b))
+    batch.close()
+
+
 def test_batch_without_particles():
     a = [_spinodal(), _spinodal()]
     b = [_spinodal(), _spinodal()]
