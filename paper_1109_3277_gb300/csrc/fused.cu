@@ -11,16 +11,16 @@
 // four-slot ring of planes; the collision of plane z reads planes z-1, z
 // and z+1 of it.  Two configurations fill the ring:
 //  - ψ formed on chip (lattices with no or few particles, batches but those of
-//    any τ in FP32): the box also holds a one-node halo (x widened to 16-byte boundaries), and each
-//    thread sums the densities of its node and of at most one halo node, so ψ
-//    of the tile and its halo comes from the stage; halo nodes beyond the
-//    lattice edge wrap around and are read from global memory.  Solid nodes
-//    take their ψ from the shell fill; a variant for lattices without any
-//    has neither types nor masks.
+//    any τ in FP32): the box also holds a one-node halo (x widened to 16-byte
+//    boundaries), and each thread sums the densities of its node and of at
+//    most one halo node, so ψ of the tile and its halo comes from the stage;
+//    halo nodes beyond the lattice edge wrap around and are read from global
+//    memory.  Solid nodes take their ψ from the shell fill; a variant for
+//    lattices without any has neither types nor masks.
 //  - ψ from memory (lattices with many particles, FP32 batches of any τ): the
-//    density pass and the shell fill have written ψ of every node a fluid node sees.  The ring
-//    entries of plane z + 2 arrive by asynchronous copies issued before the
-//    collision of plane z and waited for after it.
+//    density pass and the shell fill have written ψ of every node a fluid node
+//    sees.  The ring entries of plane z + 2 arrive by asynchronous copies
+//    issued before the collision of plane z and waited for after it.
 //
 // With τ = 1 for both components the post-collision populations are the
 // equilibria, so a node's populations are needed only for its moments, and

@@ -390,7 +390,7 @@ struct PGeom2 {
 // (quaternion) are one instruction.  Every operation and its order are those
 // of the scalar formulas.  With one thread per particle the update and the
 // geometry took 19 + 23 us for a single particle and 39 + 45 us for 25,033;
-// as one kernel of quads 15 and 58 us.
+// as one kernel of quads 12 and 50 us.
 __device__ __forceinline__ double quad(double v, int l) { return __shfl_sync(0xffffffffu, v, l, 4); }
 
 // A vector given around axis k (its components k, k+1, k+2 cyclically) in
@@ -1728,7 +1728,7 @@ __global__ void __launch_bounds__(PT_WIDE) k_reset(Lat L, Parts P, int use_old, 
 // The kernel is bound by instruction issue: rows are handled by (plane: warp,
 // row: lane) without a division, and node lists are written out once instead
 // of a search per node.  512^3 Pickering, DENSE: 965 us with a search per node
-// and divisions, 658 now; before the masks 1,420.
+// and divisions, 700 now; before the masks 1,420.
 constexpr int SHELL_ITEMS = 1024;  // nodes of a list held at once, and densities held per tile
 constexpr int SHELL_X = 30;        // nodes of a tile along x: a mask word less the halo
 constexpr int SHELL_MAX = 22;      // rows of a tile along y and z
